@@ -427,8 +427,8 @@ int layout(Plan& P) {
     if (!e) e = P.d_gfile.ensure(ng * sizeof(int32_t));
     if (!e) e = P.d_seg0.ensure(nf * sizeof(uint64_t));
     if (!e) e = P.d_sym.ensure(P.sym_total * sizeof(uint16_t));
-    if (!e) e = P.d_tok.ensure((size_t)pass1_warps((int)nc, P.wpb) * token_words_per_part() * sizeof(uint32_t));
-    if (!e) e = P.d_queue.ensure(2 * sizeof(uint32_t));
+    if (!e) e = P.d_tok.ensure((size_t)pass1_warps((int)nc, P.wpb) * token_words_per_part() * sizeof(uint32_t) + 64);
+    if (!e) e = P.d_queue.ensure(3 * sizeof(uint32_t));
     if (!e) e = P.d_order.ensure(nc * sizeof(uint32_t));
     if (!e && P.chain) e = P.d_windows.ensure(nc * (size_t)kWin);
     if (!e && P.chain) e = P.d_gmaps.ensure(ng * (size_t)kWin * sizeof(uint16_t));
@@ -486,8 +486,10 @@ int enqueue(pgz_ctx* ctx, Plan& P, cudaStream_t s, bool timed, cudaStream_t up =
     launch_inflate(df, dc, (int)nc, sym, P.d_tok.as<uint32_t>(), P.d_queue.as<uint32_t>() + 1,
                    P.d_order.as<uint32_t>(), ctx->kp, s);
     if (cudaPeekAtLastError() != cudaSuccess) return PGZ_E_CUDA;
+    launch_exec(df, dc, (int)nc, sym, P.d_queue.as<uint32_t>() + 2, P.d_order.as<uint32_t>(), ctx->kp, s);
+    if (cudaPeekAtLastError() != cudaSuccess) return PGZ_E_CUDA;
     launch_plan(df, dc, (int)nf, s);
-    k += 3;
+    k += 4;
     if (timed) cudaEventRecord(ctx->ev[2], s);
     if (P.chain) {
         launch_chain(df, dc, (int)nf, (int)ng, P.d_g0.as<int32_t>(), P.d_gn.as<int32_t>(), P.d_gfile.as<int32_t>(),
@@ -1169,7 +1171,6 @@ int pgz_create(pgz_ctx** out, const pgz_config* cfg) {
     ctx->kp.max_block = cfg->max_block;
     ctx->kp.confirm_blocks = cfg->confirm_blocks;
     ctx->kp.wpb = cfg->warps_per_block ? cfg->warps_per_block : 4;
-    ctx->kp.pipe = cfg->exec_pipelined;
     ctx->kp.tail = cfg->determined_tail;
     upload_crc_tables();
     for (int k = 0; k < 8; ++k) cudaEventCreate(&ctx->ev[k]);
@@ -1730,7 +1731,6 @@ int pgz_set_tuning(pgz_ctx* ctx, uint64_t chunk_bytes, int warps_per_block, int 
     ctx->cfg.warps_per_block = warps_per_block;
     ctx->cfg.exec_pipelined = exec_pipelined;
     ctx->kp.wpb = warps_per_block;
-    ctx->kp.pipe = exec_pipelined;
     return PGZ_OK;
 }
 
@@ -2059,7 +2059,6 @@ int pgz_autotune(pgz_ctx* ctx, pgz_job* jobs, int n_jobs, const uint64_t* chunk_
                 ctx->cfg.warps_per_block = e.warps_per_block;
                 ctx->cfg.exec_pipelined = e.exec_pipelined;
                 ctx->kp.wpb = e.warps_per_block;
-                ctx->kp.pipe = e.exec_pipelined;
                 e.status = pgz_decompress_batch(ctx, n_jobs, jobs, nullptr);   // settles buffers and plan
                 for (int r = 0; r < reps && e.status == PGZ_OK; ++r) {
                     cudaEventRecord(ctx->ev[6], ctx->stream);
@@ -2087,7 +2086,6 @@ int pgz_autotune(pgz_ctx* ctx, pgz_job* jobs, int n_jobs, const uint64_t* chunk_
     ctx->cfg.warps_per_block = pick.warps_per_block;
     ctx->cfg.exec_pipelined = pick.exec_pipelined;
     ctx->kp.wpb = pick.warps_per_block;
-    ctx->kp.pipe = pick.exec_pipelined;
     if (best) *best = pick;
     return PGZ_OK;
 }

@@ -40,8 +40,7 @@ struct KParams {
     uint32_t max_block;
     int confirm_blocks;
     int wpb;               // warps per block of the pass-1 kernels: 2, 4 or 8 (0: 4)
-    int pipe;              // k_inflate executes tokens in pipelined passes (1) or one pass at a time (0)
-    int tail;              // k_inflate stores a part's determined tail as bytes (1) or keeps u16 symbols (0)
+    int tail;              // k_exec stores a part's determined tail as bytes (1) or keeps u16 symbols (0)
 };
 
 // one gzip member
@@ -115,13 +114,17 @@ struct ChunkDesc {
 
 // host-side launch wrappers (pgz_kernels.cu)
 // tok: token_words_per_part() u32 of parallel-block-decoder scratch for each of
-//      pass1_warps(nchunks, p.wpb) warps (at most nchunks rounded up to p.wpb);
+//      pass1_warps(nchunks, p.wpb) warps (at most nchunks rounded up to p.wpb), and 64 bytes after them (read
+//      ahead, not used);
 // queue: one u32 work counter per kernel (zeroed by the launcher on the stream);
 // order (nullable): the parts in the order the work queue hands them out (nchunks entries).
 void launch_sync(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* tok,
                  uint32_t* queue, const uint32_t* order, const KParams& p, cudaStream_t s);
 void launch_inflate(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* tok,
                     uint32_t* queue, const uint32_t* order, const KParams& p, cudaStream_t s);
+// the parts' copy maps (written by the two kernels above) into symbols, in place
+void launch_exec(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* queue,
+                 const uint32_t* order, const KParams& p, cudaStream_t s);
 uint64_t token_words_per_part();
 int pass1_warps(int nchunks, int wpb);
 void launch_plan(FileDesc* files, ChunkDesc* chunks, int nfiles, cudaStream_t s);

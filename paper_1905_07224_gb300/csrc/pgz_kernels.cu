@@ -8,16 +8,19 @@
 //               a warp tests 1024 bit offsets per step (one 32-bit window per
 //               lane, bit-parallel header tests), __ballot_sync + __ffs elect
 //               the lowest candidate, and the candidate's whole block is then
-//               decoded as the final check -- into the part's own output, so
+//               decoded as the final check -- into the part's own copy map, so
 //               pass 1 resumes after it.
-//   k_inflate   pass 1b: decode(C_i, w^_i) (Algorithm "DEFLATE decompression"
-//               with the symbolic context [U_0..U_32767]) up to the next
-//               part's block start.  One warp per part: the lanes decode
-//               segments of a block in parallel and meet (see par_block), then
-//               write the tokens' symbols cooperatively.  The 32 KiB window is
-//               the part's own u16 output in global memory; a source before
-//               the part start p < 0 is the placeholder U_{32768+p}, computed,
-//               not stored.
+//   k_inflate   pass 1b: the blocks of part i up to the next part's block
+//               start.  One warp per part: the lanes decode segments of a block
+//               in parallel and meet (see par_block), then write the tokens'
+//               copy map: per output position its byte, or the distance to its
+//               source.  No symbol is read, so no window is kept.
+//   k_exec      pass 1c: decode(C_i, w^_i) (Algorithm "DEFLATE decompression"
+//               with the symbolic context [U_0..U_32767]) finished from the
+//               copy map, in place: one block per part, the last 32 KiB of the
+//               part's symbols in shared memory.  A source before the part
+//               start p < 0 is the placeholder U_{32768+p}, computed, not
+//               stored.
 //   k_plan      output offsets of the parts (prefix of their lengths), error
 //               aggregation, ISIZE and capacity checks.
 //   k_chain_*   pass 2a: w_{i+1} from w_i and the tail of D_i (Section "Full
@@ -422,160 +425,36 @@ __device__ void build_fixed(WarpSmem& S, int lane) {
 }
 
 // ---------------------------------------------------------------------------
-// symbol output of one part
+// copy map of one part: what the block decoder writes, one u16 per output
+// position -- a byte (a literal), or kPH | (distance - 1) for a position inside
+// a match.  k_exec turns it into symbols in place.
 // ---------------------------------------------------------------------------
 struct OutState {
-    uint16_t* sym;     // the part's symbols; also its window
+    uint16_t* sym;     // the part's copy map
     uint64_t cap;
-    uint64_t n;        // symbols so far (uniform)
+    uint64_t n;        // positions so far (uniform)
     bool known;        // the context before the part is empty (member start)
-    bool neg;          // this lane copied from before the part start (a placeholder source)
-    // The determined tail (Section "Undetermined context propagation technique": a placeholder is only ever
-    // copied, so once the last 32 KiB of output hold none, no later symbol can be one): symbols from det on
-    // are stored as bytes, symbol k at byte det + k of the part's buffer (det is a multiple of 8, so a lane's
-    // 8 positions are all below it or all at or above it).  ~0: no tail yet.
-    uint32_t det = 0xffffffffu;
-    uint32_t last_ph = 0;   // at or after one past the last placeholder written (uniform; kept in kTail mode)
+    bool neg;          // a match of this lane reaches before the part start (a placeholder source)
 };
 
-__device__ __forceinline__ uint8_t* tail_bytes(const OutState& o) { return reinterpret_cast<uint8_t*>(o.sym) + o.det; }
-
-__device__ __forceinline__ void cp_async4(uint32_t dst_shared, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst_shared), "l"(src) : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// the symbol at part position q: q < 0 lies in the symbolic context.  Part
-// positions are 32-bit (a part holds fewer than 2^31 symbols).
-__device__ __forceinline__ uint16_t sym_at(const uint16_t* out, int32_t q) {
-    return q >= 0 ? out[(uint32_t)q] : (uint16_t)(kPH | (uint32_t)((int32_t)kWin + q));
-}
-// the same with the determined tail: a position at or after o.det is a byte
-__device__ __forceinline__ uint16_t sym_get(const OutState& o, int32_t q) {
-    if (q >= 0 && (uint32_t)q >= o.det) return tail_bytes(o)[(uint32_t)q];
-    return sym_at(o.sym, q);
-}
-// an upper bound on one past the part's last placeholder: the end of any pass of 256 positions (from A) that
-// wrote one (uniform)
-__device__ __forceinline__ void track_placeholders(OutState& o, const uint32_t* e, uint32_t A, uint32_t end) {
-    uint32_t any = 0;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) any |= e[u];
-    if (__any_sync(0xffffffffu, (any & kPH) != 0)) o.last_ph = max(o.last_ph, min(A + 256u, end));
-}
-
-// Writes the symbols of a batch of tokens (lane t holds token t < ntok):
-// token = (1 << 16) | byte for a literal, bit 31 | length << 16 | (distance-1)
-// for a match.  Output-parallel: lane j produces output positions j, j + 32,
-// ... of the batch.  A position inside a match follows the copy to its source;
-// a source inside the batch is resolved in registers (the covering token is
-// found by binary search over the tokens' starts, an overlapping copy folds
-// back by the distance), so only sources before the batch are loaded from the
-// part's output (or are placeholders U_j before the part start).  All loads of
-// up to 256 positions are issued before their stores.
-__device__ __forceinline__ int exec_batch(OutState& o, uint32_t tok, int ntok, int lane, uint64_t& block_n) {
-    const bool valid = lane < ntok;
-    const uint32_t len = valid ? ((tok >> 16) & 0x1ffu) : 0u;
-    uint32_t incl = len;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t t = __shfl_up_sync(FULL, incl, d);
-        if (lane >= d) incl += t;
-    }
-    const uint32_t total = __shfl_sync(FULL, incl, 31);
-    const uint32_t base = (uint32_t)o.n;
-    if ((uint64_t)base + total > o.cap) return CE_OVERFLOW;
-    const uint32_t st = incl - len;          // start of my token, relative to the batch
-    uint16_t* out = o.sym;
-    bool bad = false;
-    for (uint32_t r0 = 0; r0 < total; r0 += 256) {
-        uint32_t val[8];
-        int32_t src[8];
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            uint32_t rel = r0 + 32u * r + (uint32_t)lane;
-            bool need = rel < total;
-            val[r] = 0;
-            src[r] = INT32_MIN;
-            while (__any_sync(FULL, need)) {
-                int t = 0;
-#pragma unroll
-                for (int sft = 16; sft; sft >>= 1) {
-                    const uint32_t x = __shfl_sync(FULL, st, (t + sft) & 31);
-                    if (t + sft < ntok && x <= rel) t += sft;
-                }
-                const uint32_t tk = __shfl_sync(FULL, tok, t), sk = __shfl_sync(FULL, st, t);
-                if (need) {
-                    if (!(tk >> 31)) {
-                        val[r] = tk & 0xffu;
-                        need = false;
-                    } else {
-                        const uint32_t dk = (tk & 0xffffu) + 1u;
-                        int32_t q = (int32_t)rel - (int32_t)dk;
-                        if (q >= (int32_t)sk) q = (int32_t)sk - (int32_t)dk + (int32_t)((rel - sk) % dk);
-                        if (q < 0) {
-                            src[r] = (int32_t)base + q;     // before the batch: final, or a placeholder
-                            need = false;
-                        } else {
-                            rel = (uint32_t)q;
-                        }
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            if (src[r] != INT32_MIN) {
-                if (src[r] < 0) {
-                    if (o.known) bad = true;
-                    o.neg = true;
-                }
-                val[r] = sym_at(out, src[r]);
-            }
-        }
-        if (__any_sync(FULL, bad)) return CE_DIST;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            const uint32_t rel = r0 + 32u * r + (uint32_t)lane;
-            if (rel < total) out[base + rel] = (uint16_t)val[r];
-        }
-    }
-    __syncwarp();
-    o.n = base + total;
-    block_n += total;
-    return CE_OK;
-}
-
 __device__ __forceinline__ bool allowed_has(const uint32_t* a, uint32_t b) { return (a[b >> 5] >> (b & 31)) & 1u; }
 
-// Up to 32 tokens of a Huffman block; lane t keeps token t.  SAFE: every
-// word this batch can read lies inside the member (no bounds checks).
-template <bool SAFE, bool CHECK>
-__device__ __forceinline__ int decode_batch(WarpSmem& S, BitIn& br, int lane, uint32_t& mytok, int& ntok, bool& eob) {
+// The first tokens (about kTrialTokens) of a candidate's block, every lane
+// decoding the same bits: a false candidate fails after a few tokens, before
+// the whole block is decoded in parallel.  A prefix that reaches the end of
+// the block is left to the parallel decoder to judge.
+constexpr int kTrialTokens = 64;
+
+__device__ int trial_prefix(const WarpSmem& S, BitIn br, uint64_t end_bit) {
 #pragma unroll 1
-    while (ntok < 32) {
-        br.refill<SAFE>();
+    for (int ntok = 0; ntok < kTrialTokens; ++ntok) {
+        br.refill();
         uint32_t e = S.lit[br.lo & ((1u << LB) - 1u)];
         uint32_t k = e >> 28;
-        if (k <= K_LIT2) {
-            const uint32_t b = (e >> 8) & 0xffu;
-            if (k == K_LIT2 && ntok < 31) {
-                const uint32_t b2 = (e >> 16) & 0xffu;
-                if (CHECK && !(allowed_has(S.allowed, b) && allowed_has(S.allowed, b2))) return CE_BYTE;
-                br.drop(e & 31u);
-                if (lane == ntok) mytok = 0x10000u | b;
-                if (lane == ntok + 1) mytok = 0x10000u | b2;
-                ntok += 2;
-                continue;
-            }
-            if (CHECK && !allowed_has(S.allowed, b)) return CE_BYTE;
-            br.drop(k == K_LIT ? (e & 31u) : ((e >> 24) & 15u));
-            if (lane == ntok) mytok = 0x10000u | b;
-            ++ntok;
-            continue;
-        }
         if (k >= K_LONG) {
             uint32_t L = 0;
             const int s = k == K_LONG
@@ -585,68 +464,32 @@ __device__ __forceinline__ int decode_batch(WarpSmem& S, BitIn& br, int lane, ui
             e = lit_entry((uint32_t)s, L, 0);
             k = e >> 28;
             if (k == K_BAD) return CE_DATA;
-            if (k == K_LIT) {
-                const uint32_t b = (e >> 8) & 0xffu;
-                if (CHECK && !allowed_has(S.allowed, b)) return CE_BYTE;
-                br.drop(e & 31u);
-                if (lane == ntok) mytok = 0x10000u | b;
-                ++ntok;
-                continue;
-            }
         }
-        if (k == K_EOB) {
+        if (k <= K_LIT2) {
+            if (!allowed_has(S.allowed, (e >> 8) & 0xffu)) return CE_BYTE;
+            if (k == K_LIT2 && !allowed_has(S.allowed, (e >> 16) & 0xffu)) return CE_BYTE;
             br.drop(e & 31u);
-            eob = true;
+        } else if (k == K_EOB) {
             return CE_OK;
-        }
-        uint32_t len = (e >> 8) & 0x1ffu, dn = e & 31u;
-        if (k == K_LENX) {
-            const uint32_t eb = (e >> 17) & 7u;
-            len += (br.lo >> dn) & ((1u << eb) - 1u);
-            dn += eb;
-        }
-        br.drop(dn);
-        br.refill<SAFE>();
-        uint32_t d = S.dist[br.lo & ((1u << DB) - 1u)];
-        if (d & 0x300u) {
-            if ((d & 0x300u) != (DK_LONG << 8)) return CE_DATA;
-            uint32_t L = 0;
-            const int s = decode_long(br.peek(15), DB, S.dfirst, S.dcount, S.doff, S.dsym, (int)S.dmax, L);
-            if (s < 0) return CE_DATA;
-            d = dist_entry((uint32_t)s, L);
-            if (d & 0x300u) return CE_DATA;
-        }
-        const uint32_t dl = d & 15u, de = (d >> 4) & 15u;
-        const uint32_t dist = (d >> 16) + ((br.lo >> dl) & ((1u << de) - 1u));
-        br.drop(dl + de);
-        if (lane == ntok) mytok = 0x80000000u | (len << 16) | (dist - 1u);
-        ++ntok;
-    }
-    return CE_OK;
-}
-
-constexpr int CE_MORE = 100;   // internal: the token limit was reached inside the block
-
-__device__ int huff_block(WarpSmem& S, BitIn& br, OutState& o, bool check, uint64_t max_block, uint64_t end_bit,
-                          uint64_t& block_n, int lane, uint32_t tok_limit = 0) {
-    uint32_t done = 0;
-    for (;;) {
-        uint32_t mytok = 0;
-        int ntok = 0;
-        bool eob = false;
-        const int st = check ? decode_batch<false, true>(S, br, lane, mytok, ntok, eob)
-                             : decode_batch<false, false>(S, br, lane, mytok, ntok, eob);
-        if (st) return st;
-        if (ntok) {
-            const int e = exec_batch(o, mytok, ntok, lane, block_n);
-            if (e) return e;
+        } else {
+            uint32_t dn = e & 31u;
+            if (k == K_LENX) dn += (e >> 17) & 7u;
+            br.drop(dn);
+            br.refill();
+            uint32_t d = S.dist[br.lo & ((1u << DB) - 1u)];
+            if (d & 0x300u) {
+                if ((d & 0x300u) != (DK_LONG << 8)) return CE_DATA;
+                uint32_t L = 0;
+                const int s = decode_long(br.peek(15), DB, S.dfirst, S.dcount, S.doff, S.dsym, (int)S.dmax, L);
+                if (s < 0) return CE_DATA;
+                d = dist_entry((uint32_t)s, L);
+                if (d & 0x300u) return CE_DATA;
+            }
+            br.drop((d & 15u) + ((d >> 4) & 15u));
         }
         if (br.pos() > end_bit) return CE_TRUNC;
-        if (max_block && block_n >= max_block) return CE_SIZE;
-        if (eob) return CE_OK;
-        done += (uint32_t)ntok;
-        if (tok_limit && done >= tok_limit) return CE_MORE;
     }
+    return CE_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -666,6 +509,9 @@ constexpr uint32_t kSeg = 2048;      // bits per lane per round
 constexpr uint32_t kSyncW = 1024;    // bits at the head of a segment where meeting points are looked for
 constexpr uint32_t kTokCap = 512;    // tokens a lane may keep per round (own segment + continuation)
 constexpr uint64_t kTokPerPart = 32ull * kTokCap;   // token buffer of one part (one warp)
+
+// the output length of a token
+__device__ __forceinline__ uint32_t token_len(uint32_t t) { return (t >> 16) & 0x1ffu; }
 
 enum : int { LT_ONE = 0, LT_TWO = 1, LT_EOB = 2, LT_ERR = 3 };
 
@@ -738,7 +584,7 @@ __device__ __forceinline__ void mark(uint32_t& mw, uint32_t& mwi, uint32_t* m, u
 // own segment: tokens from `my0` while the token start lies before my0 + kSeg.
 // The loop runs in lock step over the warp (one token per lane per step).
 __device__ uint32_t seg_own(const WarpSmem& S, BitIn& b, uint64_t my0, uint32_t* m, uint32_t* tb, uint32_t& n,
-                            uint64_t& stop, uint32_t& ev) {
+                            uint32_t& out_len, uint64_t& stop, uint32_t& ev) {
     uint32_t mw = 0, mwi = 0;
     uint32_t st = PS_OK;
     const uint32_t p0 = (uint32_t)my0;
@@ -760,9 +606,11 @@ __device__ uint32_t seg_own(const WarpSmem& S, BitIn& b, uint64_t my0, uint32_t*
         const int r = lane_token<false>(S, b, t0, t1, l1);
         if (r <= LT_TWO) {
             tb[n++] = t0;
+            out_len += token_len(t0);
             if (r == LT_TWO) {
                 if (rel + l1 < kSyncW) mark(mw, mwi, m, rel + l1);
                 tb[n++] = t1;
+                ++out_len;
             }
         } else {
             st = r == LT_EOB ? PS_EOB : PS_ERR;
@@ -778,7 +626,7 @@ __device__ uint32_t seg_own(const WarpSmem& S, BitIn& b, uint64_t my0, uint32_t*
 // continuation into the next segment until the parse meets one of its token
 // starts (lock step; lanes with nothing to do idle)
 __device__ uint32_t seg_next(const WarpSmem& S, BitIn& b, bool active, uint64_t nx0, const uint32_t* nm, uint32_t* tb,
-                             uint32_t n, uint32_t& n2, uint64_t& q, uint32_t& ev) {
+                             uint32_t n, uint32_t& n2, uint32_t& out_len, uint64_t& q, uint32_t& ev) {
     const uint32_t p0 = (uint32_t)nx0;
     uint32_t st = PS_NOSYNC;
     bool go = active;
@@ -799,7 +647,11 @@ __device__ uint32_t seg_next(const WarpSmem& S, BitIn& b, bool active, uint64_t 
         const int r = lane_token<false>(S, b, t0, t1, l1);
         if (r <= LT_TWO) {
             tb[n + n2++] = t0;
-            if (r == LT_TWO) tb[n + n2++] = t1;
+            out_len += token_len(t0);
+            if (r == LT_TWO) {
+                tb[n + n2++] = t1;
+                ++out_len;
+            }
         } else {
             ev = n2;
             st = r == LT_EOB ? PS_EOB : PS_ERR;
@@ -810,346 +662,90 @@ __device__ uint32_t seg_next(const WarpSmem& S, BitIn& b, bool active, uint64_t 
     return st;
 }
 
-// Stage entries of exec_range: kEntryRes | symbol when resolved; else the
-// index of the source in the same pass, or kEntryCross | its index in the
-// previous pass.
-constexpr uint32_t kEntryRes = 0x10000u, kEntryCross = 0x20000u;
-
-struct PassMasks {
-    uint32_t am, hm, cm, om;   // bit u: async copy, its upper half, cross entry, open in-pass pointer
-    uint32_t neg;              // a source lies before the part start (a placeholder)
-    uint32_t bm, bx;           // bit u: the async copy holds a tail byte; bits 2u, 2u+1: its byte in the word
+// A lane's tokens read in order, four per 16-byte load, one load ahead.
+struct TokenReader {
+    const uint4* p;
+    uint4 q, nx;
+    uint32_t left;      // tokens of q not yet taken
+    __device__ __forceinline__ void begin(const uint32_t* tb, uint32_t x) {   // tb: 16-byte aligned
+        p = reinterpret_cast<const uint4*>(tb) + (x >> 2);
+        q = p[0];
+        nx = p[1];
+        p += 2;
+        left = 4;
+        for (uint32_t k = x & 3u; k; --k) shift();
+    }
+    __device__ __forceinline__ void shift() {
+        q.x = q.y;
+        q.y = q.z;
+        q.z = q.w;
+        --left;
+    }
+    __device__ __forceinline__ uint32_t next() {
+        const uint32_t t = q.x;
+        shift();
+        if (left == 0) {
+            q = nx;
+            nx = *p++;
+            left = 4;
+        }
+        return t;
+    }
 };
 
-// The entries of the pass at A (positions A + 8 lane .. + 7) into stage buffer
-// b; positions before fin are final in the part's output and are copied
-// asynchronously into their entries (the 32-bit word holding the symbol).
-template <bool TAIL>
-__device__ __forceinline__ PassMasks build_pass(uint32_t* masks, const uint32_t* tokS, const uint32_t* stS,
-                                                uint32_t ntok, uint32_t base, uint32_t end, const uint16_t* out,
-                                                uint32_t det, uint32_t A, uint32_t fin, int b, int lane) {
-    PassMasks m{0, 0, 0, 0, 0, 0, 0};
-    uint32_t* buf = masks + 256 * b;
-    const uint32_t p0 = A + 8u * (uint32_t)lane;
-    if (!(p0 + 8u > base && p0 < end)) {
-#pragma unroll
-        for (int u = 0; u < 8; ++u) buf[8u * lane + u] = kEntryRes;
-        return m;
-    }
-    const uint32_t sh = (uint32_t)__cvta_generic_to_shared(buf);
-    const uint32_t r0 = (p0 > base ? p0 : base) - base;
-    uint32_t lo = 0, hi = ntok - 1;                        // last token starting at or before r0
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi + 1) >> 1;
-        if (stS[mid] <= r0) lo = mid;
-        else hi = mid - 1;
-    }
-    uint32_t ti = lo;
-    uint32_t next = ti + 1 < ntok ? stS[ti + 1] : 0xffffffffu;
-    uint32_t tk = tokS[ti];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-        const uint32_t P = p0 + (uint32_t)u;
-        const uint32_t slot = 8u * lane + u;
-        if (P < base || P >= end) {
-            buf[slot] = kEntryRes;
-            continue;
-        }
-        if (P - base >= next) {                            // the next token (tokens are at least 1 long)
-            ++ti;
-            next = ti + 1 < ntok ? stS[ti + 1] : 0xffffffffu;
-            tk = tokS[ti];
-        }
-        if (!(tk >> 31)) {
-            buf[slot] = kEntryRes | (tk & 0xffu);
-            continue;
-        }
-        const int32_t src = (int32_t)P - (int32_t)((tk & 0xffffu) + 1u);
-        if (src < 0) {                                     // a placeholder U_j before the part start
-            m.neg = 1;
-            buf[slot] = kEntryRes | sym_at(out, src);
-        } else if ((uint32_t)src < fin) {                  // final: copy its word into the entry
-            if (TAIL && (uint32_t)src >= det) {            // a byte of the determined tail
-                const uint32_t bo = det + (uint32_t)src;
-                cp_async4(sh + 4u * slot, reinterpret_cast<const uint8_t*>(out) + (bo & ~3u));
-                m.bm |= 1u << u;
-                m.bx |= (bo & 3u) << (2 * u);
-            } else {
-                cp_async4(sh + 4u * slot, reinterpret_cast<const uint32_t*>(out) + ((uint32_t)src >> 1));
-                m.hm |= ((uint32_t)src & 1u) << u;
-            }
-            m.am |= 1u << u;
-        } else if ((uint32_t)src < A) {                    // inside the previous pass
-            buf[slot] = kEntryCross | ((uint32_t)src - (A - 256u));
-            m.cm |= 1u << u;
-        } else {                                           // inside this pass
-            buf[slot] = (uint32_t)src - A;
-            m.om |= 1u << u;
-        }
-    }
-    return m;
-}
-
-// Execution modes of a part's blocks: kPlain, u16 symbols only; kTail, with the determined tail: an upper
-// bound on the part's last placeholder is kept, and positions at or after OutState::det (once set) are
-// bytes.  Two instantiations keep the tail's checks out of the plain decoding loop; one instantiation serves
-// every block of the tail option, so warps in different parts run the same code.
-enum : int { kPlain = 0, kTail = 1 };
-
-// A lane's 8 resolved entries (positions p0 .. p0 + 7; the low 16 bits are the symbols) into the part's
-// output, the positions inside [base, end) only: one 16-byte store of u16 symbols, or one 8-byte store of
-// bytes in the determined tail.
-template <bool TAIL>
-__device__ __forceinline__ void store8(const OutState& o, uint16_t* out, const uint32_t* e, uint32_t p0, uint32_t base,
-                                       uint32_t end) {
-    const bool all = p0 >= base && p0 + 8u <= end;
-    if (TAIL && p0 >= o.det) {
-        uint8_t* t = tail_bytes(o);
-        if (all) {
-            uint2 v;
-            v.x = (e[0] & 0xffu) | ((e[1] & 0xffu) << 8) | ((e[2] & 0xffu) << 16) | (e[3] << 24);
-            v.y = (e[4] & 0xffu) | ((e[5] & 0xffu) << 8) | ((e[6] & 0xffu) << 16) | (e[7] << 24);
-            *reinterpret_cast<uint2*>(t + p0) = v;
+// Writes the copy map of a lane's tokens [x, xe) from position `at` on: whole
+// aligned words of four positions leave as one 8-byte store; the positions of
+// the first and last word, which other lanes share, leave one by one.
+// Returns false if (check) a literal is not an allowed byte.
+__device__ __forceinline__ bool expand_tokens(const WarpSmem& S, const uint32_t* tb, uint32_t x, uint32_t xe,
+                                              uint16_t* out, uint32_t at, bool check, bool& neg) {
+    if (x >= xe) return true;
+    TokenReader rd;
+    rd.begin(tb, x);
+    bool ok = true;
+    uint64_t acc = 0;
+    uint32_t pos = at;                   // next position
+    uint32_t fill = at & 3u;             // positions of the current word before `pos`
+    uint32_t skip = fill;                // positions of the current word that are not this lane's
+    uint64_t* w = reinterpret_cast<uint64_t*>(out + (at & ~3u));
+    auto flush = [&]() {                 // the current word is full
+        if (skip) {
+            uint16_t* h = reinterpret_cast<uint16_t*>(w);
+            for (uint32_t k = skip; k < 4; ++k) h[k] = (uint16_t)(acc >> (16 * k));
+            skip = 0;
         } else {
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const uint32_t P = p0 + (uint32_t)u;
-                if (P >= base && P < end) t[P] = (uint8_t)e[u];
-            }
+            *w = acc;
         }
-    } else if (all) {
-        uint4 v;
-        v.x = (e[0] & 0xffffu) | (e[1] << 16);
-        v.y = (e[2] & 0xffffu) | (e[3] << 16);
-        v.z = (e[4] & 0xffffu) | (e[5] << 16);
-        v.w = (e[6] & 0xffffu) | (e[7] << 16);
-        *reinterpret_cast<uint4*>(out + p0) = v;
-    } else {
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const uint32_t P = p0 + (uint32_t)u;
-            if (P >= base && P < end) out[P] = (uint16_t)e[u];
+        ++w;
+    };
+    for (; x < xe; ++x) {
+        const uint32_t t = rd.next();
+        uint32_t len = 1, v = t & 0xffu;
+        if (t >> 31) {
+            len = token_len(t);
+            v = kPH | (t & 0x7fffu);
+            neg |= pos <= (t & 0x7fffu);
+        } else if (check) {
+            ok &= allowed_has(S.allowed, v);
         }
+        pos += len;
+        const uint32_t v2 = v | (v << 16);
+        const uint64_t v4 = (uint64_t)v2 | ((uint64_t)v2 << 32);
+        acc |= v4 << (16 * fill);
+        uint32_t end = fill + len;
+        while (end >= 4) {
+            flush();
+            acc = v4;
+            end -= 4;
+        }
+        fill = end;
+        acc &= (1ull << (16 * fill)) - 1ull;
     }
+    uint16_t* h = reinterpret_cast<uint16_t*>(w);
+    for (uint32_t k = skip; k < fill; ++k) h[k] = (uint16_t)(acc >> (16 * k));
+    return ok;
 }
 
-// Writes up to 256 consecutive tokens of the block (lane j loads tokens
-// 8j..8j+7).  Output positions go in passes of 256, lane l taking 8
-// consecutive ones (one 16-byte store); a position inside a match takes its
-// source: a source before the pass (the part's output so far,
-// or a placeholder U_j before the part start) is loaded; a source inside the
-// pass is resolved by pointer jumping over the pass's entries in shared memory
-// (overlapping copies included, with no division).
-// PIPE: the passes are pipelined (the next pass's final sources copied
-// asynchronously while a pass resolves); else one pass at a time with direct
-// loads.  k_sync always takes the second (its block-start search leaves fewer
-// registers); k_inflate takes either (KParams::pipe): which is faster depends
-// on the data (how far back the sources lie), so the autotuner can choose.
-template <bool PIPE, int MODE>
-__device__ __forceinline__ int exec_range(WarpSmem& S, OutState& o, const uint32_t* tks, uint32_t ntok, bool check,
-                                          uint64_t& block_n, int lane) {
-    uint32_t t[8], L[8], sum = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const uint32_t idx = 8u * lane + i;
-        t[i] = idx < ntok ? tks[idx] : 0u;
-        L[i] = idx < ntok ? ((t[i] >> 16) & 0x1ffu) : 0u;
-        sum += L[i];
-    }
-    uint32_t incl = sum;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t x = __shfl_up_sync(FULL, incl, d);
-        if (lane >= d) incl += x;
-    }
-    const uint32_t total = __shfl_sync(FULL, incl, 31);
-    const uint32_t base = (uint32_t)o.n;
-    if ((uint64_t)base + total > o.cap) return CE_OVERFLOW;
-    if (check) {
-        bool bad = false;
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            if (L[i] && !(t[i] >> 31) && !allowed_has(S.allowed, t[i] & 0xffu)) bad = true;
-        if (__any_sync(FULL, bad)) return CE_BYTE;
-    }
-    if (total == 0) return CE_OK;
-    uint32_t* tokS = S.masks + 512;                        // the batch's tokens
-    uint32_t* stS = S.masks + 768;                         // their output offsets from base
-    uint32_t s0 = incl - sum;
-    uint16_t* out = o.sym;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const uint32_t idx = 8u * lane + i;
-        if (idx < ntok) {
-            tokS[idx] = t[i];
-            stS[idx] = s0;
-            // a match's source before the batch is final already: bring its line toward L2 now, so the
-            // passes below find it there
-            const int32_t src = (int32_t)(base + s0) - (int32_t)((t[i] & 0xffffu) + 1u);
-            if ((t[i] >> 31) && src >= 0 && (uint32_t)src < base) {
-                const void* a = (MODE == kTail && (uint32_t)src >= o.det) ? (const void*)(tail_bytes(o) + src)
-                                                                         : (const void*)(out + src);
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
-            }
-        }
-        s0 += L[i];
-    }
-    __syncwarp();
-    bool bad = false;
-    const uint32_t end = base + total;
-    if constexpr (PIPE) {
-    // Passes over [A, A + 256) with A a multiple of 8; lane l takes positions A + 8l .. A + 8l + 7.  A pass's
-    // entries live in one of two stage buffers of 256 words: kRes | symbol when resolved, else the index of
-    // the source inside the same pass (strictly earlier), or kCross | index of the source in the previous
-    // pass.  While pass j is resolved, pass j + 1 is built: each of its sources that is final already (before
-    // pass j: earlier passes and batches) is copied asynchronously -- the 32-bit word holding the symbol,
-    // straight into the source's entry -- so those loads overlap pass j's work.  Pointer jumping (each entry
-    // replaced by the entry it points to) then resolves a pass; its successor's cross entries are read from
-    // it next, before its buffer is reused.
-    constexpr uint32_t kRes = kEntryRes;
-    int cur = 0;
-    uint32_t A = base & ~7u;
-    const uint32_t det = o.det;
-    PassMasks m = build_pass<MODE == kTail>(S.masks, tokS, stS, ntok, base, end, out, det, A, base, cur, lane);
-    uint32_t neg = m.neg;
-    cp_async_commit();
-    for (;;) {
-        const uint32_t A1 = A + 256u;
-        const bool more = A1 < end;
-        PassMasks m1{0, 0, 0, 0, 0, 0, 0};
-        if (more)
-            m1 = build_pass<MODE == kTail>(S.masks, tokS, stS, ntok, base, end, out, det, A1, A > base ? A : base,
-                                           cur ^ 1, lane);
-        neg |= m1.neg;
-        cp_async_commit();
-        cp_async_wait<1>();                                // this pass's copies (this lane's) have landed
-        uint32_t* buf = S.masks + 256 * cur;
-        const uint32_t p0 = A + 8u * (uint32_t)lane;
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if ((m.am >> u) & 1u) {
-                const uint32_t w = buf[8u * lane + u];
-                const uint32_t v = (MODE == kTail && ((m.bm >> u) & 1u))
-                                       ? ((w >> (8u * ((m.bx >> (2 * u)) & 3u))) & 0xffu)
-                                       : (((m.hm >> u) & 1u) ? (w >> 16) : (w & 0xffffu));
-                buf[8u * lane + u] = kRes | v;
-            }
-        __syncwarp();
-        uint32_t e[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) e[u] = buf[8u * lane + u];
-        uint32_t open = m.om;
-        while (__any_sync(FULL, open != 0)) {
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if ((open >> u) & 1u) e[u] = buf[e[u]];
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if ((open >> u) & 1u) {
-                    buf[8u * lane + u] = e[u];
-                    if (e[u] & kRes) open &= ~(1u << u);
-                }
-            __syncwarp();
-        }
-        if (more) {                                        // the next pass's sources in this one
-            uint32_t* nb = S.masks + 256 * (cur ^ 1);
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if ((m1.cm >> u) & 1u) nb[8u * lane + u] = buf[nb[8u * lane + u] & 0xffu];
-        }
-        store8<MODE == kTail>(o, out, e, p0, base, end);
-        if (MODE == kTail && o.det == 0xffffffffu) track_placeholders(o, e, A, end);
-        __syncwarp();                                      // this pass is final; its buffer may be reused
-        if (!more) break;
-        A = A1;
-        cur ^= 1;
-        m = m1;
-    }
-    cp_async_wait<0>();
-    if (neg) {
-        o.neg = true;
-        if (o.known) bad = true;
-    }
-    } else {
-    uint32_t* stage = S.masks;                             // 256 entries: the positions of one pass
-    // passes over [A, A + 256) with A a multiple of 8; lane l takes positions A + 8l .. A + 8l + 7.  A source
-    // before max(A, base) is final (earlier passes, earlier batches, or a placeholder before the part start)
-    // and is loaded; a source inside the pass is a pointer to its stage entry, strictly earlier, so pointer
-    // jumping (each entry replaced by the entry it points to) ends with every entry a symbol.  An entry is
-    // 0x10000 | symbol when resolved, else the pass index of its source.
-    for (uint32_t A = base & ~7u; A < end; A += 256u) {
-        const uint32_t p0 = A + 8u * (uint32_t)lane;
-        const uint32_t lo_pos = A > base ? A : base;       // first position of the pass that is this batch's
-        uint32_t e[8];
-        uint32_t open = 0;                                 // bit u: e[u] still a pointer
-        if (p0 + 8u > base && p0 < end) {
-            const uint32_t r0 = (p0 > base ? p0 : base) - base;
-            uint32_t lo = 0, hi = ntok - 1;                // last token starting at or before r0
-            while (lo < hi) {
-                const uint32_t mid = (lo + hi + 1) >> 1;
-                if (stS[mid] <= r0) lo = mid;
-                else hi = mid - 1;
-            }
-            uint32_t ti = lo;
-            uint32_t next = ti + 1 < ntok ? stS[ti + 1] : 0xffffffffu;
-            uint32_t tk = tokS[ti];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const uint32_t P = p0 + (uint32_t)u;
-                e[u] = 0x10000u;
-                if (P < base || P >= end) continue;
-                if (P - base >= next) {                    // the next token (tokens are at least 1 long)
-                    ++ti;
-                    next = ti + 1 < ntok ? stS[ti + 1] : 0xffffffffu;
-                    tk = tokS[ti];
-                }
-                if (!(tk >> 31)) {
-                    e[u] = 0x10000u | (tk & 0xffu);
-                    continue;
-                }
-                const int32_t src = (int32_t)P - (int32_t)((tk & 0xffffu) + 1u);
-                if (src < (int32_t)lo_pos) {
-                    if (src < 0) {
-                        if (o.known) bad = true;
-                        o.neg = true;
-                    }
-                    e[u] = 0x10000u | (MODE == kTail ? sym_get(o, src) : sym_at(out, src));
-                } else {
-                    e[u] = (uint32_t)src - A;
-                    open |= 1u << u;
-                }
-            }
-        } else {
-#pragma unroll
-            for (int u = 0; u < 8; ++u) e[u] = 0x10000u;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) stage[8u * lane + u] = e[u];
-        __syncwarp();
-        while (__any_sync(FULL, open != 0)) {
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if ((open >> u) & 1u) e[u] = stage[e[u]];
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if ((open >> u) & 1u) {
-                    stage[8u * lane + u] = e[u];
-                    if (e[u] & 0x10000u) open &= ~(1u << u);
-                }
-            __syncwarp();
-        }
-        store8<MODE == kTail>(o, out, e, p0, base, end);
-        if (MODE == kTail && o.det == 0xffffffffu) track_placeholders(o, e, A, end);
-        __syncwarp();                                      // this pass is final for the next one
-    }
-    }
-    if (__any_sync(FULL, bad)) return CE_DIST;
-    o.n = base + total;
-    block_n += total;
-    return CE_OK;
-}
-
-template <bool PIPE, int MODE>
 __device__ int par_block(WarpSmem& S, uint32_t* tokbuf, BitIn& br, OutState& o, bool check, uint64_t max_block,
                          uint64_t end_bit, uint64_t& block_n, int lane) {
     uint32_t* tb = tokbuf + (uint64_t)lane * kTokCap;
@@ -1166,12 +762,12 @@ __device__ int par_block(WarpSmem& S, uint32_t* tokbuf, BitIn& br, OutState& o, 
         }
         BitIn b = br;
         b.seek(my0);
-        uint32_t n = 0, ev1 = 0, ev2 = 0, n2 = 0;
+        uint32_t n = 0, ev1 = 0, ev2 = 0, n2 = 0, olen = 0;
         uint64_t stop = 0, q = 0;
-        const uint32_t st1 = seg_own(S, b, my0, mymask, tb, n, stop, ev1);
+        const uint32_t st1 = seg_own(S, b, my0, mymask, tb, n, olen, stop, ev1);
         __syncwarp();
         const uint32_t st2 = seg_next(S, b, st1 == PS_OK && lane < 31, my0 + kSeg, S.masks + 32 * ((lane + 1) & 31), tb,
-                                      n, n2, q, ev2);
+                                      n, n2, olen, q, ev2);
         __syncwarp();
         // the chain of meeting points, lane by lane (uniform)
         uint32_t skip = 0, my_vs = 0, my_ve = 0;
@@ -1233,16 +829,33 @@ __device__ int par_block(WarpSmem& S, uint32_t* tokbuf, BitIn& br, OutState& o, 
             break;
         }
         if (err) return err;
-        // the block's tokens of this round, in order: lane ranges one after another
-        for (int k = 0; k <= last; ++k) {
-            const uint32_t vs = __shfl_sync(FULL, my_vs, k), ve = __shfl_sync(FULL, my_ve, k);
-            const uint32_t* rng = tokbuf + (uint64_t)k * kTokCap;
-            for (uint32_t x = vs; x < ve; x += 256) {
-                const int e = exec_range<PIPE, MODE>(S, o, rng + x, ve - x < 256 ? ve - x : 256, check, block_n, lane);
-                if (e) return e;
-                if (max_block && block_n >= max_block) return CE_SIZE;
+        // the block's tokens of this round are the lane ranges [my_vs, my_ve) one after another (a lane's kept
+        // tokens end where its parse ends); each lane writes the copy map of its own
+        uint32_t len = 0;
+        if (lane <= last && my_vs < my_ve) {
+            len = olen;
+            if (my_vs) {
+                TokenReader rd;
+                rd.begin(tb, 0);
+                for (uint32_t x = 0; x < my_vs; ++x) len -= token_len(rd.next());
             }
         }
+        uint32_t incl = len;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t x = __shfl_up_sync(FULL, incl, d);
+            if (lane >= d) incl += x;
+        }
+        const uint32_t total = __shfl_sync(FULL, incl, 31);
+        if (max_block && block_n + total >= max_block) return CE_SIZE;
+        if (o.n + total > o.cap) return CE_OVERFLOW;
+        bool neg = false;
+        const bool ok = lane > last || expand_tokens(S, tb, my_vs, my_ve, o.sym, (uint32_t)o.n + incl - len, check, neg);
+        o.neg |= neg;
+        if (__any_sync(FULL, !ok)) return CE_BYTE;
+        if (o.known && __any_sync(FULL, neg)) return CE_DIST;
+        o.n += total;
+        block_n += total;
         __syncwarp();
         if (round_end > end_bit) return CE_TRUNC;
         br.seek(round_end);
@@ -1265,9 +878,7 @@ __device__ int stored_block(BitIn& br, OutState& o, bool check, const uint32_t* 
     for (uint32_t j = lane; j < len; j += 32) {
         const uint32_t v = __ldg(g + byte + 4 + j);
         if (check && !allowed_has(allowed, v)) bad = true;
-        const uint64_t P = o.n + j;
-        if (P >= o.det) tail_bytes(o)[P] = (uint8_t)v;
-        else o.sym[P] = (uint16_t)v;
+        o.sym[o.n + j] = (uint16_t)v;
     }
     if (__any_sync(FULL, bad)) return CE_BYTE;
     o.n += len;
@@ -1282,7 +893,6 @@ __device__ int stored_block(BitIn& br, OutState& o, bool check, const uint32_t* 
 // be allowed bytes.  Huffman blocks are decoded by the whole warp in parallel
 // (par_block); a candidate block start first runs a short serial prefix, so
 // that false candidates fail after a few tokens.
-template <bool PIPE, int MODE = kPlain>
 __device__ int one_block(WarpSmem& S, uint32_t* tokbuf, BitIn& br, OutState& o, bool check, uint64_t min_block,
                          uint64_t max_block, bool candidate, uint64_t end_bit, uint32_t& final, int lane) {
     br.refill();
@@ -1308,14 +918,8 @@ __device__ int one_block(WarpSmem& S, uint32_t* tokbuf, BitIn& br, OutState& o, 
             st = read_dynamic<false>(S, br, lane);
             if (st == CE_OK && br.pos() > end_bit) st = CE_TRUNC;
         }
-        if (st == CE_OK && candidate) {
-            st = huff_block(S, br, o, check, max_block, end_bit, block_n, lane, 64);
-            st = st == CE_MORE ? CE_MORE : (st == CE_OK ? CE_OK + 1000 : st);
-        }
-        if (st == CE_OK || st == CE_MORE)
-            st = par_block<PIPE, MODE>(S, tokbuf, br, o, check, max_block, end_bit, block_n, lane);
-        else if (st == CE_OK + 1000)
-            st = CE_OK;
+        if (st == CE_OK && candidate) st = trial_prefix(S, br, end_bit);
+        if (st == CE_OK) st = par_block(S, tokbuf, br, o, check, max_block, end_bit, block_n, lane);
     }
     if (st == CE_OK && max_block && block_n >= max_block) st = CE_SIZE;
     if (st == CE_OK && block_n < min_block) st = CE_SIZE;
@@ -1585,7 +1189,7 @@ __device__ void sync_part(const uint16_t* kraft3, WarpSmem& S, uint32_t* tok, co
         state = CS_EMPTY;
     } else if (o.known || C.given) {          // the member start (empty context) or a known block start
         br.seek(C.lo);
-        const int st = one_block<false>(S, tok, br, o, false, 0, 0, false, F.end_bit, final, lane);
+        const int st = one_block(S, tok, br, o, false, 0, 0, false, F.end_bit, final, lane);
         sync = C.lo;
         resume = br.pos();
         if (st) {
@@ -1603,7 +1207,7 @@ __device__ void sync_part(const uint16_t* kraft3, WarpSmem& S, uint32_t* tok, co
             br.seek(cand);
             o.n = 0;
             o.neg = false;
-            const int st = one_block<false>(S, tok, br, o, true, p.min_block, p.max_block, true, F.end_bit, final,
+            const int st = one_block(S, tok, br, o, true, p.min_block, p.max_block, true, F.end_bit, final,
                                             lane);
             if (st == CE_OK) {
                 state = CS_FOUND;
@@ -1626,8 +1230,7 @@ __device__ void sync_part(const uint16_t* kraft3, WarpSmem& S, uint32_t* tok, co
         C.resume = resume;
         C.n = state == CS_FOUND ? o.n : 0;
         C.nph = 0;
-        // a bound on one past the last placeholder: the first block's end (the member start has none)
-        C.last_ph = (state == CS_FOUND && !o.known) ? o.n : 0;
+        C.last_ph = 0;
         C.det = kNone;
         C.anyph = neg && state == CS_FOUND;
         C.blocks = state == CS_FOUND ? 1u : 0u;
@@ -1651,7 +1254,6 @@ __device__ __forceinline__ uint64_t find_stop(const FileDesc& F, const ChunkDesc
 }
 
 // Pass 1 of part c from the end of its first block up to the next part's block start.
-template <bool PIPE>
 __device__ void inflate_part(WarpSmem& S, uint32_t* tok, const FileDesc* __restrict__ files, ChunkDesc* chunks, int c,
                              uint16_t* symbuf, const KParams& p, int lane) {
     ChunkDesc& C = chunks[c];
@@ -1672,11 +1274,6 @@ __device__ void inflate_part(WarpSmem& S, uint32_t* tok, const FileDesc* __restr
     const FileDesc& F = files[C.file];
     const uint64_t stop = find_stop(F, chunks, c, C.stop_hint);
     OutState o{symbuf + C.sym_base, C.cap, C.n, C.index == 0 && C.sync == F.s0_bit, false};
-    o.det = C.det == kNone ? 0xffffffffu : (uint32_t)C.det;
-    o.last_ph = (uint32_t)C.last_ph;
-    // the determined tail when the configuration asks for it; decoding from a bit offset keeps every symbol
-    // as u16 (its caller asks for the symbols themselves)
-    const bool tail_ok = p.tail && F.mode != 1;
     uint32_t blocks = C.blocks, final = C.final, err = CE_OK, confirmed = C.confirmed;
     uint64_t end = C.resume;
     // the confirmation (Section "Detection of DEFLATE block start positions") covers the start's block and
@@ -1707,13 +1304,9 @@ __device__ void inflate_part(WarpSmem& S, uint32_t* tok, const FileDesc* __restr
                 end_stop = pos;
             }
             if (past && blocks >= window) break;
-            // no placeholder among the last 32 KiB: none can follow; the rest goes out as bytes
-            if (tail_ok && !past && o.det == 0xffffffffu && o.n >= (uint64_t)o.last_ph + kWin)
-                o.det = (uint32_t)((o.n + 7) & ~7ull);
             const bool check = !o.known && blocks < window;
             uint32_t fin = 0;
-            const int st = tail_ok ? one_block<PIPE, kTail>(S, tok, br, o, check, 0, 0, false, F.end_bit, fin, lane)
-                                   : one_block<PIPE, kPlain>(S, tok, br, o, check, 0, 0, false, F.end_bit, fin, lane);
+            const int st = one_block(S, tok, br, o, check, 0, 0, false, F.end_bit, fin, lane);
             if (st) {
                 err = (check && st != CE_OVERFLOW) ? (uint32_t)CE_CONFIRM : (uint32_t)st;
                 break;
@@ -1750,8 +1343,6 @@ __device__ void inflate_part(WarpSmem& S, uint32_t* tok, const FileDesc* __restr
         C.final = final;
         C.confirmed = confirmed;
         C.end = end;
-        C.last_ph = o.last_ph;
-        C.det = o.det < o.n ? (uint64_t)o.det : kNone;
     }
     __syncwarp();
 }
@@ -1776,7 +1367,7 @@ __global__ void __launch_bounds__(32 * WPB, pass1_min_blocks(WPB))
     }
 }
 
-template <int WPB, bool PIPE>
+template <int WPB>
 __global__ void __launch_bounds__(32 * WPB, pass1_min_blocks(WPB))
     k_inflate(const FileDesc* __restrict__ files, ChunkDesc* chunks, int nchunks, uint16_t* symbuf, uint32_t* tokbuf,
               uint32_t* queue, const uint32_t* __restrict__ order, KParams p) {
@@ -1787,7 +1378,129 @@ __global__ void __launch_bounds__(32 * WPB, pass1_min_blocks(WPB))
         const int q = next_part(queue, lane);
         if (q >= nchunks) return;
         const int c = order ? (int)__ldg(order + q) : q;
-        inflate_part<PIPE>(S, tok, files, chunks, c, symbuf, p, lane);
+        inflate_part(S, tok, files, chunks, c, symbuf, p, lane);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// k_exec: the copy map of each part into its symbols, in place
+// ---------------------------------------------------------------------------
+// One block of NT threads per part, in passes of 8 NT positions (a thread takes
+// 8 consecutive ones: one 16-byte load, one 16-byte store).  The last 32 KiB of
+// the part's symbols and the pass itself live in a ring in shared memory
+// (32768 + 8 NT u16 entries, so that a pass never overwrites a source it can
+// still need).  A position's entry is its symbol when the source lies before the
+// pass (read from the ring; U_j when it lies before the part), else kPtr | the
+// source's index inside the pass.  After one barrier every thread follows its
+// own pointers; each step shortens the chain the next reader follows (an entry
+// is replaced by the entry it points to), an entry only ever changes to an
+// earlier source or to its symbol, and indices strictly decrease, so the chase
+// needs no further barrier and ends, overlapping copies included.
+// Bound: shared-memory latency and the two barriers of a pass.  1.00 ms for the 1024 parts of a 256 MiB file
+// (268 G symbols/s; the map is read and the symbols written once, 1.1 TB/s), 0.064 ms for 8 parts of 128 K
+// symbols.  A warp that executed its tokens out of the part's output in L2 (one kernel for decoding and
+// executing) took 8.5 ms for the block starts and decoding of the same file, against 4.5 ms for decoding to
+// a map and 1.0 ms here.
+constexpr uint32_t kPtr = 0x4000u;    // neither a byte nor a placeholder; the index takes 14 bits
+
+template <int NT>
+constexpr size_t exec_smem() { return (kWin + 8 * NT) * sizeof(uint16_t); }
+
+template <int NT>
+__global__ void __launch_bounds__(NT, NT == 1024 ? 1 : (NT == 512 ? 2 : 3))
+    k_exec(const FileDesc* __restrict__ files, ChunkDesc* chunks, int nchunks, uint16_t* symbuf, uint32_t* queue,
+           const uint32_t* __restrict__ order, int tail) {
+    extern __shared__ __align__(16) uint16_t ring[];
+    __shared__ int s_q;
+    constexpr uint32_t P = 8 * NT, R = kWin + P;
+    static_assert(R % P == 0 && P <= kPtr, "whole passes in the ring, indices in 14 bits");
+    const uint32_t t8 = 8u * threadIdx.x;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_q = (int)min(atomicAdd(queue, 1u), 0x7fffffffu);
+        __syncthreads();
+        const int q = s_q;
+        if (q >= nchunks) return;
+        ChunkDesc& C = chunks[order ? (int)__ldg(order + q) : q];
+        if (C.state != CS_DONE || C.n == 0) continue;
+        const uint32_t n = (uint32_t)C.n;
+        uint16_t* sym = symbuf + C.sym_base;
+        // the determined tail when the configuration asks for it; decoding from a bit offset keeps every
+        // symbol as u16 (its caller asks for the symbols themselves)
+        const bool track = tail && files[C.file].mode != 1;
+        uint32_t det = 0xffffffffu, ph_end = 0;      // tail start; end of the last pass that held a placeholder
+        uint4 nx = t8 < n ? *reinterpret_cast<const uint4*>(sym + t8) : make_uint4(0, 0, 0, 0);
+        uint32_t sA = 0;                             // ring slot of the pass's first position
+        for (uint32_t A = 0; A < n; A += P) {
+            const uint32_t p0 = A + t8;
+            const uint4 cur = nx;
+            if (p0 + P < n) nx = *reinterpret_cast<const uint4*>(sym + p0 + P);
+            const uint32_t w4[4] = {cur.x, cur.y, cur.z, cur.w};
+            uint32_t e[8];
+            uint32_t open = 0;                       // bit u: e[u] is a pointer into the pass
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const uint32_t v = (u & 1) ? w4[u >> 1] >> 16 : w4[u >> 1] & 0xffffu;
+                e[u] = v;
+                if (p0 + (uint32_t)u >= n) {
+                    e[u] = 0;
+                } else if (v & kPH) {
+                    const int32_t rel = (int32_t)(t8 + u) - (int32_t)(v & 0x7fffu) - 1;   // source, from A
+                    if (rel >= 0) {
+                        e[u] = kPtr | (uint32_t)rel;
+                        open |= 1u << u;
+                    } else if ((int32_t)A + rel < 0) {
+                        e[u] = kPH | (uint32_t)((int32_t)kWin + (int32_t)A + rel);
+                    } else {
+                        int32_t slot = (int32_t)sA + rel;
+                        if (slot < 0) slot += (int32_t)R;
+                        e[u] = ring[slot];
+                    }
+                }
+            }
+            uint4 v4;
+            v4.x = e[0] | (e[1] << 16);
+            v4.y = e[2] | (e[3] << 16);
+            v4.z = e[4] | (e[5] << 16);
+            v4.w = e[6] | (e[7] << 16);
+            *reinterpret_cast<uint4*>(ring + sA + t8) = v4;
+            __syncthreads();
+            volatile uint16_t* pass = ring + sA;
+            if (open) {
+                while (open) {
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        if ((open >> u) & 1u) {
+                            e[u] = pass[e[u] & (kPtr - 1u)];
+                            pass[t8 + u] = (uint16_t)e[u];
+                            if ((e[u] >> 14) != 1u) open &= ~(1u << u);
+                        }
+                }
+                v4.x = e[0] | (e[1] << 16);
+                v4.y = e[2] | (e[3] << 16);
+                v4.z = e[4] | (e[5] << 16);
+                v4.w = e[6] | (e[7] << 16);
+            }
+            if (det == 0xffffffffu && track && A >= ph_end + kWin) det = A;
+            if (track) {
+                const uint32_t any = (v4.x | v4.y | v4.z | v4.w) & (kPH | (kPH << 16));
+                if (__syncthreads_or((int)any)) ph_end = A + P;
+            } else {
+                __syncthreads();
+            }
+            if (p0 < n) {
+                if (det != 0xffffffffu) {            // bytes at det + position, always behind the map still unread
+                    uint2 b;
+                    b.x = __byte_perm(v4.x, v4.y, 0x6420);
+                    b.y = __byte_perm(v4.z, v4.w, 0x6420);
+                    *reinterpret_cast<uint2*>(reinterpret_cast<uint8_t*>(sym) + det + p0) = b;
+                } else {
+                    *reinterpret_cast<uint4*>(sym + p0) = v4;
+                }
+            }
+            sA = sA + P == R ? 0u : sA + P;
+        }
+        if (threadIdx.x == 0 && det != 0xffffffffu) C.det = det;
     }
 }
 
@@ -2486,20 +2199,14 @@ static int pass1_resident_blocks_t() {
     const int slot = dev >= 0 && dev < 64 ? dev : 0;
     if (!cached[slot]) {
         const int smem = (int)(WPB * warp_smem_bytes());
-        int sms = 0, per_sm_a = 0, per_sm_b = 0, per_sm_c = 0;
+        int sms = 0, per_sm_a = 0, per_sm_b = 0;
         const bool ok =
             cudaFuncSetAttribute(k_sync<WPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
-            cudaFuncSetAttribute(k_inflate<WPB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
-                cudaSuccess &&
-            cudaFuncSetAttribute(k_inflate<WPB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+            cudaFuncSetAttribute(k_inflate<WPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_a, k_sync<WPB>, 32 * WPB, smem) == cudaSuccess &&
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_b, k_inflate<WPB, true>, 32 * WPB, smem) ==
-                cudaSuccess &&
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_c, k_inflate<WPB, false>, 32 * WPB, smem) ==
-                cudaSuccess;
-        const int per_sm_sync = per_sm_a, per_sm_inflate = std::min(per_sm_b, per_sm_c);
-        const int v = std::max(1, sms) * std::max(1, std::min(per_sm_sync, per_sm_inflate));
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_b, k_inflate<WPB>, 32 * WPB, smem) == cudaSuccess;
+        const int v = std::max(1, sms) * std::max(1, std::min(per_sm_a, per_sm_b));
         if (!ok) {
             cudaGetLastError();
             return v;                            // not cached: asked again once a device answers
@@ -2530,9 +2237,7 @@ static void launch_pass1_t(bool sync, const FileDesc* files, ChunkDesc* chunks, 
     const int grid = pass1_warps(nchunks, WPB) / WPB;
     const size_t smem = WPB * warp_smem_bytes();
     if (sync) k_sync<WPB><<<grid, 32 * WPB, smem, s>>>(files, chunks, nchunks, sym, tok, queue, order, p);
-    else if (p.pipe)
-        k_inflate<WPB, true><<<grid, 32 * WPB, smem, s>>>(files, chunks, nchunks, sym, tok, queue, order, p);
-    else k_inflate<WPB, false><<<grid, 32 * WPB, smem, s>>>(files, chunks, nchunks, sym, tok, queue, order, p);
+    else k_inflate<WPB><<<grid, 32 * WPB, smem, s>>>(files, chunks, nchunks, sym, tok, queue, order, p);
 }
 
 static void launch_pass1_any(bool sync, const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym,
@@ -2558,6 +2263,41 @@ void launch_inflate(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint1
 }
 
 uint64_t token_words_per_part() { return kTokPerPart; }
+
+// k_exec's resident blocks on the current device (0 if it cannot be asked)
+template <int NT>
+static int exec_resident() {
+    static int cached[64] = {};
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    const int slot = dev >= 0 && dev < 64 ? dev : 0;
+    if (!cached[slot]) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+            cudaFuncSetAttribute(k_exec<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)exec_smem<NT>()) ==
+                cudaSuccess &&
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_exec<NT>, NT, exec_smem<NT>()) == cudaSuccess)
+            cached[slot] = sms * per_sm;
+        else
+            cudaGetLastError();
+    }
+    return cached[slot];
+}
+
+template <int NT>
+static void launch_exec_t(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* queue,
+                          const uint32_t* order, const KParams& p, cudaStream_t s) {
+    const int cap = std::max(1, exec_resident<NT>());
+    k_exec<NT><<<std::min(nchunks, cap), NT, exec_smem<NT>(), s>>>(files, chunks, nchunks, sym, queue, order, p.tail);
+}
+
+void launch_exec(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* queue,
+                 const uint32_t* order, const KParams& p, cudaStream_t s) {
+    if (nchunks <= 0) return;
+    cudaMemsetAsync(queue, 0, sizeof(uint32_t), s);
+    // up to one block per SM, the block of 1024 threads: half the passes, so half the barriers, of a part
+    if (nchunks <= exec_resident<1024>()) launch_exec_t<1024>(files, chunks, nchunks, sym, queue, order, p, s);
+    else launch_exec_t<512>(files, chunks, nchunks, sym, queue, order, p, s);
+}
 
 void launch_plan(FileDesc* files, ChunkDesc* chunks, int nfiles, cudaStream_t s) {
     if (nfiles <= 0) return;
@@ -2639,7 +2379,7 @@ void launch_finalize(FileDesc* files, int nfiles, cudaStream_t s) {
     k_finalize<<<(nfiles + 127) / 128, 128, 0, s>>>(files, nfiles);
 }
 
-int kernels_per_run() { return 9; }
+int kernels_per_run() { return 10; }
 
 // CRC-32 constants from the polynomial (RFC 1952 section 8)
 static uint32_t h_mul(uint32_t a, uint32_t b) {

@@ -57,7 +57,7 @@ constexpr size_t kOffSym = a256(kOffWstart + (size_t)kNaMaxGroups * kWin);
 constexpr size_t kTokWords = 32 * 512;                // token buffer of one part (parallel block decoder)
 constexpr size_t kOffTok = a256(kOffSym + kNaSymbols * sizeof(uint16_t));
 constexpr size_t kOffQueue = a256(kOffTok + (size_t)kNaMaxParts * kTokWords * sizeof(uint32_t));
-constexpr size_t kScratchBytes = a256(kOffQueue + 2 * sizeof(uint32_t));   // about 23 MiB
+constexpr size_t kScratchBytes = a256(kOffQueue + 3 * sizeof(uint32_t));   // about 23 MiB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -169,7 +169,6 @@ extern "C" int pgz_decompress_noalloc(const uint8_t* gz, uint64_t gz_len, uint8_
     kp.max_block = cfg.max_block;
     kp.confirm_blocks = cfg.confirm_blocks;
     kp.wpb = 4;
-    kp.pipe = 0;
 
     const uint64_t csize = gz_len - 8 - s0, end_bit = (gz_len - 8) * 8;
     uint64_t n = (csize + kNaPartBytes - 1) / kNaPartBytes;
@@ -232,6 +231,7 @@ extern "C" int pgz_decompress_noalloc(const uint8_t* gz, uint64_t gz_len, uint8_
         cudaMemcpyAsync(d_seg0, &seg0, sizeof seg0, cudaMemcpyHostToDevice, s);
         launch_sync(d_files, d_chunks, (int)n, d_sym, d_tok, d_queue, nullptr, kp, s);
         launch_inflate(d_files, d_chunks, (int)n, d_sym, d_tok, d_queue + 1, nullptr, kp, s);
+        launch_exec(d_files, d_chunks, (int)n, d_sym, d_queue + 2, nullptr, kp, s);
         launch_plan(d_files, d_chunks, 1, s);
         launch_chain(d_files, d_chunks, 1, ng, d_g0, d_gn, d_gfile, d_sym, d_gmaps, d_wstart, d_windows, s);
         launch_translate(d_files, d_chunks, (int)n, plan[0].cap, d_sym, d_windows, nullptr, s);

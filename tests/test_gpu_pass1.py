@@ -1,0 +1,57 @@
+"""Pass 1 at the edges of its kernels' tiles: passes of the copy-map executor and segments of the block decoder."""
+import functools
+
+import numpy as np
+import pytest
+
+import deflate_writer as dw
+from gpu_util import Ctx, empty, to_device
+from paper_1905_07224_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+DISTS = [1, 2, 3, 7, 8, 9, 255, 256, 257, 2047, 2048, 4095, 4096, 4097, 8191, 8192, 8193, 16384, 24576, 32759, 32767,
+         32768]
+
+
+@functools.lru_cache(maxsize=None)
+def _copies(n, seed):
+    """A member of exactly n bytes of literals and copies whose distances lie around the executor's pass sizes (4096
+    and 8192 positions), its 16-bit pointers' and the window's ends, overlapping copies included."""
+    rng = np.random.default_rng(seed)
+    tokens, size = [], 0
+    while size < n:
+        d = int(rng.choice(DISTS))
+        if d > size or n - size < 3 or rng.random() < 0.2:
+            tokens.append(("lit", int(rng.choice(list(b"ACGT\n")))))
+            size += 1
+        else:
+            length = min(int(rng.choice([3, 4, 7, 8, 9, 31, 64, 257, 258])), n - size)
+            tokens.append(("match", length, d))
+            size += length
+    w = dw.BitWriter()
+    for a in range(0, len(tokens), 5000):
+        dw.write_dynamic(w, tokens[a:a + 5000], a + 5000 >= len(tokens))
+    text = dw.expand(tokens)
+    assert len(text) == n
+    return dw.gzip_wrap(w.tobytes(), text), text
+
+
+@pytest.mark.parametrize("tail", [0, 1])
+@pytest.mark.parametrize("members", [1, 160])
+def test_copies_across_the_executors_passes(members, tail):
+    """One member alone and many at once (the executor's block size depends on the number of parts)."""
+    sizes = [1, 7, 8, 9, 4095, 4096, 4097, 8191, 8192, 8193, 32768, 40960, 40961, 90001]
+    ctx = Ctx(determined_tail=tail)
+    try:
+        for n in sizes if members == 1 else [0]:
+            made = [_copies(n, n)] if members == 1 else [_copies(sizes[k % len(sizes)], k // 14) for k in range(members)]
+            gz = [to_device(g) for g, _ in made]
+            out = [empty(len(t)) for _, t in made]
+            st, per, _ = ctx.pgz.pgz_decompress_batch(
+                ctx.h, [(d.data_ptr(), len(g), o.data_ptr(), len(t)) for d, o, (g, t) in zip(gz, out, made)])
+            assert st == 0, (n, ctx.pgz.pgz_strerror(st))
+            for (_, t), o, (s, k) in zip(made, out, per):
+                assert s == 0 and k == len(t) and o[:k].cpu().numpy().tobytes() == t
+    finally:
+        ctx.close()
