@@ -67,14 +67,15 @@ typedef struct pgz_config {
     void* cuda_stream;          /* cudaStream_t to issue work on; NULL = default stream */
     uint64_t chunk_bytes;       /* compressed bytes per part (used when n_chunks is 0) */
     int n_chunks;               /* > 0: exactly this many parts per file (overrides chunk_bytes) */
-    int threads_per_chunk;      /* threads decoding one part: 32 (one warp) is the only value */
+    int threads_per_chunk;      /* 32 is the only value (kept from one-warp decoding; see warps_per_block) */
     uint8_t allowed[32];        /* literal bytes accepted at a block start, bit b of byte b/8 */
     int confirm_blocks;         /* blocks after a block start that must also decode (5) */
     uint32_t min_block;         /* a block start's block yields >= min_block bytes (1024) */
     uint32_t max_block;         /* ... and < max_block bytes (4 MiB) */
     uint64_t dev_mem_budget;    /* upper bound on scratch bytes; 0 = none */
     uint64_t spin_cap;          /* reserved for bounded device waits; 0 = default */
-    int warps_per_block;        /* CTA shape of the pass-1 kernels: 2, 4 or 8 warps (one part each); 0 = 4 */
+    int warps_per_block;        /* CTA shape of the pass-1 kernels: 2, 4 or 8 warps, together on one part; 0 = 4.
+                                   A run with few parts takes larger CTAs by itself */
     int exec_pipelined;         /* 0 (default) or 1; accepted, kept and swept as before, but pass 1 has one
                                    execution form now and runs the same either way */
     int determined_tail;        /* 1: once a part's last 32 KiB of output hold no placeholder (none can
@@ -211,7 +212,7 @@ int pgz_decompress_batch(pgz_ctx* ctx, int n, pgz_job* jobs, pgz_stats* st);
    bytes three (about 15 %, 70 % and 15 % of the bytes: only the first
    group's upload and the last group's download are not overlapped), from
    192 MiB two halves, else one.  Each group's part size is the one nearest
-   the context's that gives a whole number of waves of pass-1 warps
+   the context's that gives a whole number of waves of pass-1 CTAs
    (pgz_wave_chunk_bytes; the context's size as is with n_chunks set).  Every
    group is copied to device memory owned by the context, then its run's
    plan, on one upload stream in that order, so that a run waits for its own
@@ -257,7 +258,7 @@ int pgz_inspect_window(pgz_ctx* ctx, int part, uint8_t* host_dst /* 32768 bytes 
    to their own allocator at start-up, services with a fixed device-memory
    budget, loops that cannot afford cudaFree's device-wide synchronisation --
    it runs the same kernels as pgz_decompress with every scratch buffer inside
-   one fixed file-scope __device__ array of about 23 MiB, held on each GPU that
+   one fixed file-scope __device__ array of about 24 MiB, held on each GPU that
    loads the library until the process exits.  No cudaMalloc, cudaFree or other
    allocating routine is called.
    gz [device, 4-byte aligned, gz_len bytes], out [device, out_cap bytes] on
@@ -328,10 +329,10 @@ int pgz_autotune(pgz_ctx* ctx, pgz_job* jobs, int n_jobs, const uint64_t* chunk_
 
 /* The part size that cuts the jobs' members (gz_len of each; one member per
    job, 10-byte gzip headers assumed) into about waves x R parts, where R is
-   the number of pass-1 warps the device holds at once with the given CTA
-   shape (*resident_warps, nullable): the pass-1 kernels are persistent grids
-   of R warps, one part per warp at a time, so a part count of whole waves
-   leaves no warp idle at the end of a launch.  *chunk_bytes: the smallest
+   the number of parts the pass-1 kernels hold at once with the given CTA
+   shape (*resident_warps, nullable): they are persistent grids of R CTAs, one
+   part per CTA at a time, so a part count of whole waves leaves none idle at
+   the end of a launch.  *chunk_bytes: the smallest
    size (>= 4096) whose part count does not exceed the target.  For the
    autotuner's list of sizes; no device work.  PGZ_E_ARG for bad arguments
    (warps_per_block not 2, 4 or 8; waves <= 0). */

@@ -240,7 +240,7 @@ struct Plan {
     bool results_valid = false;   // the device chunk array holds the last run's results
     int wpb = 4;                  // warps per block of the pass-1 kernels (sizes the token scratch)
     const uint8_t* fill = nullptr;   // device window of fill bytes (mode 1)
-    DBuf d_files, d_chunks, d_g0, d_gn, d_gfile, d_seg0, d_sym, d_windows, d_gmaps, d_wstart, d_tok, d_queue, d_order;
+    DBuf d_files, d_chunks, d_g0, d_gn, d_gfile, d_seg0, d_sym, d_windows, d_gmaps, d_wstart, d_tok, d_start, d_queue, d_order;
     PBuf h_files, h_chunks, h_static;
     cudaGraphExec_t graph = nullptr;
     void release() {
@@ -255,6 +255,7 @@ struct Plan {
         d_gmaps.release();
         d_wstart.release();
         d_tok.release();
+        d_start.release();
         d_queue.release();
         d_order.release();
         h_files.release();
@@ -389,7 +390,7 @@ void plan_member(pgz_ctx* ctx, Plan& P, const uint8_t* gz, uint64_t gz_len, uint
 int layout(Plan& P) {
     uint64_t base = 0, mx = 0;
     for (auto& C : P.chunks) {
-        C.cap = round_up(C.cap, 8);
+        C.cap = round_up(C.cap, 32);
         C.sym_base = base;
         base += C.cap;
         mx = std::max(mx, C.cap);
@@ -427,7 +428,8 @@ int layout(Plan& P) {
     if (!e) e = P.d_gfile.ensure(ng * sizeof(int32_t));
     if (!e) e = P.d_seg0.ensure(nf * sizeof(uint64_t));
     if (!e) e = P.d_sym.ensure(P.sym_total * sizeof(uint16_t));
-    if (!e) e = P.d_tok.ensure((size_t)pass1_warps((int)nc, P.wpb) * token_words_per_part() * sizeof(uint32_t) + 64);
+    if (!e) e = P.d_tok.ensure((size_t)token_words((int)nc, P.wpb) * sizeof(uint32_t));
+    if (!e) e = P.d_start.ensure(P.sym_total / 8);
     if (!e) e = P.d_queue.ensure(3 * sizeof(uint32_t));
     if (!e) e = P.d_order.ensure(nc * sizeof(uint32_t));
     if (!e && P.chain) e = P.d_windows.ensure(nc * (size_t)kWin);
@@ -479,14 +481,16 @@ int enqueue(pgz_ctx* ctx, Plan& P, cudaStream_t s, bool timed, cudaStream_t up =
     uint16_t* sym = P.d_sym.as<uint16_t>();
     int k = 0;
     if (timed) cudaEventRecord(ctx->ev[0], s);
-    launch_sync(df, dc, (int)nc, sym, P.d_tok.as<uint32_t>(), P.d_queue.as<uint32_t>(), P.d_order.as<uint32_t>(),
-                ctx->kp, s);
+    uint32_t* start = P.d_start.as<uint32_t>();
+    cudaMemsetAsync(start, 0, P.sym_total / 8, s);
+    launch_sync(df, dc, (int)nc, sym, start, P.d_tok.as<uint32_t>(), P.d_queue.as<uint32_t>(),
+                P.d_order.as<uint32_t>(), ctx->kp, s);
     if (cudaPeekAtLastError() != cudaSuccess) return PGZ_E_CUDA;
     if (timed) cudaEventRecord(ctx->ev[1], s);
-    launch_inflate(df, dc, (int)nc, sym, P.d_tok.as<uint32_t>(), P.d_queue.as<uint32_t>() + 1,
+    launch_inflate(df, dc, (int)nc, sym, start, P.d_tok.as<uint32_t>(), P.d_queue.as<uint32_t>() + 1,
                    P.d_order.as<uint32_t>(), ctx->kp, s);
     if (cudaPeekAtLastError() != cudaSuccess) return PGZ_E_CUDA;
-    launch_exec(df, dc, (int)nc, sym, P.d_queue.as<uint32_t>() + 2, P.d_order.as<uint32_t>(), ctx->kp, s);
+    launch_exec(df, dc, (int)nc, sym, start, P.d_queue.as<uint32_t>() + 2, P.d_order.as<uint32_t>(), ctx->kp, s);
     if (cudaPeekAtLastError() != cudaSuccess) return PGZ_E_CUDA;
     launch_plan(df, dc, (int)nf, s);
     k += 4;
@@ -1422,11 +1426,11 @@ int pgz_decompress_batch_host(pgz_ctx* ctx, int n, pgz_job* jobs, pgz_stats* st)
     int status = PGZ_OK;
     std::vector<char> started((size_t)ng, 0);
     const pgz_config saved = ctx->cfg;
-    const uint64_t W = ctx->cfg.n_chunks > 0 ? 0 : (uint64_t)pass1_warps(1 << 30, ctx->kp.wpb);
+    const uint64_t W = ctx->cfg.n_chunks > 0 ? 0 : (uint64_t)pass1_parts(ctx->kp.wpb);
     for (int g = 0; g < ng; ++g) {
         Plan& P = ctx->hb_plan[g];
         begin_plan(P);
-        if (W) {   // the group's parts in a whole number of waves of pass-1 warps, near the context's part size
+        if (W) {   // the group's parts in a whole number of waves of pass-1 teams, near the context's part size
             std::vector<uint64_t> lens;
             for (int k = gfirst[g]; k < gfirst[g + 1]; ++k)
                 if (valid[k]) lens.push_back(jobs[k].gz_len);
@@ -1713,7 +1717,7 @@ int pgz_wave_chunk_bytes(pgz_ctx* ctx, const pgz_job* jobs, int n_jobs, int warp
         (warps_per_block != 2 && warps_per_block != 4 && warps_per_block != 8))
         return PGZ_E_ARG;
     cudaSetDevice(ctx->cfg.device);
-    const uint64_t W = (uint64_t)pass1_warps(1 << 30, warps_per_block);
+    const uint64_t W = (uint64_t)pass1_parts(warps_per_block);
     if (resident_warps) *resident_warps = (int)W;
     const uint64_t target = std::max<uint64_t>(1, (uint64_t)std::llround(waves * (double)W));
     std::vector<uint64_t> lens((size_t)n_jobs);

@@ -39,7 +39,9 @@ struct KParams {
     uint32_t min_block;
     uint32_t max_block;
     int confirm_blocks;
-    int wpb;               // warps per block of the pass-1 kernels: 2, 4 or 8 (0: 4)
+    int wpb;               // warps per block of the pass-1 kernels: 2, 4 or 8 (0: 4); more with few parts
+    int team;              // != 0: exactly this many warps per block (2, 4, 8 or 16), and
+    uint32_t tok_rows;     // this many rows of tokens per team; 0: the launcher's choice
     int tail;              // k_exec stores a part's determined tail as bytes (1) or keeps u16 symbols (0)
 };
 
@@ -82,7 +84,7 @@ struct FileDesc {
 struct ChunkDesc {
     // plan
     uint64_t lo, hi;       // scan range of the block start, bits [lo, hi)
-    uint64_t sym_base;     // offset of the part's symbols in the scratch (u16 units)
+    uint64_t sym_base;     // offset of the part's symbols in the scratch (u16 units; a multiple of 32)
     uint64_t cap;          // symbol capacity
     int32_t file;
     int32_t index;         // part number within the member
@@ -113,20 +115,22 @@ struct ChunkDesc {
 };
 
 // host-side launch wrappers (pgz_kernels.cu)
-// tok: token_words_per_part() u32 of parallel-block-decoder scratch for each of
-//      pass1_warps(nchunks, p.wpb) warps (at most nchunks rounded up to p.wpb), and 64 bytes after them (read
-//      ahead, not used);
+// start: the parts' start bits, one per symbol (the bits of part c from word sym_base / 32 on, sym_base a multiple of
+//        32), zero before launch_sync;
+// tok: token_words(nchunks, p.wpb) u32 of the block decoder's scratch (p.team set: p.tok_rows rows of 32 p.team u32 for
+//      each of at most nchunks teams);
 // queue: one u32 work counter per kernel (zeroed by the launcher on the stream);
 // order (nullable): the parts in the order the work queue hands them out (nchunks entries).
-void launch_sync(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* tok,
+void launch_sync(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* start, uint32_t* tok,
                  uint32_t* queue, const uint32_t* order, const KParams& p, cudaStream_t s);
-void launch_inflate(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* tok,
-                    uint32_t* queue, const uint32_t* order, const KParams& p, cudaStream_t s);
+void launch_inflate(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* start,
+                    uint32_t* tok, uint32_t* queue, const uint32_t* order, const KParams& p, cudaStream_t s);
 // the parts' copy maps (written by the two kernels above) into symbols, in place
-void launch_exec(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* queue,
+void launch_exec(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* start, uint32_t* queue,
                  const uint32_t* order, const KParams& p, cudaStream_t s);
-uint64_t token_words_per_part();
-int pass1_warps(int nchunks, int wpb);
+uint64_t token_words(int nchunks, int wpb);
+int pass1_team(int nchunks, int wpb);   // warps per part for a launch of nchunks parts
+int pass1_parts(int wpb);               // parts resident at once with many parts (teams of wpb warps)
 void launch_plan(FileDesc* files, ChunkDesc* chunks, int nfiles, cudaStream_t s);
 void launch_chain(const FileDesc* files, const ChunkDesc* chunks, int nfiles, int ngroups,
                   const int32_t* group_chunk0, const int32_t* group_n, const int32_t* group_file,

@@ -5,16 +5,17 @@
 //   k_sync      pass 1a: per part, the first bit of [lo, hi) where a DEFLATE
 //               block starts (Section "Detection of DEFLATE block start
 //               positions", Appendix "DEFLATE block decompression checks"):
-//               a warp tests 1024 bit offsets per step (one 32-bit window per
-//               lane, bit-parallel header tests), __ballot_sync + __ffs elect
-//               the lowest candidate, and the candidate's whole block is then
-//               decoded as the final check -- into the part's own copy map, so
-//               pass 1 resumes after it.
+//               each warp of the part's team filters windows of 1024 bit
+//               offsets (32 per lane, bit-parallel header tests), the survivors'
+//               headers are checked one per lane, and the lowest valid
+//               candidate's whole block is then decoded as the final check --
+//               into the part's own copy map, so pass 1 resumes after it.
 //   k_inflate   pass 1b: the blocks of part i up to the next part's block
-//               start.  One warp per part: the lanes decode segments of a block
-//               in parallel and meet (see par_block), then write the tokens'
-//               copy map: per output position its byte, or the distance to its
-//               source.  No symbol is read, so no window is kept.
+//               start.  One team (a block of 2 to 16 warps) per part: the lanes
+//               decode segments of a DEFLATE block in parallel and meet (see
+//               par_block), then write the tokens' copy map: where a token's
+//               output starts, its byte or the distance to its source.  No
+//               symbol is read, so no window is kept.
 //   k_exec      pass 1c: decode(C_i, w^_i) (Algorithm "DEFLATE decompression"
 //               with the symbolic context [U_0..U_32767]) finished from the
 //               copy map, in place: one block per part, the last 32 KiB of the
@@ -52,16 +53,6 @@ constexpr int LB = 10;          // literal/length lookup bits
 constexpr int DB = 8;           // distance lookup bits
 constexpr uint32_t kPoly = 0xEDB88320u;
 
-// RFC 1951 3.2.5: length codes 257..285 and distance codes 0..29
-__constant__ uint16_t c_lbase[29] = {3, 4, 5, 6, 7, 8, 9, 10, 11, 13, 15, 17, 19, 23, 27, 31,
-                                     35, 43, 51, 59, 67, 83, 99, 115, 131, 163, 195, 227, 258};
-__constant__ uint8_t c_lext[29] = {0, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1, 2, 2, 2, 2,
-                                   3, 3, 3, 3, 4, 4, 4, 4, 5, 5, 5, 5, 0};
-__constant__ uint16_t c_dbase[30] = {1, 2, 3, 4, 5, 7, 9, 13, 17, 25, 33, 49, 65, 97, 129,
-                                     193, 257, 385, 513, 769, 1025, 1537, 2049, 3073, 4097,
-                                     6145, 8193, 12289, 16385, 24577};
-__constant__ uint8_t c_dext[30] = {0, 0, 0, 0, 1, 1, 2, 2, 3, 3, 4, 4, 5, 5, 6, 6,
-                                   7, 7, 8, 8, 9, 9, 10, 10, 11, 11, 12, 12, 13, 13};
 // RFC 1951 3.2.7: order of the code-length code lengths
 __constant__ uint8_t c_clorder[19] = {16, 17, 18, 0, 8, 7, 9, 6, 10, 5, 11, 4, 12, 3, 13, 2, 14, 1, 15};
 // CRC-32 tables (filled by upload_crc_tables)
@@ -70,31 +61,70 @@ __constant__ uint32_t c_x2k[64];           // x^(2^k) mod P
 __constant__ uint32_t c_lane_shift[32];    // x^(8*kPiece*k) mod P
 __constant__ uint32_t c_seg_shift[4][256]; // [j][b]: (byte b at byte j of a register) x^(8*kCrcSeg) mod P
 
-// literal/length lookup entry: bits 0-4 bits to drop, 8-16 value, 17-19
-// extra-bit count (K_LENX), 28-31 kind.  K_LEN carries the exact length
-// (code and extra bits both inside the lookup width), K_LENX the base.
-// K_LIT2: two literals whose codes both fit the lookup width: bits 8-15 and
-// 16-23 the bytes, 24-27 the first code's length, 0-4 both lengths.
-enum : uint32_t { K_LIT = 0, K_LIT2 = 1, K_LEN = 2, K_LENX = 3, K_EOB = 4, K_LONG = 5, K_BAD = 6 };
-// distance lookup entry: bits 0-3 code length, 4-7 extra bits, 8-9 kind, 16-31 base
-enum : uint32_t { DK_OK = 0, DK_LONG = 1, DK_BAD = 2 };
+// Lookup entry of either code, one layout, so that a lane's step is the same
+// for both: bits 0-4 the bits to drop (code and extra bits; both codes of two
+// literals), 5-8 the code's length (the first literal's), 9-11 the kind, 12-31
+// the payload -- LIT: the token (bytes in its low 16 bits, their count above),
+// two literals when both codes fit the lookup width; LEN, DIST: the base to
+// which the extra bits are added.
+enum : uint32_t { K_LIT = 0, K_LEN = 1, K_DIST = 2, K_EOB = 3, K_LONG = 4, K_BAD = 5 };
 
-struct WarpSmem {
-    uint32_t lit[1 << LB];
-    uint32_t dist[1 << DB];
-    uint16_t lsym[288];
-    uint16_t dsym[32];
-    uint16_t lfirst[16], lcount[16], loff[16];
-    uint16_t dfirst[16], dcount[16], doff[16];
-    uint32_t cnt[16];
+// Shared memory of a team: the NW warps of one block, all on one part.
+template <int NW>
+struct TeamSmem {
+    static constexpr uint32_t T = 32 * NW;
+    // longest segment of a lane, in words; odd, so that the lanes' equal places lie in different banks
+    static constexpr uint32_t kSegWords = NW <= 4 ? 29 : (NW == 8 ? 25 : 15);
+    // token starts of a lane that the lanes before it can meet: every second one
+    static constexpr uint32_t kList = NW <= 8 ? 48 : 40;
+    // a round's words, or a block's header (at most 4510 bits) and its first round's
+    static constexpr uint32_t kBits = T * kSegWords + 160;
+    uint32_t tab[(1 << LB) + (1 << DB)];   // literal/length entries, then distance entries
+    // the two codes (0 literal/length, 1 distance): entries of the symbols in (length, value) order, the
+    // distance code's from kDistEnt on; ends of the codes of each length, left-aligned in 15 bits; index of a
+    // length's first entry minus its first code
+    static constexpr uint32_t kDistEnt = 288;
+    uint32_t ent[kDistEnt + 32];
+    uint32_t lim[2][16];
+    int32_t sb[2][16];
     uint32_t allowed[8];
-    uint32_t lmax, dmax, table_kind, pad;
-    uint8_t lens[320];
-    uint8_t cllens[32];
-    uint32_t masks[32 * 32];   // parallel decoding: token starts in the first 1024 bits of each lane's segment;
-                               // reused by exec_range: words 0-511 the entries of two passes of 256
-                               // positions, 512-767 the batch's tokens, 768-1023 their output offsets
+    uint32_t table_kind;
+    // a header's results, a round's results
+    int32_t h_status;
+    uint32_t h_hlit, h_hdist, h_bits;
+    uint16_t r_next[T], r_j[T];            // the lane a lane met (T: none), and at which of its tokens
+    uint8_t r_cnt[T];                      // a lane's listed token starts
+    uint32_t r_exc[NW], r_sum[NW], r_flags, r_end;
+    // block-start search
+    static constexpr uint32_t kCand = 4;                           // valid headers a warp reports per step
+    static constexpr uint32_t kScanWindows = NW <= 8 ? 16 : 8;     // windows of 1024 bits a warp filters per step
+    uint32_t c_n[NW], c_done[NW], c_at[NW][kCand];
+    uint64_t c_resume[NW];
+    int32_t q;                             // queue position
+    union {
+        uint8_t list[kList][T];            // every second token start of each lane's own parse, from its segment's
+                                           // start, modulo 256 (a token takes at most 48 bits)
+        struct {                           // a header's code-length code, its symbols, the lengths and their counts
+            uint16_t cl[128], hs[320];
+            uint8_t lens[320];
+            uint32_t cnt[2][16];
+        };
+    };
+    uint32_t bits[kBits + 2];              // staged words of the compressed data (during the block-start search, its
+                                           // table of Kraft sums takes the last 256)
+    __device__ __forceinline__ uint16_t* kraft3() { return reinterpret_cast<uint16_t*>(bits + kBits + 2 - 256); }
 };
+
+template <int NW>
+__device__ __forceinline__ void team_sync() {
+    if (NW == 1) __syncwarp();
+    else __syncthreads();
+}
+template <int NW>
+__device__ __forceinline__ bool team_or(bool x) {
+    if (NW == 1) return __any_sync(FULL, x);
+    return __syncthreads_or(x);
+}
 
 __device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) {
     uint32_t lo = __shfl_sync(FULL, (uint32_t)v, src), hi = __shfl_sync(FULL, (uint32_t)(v >> 32), src);
@@ -102,25 +132,19 @@ __device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) {
 }
 
 // ---------------------------------------------------------------------------
-// bit input: RFC 1951 3.1.1, LSB first; 32-bit words, bounds-checked; the
-// next word is loaded one refill ahead
+// bit input: RFC 1951 3.1.1, LSB first; 32-bit words, bounds-checked, staged in
+// shared memory.  Each lane of the parallel decoder reads at its own place: a
+// load from global memory there would stall the whole warp on whichever lane's
+// line is missing, at every step.
 // ---------------------------------------------------------------------------
-struct BitIn {
+struct Input {
     const uint32_t* w;   // the member's bytes as 32-bit words (4-byte aligned)
     const uint8_t* b;
     uint64_t nbytes;
-    uint32_t nfull;      // words wholly inside the member
-    uint32_t lo, hi;     // buffered bits [0, 32) and [32, 64); zero above cnt
-    uint32_t cnt;        // buffered bits
-    uint32_t nxt;        // word(wi), loaded one refill ahead
-    uint32_t wi;         // next word to merge into the buffer
+    uint64_t nfull;      // words wholly inside the member
 
-    __device__ __forceinline__ void setup(const uint8_t* gz, uint64_t len) {
-        w = reinterpret_cast<const uint32_t*>(gz);
-        b = gz;
-        nbytes = len;
-        nfull = (uint32_t)((len >> 2) < 0xffffffffull ? (len >> 2) : 0xffffffffull);
-    }
+    __device__ __forceinline__ Input(const uint8_t* gz, uint64_t len)
+        : w(reinterpret_cast<const uint32_t*>(gz)), b(gz), nbytes(len), nfull(len >> 2) {}
     __device__ __forceinline__ uint32_t word(uint64_t i) const {
         if (i < nfull) return __ldg(w + i);
         uint32_t v = 0;
@@ -131,308 +155,341 @@ struct BitIn {
         }
         return v;
     }
-    // SAFE: the caller has checked that word wi lies inside the member
-    template <bool SAFE = false>
-    __device__ __forceinline__ void refill() {
-        if (cnt <= 32) {
-            lo |= __funnelshift_lc(0u, nxt, cnt);    // nxt << cnt, 0 when cnt = 32
-            hi |= __funnelshift_lc(nxt, 0u, cnt);    // nxt >> (32 - cnt), nxt when cnt = 32
-            cnt += 32;
-            ++wi;
-            nxt = SAFE ? __ldg(w + wi) : word(wi);
+};
+
+// n words of the input from word w0 on into S.bits, by the whole team (zeros past the member's end)
+template <int NW>
+__device__ void stage(TeamSmem<NW>& S, const Input& in, uint64_t w0, uint32_t n) {
+    constexpr uint32_t T = 32 * NW;
+    team_sync<NW>();
+    uint32_t i = threadIdx.x;
+    if (w0 + n <= in.nfull) {
+        for (; i + 7 * T < n; i += 8 * T) {
+            uint32_t v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = __ldg(in.w + w0 + i + k * T);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) S.bits[i + k * T] = v[k];
         }
     }
-    __device__ __forceinline__ void seek(uint64_t bit) {
-        wi = (uint32_t)(bit >> 5);
-        const uint32_t s = (uint32_t)(bit & 31);
-        lo = word(wi) >> s;
-        hi = 0;
-        cnt = 32 - s;
-        ++wi;
-        nxt = word(wi);
-        refill();
+    for (; i < n; i += T) S.bits[i] = in.word(w0 + i);
+    team_sync<NW>();
+}
+
+// a reader at bit p of the staged words: 32 bits from p on in x()
+struct Bits {
+    uint32_t p, w0, w1;
+    __device__ __forceinline__ void seek(const uint32_t* bits, uint32_t at) {
+        p = at;
+        w0 = bits[at >> 5];
+        w1 = bits[(at >> 5) + 1];
     }
-    __device__ __forceinline__ uint64_t pos() const { return (uint64_t)wi * 32 - cnt; }
-    __device__ __forceinline__ uint32_t peek(uint32_t n) const { return lo & ((1u << n) - 1u); }   // n < 32
-    __device__ __forceinline__ void drop(uint32_t n) {                                           // n < 32
-        lo = __funnelshift_r(lo, hi, n);
-        hi >>= n;
-        cnt -= n;
+    __device__ __forceinline__ uint32_t x() const { return __funnelshift_r(w0, w1, p); }
+    __device__ __forceinline__ void drop(const uint32_t* bits, uint32_t n) {   // n <= 32
+        const uint32_t q = p + n;
+        if ((q ^ p) >> 5) {
+            w0 = w1;
+            w1 = bits[(q >> 5) + 1];
+        }
+        p = q;
     }
 };
 
 // ---------------------------------------------------------------------------
-// canonical Huffman codes (RFC 1951 3.2.2), built by one warp
+// canonical Huffman codes (RFC 1951 3.2.2)
 // ---------------------------------------------------------------------------
-struct CodeInfo {
-    int status;   // 0 complete, 1 incomplete, -1 over-subscribed
-    int ncodes;
-    int maxlen;
-};
+// entries of the two codes (RFC 1951 3.2.5): length codes 257..285 and distance codes 0..29 by their rule --
+// four (two) codes per number of extra bits
+__device__ __forceinline__ uint32_t lit_entry(uint32_t s, uint32_t L) {
+    if (s < 256) return ((0x10000u | s) << 12) | (K_LIT << 9) | (L << 5) | L;
+    if (s == 256) return (K_EOB << 9) | (L << 5) | L;
+    if (s > 285) return (K_BAD << 9) | 1u;
+    const uint32_t k = s - 257;
+    if (k < 8) return ((k + 3) << 12) | (K_LEN << 9) | (L << 5) | L;
+    if (k == 28) return (258u << 12) | (K_LEN << 9) | (L << 5) | L;
+    const uint32_t E = (k - 4) >> 2;
+    return ((((4 + (k & 3u)) << E) + 3) << 12) | (K_LEN << 9) | (L << 5) | (L + E);
+}
+__device__ __forceinline__ uint32_t dist_entry(uint32_t s, uint32_t L) {
+    if (s > 29) return (K_BAD << 9) | 1u;
+    if (s < 4) return ((s + 1) << 12) | (K_DIST << 9) | (L << 5) | L;
+    const uint32_t E = (s - 2) >> 1;
+    return ((((2 + (s & 1u)) << E) + 1) << 12) | (K_DIST << 9) | (L << 5) | (L + E);
+}
 
-__device__ CodeInfo build_code(WarpSmem& S, const uint8_t* lens, int n, uint16_t* first, uint16_t* count,
-                               uint16_t* off, uint16_t* sym, int lane) {
-    if (lane < 16) S.cnt[lane] = 0;
-    __syncwarp();
-    for (int s = lane; s < n; s += 32) {
-        const uint32_t l = lens[s];
-        if (l) atomicAdd(&S.cnt[l], 1u);
-    }
-    __syncwarp();
-    CodeInfo ci{0, 0, 0};
-    int left = 1;
-    uint32_t code = 0, o = 0, prev = 0;
+// the code that prefixes v (15 code bits, first bit most significant): its length (16: none) from the ends of
+// the codes of each length
+__device__ __forceinline__ uint32_t code_length(uint32_t v, const uint32_t* lim) {
+    uint32_t L = 1;
+#pragma unroll
+    for (int l = 1; l <= 15; ++l) L += v >= lim[l];
+    return L;
+}
+
+// a code longer than the lookup width (or none) of code d: its entry
+template <int NW>
+__device__ __forceinline__ uint32_t long_entry(const TeamSmem<NW>& S, uint32_t x, uint32_t d) {
+    const uint32_t v = __brev(x) >> 17;
+    const uint32_t* lim = S.lim[d];
+    uint32_t L = DB + 1;
+#pragma unroll
+    for (int l = DB + 1; l <= 15; ++l) L += v >= lim[l];
+    if (L > 15) return (K_BAD << 9) | 1u;
+    return S.ent[(int32_t)(v >> (15 - L)) + S.sb[d][L]];
+}
+
+// One warp: code ends of n code lengths whose counts per length are known, and the entries of the symbols in
+// (length, value) order, from ent[off] on.
+template <typename Make>
+__device__ __forceinline__ void sort_code(const uint8_t* lens, int n, uint32_t* cnt, uint32_t* lim, int32_t* sb,
+                                          uint32_t* ent, uint32_t off, Make make, int lane) {
+    uint32_t code = 0, prev = 0, my_off = 0;
+#pragma unroll
     for (int L = 1; L <= 15; ++L) {
-        const uint32_t c = S.cnt[L];
-        left = 2 * left - (int)c;
-        if (left < 0) ci.status = -1;
-        if (c) ci.maxlen = L;
-        ci.ncodes += (int)c;
+        const uint32_t c = cnt[L];
         code = (code + prev) << 1;
         prev = c;
-        if (lane == 0) {
-            first[L] = (uint16_t)code;
-            count[L] = (uint16_t)c;
-            off[L] = (uint16_t)o;
+        if (lane == L) {
+            lim[L] = (code + c) << (15 - L);
+            sb[L] = (int32_t)off - (int32_t)code;
+            my_off = off;
         }
-        o += c;
+        off += c;
     }
-    if (lane == 0) first[0] = count[0] = off[0] = 0;
-    if (ci.status == 0 && left > 0) ci.status = 1;
     __syncwarp();
-    if (ci.status < 0) return ci;
-    if (lane < 16) S.cnt[lane] = off[lane];
+    if (lane < 16) cnt[lane] = my_off;             // next index of each length
     __syncwarp();
-    for (int s0 = 0; s0 < n; s0 += 32) {          // symbols in (length, value) order
+    for (int s0 = 0; s0 < n; s0 += 32) {
         const int s = s0 + lane;
         const uint32_t l = (s < n) ? lens[s] : 0u;
         const uint32_t peers = __match_any_sync(FULL, l);
         const uint32_t rank = __popc(peers & ((1u << lane) - 1u));
-        const uint32_t base = S.cnt[l];
-        if (s < n && l) sym[base + rank] = (uint16_t)s;
+        const uint32_t base = cnt[l];
+        if (s < n && l) ent[base + rank] = make((uint32_t)s, l);
         __syncwarp();
-        if (rank == 0 && l) S.cnt[l] = base + __popc(peers);
+        if (rank == 0 && l) cnt[l] = base + __popc(peers);
         __syncwarp();
     }
-    return ci;
 }
 
-// lut[x] for every NB-bit stream pattern x: the code of length <= NB that
-// prefixes it (make(symbol, length, x)), else `miss` (a longer code, or none)
-template <int NB, typename Make>
-__device__ void fill_lut(uint32_t* lut, const uint16_t* first, const uint16_t* count, const uint16_t* off,
-                         const uint16_t* sym, int maxlen, uint32_t miss, Make make, int lane) {
-    const int top = maxlen < NB ? maxlen : NB;
-    for (uint32_t v = lane; v < (1u << NB); v += 32) {      // v: NB code bits, first bit most significant
-        const uint32_t x = __brev(v) >> (32 - NB);
-        uint32_t e = miss;
-        for (int L = 1; L <= top; ++L) {
-            const uint32_t d = (v >> (NB - L)) - first[L];
-            if (d < count[L]) {
-                e = make(sym[off[L] + d], (uint32_t)L, x, v);
-                break;
+// Both codes of a block from their lengths (S.lens: hlit literal/length, then hdist distance lengths), by the
+// whole team: counts, then one warp per code sorts, then every thread fills its share of the lookup table by
+// the ends of the codes.  A sum of lengths at most 1 has been checked (or is that of the fixed code).
+template <int NW>
+__device__ void build_tables(TeamSmem<NW>& S, uint32_t hlit, uint32_t hdist) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid < 32) S.cnt[tid >> 4][tid & 15] = 0;
+    team_sync<NW>();
+    for (uint32_t s = tid; s < hlit + hdist; s += 32 * NW) {
+        const uint32_t l = S.lens[s];
+        if (l) atomicAdd(&S.cnt[s >= hlit][l], 1u);
+    }
+    team_sync<NW>();
+    if (warp == 0) sort_code(S.lens, (int)hlit, S.cnt[0], S.lim[0], S.sb[0], S.ent, 0, lit_entry, lane);
+    if (warp == (NW > 1 ? 1 : 0))
+        sort_code(S.lens + hlit, (int)hdist, S.cnt[1], S.lim[1], S.sb[1], S.ent, TeamSmem<NW>::kDistEnt, dist_entry, lane);
+    team_sync<NW>();
+    for (uint32_t x = tid; x < (1u << LB); x += 32 * NW) {         // x: stream bits, the first least significant
+        const uint32_t v = __brev(x) >> 17;                        // the same, left-aligned in 15 bits
+        const uint32_t L = code_length(v, S.lim[0]);
+        uint32_t e = K_LONG << 9;
+        if (L <= LB) {
+            e = S.ent[(int32_t)(v >> (15 - L)) + S.sb[0][L]];
+            if (((e >> 9) & 7u) == K_LIT) {                        // a second literal inside the lookup width?
+                const uint32_t v2 = (v << L) & 0x7fffu, L2 = code_length(v2, S.lim[0]);
+                if (L + L2 <= LB) {
+                    const uint32_t e2 = S.ent[(int32_t)(v2 >> (15 - L2)) + S.sb[0][L2]];
+                    if (((e2 >> 9) & 7u) == K_LIT)
+                        e = (0x20000u << 12) | ((e2 & 0xff000u) << 8) | (e & 0xff000u) | (K_LIT << 9) | (L << 5) | (L + L2);
+                }
             }
         }
-        lut[x] = e;
+        S.tab[x] = e;
     }
+    for (uint32_t x = tid; x < (1u << DB); x += 32 * NW) {
+        const uint32_t v = __brev(x) >> 17;
+        const uint32_t L = code_length(v, S.lim[1]);
+        S.tab[(1 << LB) + x] = L <= DB ? S.ent[(int32_t)(v >> (15 - L)) + S.sb[1][L]] : K_LONG << 9;
+    }
+    team_sync<NW>();
 }
 
-// codes longer than the lookup width: compare the first L bits with each
-// length's code range
-__device__ __forceinline__ int decode_long(uint32_t bits15, int nb, const uint16_t* first, const uint16_t* count,
-                                           const uint16_t* off, const uint16_t* sym, int maxlen, uint32_t& len) {
-    const uint32_t v = __brev(bits15) >> 17;
-    for (int L = nb + 1; L <= maxlen; ++L) {
-        const uint32_t d = (v >> (15 - L)) - first[L];
-        if (d < count[L]) {
-            len = (uint32_t)L;
-            return sym[off[L] + d];
-        }
-    }
-    return -1;
-}
-
-// x: the lookup index (stream bits), whose bits after the code are the
-// length's extra bits when they fit
-__device__ __forceinline__ uint32_t lit_entry(uint32_t s, uint32_t L, uint32_t x) {
-    if (s < 256) return (K_LIT << 28) | (s << 8) | L;
-    if (s == 256) return (K_EOB << 28) | L;
-    if (s < 286) {
-        const uint32_t k = s - 257, base = c_lbase[k], E = c_lext[k];
-        if (L + E <= (uint32_t)LB) return (K_LEN << 28) | ((base + ((x >> L) & ((1u << E) - 1u))) << 8) | (L + E);
-        return (K_LENX << 28) | (E << 17) | (base << 8) | L;
-    }
-    return (K_BAD << 28) | L;
-}
-
-__device__ __forceinline__ uint32_t dist_entry(uint32_t s, uint32_t L) {
-    if (s < 30) return ((uint32_t)c_dbase[s] << 16) | ((uint32_t)c_dext[s] << 4) | L;
-    return (DK_BAD << 8) | L;
-}
-
-// a literal followed, inside the lookup width, by a second literal: one entry
-struct LitMake {
-    const uint16_t *first, *count, *off, *sym;
-    __device__ uint32_t operator()(uint32_t s, uint32_t L, uint32_t x, uint32_t v) const {
-        const uint32_t e = lit_entry(s, L, x);
-        if (s >= 256 || L >= (uint32_t)LB - 1) return e;
-        const uint32_t rest = LB - L, v2 = v & ((1u << rest) - 1u);   // the next code bits, first bit most significant
-        for (uint32_t L2 = 1; L2 <= rest; ++L2) {
-            const uint32_t d = (v2 >> (rest - L2)) - first[L2];
-            if (d < count[L2]) {
-                const uint32_t s2 = sym[off[L2] + d];
-                if (s2 >= 256) return e;
-                return (K_LIT2 << 28) | (L << 24) | (s2 << 16) | (s << 8) | (L + L2);
-            }
-        }
-        return e;
-    }
-};
-struct DistMake {
-    __device__ uint32_t operator()(uint32_t s, uint32_t L, uint32_t, uint32_t) const { return dist_entry(s, L); }
-};
-struct ClMake {
-    __device__ uint32_t operator()(uint32_t s, uint32_t L, uint32_t, uint32_t) const { return s | (L << 8); }
-};
-
-// Reading of valid codes, as RFC 1951 3.2.7 and its producer zlib use them:
-// code-length code complete; literal/length code complete or one code of
-// length 1, with an end-of-block code; distance code complete, one code of
-// length 1, or empty.  HDR_ONLY: stop after the checks (block-start search);
-// an over-subscribed length set ends the decoding early either way.
-template <bool HDR_ONLY>
-__device__ int read_dynamic(WarpSmem& S, BitIn& br, int lane) {
-    if (lane == 0) S.table_kind = 0;
-    br.refill();
-    const uint32_t hlit = br.peek(5) + 257;
-    br.drop(5);
-    const uint32_t hdist = br.peek(5) + 1;
-    br.drop(5);
-    const uint32_t hclen = br.peek(4) + 4;
-    br.drop(4);
+// A dynamic block's header up to its code lengths, by one warp (RFC 1951
+// 3.2.7).  Reading of valid codes, as its producer zlib uses them: code-length
+// code complete; literal/length code complete or one code of length 1, with an
+// end-of-block code; distance code complete, one code of length 1, or empty.
+template <int NW>
+__device__ int read_lengths(TeamSmem<NW>& S, Bits& br, int lane, uint32_t& hlit, uint32_t& hdist) {
+    uint32_t x = br.x();
+    hlit = (x & 31u) + 257;
+    hdist = ((x >> 5) & 31u) + 1;
+    const uint32_t hclen = ((x >> 10) & 15u) + 4;
+    br.drop(S.bits, 14);
     if (hlit > 286 || hdist > 30) return CE_DATA;
-    S.cllens[lane] = 0;
-    __syncwarp();
-    br.refill();
+    // lane k reads the k-th code-length length; lane s then holds that of symbol s
+    uint32_t mine = 0;
     const uint32_t n1 = hclen < 10 ? hclen : 10;
-    if ((uint32_t)lane < n1) S.cllens[c_clorder[lane]] = (uint8_t)((br.lo >> (3 * lane)) & 7);
-    br.drop(3 * n1);
-    br.refill();
+    if ((uint32_t)lane < n1) mine = (br.x() >> (3 * lane)) & 7;
+    br.drop(S.bits, 3 * n1);
     if (hclen > 10) {
-        if ((uint32_t)lane >= 10 && (uint32_t)lane < hclen)
-            S.cllens[c_clorder[lane]] = (uint8_t)((br.lo >> (3 * (lane - 10))) & 7);
-        br.drop(3 * (hclen - 10));
+        if ((uint32_t)lane >= 10 && (uint32_t)lane < hclen) mine = (br.x() >> (3 * (lane - 10))) & 7;
+        br.drop(S.bits, 3 * (hclen - 10));
     }
+    uint32_t len = 0;
+#pragma unroll
+    for (int k = 0; k < 19; ++k) {
+        const uint32_t l = __shfl_sync(FULL, mine, k);
+        if (lane == c_clorder[k]) len = l;
+    }
+    if (__reduce_add_sync(FULL, len ? 128u >> len : 0u) != 128u) return CE_DATA;   // complete
+    uint32_t lim[8], base[8], code = 0, off = 0, prev = 0, at = 0;
+#pragma unroll
+    for (int L = 1; L <= 7; ++L) {
+        const uint32_t m = __ballot_sync(FULL, len == (uint32_t)L), c = __popc(m);
+        code = (code + prev) << 1;
+        prev = c;
+        lim[L] = (code + c) << (7 - L);
+        base[L] = off - code;
+        if (len == (uint32_t)L) at = off + __popc(m & ((1u << lane) - 1u));
+        off += c;
+    }
+    if (len) S.ent[at] = (uint32_t)lane;
     __syncwarp();
-    CodeInfo ci = build_code(S, S.cllens, 19, S.dfirst, S.dcount, S.doff, S.dsym, lane);
-    if (ci.status != 0) return CE_DATA;
-    __syncwarp();
-    fill_lut<7>(S.dist, S.dfirst, S.dcount, S.doff, S.dsym, ci.maxlen, 0u, ClMake(), lane);
-    __syncwarp();
-    const uint32_t total = hlit + hdist;
-    uint32_t i = 0, prev = 0;
-    uint32_t kl = 0, kd = 0, nl = 0, nd = 0, ml = 0, md = 0;   // Kraft sums (units of 2^-15), counts, max lengths
-    bool eob = false;
-    while (i < total) {
-        br.refill();
-        const uint32_t e = S.dist[br.peek(7)];
-        const uint32_t s = e & 0xffu;
-        br.drop(e >> 8);
-        uint32_t rep = 1, val;
-        if (s < 16) {
-            val = s;
-            prev = s;
-        } else if (s == 16) {
-            if (i == 0) return CE_DATA;
-            val = prev;
-            rep = 3 + br.peek(2);
-            br.drop(2);
-        } else if (s == 17) {
-            val = 0;
-            rep = 3 + br.peek(3);
-            br.drop(3);
-            prev = 0;
-        } else {
-            val = 0;
-            rep = 11 + br.peek(7);
-            br.drop(7);
-            prev = 0;
-        }
-        if (i + rep > total) return CE_DATA;
-        if (val) {
-            const uint32_t e2 = i + rep;
-            const uint32_t nlit = i < hlit ? ((e2 < hlit ? e2 : hlit) - i) : 0u;
-            const uint32_t ndst = rep - nlit;
-            kl += nlit * (32768u >> val);
-            kd += ndst * (32768u >> val);
-            nl += nlit;
-            nd += ndst;
-            if (nlit && val > ml) ml = val;
-            if (ndst && val > md) md = val;
-            if (i <= 256 && 256 < e2) eob = true;
-            if (kl > 32768u || kd > 32768u) return CE_DATA;       // over-subscribed
-        }
-        if (!HDR_ONLY) {
-            if (rep == 1) {
-                if (lane == 0) S.lens[i] = (uint8_t)val;
-            } else {
-                for (uint32_t j = lane; j < rep; j += 32) S.lens[i + j] = (uint8_t)val;
+    // entry: bits 0-3 the bits to drop (code and repeat count), 4-6 the code's length, 7-10 the least repeat
+    // count, 11-15 the symbol
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t x = (uint32_t)lane + 32u * k, v = __brev(x) >> 25;
+        uint32_t L = 1, b = base[1];
+#pragma unroll
+        for (int l = 1; l <= 6; ++l)
+            if (v >= lim[l]) {
+                L = l + 1;
+                b = base[l + 1];
             }
+        const uint32_t y = S.ent[(v >> (7 - L)) + b];
+        const uint32_t ex = y < 16 ? 0u : (y == 16 ? 2u : (y == 17 ? 3u : 7u));
+        S.cl[x] = (uint16_t)((L + ex) | (L << 4) | ((y < 16 ? 1u : (y == 18 ? 11u : 3u)) << 7) | (y << 11));
+    }
+    __syncwarp();
+    // the chain of symbols, kept as short as it can be (every lane the same): symbol | repeat count << 5
+    const uint32_t total = hlit + hdist;
+    uint32_t i = 0, n = 0;
+    while (i < total) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (u && i >= total) break;
+            const uint32_t w = br.x(), e = S.cl[w & 127u], drop = e & 15u;
+            const uint32_t rep = ((e >> 7) & 15u) + ((w & ((1u << drop) - 1u)) >> ((e >> 4) & 7u));
+            br.drop(S.bits, drop);
+            if (lane == 0) S.hs[n] = (uint16_t)((e >> 11) | (rep << 5));
+            ++n;
+            i += rep;
         }
-        i += rep;
     }
-    if (!eob) return CE_DATA;
-    if (!(kl == 32768u || (nl == 1 && ml == 1))) return CE_DATA;
-    if (!(kd == 32768u || nd == 0 || (nd == 1 && md == 1))) return CE_DATA;
-    if (HDR_ONLY) return CE_OK;
+    if (i != total) return CE_DATA;
     __syncwarp();
-    ci = build_code(S, S.lens, (int)hlit, S.lfirst, S.lcount, S.loff, S.lsym, lane);
-    if (ci.status < 0) return CE_DATA;
-    __syncwarp();
-    fill_lut<LB>(S.lit, S.lfirst, S.lcount, S.loff, S.lsym, ci.maxlen, K_LONG << 28,
-                 LitMake{S.lfirst, S.lcount, S.loff, S.lsym}, lane);
-    if (lane == 0) S.lmax = (uint32_t)ci.maxlen;
-    ci = build_code(S, S.lens + hlit, (int)hdist, S.dfirst, S.dcount, S.doff, S.dsym, lane);
-    if (ci.status < 0) return CE_DATA;
-    __syncwarp();
-    fill_lut<DB>(S.dist, S.dfirst, S.dcount, S.doff, S.dsym, ci.maxlen, DK_LONG << 8, DistMake(), lane);
-    if (lane == 0) {
-        S.dmax = (uint32_t)ci.maxlen;
-        S.table_kind = 2;
+    // the lengths, 32 symbols at a time: places by a prefix sum of the counts, a repeat's value from the last
+    // symbol before it that is no repeat
+    uint32_t at0 = 0, prev_val = 0xffu;
+    bool bad = false;
+    for (uint32_t k0 = 0; k0 < n; k0 += 32) {
+        const uint32_t h = k0 + lane < n ? S.hs[k0 + lane] : 0u, y = h & 31u, rep = h >> 5;
+        uint32_t incl = rep;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t x = __shfl_up_sync(FULL, incl, d);
+            if (lane >= d) incl += x;
+        }
+        const uint32_t own = __ballot_sync(FULL, y != 16) & (FULL >> (31 - lane));   // values at or before mine
+        const uint32_t from = __shfl_sync(FULL, y < 16 ? y : 0u, own ? 31 - __clz(own) : 0);
+        const uint32_t val = own ? from : prev_val;
+        bad |= val == 0xffu && rep;                    // a repeat before the first length
+        const uint32_t at1 = at0 + incl - rep;
+        for (uint32_t j = 0; j < rep; ++j) S.lens[at1 + j] = (uint8_t)val;
+        at0 += __shfl_sync(FULL, incl, 31);
+        prev_val = __shfl_sync(FULL, val, 31);
     }
+    if (__any_sync(FULL, bad)) return CE_DATA;
     __syncwarp();
+    // Kraft sums (units of 2^-15) with the counts above bit 20, longest lengths
+    uint32_t kl = 0, kd = 0, ml = 0, md = 0;
+    for (uint32_t k = lane; k < total; k += 32) {
+        const uint32_t l = S.lens[k];
+        const uint32_t v = l ? (1u << 20 << 3) + (32768u >> l) : 0u;
+        if (k < hlit) {
+            kl += v;
+            ml = max(ml, l);
+        } else {
+            kd += v;
+            md = max(md, l);
+        }
+    }
+    kl = __reduce_add_sync(FULL, kl);
+    kd = __reduce_add_sync(FULL, kd);
+    ml = __reduce_max_sync(FULL, ml);
+    md = __reduce_max_sync(FULL, md);
+    const uint32_t sl = kl & 0x7fffffu, nl = kl >> 23, sd = kd & 0x7fffffu, nd = kd >> 23;
+    if (S.lens[256] == 0) return CE_DATA;
+    if (!(sl == 32768u || (nl == 1 && ml == 1))) return CE_DATA;
+    if (!(sd == 32768u || nd == 0 || (nd == 1 && md == 1))) return CE_DATA;
+    return CE_OK;
+}
+
+// the header of a dynamic block (at bit `at` of the staged words) and its tables; *bits: the header's bits
+template <int NW>
+__device__ int read_dynamic(TeamSmem<NW>& S, uint32_t at, uint32_t* bits) {
+    if (threadIdx.x < 32) {
+        uint32_t hlit = 0, hdist = 0;
+        Bits br;
+        br.seek(S.bits, at);
+        const int st = read_lengths<NW>(S, br, threadIdx.x, hlit, hdist);
+        if (threadIdx.x == 0) {
+            S.h_status = st;
+            S.h_hlit = hlit;
+            S.h_hdist = hdist;
+            S.h_bits = br.p - at;
+            S.table_kind = 0;
+        }
+    }
+    team_sync<NW>();
+    const int st = S.h_status;
+    *bits = S.h_bits;
+    if (st) {
+        team_sync<NW>();                       // S.h_* may be rewritten
+        return st;
+    }
+    build_tables<NW>(S, S.h_hlit, S.h_hdist);
     return CE_OK;
 }
 
 // the fixed code of RFC 1951 3.2.6
-__device__ void build_fixed(WarpSmem& S, int lane) {
-    for (int s = lane; s < 320; s += 32)
+template <int NW>
+__device__ void build_fixed(TeamSmem<NW>& S) {
+    team_sync<NW>();
+    for (int s = threadIdx.x; s < 320; s += 32 * NW)
         S.lens[s] = (uint8_t)(s < 144 ? 8 : s < 256 ? 9 : s < 280 ? 7 : s < 288 ? 8 : 5);
-    __syncwarp();
-    CodeInfo ci = build_code(S, S.lens, 288, S.lfirst, S.lcount, S.loff, S.lsym, lane);
-    __syncwarp();
-    fill_lut<LB>(S.lit, S.lfirst, S.lcount, S.loff, S.lsym, ci.maxlen, K_LONG << 28,
-                 LitMake{S.lfirst, S.lcount, S.loff, S.lsym}, lane);
-    if (lane == 0) S.lmax = (uint32_t)ci.maxlen;
-    ci = build_code(S, S.lens + 288, 32, S.dfirst, S.dcount, S.doff, S.dsym, lane);
-    __syncwarp();
-    fill_lut<DB>(S.dist, S.dfirst, S.dcount, S.doff, S.dsym, ci.maxlen, DK_LONG << 8, DistMake(), lane);
-    if (lane == 0) {
-        S.dmax = (uint32_t)ci.maxlen;
-        S.table_kind = 1;
-    }
-    __syncwarp();
+    if (threadIdx.x == 0) S.table_kind = 1;
+    team_sync<NW>();
+    build_tables<NW>(S, 288, 32);
 }
 
 // ---------------------------------------------------------------------------
-// copy map of one part: what the block decoder writes, one u16 per output
-// position -- a byte (a literal), or kPH | (distance - 1) for a position inside
-// a match.  k_exec turns it into symbols in place.
+// copy map of one part: what the block decoder writes and k_exec turns into
+// symbols in place.  At the position where a token's output starts, a u16: a
+// byte (each literal), or kPH | (distance - 1) (a match), and the position's bit
+// in the start bits (zero before the run); a match also starts anew at every
+// multiple of kRestart positions inside it, so that k_exec finds the code in
+// force without looking back.  The other positions hold nothing.
 // ---------------------------------------------------------------------------
+constexpr uint32_t kRestart = 256;
+
 struct OutState {
     uint16_t* sym;     // the part's copy map
+    uint32_t* start;   // its start bits
     uint64_t cap;
     uint64_t n;        // positions so far (uniform)
+    uint64_t hi;       // positions written, or tried (uniform): n, or more after a failed block
     bool known;        // the context before the part is empty (member start)
     bool neg;          // a match of this lane reaches before the part start (a placeholder source)
 };
@@ -443,483 +500,487 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 
 __device__ __forceinline__ bool allowed_has(const uint32_t* a, uint32_t b) { return (a[b >> 5] >> (b & 31)) & 1u; }
 
-// The first tokens (about kTrialTokens) of a candidate's block, every lane
-// decoding the same bits: a false candidate fails after a few tokens, before
-// the whole block is decoded in parallel.  A prefix that reaches the end of
-// the block is left to the parallel decoder to judge.
-constexpr int kTrialTokens = 64;
+// The entry of the next Huffman symbol at 32 bits x: of a distance when `pend`
+// (the length of a match whose distance is next), else of a literal or length.
+// One table and one entry layout, so that the lanes of a warp take the same step
+// whatever their symbols' kinds.
+template <int NW>
+__device__ __forceinline__ uint32_t symbol_entry(const TeamSmem<NW>& S, uint32_t x, uint32_t pend) {
+    uint32_t e = S.tab[pend ? (1u << LB) + (x & ((1u << DB) - 1u)) : (x & ((1u << LB) - 1u))];
+    if (((e >> 9) & 7u) == K_LONG) e = long_entry<NW>(S, x, pend ? 1u : 0u);
+    return e;
+}
+__device__ __forceinline__ uint32_t entry_kind(uint32_t e) { return (e >> 9) & 7u; }
+// base and extra bits of a length or distance
+__device__ __forceinline__ uint32_t entry_value(uint32_t e, uint32_t x) {
+    return (e >> 12) + ((x & ((1u << (e & 31u)) - 1u)) >> ((e >> 5) & 15u));
+}
+// output length of a literal entry (one or two)
+__device__ __forceinline__ uint32_t lit_count(uint32_t e) { return e >> 28; }
 
-__device__ int trial_prefix(const WarpSmem& S, BitIn br, uint64_t end_bit) {
+// The first tokens of a candidate's block, by one warp whose lanes decode the
+// same bits: a false candidate fails after a few tokens (its literals must be
+// allowed bytes), before the whole block is decoded in parallel.  A prefix that
+// reaches the end of the block is left to the parallel decoder to judge.
+constexpr int kTrialTokens = 24;
+
+template <int NW>
+__device__ int trial_prefix(const TeamSmem<NW>& S, uint32_t at) {
+    uint32_t dist = 0;                                 // 1: a distance is next
+    Bits br;
+    br.seek(S.bits, at);
 #pragma unroll 1
     for (int ntok = 0; ntok < kTrialTokens; ++ntok) {
-        br.refill();
-        uint32_t e = S.lit[br.lo & ((1u << LB) - 1u)];
-        uint32_t k = e >> 28;
-        if (k >= K_LONG) {
-            uint32_t L = 0;
-            const int s = k == K_LONG
-                              ? decode_long(br.peek(15), LB, S.lfirst, S.lcount, S.loff, S.lsym, (int)S.lmax, L)
-                              : -1;
-            if (s < 0) return CE_DATA;
-            e = lit_entry((uint32_t)s, L, 0);
-            k = e >> 28;
-            if (k == K_BAD) return CE_DATA;
+        const uint32_t x = br.x();
+        const uint32_t e = symbol_entry<NW>(S, x, dist), k = entry_kind(e);
+        if (k == K_BAD) return CE_DATA;
+        if (k == K_EOB) return CE_OK;
+        if (k == K_LIT) {
+            if (!allowed_has(S.allowed, (e >> 12) & 0xffu)) return CE_BYTE;
+            if ((e >> 29) & 1u)
+                if (!allowed_has(S.allowed, (e >> 20) & 0xffu)) return CE_BYTE;
         }
-        if (k <= K_LIT2) {
-            if (!allowed_has(S.allowed, (e >> 8) & 0xffu)) return CE_BYTE;
-            if (k == K_LIT2 && !allowed_has(S.allowed, (e >> 16) & 0xffu)) return CE_BYTE;
-            br.drop(e & 31u);
-        } else if (k == K_EOB) {
-            return CE_OK;
-        } else {
-            uint32_t dn = e & 31u;
-            if (k == K_LENX) dn += (e >> 17) & 7u;
-            br.drop(dn);
-            br.refill();
-            uint32_t d = S.dist[br.lo & ((1u << DB) - 1u)];
-            if (d & 0x300u) {
-                if ((d & 0x300u) != (DK_LONG << 8)) return CE_DATA;
-                uint32_t L = 0;
-                const int s = decode_long(br.peek(15), DB, S.dfirst, S.dcount, S.doff, S.dsym, (int)S.dmax, L);
-                if (s < 0) return CE_DATA;
-                d = dist_entry((uint32_t)s, L);
-                if (d & 0x300u) return CE_DATA;
-            }
-            br.drop((d & 15u) + ((d >> 4) & 15u));
-        }
-        if (br.pos() > end_bit) return CE_TRUNC;
+        dist = k == K_LEN;
+        br.drop(S.bits, e & 31u);
     }
     return CE_OK;
 }
 
 // ---------------------------------------------------------------------------
-// parallel decoding of one Huffman block by the 32 lanes of a warp.
-// Round: lane k decodes its own kSeg-bit segment from bit start + k*kSeg with
-// the block's codes (a guess: it may begin inside a code), storing its tokens
-// and marking its token starts among the first kSyncW bits.  Lane k then
-// continues into segment k+1 until its parse meets a token start of lane
-// k+1's parse: from there the two parses are identical (Huffman codes
-// resynchronise), so lane k+1's tokens from that bit on are the block's.
-// Lane 0 starts at a known token start, so the chain of meeting points gives
-// the true token sequence; the warp then writes those tokens in order.  A
-// lane that does not meet its successor within kSyncW bits ends the round
-// there; the next round starts at that known position.
+// parallel decoding of one Huffman block by the T = 32 NW lanes of a team.
+// Round, over a stretch of the block staged in shared memory:
+//  A. lane k parses its own segment of `seg` bits from bit start + k*seg with
+//     the block's codes (a guess: it may begin inside a code), keeping its tokens
+//     and listing where the first of them start;
+//  B. it parses on through the next segments until it reaches a token start
+//     listed by some lane j > k (nearly always k+1): from there the two parses are
+//     identical (Huffman codes resynchronise), so lane j's tokens from that one
+//     on are the block's, and the lanes between hold nothing.  Lane 0 starts at
+//     a known token start, so the lanes on the path 0 -> next(0) -> ... hold the
+//     block's tokens, up to the first that meets nobody (the block's end, or the
+//     round's);
+//  C. each lane on the path drops its tokens before its meeting point; a prefix
+//     sum of the output lengths gives its place in the output, and it writes the
+//     copy map of its tokens.
+// The next round starts where the last lane of the path stopped.
+// Tokens are kept in global memory, row by row over the lanes: the stores wait
+// for nothing, and in C the lanes read along together.
+// seg follows the length of the part's previous block, so that its rounds have
+// few lanes left over.
 // ---------------------------------------------------------------------------
-constexpr uint32_t kSeg = 2048;      // bits per lane per round
-constexpr uint32_t kSyncW = 1024;    // bits at the head of a segment where meeting points are looked for
-constexpr uint32_t kTokCap = 512;    // tokens a lane may keep per round (own segment + continuation)
-constexpr uint64_t kTokPerPart = 32ull * kTokCap;   // token buffer of one part (one warp)
+constexpr uint32_t kSegWordsMin = 3;
 
-// the output length of a token
+// token: bits 16-24 the output length, bit 31 a match (bits 0-14 distance - 1), else one or two bytes
 __device__ __forceinline__ uint32_t token_len(uint32_t t) { return (t >> 16) & 0x1ffu; }
 
-enum : int { LT_ONE = 0, LT_TWO = 1, LT_EOB = 2, LT_ERR = 3 };
+enum : uint32_t { PS_OK = 0, PS_EOB = 1, PS_ERR = 2, PS_SYNC = 3, PS_NOSYNC = 4, PS_CAP = 5 };
 
-// one token by one lane: t0 (and t1 for two literals, the first l1 bits long)
-template <bool SAFE>
-__device__ __forceinline__ int lane_token(const WarpSmem& S, BitIn& b, uint32_t& t0, uint32_t& t1, uint32_t& l1) {
-    b.refill<SAFE>();
-    uint32_t e = S.lit[b.lo & ((1u << LB) - 1u)];
-    uint32_t k = e >> 28;
-    if (k == K_LIT2) {
-        t0 = 0x10000u | ((e >> 8) & 0xffu);
-        t1 = 0x10000u | ((e >> 16) & 0xffu);
-        l1 = (e >> 24) & 15u;
-        b.drop(e & 31u);
-        return LT_TWO;
-    }
-    if (k >= K_LONG) {
-        uint32_t L = 0;
-        const int s = k == K_LONG ? decode_long(b.peek(15), LB, S.lfirst, S.lcount, S.loff, S.lsym, (int)S.lmax, L) : -1;
-        if (s < 0) return LT_ERR;
-        e = lit_entry((uint32_t)s, L, 0);
-        k = e >> 28;
-        if (k == K_BAD) return LT_ERR;
-    }
-    if (k == K_LIT) {
-        t0 = 0x10000u | ((e >> 8) & 0xffu);
-        b.drop(e & 31u);
-        return LT_ONE;
-    }
-    if (k == K_EOB) {
-        b.drop(e & 31u);
-        return LT_EOB;
-    }
-    uint32_t len = (e >> 8) & 0x1ffu, dn = e & 31u;
-    if (k == K_LENX) {
-        const uint32_t eb = (e >> 17) & 7u;
-        len += (b.lo >> dn) & ((1u << eb) - 1u);
-        dn += eb;
-    }
-    b.drop(dn);
-    b.refill<SAFE>();
-    uint32_t d = S.dist[b.lo & ((1u << DB) - 1u)];
-    if (d & 0x300u) {
-        if ((d & 0x300u) != (DK_LONG << 8)) return LT_ERR;
-        uint32_t L = 0;
-        const int s = decode_long(b.peek(15), DB, S.dfirst, S.dcount, S.doff, S.dsym, (int)S.dmax, L);
-        if (s < 0) return LT_ERR;
-        d = dist_entry((uint32_t)s, L);
-        if (d & 0x300u) return LT_ERR;
-    }
-    const uint32_t dl = d & 15u, de = (d >> 4) & 15u;
-    const uint32_t dist = (d >> 16) + ((b.lo >> dl) & ((1u << de) - 1u));
-    b.drop(dl + de);
-    t0 = 0x80000000u | (len << 16) | (dist - 1u);
-    return LT_ONE;
-}
-
-enum : uint32_t { PS_OK = 0, PS_EOB = 1, PS_ERR = 2, PS_CAP = 3, PS_SYNC = 4, PS_NOSYNC = 5 };
-
-__device__ __forceinline__ void mark(uint32_t& mw, uint32_t& mwi, uint32_t* m, uint32_t rel) {
-    const uint32_t wi = rel >> 5;
-    if (wi != mwi) {
-        m[mwi] = mw;
-        mw = 0;
-        mwi = wi;
-    }
-    mw |= 1u << (rel & 31);
-}
-
-// own segment: tokens from `my0` while the token start lies before my0 + kSeg.
-// The loop runs in lock step over the warp (one token per lane per step).
-__device__ uint32_t seg_own(const WarpSmem& S, BitIn& b, uint64_t my0, uint32_t* m, uint32_t* tb, uint32_t& n,
-                            uint32_t& out_len, uint64_t& stop, uint32_t& ev) {
-    uint32_t mw = 0, mwi = 0;
-    uint32_t st = PS_OK;
-    const uint32_t p0 = (uint32_t)my0;
-    bool go = true;
-    while (__any_sync(FULL, go)) {
-        if (!go) continue;
-        const uint32_t rel = (uint32_t)(b.wi * 32u - b.cnt) - p0;
-        if (rel >= kSeg) {
-            go = false;
-            continue;
-        }
-        if (rel < kSyncW) mark(mw, mwi, m, rel);
-        if (n + 2 > kTokCap) {
-            st = PS_CAP;
-            go = false;
-            continue;
-        }
-        uint32_t t0, t1, l1;
-        const int r = lane_token<false>(S, b, t0, t1, l1);
-        if (r <= LT_TWO) {
-            tb[n++] = t0;
-            out_len += token_len(t0);
-            if (r == LT_TWO) {
-                if (rel + l1 < kSyncW) mark(mw, mwi, m, rel + l1);
-                tb[n++] = t1;
-                ++out_len;
-            }
-        } else {
-            st = r == LT_EOB ? PS_EOB : PS_ERR;
-            ev = n;
-            go = false;
-        }
-    }
-    m[mwi] = mw;
-    stop = b.pos();
-    return st;
-}
-
-// continuation into the next segment until the parse meets one of its token
-// starts (lock step; lanes with nothing to do idle)
-__device__ uint32_t seg_next(const WarpSmem& S, BitIn& b, bool active, uint64_t nx0, const uint32_t* nm, uint32_t* tb,
-                             uint32_t n, uint32_t& n2, uint32_t& out_len, uint64_t& q, uint32_t& ev) {
-    const uint32_t p0 = (uint32_t)nx0;
-    uint32_t st = PS_NOSYNC;
-    bool go = active;
-    while (__any_sync(FULL, go)) {
-        if (!go) continue;
-        const uint32_t rel = (uint32_t)(b.wi * 32u - b.cnt) - p0;
-        if (rel >= kSyncW || n + n2 + 2 > kTokCap) {
-            st = PS_NOSYNC;
-            go = false;
-            continue;
-        }
-        if ((nm[rel >> 5] >> (rel & 31)) & 1u) {
-            st = PS_SYNC;
-            go = false;
-            continue;
-        }
-        uint32_t t0, t1, l1;
-        const int r = lane_token<false>(S, b, t0, t1, l1);
-        if (r <= LT_TWO) {
-            tb[n + n2++] = t0;
-            out_len += token_len(t0);
-            if (r == LT_TWO) {
-                tb[n + n2++] = t1;
-                ++out_len;
-            }
-        } else {
-            ev = n2;
-            st = r == LT_EOB ? PS_EOB : PS_ERR;
-            go = false;
-        }
-    }
-    q = b.pos();
-    return st;
-}
-
-// A lane's tokens read in order, four per 16-byte load, one load ahead.
-struct TokenReader {
-    const uint4* p;
-    uint4 q, nx;
-    uint32_t left;      // tokens of q not yet taken
-    __device__ __forceinline__ void begin(const uint32_t* tb, uint32_t x) {   // tb: 16-byte aligned
-        p = reinterpret_cast<const uint4*>(tb) + (x >> 2);
-        q = p[0];
-        nx = p[1];
-        p += 2;
-        left = 4;
-        for (uint32_t k = x & 3u; k; --k) shift();
-    }
-    __device__ __forceinline__ void shift() {
-        q.x = q.y;
-        q.y = q.z;
-        q.z = q.w;
-        --left;
-    }
-    __device__ __forceinline__ uint32_t next() {
-        const uint32_t t = q.x;
-        shift();
-        if (left == 0) {
-            q = nx;
-            nx = *p++;
-            left = 4;
-        }
-        return t;
-    }
+// A lane's parse and what it has found so far.
+struct LaneParse {
+    uint32_t p;           // bit of the staged words
+    uint32_t n, out_len;  // tokens kept (rows of T), their output length
+    uint32_t st;
 };
 
-// Writes the copy map of a lane's tokens [x, xe) from position `at` on: whole
-// aligned words of four positions leave as one 8-byte store; the positions of
-// the first and last word, which other lanes share, leave one by one.
-// Returns false if (check) a literal is not an allowed byte.
-__device__ __forceinline__ bool expand_tokens(const WarpSmem& S, const uint32_t* tb, uint32_t x, uint32_t xe,
-                                              uint16_t* out, uint32_t at, bool check, bool& neg) {
-    if (x >= xe) return true;
-    TokenReader rd;
-    rd.begin(tb, x);
-    bool ok = true;
-    uint64_t acc = 0;
-    uint32_t pos = at;                   // next position
-    uint32_t fill = at & 3u;             // positions of the current word before `pos`
-    uint32_t skip = fill;                // positions of the current word that are not this lane's
-    uint64_t* w = reinterpret_cast<uint64_t*>(out + (at & ~3u));
-    auto flush = [&]() {                 // the current word is full
-        if (skip) {
-            uint16_t* h = reinterpret_cast<uint16_t*>(w);
-            for (uint32_t k = skip; k < 4; ++k) h[k] = (uint16_t)(acc >> (16 * k));
-            skip = 0;
-        } else {
-            *w = acc;
-        }
-        ++w;
-    };
-    for (; x < xe; ++x) {
-        const uint32_t t = rd.next();
-        uint32_t len = 1, v = t & 0xffu;
-        if (t >> 31) {
-            len = token_len(t);
-            v = kPH | (t & 0x7fffu);
-            neg |= pos <= (t & 0x7fffu);
-        } else if (check) {
-            ok &= allowed_has(S.allowed, v);
-        }
-        pos += len;
-        const uint32_t v2 = v | (v << 16);
-        const uint64_t v4 = (uint64_t)v2 | ((uint64_t)v2 << 32);
-        acc |= v4 << (16 * fill);
-        uint32_t end = fill + len;
-        while (end >= 4) {
-            flush();
-            acc = v4;
-            end -= 4;
-        }
-        fill = end;
-        acc &= (1ull << (16 * fill)) - 1ull;
+// The token at P.p of the lanes with `go` (two literals at once if PAIRS), kept in tok[P.n]; false at a symbol that
+// ends the parse (P.p stays at it; P.st says why).  One step for a literal, a match, or two literals: the words
+// around P.p are loaded anew (three loads that conflict little cost less than carrying them from step to step).
+template <int NW, bool PAIRS>
+__device__ __forceinline__ bool next_token(const TeamSmem<NW>& S, LaneParse& P, uint32_t* tok) {
+    const uint32_t* w = S.bits + (P.p >> 5);
+    const uint32_t w0 = w[0], w1 = w[1], w2 = w[2];
+    const uint32_t x = __funnelshift_r(w0, w1, P.p);
+    uint32_t e = S.tab[x & ((1u << LB) - 1u)];
+    if (entry_kind(e) == K_LONG) e = long_entry<NW>(S, x, 0);
+    uint32_t kind = entry_kind(e);
+    uint32_t t = PAIRS ? e >> 12 : 0x10000u | ((e >> 12) & 0xffu), drop = PAIRS ? e & 31u : (e >> 5) & 15u;
+    if (kind == K_LEN) {
+        const uint32_t q = (P.p & 31u) + (e & 31u);
+        const uint32_t y = __funnelshift_r(q < 32 ? w0 : w1, q < 32 ? w1 : w2, q);
+        uint32_t d = S.tab[(1u << LB) + (y & ((1u << DB) - 1u))];
+        if (entry_kind(d) == K_LONG) d = long_entry<NW>(S, y, 1);
+        kind = entry_kind(d);
+        t = 0x80000000u | (entry_value(e, x) << 16) | (entry_value(d, y) - 1u);
+        drop = (e & 31u) + (d & 31u);
     }
-    uint16_t* h = reinterpret_cast<uint16_t*>(w);
-    for (uint32_t k = skip; k < fill; ++k) h[k] = (uint16_t)(acc >> (16 * k));
+    if (kind >= K_EOB) {
+        P.st = kind == K_EOB ? PS_EOB : PS_ERR;
+        return false;
+    }
+    P.p += drop;
+    P.out_len += token_len(t);
+    tok[P.n] = t;
+    P.n += 32 * NW;
+    return true;
+}
+
+// In the loops below the lanes of a warp take every step together (the vote at its end): left to themselves, lanes
+// that took different branches run apart for the rest of the loop, and the warp does each group's steps in turn.
+
+// A: the tokens that start before p0 + seg, kept in tok[0], tok[T], ... up to tok[cap]
+template <int NW>
+__device__ __forceinline__ void parse_own(TeamSmem<NW>& S, LaneParse& P, uint32_t tl, uint32_t seg, uint32_t* tok,
+                                          uint32_t cap) {
+    constexpr uint32_t T = 32 * NW;
+    const uint32_t p0 = P.p, p1 = p0 + seg;
+    uint8_t* list = &S.list[0][0] + tl;
+    bool go = true;
+    while (__any_sync(FULL, go)) {
+        if (go) {
+            const uint32_t rel = P.p - p0, n = P.n;
+            go = next_token<NW, true>(S, P, tok);
+            if (!(n & T) && n < 2 * TeamSmem<NW>::kList * T) list[n / 2] = (uint8_t)rel;
+            if (P.n >= cap) {
+                P.st = PS_CAP;
+                go = false;
+            }
+            go = go && P.p < p1;
+        }
+    }
+}
+
+// B: on through the segments after lane tl's (rel: the place in the first), literals one at a time, until a listed
+// token start; m and j: that lane and list entry.  A parse that meets nobody over kMeetBits bits gives up (a lane past
+// the block's end can otherwise go on to the round's).
+constexpr uint32_t kMeetBits = 8192;
+
+template <int NW>
+__device__ __forceinline__ void parse_on(TeamSmem<NW>& S, LaneParse& P, bool go, uint32_t tl, uint32_t seg, uint32_t rel,
+                                         uint32_t* tok, uint32_t cap, uint32_t& m, uint32_t& j) {
+    constexpr uint32_t T = 32 * NW;
+    const uint32_t give_up = min(T, tl + 2 + kMeetBits / seg);
+    m = tl + 1;
+    j = 0;
+    uint32_t at = 0, cnt = m < T ? S.r_cnt[m] : 0u;    // place of entry j of lane m's list; its entries
+    while (__any_sync(FULL, go)) {
+        if (go) {
+            if (rel >= seg) {
+                rel -= seg;
+                ++m;
+                j = at = 0;
+                cnt = m < T ? S.r_cnt[m] : 0u;
+            }
+            while (at < rel && j + 1 < cnt) {
+                ++j;
+                at += (S.list[j][m] - at) & 255u;
+            }
+            if (m >= give_up || P.n >= cap) {
+                P.st = PS_NOSYNC;
+                go = false;
+            } else if (at == rel) {
+                P.st = PS_SYNC;
+                go = false;
+            } else {
+                const uint32_t p = P.p;
+                go = next_token<NW, false>(S, P, tok);
+                rel += P.p - p;
+            }
+        }
+    }
+}
+
+// output length of the tokens [0, z)
+template <int NW>
+__device__ __forceinline__ uint32_t tokens_length(const uint32_t* tok, uint32_t z) {
+    constexpr uint32_t T = 32 * NW;
+    uint32_t len = 0;
+    for (uint32_t n = 0; __any_sync(FULL, n < z); n += 4 * T) {
+        uint32_t t[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) t[k] = n + k * T < z ? tok[n + k * T] : 0u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) len += token_len(t[k]);
+    }
+    return len;
+}
+
+// whether every literal among the tokens [n, z) is an allowed byte
+template <int NW>
+__device__ __noinline__ bool tokens_allowed(const TeamSmem<NW>& S, const uint32_t* tok, uint32_t n, uint32_t z) {
+    bool ok = true;
+    for (; n < z; n += 32 * NW) {
+        const uint32_t t = tok[n];
+        if (!(t >> 31))
+            ok &= allowed_has(S.allowed, t & 0xffu) && (token_len(t) < 2 || allowed_has(S.allowed, (t >> 8) & 0xffu));
+    }
     return ok;
 }
 
-__device__ int par_block(WarpSmem& S, uint32_t* tokbuf, BitIn& br, OutState& o, bool check, uint64_t max_block,
-                         uint64_t end_bit, uint64_t& block_n, int lane) {
-    uint32_t* tb = tokbuf + (uint64_t)lane * kTokCap;
-    uint32_t* mymask = S.masks + 32 * lane;
-    for (;;) {
-        const uint64_t start = br.pos();
-        const uint64_t my0 = start + (uint64_t)lane * kSeg;
+// C: the copy map of the tokens [n, z), from position `pos` on.  Only the places where a token starts are written
+// (a u16 each, and its start bit): k_exec spreads the matches, many threads to each.  The start bits go to shared
+// memory (sb, from bit 0 of position pos0's word on) when the round's fit there (sb not null), else to `start`.
+// Returns false if (check) a literal is not an allowed byte.
+template <int NW>
+__device__ __forceinline__ bool write_map(const TeamSmem<NW>& S, const uint32_t* tok, uint32_t n, uint32_t z,
+                                          uint16_t* map, uint32_t* start, uint32_t* sb, uint32_t pos0, uint32_t pos,
+                                          bool check, bool& neg) {
+    constexpr uint32_t T = 32 * NW;
+    constexpr int kAhead = 4;
+    bool ok = true;
+    uint32_t* words = sb ? sb - (pos0 >> 5) : start;
+    uint32_t nx[kAhead];
 #pragma unroll
-        for (int w = 0; w < 32; ++w) mymask[w] = 0;
-        {   // bring the lane's segment (and the continuation window) into L1
-            const uint64_t b0 = my0 >> 3, b1 = (my0 + kSeg + kSyncW + 128) >> 3;
-            for (uint64_t a = b0 & ~127ull; a < b1; a += 128)
-                if (a < br.nbytes) asm volatile("prefetch.global.L1 [%0];" ::"l"(br.b + a));
-        }
-        BitIn b = br;
-        b.seek(my0);
-        uint32_t n = 0, ev1 = 0, ev2 = 0, n2 = 0, olen = 0;
-        uint64_t stop = 0, q = 0;
-        const uint32_t st1 = seg_own(S, b, my0, mymask, tb, n, olen, stop, ev1);
-        __syncwarp();
-        const uint32_t st2 = seg_next(S, b, st1 == PS_OK && lane < 31, my0 + kSeg, S.masks + 32 * ((lane + 1) & 31), tb,
-                                      n, n2, olen, q, ev2);
-        __syncwarp();
-        // the chain of meeting points, lane by lane (uniform)
-        uint32_t skip = 0, my_vs = 0, my_ve = 0;
-        int last = -1;
-        bool block_end = false;
-        int err = CE_OK;
-        uint64_t round_end = 0;
-        for (int k = 0; k < 32; ++k) {
-            const uint32_t s1 = __shfl_sync(FULL, st1, k), nk = __shfl_sync(FULL, n, k);
-            uint32_t ve;
-            bool stop_here = true;
-            if (s1 == PS_EOB) {
-                ve = __shfl_sync(FULL, ev1, k);
-                block_end = true;
-                round_end = shfl64(stop, k);
-            } else if (s1 == PS_ERR) {
-                err = CE_DATA;
-                ve = skip;
-            } else if (s1 == PS_CAP || k == 31) {
-                ve = nk;
-                round_end = shfl64(stop, k);
-            } else {
-                const uint32_t s2 = __shfl_sync(FULL, st2, k), n2k = __shfl_sync(FULL, n2, k);
-                const uint64_t qk = shfl64(q, k);
-                if (s2 == PS_EOB) {
-                    ve = nk + __shfl_sync(FULL, ev2, k);
-                    block_end = true;
-                    round_end = qk;
-                } else if (s2 == PS_ERR) {
-                    err = CE_DATA;
-                    ve = skip;
-                } else if (s2 == PS_NOSYNC) {
-                    ve = nk + n2k;
-                    round_end = qk;
-                } else {                                   // met lane k+1 at qk
-                    ve = nk + n2k;
-                    stop_here = false;
+    for (int k = 0; k < kAhead; ++k) nx[k] = n + k * T < z ? tok[n + k * T] : 0u;
+    while (__any_sync(FULL, n < z)) {
+        uint32_t q[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) q[k] = nx[k];
+        n += kAhead * T;
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) nx[k] = n + k * T < z ? tok[n + k * T] : 0u;
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {
+            const uint32_t t = q[k], len = token_len(t), d = t & 0x7fffu;   // (len 0: past the lane's last token)
+            const bool match = t >> 31, two = !match && len > 1;
+            const uint32_t code = match ? kPH | d : t & 0xffu, b1 = (t >> 8) & 0xffu;
+            if (check && !match && len) ok &= allowed_has(S.allowed, code) && (!two || allowed_has(S.allowed, b1));
+            neg |= match && pos <= d;
+            if (len) {
+                atomicOr(words + (pos >> 5), (two ? 3u : 1u) << (pos & 31u));
+                map[pos] = (uint16_t)code;
+            }
+            if (two) map[pos + 1] = (uint16_t)b1;
+            const uint32_t r = (pos | (kRestart - 1)) + 1, e = pos + len;
+            if (r < e) {                        // the second literal, or the match, starts anew at r
+                for (uint32_t a = r; a < e; a += kRestart) {
+                    if (match) map[a] = (uint16_t)code;
+                    atomicOr(words + (a >> 5), 1u);
                 }
-                if (!stop_here) {
-                    // lane k+1's tokens that start before qk are not the block's
-                    const uint32_t rel = (uint32_t)(qk - (start + (uint64_t)(k + 1) * kSeg));
-                    const uint32_t w = S.masks[32 * (k + 1) + lane];
-                    const uint32_t below = (uint32_t)lane < (rel >> 5) ? __popc(w)
-                                         : ((uint32_t)lane == (rel >> 5) ? __popc(w & ((1u << (rel & 31)) - 1u)) : 0u);
-                    const uint32_t nskip = __reduce_add_sync(FULL, below);
-                    if (lane == k) {
-                        my_vs = skip;
-                        my_ve = ve;
-                    }
-                    skip = nskip;
-                    continue;
-                }
+            } else if (two && !(~pos & 31u)) {  // the second literal's bit is the next word's
+                atomicOr(words + (pos >> 5) + 1, 1u);
             }
-            if (lane == k) {
-                my_vs = skip;
-                my_ve = ve;
-            }
-            last = k;
-            break;
+            pos = e;
         }
-        if (err) return err;
-        // the block's tokens of this round are the lane ranges [my_vs, my_ve) one after another (a lane's kept
-        // tokens end where its parse ends); each lane writes the copy map of its own
-        uint32_t len = 0;
-        if (lane <= last && my_vs < my_ve) {
-            len = olen;
-            if (my_vs) {
-                TokenReader rd;
-                rd.begin(tb, 0);
-                for (uint32_t x = 0; x < my_vs; ++x) len -= token_len(rd.next());
-            }
+    }
+    return ok;
+}
+
+// What a part's blocks share.
+struct TeamState {
+    uint32_t* tok;       // the team's tokens: row k holds every lane's k-th
+    uint32_t cap;        // rows
+    uint32_t est;        // bits of the part's previous block (0: not known)
+    uint32_t segw_lim;   // longest segment in words, shortened while tokens fill the rows first
+};
+
+// The tokens of a Huffman block whose tables are in S, from bit `pos` of the
+// member on; [s0, s1) are the staged words.
+template <int NW>
+__device__ int par_block(TeamSmem<NW>& S, const Input& in, uint64_t s0, uint64_t s1, uint64_t& pos, TeamState& ts,
+                         OutState& o, bool check, uint64_t max_block, uint64_t end_bit, uint64_t& block_n) {
+    constexpr uint32_t T = 32 * NW, kSegWords = TeamSmem<NW>::kSegWords;
+    const uint32_t tl = threadIdx.x, lane = tl & 31, warp = tl >> 5;
+    const uint64_t block0 = pos;
+    for (;;) {
+        uint32_t segw = ts.segw_lim;
+        if (ts.est) {                                  // what is expected to be left, in equal rounds
+            const uint64_t done = pos - block0;
+            uint32_t left = done < ts.est ? ts.est - (uint32_t)done : ts.est >> 4;
+            left = (left + left / 32) / 32 + 1;
+            const uint32_t rounds = (left + T * segw - 1) / (T * segw);
+            segw = min(segw, max(5u, (left / rounds + T - 1) / T) | 1u);
         }
+        const uint32_t seg = 32 * segw, need = T * segw + 4;   // a token may end 48 bits past the last segment
+        const uint64_t w = pos >> 5;
+        if (w < s0 || w + need > s1) {
+            s0 = w;
+            s1 = w + TeamSmem<NW>::kBits;
+            stage<NW>(S, in, s0, TeamSmem<NW>::kBits);
+        }
+        const uint64_t base = s0 << 5;                 // member bit of staged bit 0
+        const uint32_t start = (uint32_t)(pos - base), p0 = start + tl * seg;
+        LaneParse P{p0, 0, 0, PS_OK};
+        uint32_t* tok = ts.tok + tl;
+        const uint32_t cap = ts.cap * T;
+        team_sync<NW>();                               // the lists' place is free
+        parse_own<NW>(S, P, tl, seg, tok, cap);
+        S.r_cnt[tl] = (uint8_t)min((P.n / T + 1) / 2, TeamSmem<NW>::kList);
+        team_sync<NW>();
+        uint32_t m, j;
+        parse_on<NW>(S, P, P.st == PS_OK && tl + 1 < T, tl, seg, P.p - p0 - seg, tok, cap, m, j);
+        const bool met = P.st == PS_SYNC;
+        const uint32_t n = P.n;
+        S.r_next[tl] = (uint16_t)(met ? m : T);
+        S.r_j[tl] = (uint16_t)(2 * j);
+        const uint32_t exc = __ballot_sync(FULL, !met || m != tl + 1);
+        if (lane == 0) S.r_exc[warp] = exc;
+        team_sync<NW>();
+        // the path from lane 0 (uniform): runs of lanes that met the next one, up to a lane that met another or
+        // nobody (the last)
+        uint32_t path = 0, last = 0, pred = tl - 1;    // my warp's lanes on the path; mine's predecessor
+        for (uint32_t cur = 0;;) {
+            uint32_t v = cur >> 5, x = S.r_exc[v] & (FULL << (cur & 31));
+            while (!x) {                               // ends: the team's last lane met nobody
+                if (v == warp) path |= FULL << (cur & 31);
+                cur = 32 * ++v;
+                x = S.r_exc[v];
+            }
+            const uint32_t e = 32 * v + (uint32_t)(__ffs(x) - 1);
+            if (v == warp) path |= (FULL << (cur & 31)) & (FULL >> (31 - (e & 31)));
+            const uint32_t nx = S.r_next[e];
+            if (nx >= T) {
+                last = e;
+                break;
+            }
+            if (nx == tl) pred = e;
+            cur = nx;
+        }
+        const bool mine = (path >> lane) & 1u;
+        // my tokens before my predecessor's meeting point are not the block's
+        const uint32_t skip = mine && tl ? T * S.r_j[pred] : 0u;
+        const uint32_t skipped = tokens_length<NW>(tok, skip);
+        const uint32_t len = mine ? P.out_len - skipped : 0u;
         uint32_t incl = len;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const uint32_t x = __shfl_up_sync(FULL, incl, d);
-            if (lane >= d) incl += x;
+            if ((int)lane >= d) incl += x;
         }
-        const uint32_t total = __shfl_sync(FULL, incl, 31);
-        if (max_block && block_n + total >= max_block) return CE_SIZE;
-        if (o.n + total > o.cap) return CE_OVERFLOW;
+        if (lane == 31) S.r_sum[warp] = incl;
+        if (tl == last) {
+            S.r_flags = P.st;
+            Bits b;
+            b.seek(S.bits, P.p);
+            S.r_end = P.p + (P.st == PS_EOB ? symbol_entry<NW>(S, b.x(), 0) & 31u : 0u);
+        }
+        team_sync<NW>();
+        uint32_t before = 0, total = 0;
+#pragma unroll
+        for (int v = 0; v < NW; ++v) {
+            const uint32_t x = S.r_sum[v];
+            if (v < (int)warp) before += x;
+            total += x;                                // lanes off the path add nothing
+        }
+        const uint32_t st = S.r_flags;
+        const uint64_t round_end = base + S.r_end;
+        int err = CE_OK;
+        if (st == PS_ERR) err = CE_DATA;
+        else if (max_block && block_n + total >= max_block) err = CE_SIZE;
+        else if (o.n + total > o.cap) err = CE_OVERFLOW;
+        if (err) {
+            // a false candidate is told by its literals before it is given more room
+            if (team_or<NW>(err == CE_OVERFLOW && check && mine && !tokens_allowed<NW>(S, tok, skip, n)))
+                return CE_BYTE;
+            return err;
+        }
         bool neg = false;
-        const bool ok = lane > last || expand_tokens(S, tb, my_vs, my_ve, o.sym, (uint32_t)o.n + incl - len, check, neg);
+        o.hi = max(o.hi, o.n + total);
+        // the round's start bits, in the lists' place if they fit
+        const uint32_t pos0 = (uint32_t)o.n, nw = (uint32_t)((o.n + total + 31) / 32 - o.n / 32);
+        uint32_t* sb = nw <= sizeof(S.list) / 4 ? reinterpret_cast<uint32_t*>(&S.list[0][0]) : nullptr;
+        if (sb) {
+            for (uint32_t k = tl; k < nw; k += T) sb[k] = 0;
+            team_sync<NW>();
+        }
+        const bool ok = write_map<NW>(S, tok, skip, mine ? n : skip, o.sym, o.start, sb, pos0,
+                                      pos0 + before + incl - len, check, neg);
+        const bool bad = team_or<NW>(!ok);
+        if (sb)
+            for (uint32_t k = tl; k < nw; k += T) {
+                uint32_t* g = o.start + (pos0 >> 5) + k;
+                if (k == 0 || k + 1 == nw) atomicOr(g, sb[k]);    // words shared with the rounds before and after
+                else *g = sb[k];
+            }
         o.neg |= neg;
-        if (__any_sync(FULL, !ok)) return CE_BYTE;
-        if (o.known && __any_sync(FULL, neg)) return CE_DIST;
+        if (bad) return CE_BYTE;
+        if (o.known && team_or<NW>(neg)) return CE_DIST;
         o.n += total;
         block_n += total;
-        __syncwarp();
         if (round_end > end_bit) return CE_TRUNC;
-        br.seek(round_end);
-        if (block_end) return CE_OK;
+        pos = round_end;
+        if (st == PS_EOB) {
+            ts.est = (uint32_t)min(round_end - block0, (uint64_t)0xfffffffu);
+            ts.segw_lim = min(kSegWords, 2 * ts.segw_lim + 1);
+            return CE_OK;
+        }
+        if (st == PS_CAP) ts.segw_lim = max(kSegWordsMin, segw / 2 | 1u);
     }
 }
 
-__device__ int stored_block(BitIn& br, OutState& o, bool check, const uint32_t* allowed, uint64_t end_bit,
-                            uint64_t& block_n, int lane) {
-    const uint64_t p = (br.pos() + 7) & ~7ull;
+// a stored block; pos is after its three header bits
+template <int NW>
+__device__ int stored_block(const Input& in, uint64_t& pos, OutState& o, bool check, const uint32_t* allowed,
+                            uint64_t end_bit, uint64_t& block_n) {
+    const uint64_t p = (pos + 7) & ~7ull;
     if (p + 32 > end_bit) return CE_TRUNC;
     const uint64_t byte = p >> 3;
-    const uint8_t* g = br.b;
+    const uint8_t* g = in.b;
     const uint32_t len = (uint32_t)__ldg(g + byte) | ((uint32_t)__ldg(g + byte + 1) << 8);
     const uint32_t nlen = (uint32_t)__ldg(g + byte + 2) | ((uint32_t)__ldg(g + byte + 3) << 8);
     if ((len ^ 0xffffu) != nlen) return CE_DATA;
     if (p + 32 + 8ull * len > end_bit) return CE_TRUNC;
     if (o.n + len > o.cap) return CE_OVERFLOW;
     bool bad = false;
-    for (uint32_t j = lane; j < len; j += 32) {
+    for (uint32_t j = threadIdx.x; j < len; j += 32 * NW) {
         const uint32_t v = __ldg(g + byte + 4 + j);
         if (check && !allowed_has(allowed, v)) bad = true;
         o.sym[o.n + j] = (uint16_t)v;
     }
-    if (__any_sync(FULL, bad)) return CE_BYTE;
+    if (len) {                                  // every position a start
+        const uint32_t a = (uint32_t)o.n, z = a + len;
+        for (uint32_t k = (a >> 5) + threadIdx.x; k <= (z - 1) >> 5; k += 32 * NW) {
+            const uint32_t lo = k == a >> 5 ? FULL << (a & 31u) : FULL, hi = k == (z - 1) >> 5 ? FULL >> (31u - ((z - 1) & 31u)) : FULL;
+            atomicOr(o.start + k, lo & hi);
+        }
+    }
+    o.hi = max(o.hi, o.n + len);
+    if (team_or<NW>(bad)) return CE_BYTE;
     o.n += len;
     block_n += len;
-    br.seek(p + 32 + 8ull * len);
-    __syncwarp();
+    pos = p + 32 + 8ull * len;
     return CE_OK;
 }
 
-// one block.  candidate: the block must be a non-final dynamic block (the
-// block-start checks); min/max_block bound its size; check: its literals must
-// be allowed bytes.  Huffman blocks are decoded by the whole warp in parallel
-// (par_block); a candidate block start first runs a short serial prefix, so
-// that false candidates fail after a few tokens.
-__device__ int one_block(WarpSmem& S, uint32_t* tokbuf, BitIn& br, OutState& o, bool check, uint64_t min_block,
-                         uint64_t max_block, bool candidate, uint64_t end_bit, uint32_t& final, int lane) {
-    br.refill();
-    final = br.peek(1);
-    const uint32_t type = br.peek(3) >> 1;
-    br.drop(3);
-    if (br.pos() > end_bit) return CE_TRUNC;
+// The block at bit `pos`, which moves past it.  candidate: the block must be a
+// non-final dynamic block (the block-start checks); min/max_block bound its
+// size; check: its literals must be allowed bytes.  Huffman blocks are decoded
+// by the whole team in parallel (par_block); a candidate block start first runs
+// a short serial prefix, so that false candidates fail after a few tokens.
+template <int NW>
+__device__ int one_block(TeamSmem<NW>& S, const Input& in, uint64_t& pos, TeamState& ts, OutState& o, bool check,
+                         uint64_t min_block, uint64_t max_block, bool candidate, uint64_t end_bit, uint32_t& final) {
+    const uint64_t s0 = pos >> 5, s1 = s0 + TeamSmem<NW>::kBits;
+    // a candidate's header and prefix first; its block's words follow if they pass
+    const uint32_t ns = candidate ? 256u : TeamSmem<NW>::kBits;
+    stage<NW>(S, in, s0, ns);
+    uint32_t at = (uint32_t)pos & 31u;
+    const uint32_t h = __funnelshift_r(S.bits[0], S.bits[1], at) & 7u;
+    final = h & 1u;
+    const uint32_t type = h >> 1;
+    pos += 3;
+    at += 3;
+    if (pos > end_bit) return CE_TRUNC;
     if (candidate) {
         if (final) return CE_FINAL;
         if (type != 2) return CE_TYPE;
     }
     uint64_t block_n = 0;
-    int st;
+    int st = CE_OK;
     if (type == 0) {
-        st = stored_block(br, o, check, S.allowed, end_bit, block_n, lane);
+        st = stored_block<NW>(in, pos, o, check, S.allowed, end_bit, block_n);
     } else if (type == 3) {
         st = CE_DATA;
     } else {
         if (type == 1) {
-            if (S.table_kind != 1) build_fixed(S, lane);
-            st = CE_OK;
+            if (S.table_kind != 1) build_fixed<NW>(S);
         } else {
-            st = read_dynamic<false>(S, br, lane);
-            if (st == CE_OK && br.pos() > end_bit) st = CE_TRUNC;
+            uint32_t bits = 0;
+            st = read_dynamic<NW>(S, at, &bits);
+            pos += bits;
+            at += bits;
+            if (st == CE_OK && pos > end_bit) st = CE_TRUNC;
         }
-        if (st == CE_OK && candidate) st = trial_prefix(S, br, end_bit);
-        if (st == CE_OK) st = par_block(S, tokbuf, br, o, check, max_block, end_bit, block_n, lane);
+        if (st == CE_OK && candidate) {
+            if (threadIdx.x < 32) {
+                const int t = trial_prefix<NW>(S, at);
+                if (threadIdx.x == 0) S.h_status = t;
+            }
+            team_sync<NW>();
+            st = S.h_status;
+            team_sync<NW>();
+        }
+        if (st == CE_OK)
+            st = par_block<NW>(S, in, s0, candidate ? s0 : s1, pos, ts, o, check, max_block, end_bit, block_n);
     }
     if (st == CE_OK && max_block && block_n >= max_block) st = CE_SIZE;
     if (st == CE_OK && block_n < min_block) st = CE_SIZE;
@@ -932,8 +993,8 @@ __device__ int one_block(WarpSmem& S, uint32_t* tokbuf, BitIn& br, OutState& o, 
 //     32 offsets of a lane;
 //  2. the code-length code is complete: sum of 2^-l over its lengths is 1,
 //     from a 512-entry table of three-field sums;
-//  3. the whole dynamic header is valid (the checks of read_dynamic<true>),
-//     32 listed offsets at a time, one per lane (hdr_ok_lane).
+//  3. the dynamic header is valid (the checks of read_lengths), up to 32 listed
+//     offsets at a time, one per lane (headers_ok).
 // The full block decode then follows in k_sync, lowest offset first.  Stages
 // 1-3 are implied by the complete checks, so no offset that passes those is
 // dropped here.
@@ -959,166 +1020,135 @@ __device__ uint32_t cl_complete(const uint16_t* kraft3, uint32_t w0, uint32_t w1
     return kr == 128u;
 }
 
-// The whole dynamic-header check of one candidate by one lane, with no
-// shared state (the checks of read_dynamic<true>): the code-length code is
-// decoded canonically from its lengths -- code length by comparing the next
-// 7 bits (MSB first) against the left-aligned limits of lengths 1..6, symbol
-// from the lengths' offsets and the symbols sorted by (length, value) -- and
-// the literal/length and distance length sets are checked as they are read.
-// The caller has already checked that the code-length code is complete.
-__device__ bool hdr_ok_lane(const FileDesc& F, uint64_t p) {
-    BitIn br;
-    br.setup(F.gz, F.gz_len);
-    br.seek(p + 3);
-    br.refill();
-    const uint32_t hlit = br.peek(5) + 257;
-    br.drop(5);
-    const uint32_t hdist = br.peek(5) + 1;
-    br.drop(5);
-    const uint32_t hclen = br.peek(4) + 4;
-    br.drop(4);
-    if (hlit > 286 || hdist > 30) return false;
-    uint64_t lens = 0;                                     // 3 bits per code-length symbol 0..18
-    br.refill();
+// The whole dynamic-header check of up to 32 candidates by one warp, one per
+// lane (mine: its bit of the staged words; the caller has checked that its
+// code-length code is complete).  The warp first builds each candidate's lookup
+// table of the code-length code, one candidate at a time (128 bytes: length,
+// symbol << 3), in tabs, candidate i's at i mod kTabs; then every lane reads its
+// candidate's lengths symbol by symbol, the checks of read_lengths made as they
+// come, nearly every false candidate failing long before its end.  Returns the
+// lanes whose headers are valid.
+__device__ uint32_t headers_ok(const uint32_t* bits, uint8_t* tabs, uint32_t kTabs, uint32_t n, uint32_t mine,
+                               uint64_t base_bit, uint64_t end_bit, int lane) {
+    uint32_t ok = 0;
+    for (uint32_t c0 = 0; c0 < n; c0 += kTabs) {
+        const uint32_t c1 = min(n, c0 + kTabs);
+        __syncwarp();
+        for (uint32_t c = c0; c < c1; ++c) {
+            Bits br;
+            br.seek(bits, __shfl_sync(FULL, mine, (int)c) + 3);
+            const uint32_t hclen = ((br.x() >> 10) & 15u) + 4;
+            br.drop(bits, 14);
+            const uint32_t f1 = br.x();
+            br.drop(bits, 30);
+            const uint32_t f2 = br.x();
+            uint32_t len = 0;                              // of symbol `lane`
 #pragma unroll
-    for (uint32_t k = 0; k < 19; ++k) {
-        if (k == 10) br.refill();
-        if (k < hclen) {
-            lens |= (uint64_t)br.peek(3) << (3 * c_clorder[k]);
-            br.drop(3);
+            for (uint32_t k = 0; k < 19; ++k)
+                if (lane == c_clorder[k] && k < hclen) len = (k < 10 ? f1 >> (3 * k) : f2 >> (3 * (k - 10))) & 7u;
+            uint32_t code = 0, prev = 0, first = 0;        // first code of my length
+            uint32_t rank = 0;
+#pragma unroll
+            for (uint32_t L = 1; L <= 7; ++L) {
+                const uint32_t m = __ballot_sync(FULL, len == L);
+                code = (code + prev) << 1;
+                prev = __popc(m);
+                if (len == L) {
+                    first = code;
+                    rank = __popc(m & ((1u << lane) - 1u));
+                }
+            }
+            uint8_t* tab = tabs + 128 * (c - c0);
+            if (len) {
+                const uint32_t lo = __brev(first + rank) >> (32 - len);
+                for (uint32_t v = lo; v < 128; v += 1u << len) tab[v] = (uint8_t)(len | (lane << 3));
+            }
         }
-    }
-    uint64_t cnt8 = 0;                                     // symbols of each length (8 bits per length)
-#pragma unroll
-    for (int t = 0; t < 19; ++t) {
-        const uint32_t l = (uint32_t)(lens >> (3 * t)) & 7u;
-        if (l) cnt8 += 1ull << (8 * l);
-    }
-    uint32_t first = 0, offs = 0, limA = 0, limB = 0xffff0000u;
-    uint64_t base8 = 0, next8 = 0;
-#pragma unroll
-    for (int l = 1; l <= 7; ++l) {
-        const uint32_t cprev = (uint32_t)(cnt8 >> (8 * (l - 1))) & 0xffu, c = (uint32_t)(cnt8 >> (8 * l)) & 0xffu;
-        first = (first + cprev) << 1;                     // first code of length l
-        const uint32_t lim = (first + c) << (7 - l);      // left-aligned end of the length-l codes
-        if (l <= 4) limA |= (lim > 255u ? 255u : lim) << (8 * (l - 1));
-        else if (l <= 6) limB |= (lim > 255u ? 255u : lim) << (8 * (l - 5));
-        base8 |= (uint64_t)((offs - first + 128u) & 0xffu) << (8 * l);
-        next8 |= (uint64_t)offs << (8 * l);
-        offs += c;
-    }
-    uint64_t slo = 0, shi = 0;                             // symbols sorted by (length, value), 5 bits each
-#pragma unroll
-    for (int t = 0; t < 19; ++t) {
-        const uint32_t l = (uint32_t)(lens >> (3 * t)) & 7u;
-        if (l) {
-            const uint32_t i = (uint32_t)(next8 >> (8 * l)) & 0xffu;
-            next8 += 1ull << (8 * l);
-            if (i < 12) slo |= (uint64_t)t << (5 * i);
-            else shi |= (uint64_t)t << (5 * (i - 12));
-        }
-    }
-    const uint32_t total = hlit + hdist;
-    uint32_t i = 0, prev = 0, kl = 0, kd = 0, nl = 0, nd = 0, ml = 0, md = 0;
-    bool eob = false;
-    while (i < total) {
-        br.refill();
-        const uint32_t v = __brev(br.peek(7)) >> 25;      // the next 7 bits, first bit most significant
-        const uint32_t vv = v * 0x01010101u;
-        const uint32_t l = 1u + ((__popc(__vcmpgeu4(vv, limA)) + __popc(__vcmpgeu4(vv, limB))) >> 3);
-        const uint32_t ix = ((uint32_t)(base8 >> (8 * l)) & 0xffu) - 128u + (v >> (7 - l));
-        const uint32_t sym = ix < 12 ? (uint32_t)(slo >> (5 * ix)) & 31u : (uint32_t)(shi >> (5 * (ix - 12))) & 31u;
-        br.drop(l);
-        uint32_t rep = 1, val;
-        if (sym < 16) {
-            val = sym;
-            prev = sym;
-        } else if (sym == 16) {
-            if (i == 0) return false;
-            val = prev;
-            rep = 3 + br.peek(2);
-            br.drop(2);
-        } else if (sym == 17) {
-            val = 0;
-            rep = 3 + br.peek(3);
-            br.drop(3);
-            prev = 0;
-        } else {
-            val = 0;
-            rep = 11 + br.peek(7);
-            br.drop(7);
-            prev = 0;
-        }
-        if (i + rep > total) return false;
-        if (val) {
+        __syncwarp();
+        bool go = (uint32_t)lane >= c0 && (uint32_t)lane < c1;
+        const uint8_t* tab = tabs + 128 * (go ? lane - c0 : 0);
+        Bits br;
+        br.seek(bits, mine + 3);
+        const uint32_t x0 = br.x();
+        const uint32_t hlit = (x0 & 31u) + 257, total = hlit + ((x0 >> 5) & 31u) + 1, hclen = ((x0 >> 10) & 15u) + 4;
+        go = go && hlit <= 286 && total - hlit <= 30;
+        br.seek(bits, go ? mine + 17 + 3 * hclen : 0);
+        bool good = go;
+        uint32_t i = 0, prev = 0, kl = 0, kd = 0;          // Kraft sums (units of 2^-15), codes of length 1 at bit 20
+        bool eob = false;
+        while (__any_sync(FULL, go)) {
+            const uint32_t x = br.x(), e = tab[x & 127u], l = e & 7u, sym = e >> 3, y = x >> l;
+            const uint32_t ex = sym < 16 ? 0u : (sym == 16 ? 2u : (sym == 17 ? 3u : 7u));
+            const uint32_t rep = (sym < 16 ? 1u : (sym == 18 ? 11u : 3u)) + (y & ((1u << ex) - 1u));
+            const uint32_t val = sym < 16 ? sym : (sym == 16 ? prev : 0u);
+            prev = val;
             const uint32_t e2 = i + rep;
-            const uint32_t nlit = i < hlit ? ((e2 < hlit ? e2 : hlit) - i) : 0u;
-            const uint32_t ndst = rep - nlit;
-            kl += nlit * (32768u >> val);
-            kd += ndst * (32768u >> val);
-            nl += nlit;
-            nd += ndst;
-            if (nlit && val > ml) ml = val;
-            if (ndst && val > md) md = val;
-            if (i <= 256 && 256 < e2) eob = true;
-            if (kl > 32768u || kd > 32768u) return false;
+            const uint32_t nlit = i < hlit ? min(e2, hlit) - i : 0u, w = val ? 32768u >> val : 0u;
+            const bool bad = (sym == 16 && i == 0) || e2 > total;
+            if (go) {
+                kl += nlit * w;
+                kd += (rep - nlit) * w;
+                eob |= val && i <= 256 && 256 < e2;
+                good = !bad && kl <= 32768u && kd <= 32768u;
+                i = e2;
+                go = good && i < total;
+            }
+            br.drop(bits, go ? l + ex : 0u);
         }
-        i += rep;
+        // complete, or one code of length 1 (a sum of one half can also be that of longer codes: the team's own
+        // check of the header tells), or no distance code at all
+        good = good && eob && (kl == 32768u || kl == 16384u) && (kd == 32768u || kd == 16384u || kd == 0);
+        ok |= __ballot_sync(FULL, good && base_bit + br.p <= end_bit);
     }
-    if (!eob) return false;
-    if (!(kl == 32768u || (nl == 1 && ml == 1))) return false;
-    if (!(kd == 32768u || nd == 0 || (nd == 1 && md == 1))) return false;
-    return br.pos() <= F.end_bit;
+    return ok;
 }
 
-// Search state of a part, kept by the caller between candidates: the next
-// window to filter, and a list of up to 32 filtered offsets (one per lane,
-// relative to the part's scan start) whose header checks are done.
-struct ScanState {
-    uint64_t next;       // first bit not yet filtered
-    uint64_t mine;       // this lane's list entry
-    uint32_t pass;       // list entries whose whole header passed, not yet returned
-};
+// One step of the search from bit `next`: each warp filters kScanWindows
+// consecutive windows of 1024 bits (each lane tests 32 offsets with bit masks,
+// then the completeness of the code-length code); the survivors are gathered,
+// one per lane, and their whole headers are checked at once, one per lane.  A
+// warp that finds valid headers stops there.  The results are in S.c_*: per warp
+// the offsets from T (the step's first window) whose headers are valid, lowest
+// first, and the bit where its search resumes.
 
-__device__ __forceinline__ void scan_begin(ScanState& st, uint64_t lo) {
-    st.next = lo;
-    st.mine = 0;
-    st.pass = 0;
-}
-
-// The next block-start candidate at or after the state's position, lowest
-// first: windows of 1024 bits are filtered (each lane tests 32 offsets with
-// bit masks, then the completeness of the code-length code); the survivors
-// are gathered, one per lane, until 32 are listed or the range ends, and then
-// all whole-header checks of the list run at once, one per lane.
-__device__ uint64_t find_candidate(const uint16_t* kraft3, const FileDesc& F, uint64_t lo, uint64_t hi, int lane,
-                                   ScanState& st) {
-    BitIn w;
-    w.setup(F.gz, F.gz_len);
-    if (hi > F.end_bit) hi = F.end_bit;
-    for (;;) {
-        if (st.pass) {
-            const int k = __ffs(st.pass) - 1;
-            st.pass &= st.pass - 1;
-            return lo + shfl64(st.mine, k);
-        }
-        if (st.next >= hi) return kNone;
-        uint32_t n = 0;                                    // entries listed
-        while (n < 32 && st.next < hi) {
-            const uint64_t T = st.next & ~1023ull;
+template <int NW>
+__device__ void scan_step(TeamSmem<NW>& S, const Input& in, uint64_t next, uint64_t hi, uint64_t end_bit) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr uint32_t kScanWindows = TeamSmem<NW>::kScanWindows;
+    constexpr uint32_t kWords = NW * kScanWindows * 32 + 148;      // the windows, and a header after the last bit
+    static_assert(kWords + 256 <= TeamSmem<NW>::kBits + 2, "a step's words are staged at once");
+    const uint64_t T0 = next & ~1023ull;
+    uint16_t* kraft3 = S.kraft3();
+    team_sync<NW>();
+    for (uint32_t v = threadIdx.x; v < 512; v += 32 * NW)
+        kraft3[v] = (uint16_t)(kraft1(v & 7) + kraft1((v >> 3) & 7) + kraft1(v >> 6));
+    stage<NW>(S, in, T0 >> 5, kWords);
+    const uint64_t lo_w = T0 + (uint64_t)warp * (kScanWindows * 1024u);
+    uint64_t end_w = min(hi, lo_w + kScanWindows * 1024u);
+    uint64_t at = max(next, lo_w);             // this warp's first bit not yet filtered
+    // the warps' header tables take the place between the step's words and the Kraft sums
+    constexpr uint32_t kTabs = (TeamSmem<NW>::kBits + 2 - 256 - kWords) / NW / 32;
+    static_assert(kTabs >= 4, "a header table is 32 words");
+    uint8_t* tabs = reinterpret_cast<uint8_t*>(S.bits + kWords + warp * (32 * kTabs));
+    uint32_t found = 0, mine = 0;
+    uint32_t pass = 0;
+    while (!pass && at < end_w) {
+        uint32_t n = 0;                        // offsets listed
+        while (n < 32 && at < end_w) {
+            const uint64_t T = at & ~1023ull;
             const uint64_t base = T + 32ull * (uint64_t)lane;
-            const uint64_t wi = base >> 5;
-            const uint32_t w0 = w.word(wi), w1 = w.word(wi + 1), w2 = w.word(wi + 2), w3 = w.word(wi + 3);
+            const uint32_t* wp = S.bits + (uint32_t)((base - T0) >> 5);
+            const uint32_t w0 = wp[0], w1 = wp[1], w2 = wp[2], w3 = wp[3];
             const uint64_t x = (uint64_t)w0 | ((uint64_t)w1 << 32);
             uint64_t y = ~x & ~(x >> 1) & (x >> 2);                // BFINAL = 0, BTYPE = 10
             y &= ~((x >> 4) & (x >> 5) & (x >> 6) & (x >> 7));     // HLIT <= 29
             y &= ~((x >> 9) & (x >> 10) & (x >> 11) & (x >> 12));  // HDIST <= 29
             uint32_t m = (uint32_t)y;
-            if (base < st.next) {
-                const uint64_t d = st.next - base;
+            if (base < at) {
+                const uint64_t d = at - base;
                 m = d >= 32 ? 0u : (m & (~0u << d));
             }
-            if (base + 32 > hi) m = base >= hi ? 0u : (m & ((1u << (uint32_t)(hi - base)) - 1u));
+            if (base + 32 > end_w) m = base >= end_w ? 0u : (m & ((1u << (uint32_t)(end_w - base)) - 1u));
             uint32_t c = 0;
             for (uint32_t mm = m; mm; mm &= mm - 1) {
                 const uint32_t k = __ffs(mm) - 1;
@@ -1131,67 +1161,94 @@ __device__ uint64_t find_candidate(const uint16_t* kraft3, const FileDesc& F, ui
                 const uint32_t cl = __shfl_sync(FULL, c, l);
                 const uint32_t k = __ffs(cl) - 1;
                 const uint64_t pos = T + 32ull * (uint64_t)l + k;
-                if (n == 32) {                            // full: this window resumes here
+                if (n == 32) {                                    // full: this window resumes here
                     resume = pos;
                     break;
                 }
                 if (lane == l) c &= c - 1;
-                if ((uint32_t)lane == n) st.mine = pos - lo;
+                if ((uint32_t)lane == n) mine = (uint32_t)(pos - T0);
                 ++n;
             }
-            st.next = resume < hi ? resume : hi;
+            at = resume;
         }
-        const bool ok = (uint32_t)lane < n && hdr_ok_lane(F, lo + st.mine);
-        st.pass = __ballot_sync(FULL, ok);
+        pass = headers_ok(S.bits, tabs, kTabs, n, mine, T0, end_bit, lane);
     }
+    constexpr uint32_t kCand = TeamSmem<NW>::kCand;
+    found = __popc(pass);
+    const uint32_t ix = __popc(pass & ((1u << lane) - 1u));
+    if (((pass >> lane) & 1u) && ix < kCand) S.c_at[warp][ix] = mine;
+    if (found > kCand) {                       // the search resumes at the first one left out
+        at = T0 + __shfl_sync(FULL, mine, (int)__fns(pass, 0, kCand + 1));
+        end_w = ~0ull;
+        found = kCand;
+    }
+    if (lane == 0) {
+        S.c_n[warp] = found;
+        S.c_done[warp] = at >= end_w;
+        S.c_resume[warp] = at;
+    }
+    team_sync<NW>();
 }
 
-__device__ __forceinline__ WarpSmem& warp_smem() {
+template <int NW>
+__device__ __forceinline__ TeamSmem<NW>& team_smem() {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    return reinterpret_cast<WarpSmem*>(smem_raw)[threadIdx.x >> 5];
+    return *reinterpret_cast<TeamSmem<NW>*>(smem_raw);
 }
 
-__device__ __forceinline__ void init_smem(WarpSmem& S, const KParams& p, int lane) {
-    if (lane < 8) S.allowed[lane] = p.allowed[lane];
-    if (lane == 0) S.table_kind = 0;
-    __syncwarp();
-}
-
-// pass-1 CTA shapes: warps per block and the blocks per SM the register
-// budget is set for (about 20 resident warps per SM, 96 registers a thread)
-constexpr int pass1_min_blocks(int wpb) { return wpb == 2 ? 10 : (wpb == 4 ? 5 : 2); }
-
-// Work queue of the pass-1 kernels: each resident warp takes the next queue
+// Work queue of the pass-1 kernels: each resident team takes the next queue
 // position until the parts run out, so parts of uneven work (many members of
-// different sizes in one launch) balance over the warps.  Position q holds
+// different sizes in one launch) balance over the teams.  Position q holds
 // part order[q] (the parts with the most expected output first, so that the
 // short ones fill the end of the launch), or part q without an order.  The
 // counter is zeroed on the stream before each launch.
-__device__ __forceinline__ int next_part(uint32_t* queue, int lane) {
-    uint32_t c = 0;
-    if (lane == 0) c = atomicAdd(queue, 1u);
-    return (int)min(__shfl_sync(FULL, c, 0), 0x7fffffffu);
+template <int NW>
+__device__ __forceinline__ int next_part(TeamSmem<NW>& S, uint32_t* queue) {
+    team_sync<NW>();
+    if (threadIdx.x == 0) S.q = (int)min(atomicAdd(queue, 1u), 0x7fffffffu);
+    team_sync<NW>();
+    return S.q;
+}
+
+template <int NW>
+__device__ __forceinline__ void init_smem(TeamSmem<NW>& S, const KParams& p) {
+    if (threadIdx.x < 8) S.allowed[threadIdx.x] = p.allowed[threadIdx.x];
+    if (threadIdx.x == 0) S.table_kind = 0;
+    team_sync<NW>();
 }
 
 // ---------------------------------------------------------------------------
 // k_sync: block start of each part and its first block; k_inflate: the rest of each part
 // ---------------------------------------------------------------------------
+template <int NW>
+__device__ __forceinline__ TeamState team_state(uint32_t* tok, const KParams& p, uint32_t est) {
+    return TeamState{tok + (uint64_t)blockIdx.x * (32 * NW) * p.tok_rows, p.tok_rows, est, TeamSmem<NW>::kSegWords};
+}
+
+// the start bits of a block that failed
+template <int NW>
+__device__ void clear_starts(OutState& o) {
+    team_sync<NW>();
+    for (uint64_t k = threadIdx.x; k < (o.hi + 31) / 32; k += 32 * NW) o.start[k] = 0;
+    o.hi = 0;
+    team_sync<NW>();
+}
+
 // The block start of part c and its first block (Section "Detection of DEFLATE block start positions").
-__device__ void sync_part(const uint16_t* kraft3, WarpSmem& S, uint32_t* tok, const FileDesc& F, ChunkDesc& C,
-                          uint16_t* symbuf, const KParams& p, int lane) {
-    init_smem(S, p, lane);
-    OutState o{symbuf + C.sym_base, C.cap, 0, C.index == 0 && C.lo <= F.s0_bit, false};
-    BitIn br;
-    br.setup(F.gz, F.gz_len);
+template <int NW>
+__device__ void sync_part(TeamSmem<NW>& S, const FileDesc& F, ChunkDesc& C, uint16_t* symbuf,
+                          uint32_t* start_bits, uint32_t* tok, const KParams& p) {
+    init_smem<NW>(S, p);
+    OutState o{symbuf + C.sym_base, start_bits + C.sym_base / 32, C.cap, 0, 0, C.index == 0 && C.lo <= F.s0_bit, false};
+    const Input in(F.gz, F.gz_len);
+    TeamState ts = team_state<NW>(tok, p, 0);
     uint32_t state = CS_EMPTY, err = CE_OK, final = 0;
     uint64_t sync = kNone, resume = 0;
     if (C.disabled) {
         state = CS_EMPTY;
     } else if (o.known || C.given) {          // the member start (empty context) or a known block start
-        br.seek(C.lo);
-        const int st = one_block(S, tok, br, o, false, 0, 0, false, F.end_bit, final, lane);
-        sync = C.lo;
-        resume = br.pos();
+        sync = resume = C.lo;
+        const int st = one_block<NW>(S, in, resume, ts, o, false, 0, 0, false, F.end_bit, final);
         if (st) {
             state = CS_ERROR;
             err = (uint32_t)st;
@@ -1199,32 +1256,49 @@ __device__ void sync_part(const uint16_t* kraft3, WarpSmem& S, uint32_t* tok, co
             state = CS_FOUND;
         }
     } else {
-        ScanState scan;
-        scan_begin(scan, C.lo);
-        for (;;) {
-            const uint64_t cand = find_candidate(kraft3, F, C.lo, C.hi, lane, scan);
-            if (cand == kNone) break;
-            br.seek(cand);
-            o.n = 0;
-            o.neg = false;
-            const int st = one_block(S, tok, br, o, true, p.min_block, p.max_block, true, F.end_bit, final,
-                                            lane);
-            if (st == CE_OK) {
-                state = CS_FOUND;
-                sync = cand;
-                resume = br.pos();
-                break;
+        const uint64_t hi = min(C.hi, F.end_bit);
+        uint64_t next = C.lo;
+        bool go = true;
+        while (go && next < hi) {
+            scan_step<NW>(S, in, next, hi, F.end_bit);
+            const uint64_t T0 = next & ~1023ull;
+            next = T0 + NW * TeamSmem<NW>::kScanWindows * 1024ull;
+            for (int w = 0; w < NW && go; ++w) {
+                const uint32_t n = S.c_n[w];
+                for (uint32_t k = 0; k < n; ++k) {
+                    const uint64_t cand = T0 + S.c_at[w][k];
+                    uint64_t pos = cand;
+                    o.n = 0;
+                    o.neg = false;
+                    ts = team_state<NW>(tok, p, 0);
+                    const int st = one_block<NW>(S, in, pos, ts, o, true, p.min_block, p.max_block, true, F.end_bit,
+                                                 final);
+                    if (st == CE_OK) {
+                        state = CS_FOUND;
+                        sync = cand;
+                        resume = pos;
+                        go = false;
+                        break;
+                    }
+                    clear_starts<NW>(o);
+                    if (st == CE_OVERFLOW) {     // the candidate's block does not fit: cannot judge it here
+                        state = CS_ERROR;
+                        err = CE_OVERFLOW;
+                        sync = cand;
+                        go = false;
+                        break;
+                    }
+                }
+                if (go && !S.c_done[w]) {        // that warp's search stopped short: the next step starts there
+                    next = S.c_resume[w];
+                    break;
+                }
             }
-            if (st == CE_OVERFLOW) {             // the candidate's block does not fit: cannot judge it here
-                state = CS_ERROR;
-                err = CE_OVERFLOW;
-                sync = cand;
-                break;
-            }
+            team_sync<NW>();                     // S.c_* may be rewritten
         }
     }
-    const bool neg = __any_sync(FULL, o.neg);
-    if (lane == 0) {
+    const bool neg = team_or<NW>(o.neg);
+    if (threadIdx.x == 0) {
         C.err = err;
         C.sync = sync;
         C.resume = resume;
@@ -1239,7 +1313,6 @@ __device__ void sync_part(const uint16_t* kraft3, WarpSmem& S, uint32_t* tok, co
         C.end = resume;
         C.state = state;
     }
-    __syncwarp();
 }
 
 // Where part c's decoding stops: the start of the next part that holds one (`sync` is final after k_sync and
@@ -1254,12 +1327,14 @@ __device__ __forceinline__ uint64_t find_stop(const FileDesc& F, const ChunkDesc
 }
 
 // Pass 1 of part c from the end of its first block up to the next part's block start.
-__device__ void inflate_part(WarpSmem& S, uint32_t* tok, const FileDesc* __restrict__ files, ChunkDesc* chunks, int c,
-                             uint16_t* symbuf, const KParams& p, int lane) {
+template <int NW>
+__device__ void inflate_part(TeamSmem<NW>& S, const FileDesc* __restrict__ files, ChunkDesc* chunks, int c,
+                             uint16_t* symbuf, uint32_t* start_bits, uint32_t* tok, const KParams& p) {
     ChunkDesc& C = chunks[c];
     if (C.state != CS_FOUND) return;
     if (C.probe) {                    // a streamed segment's end: the block start found is all it gives
-        if (lane == 0) {
+        team_sync<NW>();
+        if (threadIdx.x == 0) {
             C.state = CS_DONE;
             C.n = 0;
             C.anyph = 0;
@@ -1268,12 +1343,11 @@ __device__ void inflate_part(WarpSmem& S, uint32_t* tok, const FileDesc* __restr
             C.confirmed = 0;
             C.end = C.sync;
         }
-        __syncwarp();
         return;
     }
     const FileDesc& F = files[C.file];
     const uint64_t stop = find_stop(F, chunks, c, C.stop_hint);
-    OutState o{symbuf + C.sym_base, C.cap, C.n, C.index == 0 && C.sync == F.s0_bit, false};
+    OutState o{symbuf + C.sym_base, start_bits + C.sym_base / 32, C.cap, C.n, C.n, C.index == 0 && C.sync == F.s0_bit, false};
     uint32_t blocks = C.blocks, final = C.final, err = CE_OK, confirmed = C.confirmed;
     uint64_t end = C.resume;
     // the confirmation (Section "Detection of DEFLATE block start positions") covers the start's block and
@@ -1282,17 +1356,17 @@ __device__ void inflate_part(WarpSmem& S, uint32_t* tok, const FileDesc* __restr
     if (final) {
         if (stop != kNone && !F.open_end) err = CE_CHAIN;
     } else if (!(stop != kNone && C.resume == stop) || (C.confirm_ext && !confirmed)) {
-        init_smem(S, p, lane);
-        BitIn br;
-        br.setup(F.gz, F.gz_len);
-        br.seek(C.resume);
+        init_smem<NW>(S, p);
+        TeamState ts = team_state<NW>(tok, p, (uint32_t)min(C.resume - C.sync, (uint64_t)0xfffffffu));
+        const Input in(F.gz, F.gz_len);
+        uint64_t bit = C.resume;
         // past the stop (confirm_ext): blocks decoded only to finish the confirmation; the part's own
         // output, end and status are those at the stop
         bool past = false;
         uint32_t err_stop = CE_OK;
         uint64_t n_stop = 0, end_stop = 0;
         for (;;) {
-            const uint64_t pos = br.pos();
+            const uint64_t pos = bit;
             if (!past && stop != kNone && pos >= stop) {
                 err_stop = pos != stop ? (uint32_t)CE_CHAIN : (uint32_t)CE_OK;
                 if (!C.confirm_ext || blocks >= window) {
@@ -1306,7 +1380,7 @@ __device__ void inflate_part(WarpSmem& S, uint32_t* tok, const FileDesc* __restr
             if (past && blocks >= window) break;
             const bool check = !o.known && blocks < window;
             uint32_t fin = 0;
-            const int st = one_block(S, tok, br, o, check, 0, 0, false, F.end_bit, fin, lane);
+            const int st = one_block<NW>(S, in, bit, ts, o, check, 0, 0, false, F.end_bit, fin);
             if (st) {
                 err = (check && st != CE_OVERFLOW) ? (uint32_t)CE_CONFIRM : (uint32_t)st;
                 break;
@@ -1320,7 +1394,7 @@ __device__ void inflate_part(WarpSmem& S, uint32_t* tok, const FileDesc* __restr
                 break;
             }
         }
-        end = br.pos();
+        end = bit;
         if (blocks >= window && err != CE_CONFIRM) confirmed = 1;
         if (past) {
             if (err == CE_OK) err = err_stop;
@@ -1330,11 +1404,11 @@ __device__ void inflate_part(WarpSmem& S, uint32_t* tok, const FileDesc* __restr
             }
         }
     }
-    const bool neg = __any_sync(FULL, o.neg);
+    const bool neg = team_or<NW>(o.neg);
     if (err == CE_OK && final && F.mode != 2 && !F.open_end) {   // the trailer must follow the final block
         if (((end + 7) >> 3) + 8 != F.gz_len) err = CE_TRAIL;
     }
-    if (lane == 0) {
+    if (threadIdx.x == 0) {
         C.state = err ? CS_ERROR : CS_DONE;
         C.err = err;
         C.n = o.n;
@@ -1344,41 +1418,35 @@ __device__ void inflate_part(WarpSmem& S, uint32_t* tok, const FileDesc* __restr
         C.confirmed = confirmed;
         C.end = end;
     }
-    __syncwarp();
 }
 
-// Work queue over the parts (one per warp at a time), for both kernels.
-template <int WPB>
-__global__ void __launch_bounds__(32 * WPB, pass1_min_blocks(WPB))
-    k_sync(const FileDesc* __restrict__ files, ChunkDesc* chunks, int nchunks, uint16_t* symbuf, uint32_t* tokbuf,
-           uint32_t* queue, const uint32_t* __restrict__ order, KParams p) {
-    __shared__ uint16_t kraft3[512];
-    for (uint32_t v = threadIdx.x; v < 512; v += blockDim.x)
-        kraft3[v] = (uint16_t)(kraft1(v & 7) + kraft1((v >> 3) & 7) + kraft1(v >> 6));
-    __syncthreads();
-    WarpSmem& S = warp_smem();
-    const int lane = threadIdx.x & 31;
-    uint32_t* tok = tokbuf + (uint64_t)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kTokPerPart;
+// Launch bounds of the pass-1 kernels: 64 registers a thread; shared memory then holds 7 teams of 4 warps per SM,
+// 4 of 8, 2 of 16.
+constexpr int pass1_min_blocks(int nw) { return 32 / nw; }
+
+template <int NW>
+__global__ void __launch_bounds__(32 * NW, pass1_min_blocks(NW))
+    k_sync(const FileDesc* __restrict__ files, ChunkDesc* chunks, int nchunks, uint16_t* symbuf, uint32_t* start_bits,
+           uint32_t* tok, uint32_t* queue, const uint32_t* __restrict__ order, KParams p) {
+    TeamSmem<NW>& S = team_smem<NW>();
     for (;;) {
-        const int q = next_part(queue, lane);
+        const int q = next_part<NW>(S, queue);
         if (q >= nchunks) return;
         const int c = order ? (int)__ldg(order + q) : q;
-        sync_part(kraft3, S, tok, files[chunks[c].file], chunks[c], symbuf, p, lane);
+        sync_part<NW>(S, files[chunks[c].file], chunks[c], symbuf, start_bits, tok, p);
     }
 }
 
-template <int WPB>
-__global__ void __launch_bounds__(32 * WPB, pass1_min_blocks(WPB))
-    k_inflate(const FileDesc* __restrict__ files, ChunkDesc* chunks, int nchunks, uint16_t* symbuf, uint32_t* tokbuf,
-              uint32_t* queue, const uint32_t* __restrict__ order, KParams p) {
-    WarpSmem& S = warp_smem();
-    const int lane = threadIdx.x & 31;
-    uint32_t* tok = tokbuf + (uint64_t)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kTokPerPart;
+template <int NW>
+__global__ void __launch_bounds__(32 * NW, pass1_min_blocks(NW))
+    k_inflate(const FileDesc* __restrict__ files, ChunkDesc* chunks, int nchunks, uint16_t* symbuf, uint32_t* start_bits,
+              uint32_t* tok, uint32_t* queue, const uint32_t* __restrict__ order, KParams p) {
+    TeamSmem<NW>& S = team_smem<NW>();
     for (;;) {
-        const int q = next_part(queue, lane);
+        const int q = next_part<NW>(S, queue);
         if (q >= nchunks) return;
         const int c = order ? (int)__ldg(order + q) : q;
-        inflate_part(S, tok, files, chunks, c, symbuf, p, lane);
+        inflate_part<NW>(S, files, chunks, c, symbuf, start_bits, tok, p);
     }
 }
 
@@ -1386,7 +1454,9 @@ __global__ void __launch_bounds__(32 * WPB, pass1_min_blocks(WPB))
 // k_exec: the copy map of each part into its symbols, in place
 // ---------------------------------------------------------------------------
 // One block of NT threads per part, in passes of 8 NT positions (a thread takes
-// 8 consecutive ones: one 16-byte load, one 16-byte store).  The last 32 KiB of
+// 8 consecutive ones: one 16-byte load, one 16-byte store; a warp's 256 begin at
+// a multiple of kRestart, so the code in force at each comes from the start
+// bits and codes of its own lanes).  The last 32 KiB of
 // the part's symbols and the pass itself live in a ring in shared memory
 // (32768 + 8 NT u16 entries, so that a pass never overwrites a source it can
 // still need).  A position's entry is its symbol when the source lies before the
@@ -1408,13 +1478,15 @@ constexpr size_t exec_smem() { return (kWin + 8 * NT) * sizeof(uint16_t); }
 
 template <int NT>
 __global__ void __launch_bounds__(NT, NT == 1024 ? 1 : (NT == 512 ? 2 : 3))
-    k_exec(const FileDesc* __restrict__ files, ChunkDesc* chunks, int nchunks, uint16_t* symbuf, uint32_t* queue,
-           const uint32_t* __restrict__ order, int tail) {
+    k_exec(const FileDesc* __restrict__ files, ChunkDesc* chunks, int nchunks, uint16_t* symbuf,
+           const uint32_t* __restrict__ start_bits, uint32_t* queue, const uint32_t* __restrict__ order, int tail) {
     extern __shared__ __align__(16) uint16_t ring[];
     __shared__ int s_q;
     constexpr uint32_t P = 8 * NT, R = kWin + P;
     static_assert(R % P == 0 && P <= kPtr, "whole passes in the ring, indices in 14 bits");
+    static_assert(kRestart == 256, "a warp's positions of a pass");
     const uint32_t t8 = 8u * threadIdx.x;
+    const uint32_t below = (1u << (threadIdx.x & 31)) - 1u;
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0) s_q = (int)min(atomicAdd(queue, 1u), 0x7fffffffu);
@@ -1429,33 +1501,49 @@ __global__ void __launch_bounds__(NT, NT == 1024 ? 1 : (NT == 512 ? 2 : 3))
         // symbol as u16 (its caller asks for the symbols themselves)
         const bool track = tail && files[C.file].mode != 1;
         uint32_t det = 0xffffffffu, ph_end = 0;      // tail start; end of the last pass that held a placeholder
-        uint4 nx = t8 < n ? *reinterpret_cast<const uint4*>(sym + t8) : make_uint4(0, 0, 0, 0);
+        const uint8_t* start = reinterpret_cast<const uint8_t*>(start_bits) + C.sym_base / 8;
+        uint4 nx = make_uint4(0, 0, 0, 0);
+        uint32_t nst = 0;
+        if (t8 < n) {
+            nx = *reinterpret_cast<const uint4*>(sym + t8);
+            nst = start[t8 >> 3];
+        }
         uint32_t sA = 0;                             // ring slot of the pass's first position
         for (uint32_t A = 0; A < n; A += P) {
             const uint32_t p0 = A + t8;
-            const uint4 cur = nx;
-            if (p0 + P < n) nx = *reinterpret_cast<const uint4*>(sym + p0 + P);
-            const uint32_t w4[4] = {cur.x, cur.y, cur.z, cur.w};
-            uint32_t e[8];
+            const uint32_t w4[4] = {nx.x, nx.y, nx.z, nx.w}, st = nst;
+            if (p0 + P < n) {
+                nx = *reinterpret_cast<const uint4*>(sym + p0 + P);
+                nst = start[(p0 + P) >> 3];
+            } else {
+                nst = 0;
+            }
+            // the last code of the lanes below is in force at my first position
+            const uint32_t top = st ? 31u - __clz(st) : 0u, tw = w4[0], th = 16u * (top & 1u);
+            const uint32_t mine = (top < 4 ? (top < 2 ? tw : w4[1]) : (top < 6 ? w4[2] : w4[3])) >> th;
+            const uint32_t has = __ballot_sync(FULL, st != 0) & below;
+            uint32_t v = __shfl_sync(FULL, mine, has ? 31 - __clz(has) : 0) & 0xffffu;
+            uint32_t e[8], slot[8];
             uint32_t open = 0;                       // bit u: e[u] is a pointer into the pass
+            // (selections, not branches: the eight loads of a thread are in flight together, here and below)
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const uint32_t v = (u & 1) ? w4[u >> 1] >> 16 : w4[u >> 1] & 0xffffu;
-                e[u] = v;
-                if (p0 + (uint32_t)u >= n) {
-                    e[u] = 0;
-                } else if (v & kPH) {
-                    const int32_t rel = (int32_t)(t8 + u) - (int32_t)(v & 0x7fffu) - 1;   // source, from A
-                    if (rel >= 0) {
-                        e[u] = kPtr | (uint32_t)rel;
-                        open |= 1u << u;
-                    } else if ((int32_t)A + rel < 0) {
-                        e[u] = kPH | (uint32_t)((int32_t)kWin + (int32_t)A + rel);
-                    } else {
-                        int32_t slot = (int32_t)sA + rel;
-                        if (slot < 0) slot += (int32_t)R;
-                        e[u] = ring[slot];
-                    }
+                if ((st >> u) & 1u) v = (u & 1) ? w4[u >> 1] >> 16 : w4[u >> 1] & 0xffffu;
+                e[u] = p0 + (uint32_t)u < n ? v : 0u;
+                const int32_t rel = (int32_t)(t8 + u) - (int32_t)(e[u] & 0x7fffu) - 1;   // a match's source, from A
+                const int32_t a = (int32_t)sA + rel;
+                slot[u] = (e[u] & kPH) && rel < 0 ? (uint32_t)(a < 0 ? a + (int32_t)R : a) : sA;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) slot[u] = ring[slot[u]];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (e[u] & kPH) {
+                    const int32_t rel = (int32_t)(t8 + u) - (int32_t)(e[u] & 0x7fffu) - 1;
+                    const bool in = rel >= 0;
+                    open |= in ? 1u << u : 0u;
+                    e[u] = in ? kPtr | (uint32_t)rel
+                              : ((int32_t)A + rel < 0 ? kPH | (uint32_t)((int32_t)kWin + (int32_t)A + rel) : slot[u]);
                 }
             }
             uint4 v4;
@@ -1466,20 +1554,19 @@ __global__ void __launch_bounds__(NT, NT == 1024 ? 1 : (NT == 512 ? 2 : 3))
             *reinterpret_cast<uint4*>(ring + sA + t8) = v4;
             __syncthreads();
             volatile uint16_t* pass = ring + sA;
-            if (open) {
-                while (open) {
+            while (__any_sync(FULL, open)) {
 #pragma unroll
-                    for (int u = 0; u < 8; ++u)
-                        if ((open >> u) & 1u) {
-                            e[u] = pass[e[u] & (kPtr - 1u)];
-                            pass[t8 + u] = (uint16_t)e[u];
-                            if ((e[u] >> 14) != 1u) open &= ~(1u << u);
-                        }
+                for (int u = 0; u < 8; ++u) slot[u] = pass[(open >> u) & 1u ? e[u] & (kPtr - 1u) : t8 + u];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    e[u] = (open >> u) & 1u ? slot[u] : e[u];
+                    if ((e[u] >> 14) != 1u) open &= ~(1u << u);
                 }
                 v4.x = e[0] | (e[1] << 16);
                 v4.y = e[2] | (e[3] << 16);
                 v4.z = e[4] | (e[5] << 16);
                 v4.w = e[6] | (e[7] << 16);
+                *reinterpret_cast<uint4*>(ring + sA + t8) = v4;   // a thread's entries change only by its own hand
             }
             if (det == 0xffffffffu && track && A >= ph_end + kWin) det = A;
             if (track) {
@@ -2183,29 +2270,23 @@ void launch_sequences(const uint16_t* sym, uint64_t n, uint32_t min_len, uint64_
     k_sequences<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(sym, n, min_len, spans, max_spans, counts);
 }
 
-static size_t warp_smem_bytes() { return sizeof(WarpSmem); }
-
-static int wpb_of(const KParams& p) { return p.wpb == 2 || p.wpb == 8 ? p.wpb : 4; }
-static int wpb_slot(int wpb) { return wpb == 2 ? 0 : (wpb == 4 ? 1 : 2); }
-
-// resident blocks of the pass-1 kernels of a CTA shape on the current device
-// (both kernels have the same launch bounds and shared memory); also raises
-// the kernels' dynamic shared-memory limit once
-template <int WPB>
-static int pass1_resident_blocks_t() {
+// resident teams of a size on the current device (both pass-1 kernels have the same launch bounds and shared
+// memory); also raises the kernels' dynamic shared-memory limit once
+template <int NW>
+static int pass1_resident_t() {
     static int cached[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     const int slot = dev >= 0 && dev < 64 ? dev : 0;
     if (!cached[slot]) {
-        const int smem = (int)(WPB * warp_smem_bytes());
+        const int smem = (int)sizeof(TeamSmem<NW>);
         int sms = 0, per_sm_a = 0, per_sm_b = 0;
         const bool ok =
-            cudaFuncSetAttribute(k_sync<WPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
-            cudaFuncSetAttribute(k_inflate<WPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+            cudaFuncSetAttribute(k_sync<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+            cudaFuncSetAttribute(k_inflate<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_a, k_sync<WPB>, 32 * WPB, smem) == cudaSuccess &&
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_b, k_inflate<WPB>, 32 * WPB, smem) == cudaSuccess;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_a, k_sync<NW>, 32 * NW, smem) == cudaSuccess &&
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_b, k_inflate<NW>, 32 * NW, smem) == cudaSuccess;
         const int v = std::max(1, sms) * std::max(1, std::min(per_sm_a, per_sm_b));
         if (!ok) {
             cudaGetLastError();
@@ -2216,53 +2297,72 @@ static int pass1_resident_blocks_t() {
     return cached[slot];
 }
 
-static int pass1_resident_blocks(int wpb) {
-    switch (wpb_slot(wpb)) {
-        case 0: return pass1_resident_blocks_t<2>();
-        case 1: return pass1_resident_blocks_t<4>();
-        default: return pass1_resident_blocks_t<8>();
+static int pass1_resident(int nw) {
+    switch (nw) {
+        case 2: return pass1_resident_t<2>();
+        case 8: return pass1_resident_t<8>();
+        case 16: return pass1_resident_t<16>();
+        default: return pass1_resident_t<4>();
     }
 }
 
-int pass1_warps(int nchunks, int wpb) {
-    if (nchunks <= 0) return 0;
-    wpb = wpb == 2 || wpb == 8 ? wpb : 4;
-    const int blocks = std::min((nchunks + wpb - 1) / wpb, pass1_resident_blocks(wpb));
-    return blocks * wpb;
+// Rows of the teams' token buffers: twice the tokens of a segment of ordinary text (about 8 bits each).  Data of
+// fewer bits a token ends its rounds early and shortens its segments.
+static uint32_t team_rows(int nw) { return nw <= 8 ? 384 : 256; }
+
+// Warps per part: with few parts the largest team whose launch still holds every part at once (the time of a part
+// falls with its team's size: 8 parts of a 1 MiB file take 0.25 ms of block-start search and 0.2 ms of decoding with
+// teams of 16, against 0.86 and 1.36 ms with one warp each); with more parts than that the configured size, whose
+// rounds spend less on lanes left over.
+int pass1_team(int nchunks, int wpb) {
+    const int base = wpb == 2 || wpb == 8 ? wpb : 4;
+    for (int nw = 16; nw > base; nw >>= 1)
+        if (nchunks <= pass1_resident(nw)) return nw;
+    return base;
 }
 
-template <int WPB>
+int pass1_parts(int wpb) { return pass1_resident(wpb == 2 || wpb == 8 ? wpb : 4); }
+
+static int pass1_grid(int nchunks, int nw) { return std::min(nchunks, pass1_resident(nw)); }
+
+uint64_t token_words(int nchunks, int wpb) {
+    if (nchunks <= 0) return 0;
+    const int nw = pass1_team(nchunks, wpb);
+    return (uint64_t)pass1_grid(nchunks, nw) * 32 * nw * team_rows(nw);
+}
+
+template <int NW>
 static void launch_pass1_t(bool sync, const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym,
-                         uint32_t* tok, uint32_t* queue, const uint32_t* order, const KParams& p, cudaStream_t s) {
-    const int grid = pass1_warps(nchunks, WPB) / WPB;
-    const size_t smem = WPB * warp_smem_bytes();
-    if (sync) k_sync<WPB><<<grid, 32 * WPB, smem, s>>>(files, chunks, nchunks, sym, tok, queue, order, p);
-    else k_inflate<WPB><<<grid, 32 * WPB, smem, s>>>(files, chunks, nchunks, sym, tok, queue, order, p);
+                           uint32_t* start, uint32_t* tok, uint32_t* queue, const uint32_t* order, const KParams& p, cudaStream_t s) {
+    const int grid = pass1_grid(nchunks, NW);
+    KParams q = p;
+    if (!p.team) q.tok_rows = team_rows(NW);
+    if (sync) k_sync<NW><<<grid, 32 * NW, sizeof(TeamSmem<NW>), s>>>(files, chunks, nchunks, sym, start, tok, queue, order, q);
+    else k_inflate<NW><<<grid, 32 * NW, sizeof(TeamSmem<NW>), s>>>(files, chunks, nchunks, sym, start, tok, queue, order, q);
 }
 
 static void launch_pass1_any(bool sync, const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym,
-                             uint32_t* tok, uint32_t* queue, const uint32_t* order, const KParams& p,
+                             uint32_t* start, uint32_t* tok, uint32_t* queue, const uint32_t* order, const KParams& p,
                              cudaStream_t s) {
     if (nchunks <= 0) return;
     cudaMemsetAsync(queue, 0, sizeof(uint32_t), s);
-    switch (wpb_slot(wpb_of(p))) {
-        case 0: launch_pass1_t<2>(sync, files, chunks, nchunks, sym, tok, queue, order, p, s); break;
-        case 1: launch_pass1_t<4>(sync, files, chunks, nchunks, sym, tok, queue, order, p, s); break;
-        default: launch_pass1_t<8>(sync, files, chunks, nchunks, sym, tok, queue, order, p, s); break;
+    switch (p.team ? p.team : pass1_team(nchunks, p.wpb)) {
+        case 2: launch_pass1_t<2>(sync, files, chunks, nchunks, sym, start, tok, queue, order, p, s); break;
+        case 8: launch_pass1_t<8>(sync, files, chunks, nchunks, sym, start, tok, queue, order, p, s); break;
+        case 16: launch_pass1_t<16>(sync, files, chunks, nchunks, sym, start, tok, queue, order, p, s); break;
+        default: launch_pass1_t<4>(sync, files, chunks, nchunks, sym, start, tok, queue, order, p, s); break;
     }
 }
 
-void launch_sync(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* tok,
+void launch_sync(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* start, uint32_t* tok,
                  uint32_t* queue, const uint32_t* order, const KParams& p, cudaStream_t s) {
-    launch_pass1_any(true, files, chunks, nchunks, sym, tok, queue, order, p, s);
+    launch_pass1_any(true, files, chunks, nchunks, sym, start, tok, queue, order, p, s);
 }
 
-void launch_inflate(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* tok,
-                    uint32_t* queue, const uint32_t* order, const KParams& p, cudaStream_t s) {
-    launch_pass1_any(false, files, chunks, nchunks, sym, tok, queue, order, p, s);
+void launch_inflate(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* start,
+                    uint32_t* tok, uint32_t* queue, const uint32_t* order, const KParams& p, cudaStream_t s) {
+    launch_pass1_any(false, files, chunks, nchunks, sym, start, tok, queue, order, p, s);
 }
-
-uint64_t token_words_per_part() { return kTokPerPart; }
 
 // k_exec's resident blocks on the current device (0 if it cannot be asked)
 template <int NT>
@@ -2284,19 +2384,19 @@ static int exec_resident() {
 }
 
 template <int NT>
-static void launch_exec_t(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* queue,
+static void launch_exec_t(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* start, uint32_t* queue,
                           const uint32_t* order, const KParams& p, cudaStream_t s) {
     const int cap = std::max(1, exec_resident<NT>());
-    k_exec<NT><<<std::min(nchunks, cap), NT, exec_smem<NT>(), s>>>(files, chunks, nchunks, sym, queue, order, p.tail);
+    k_exec<NT><<<std::min(nchunks, cap), NT, exec_smem<NT>(), s>>>(files, chunks, nchunks, sym, start, queue, order, p.tail);
 }
 
-void launch_exec(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* queue,
+void launch_exec(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* start, uint32_t* queue,
                  const uint32_t* order, const KParams& p, cudaStream_t s) {
     if (nchunks <= 0) return;
     cudaMemsetAsync(queue, 0, sizeof(uint32_t), s);
     // up to one block per SM, the block of 1024 threads: half the passes, so half the barriers, of a part
-    if (nchunks <= exec_resident<1024>()) launch_exec_t<1024>(files, chunks, nchunks, sym, queue, order, p, s);
-    else launch_exec_t<512>(files, chunks, nchunks, sym, queue, order, p, s);
+    if (nchunks <= exec_resident<1024>()) launch_exec_t<1024>(files, chunks, nchunks, sym, start, queue, order, p, s);
+    else launch_exec_t<512>(files, chunks, nchunks, sym, start, queue, order, p, s);
 }
 
 void launch_plan(FileDesc* files, ChunkDesc* chunks, int nfiles, cudaStream_t s) {

@@ -54,10 +54,11 @@ constexpr size_t kOffWindows = a256(kOffSeg0 + sizeof(uint64_t));
 constexpr size_t kOffGmaps = a256(kOffWindows + (size_t)kNaMaxParts * kWin);
 constexpr size_t kOffWstart = a256(kOffGmaps + (size_t)kNaMaxGroups * kWin * sizeof(uint16_t));
 constexpr size_t kOffSym = a256(kOffWstart + (size_t)kNaMaxGroups * kWin);
-constexpr size_t kTokWords = 32 * 512;                // token buffer of one part (parallel block decoder)
-constexpr size_t kOffTok = a256(kOffSym + kNaSymbols * sizeof(uint16_t));
+constexpr size_t kOffStart = a256(kOffSym + kNaSymbols * sizeof(uint16_t));
+constexpr size_t kTokWords = 32 * 512;                // token rows of one of kNaMaxParts parts
+constexpr size_t kOffTok = a256(kOffStart + kNaSymbols / 8);
 constexpr size_t kOffQueue = a256(kOffTok + (size_t)kNaMaxParts * kTokWords * sizeof(uint32_t));
-constexpr size_t kScratchBytes = a256(kOffQueue + 3 * sizeof(uint32_t));   // about 23 MiB
+constexpr size_t kScratchBytes = a256(kOffQueue + 3 * sizeof(uint32_t));   // about 24 MiB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -156,9 +157,9 @@ extern "C" int pgz_decompress_noalloc(const uint8_t* gz, uint64_t gz_len, uint8_
     uint16_t* d_gmaps = reinterpret_cast<uint16_t*>(base + kOffGmaps);
     uint8_t* d_wstart = base + kOffWstart;
     uint16_t* d_sym = reinterpret_cast<uint16_t*>(base + kOffSym);
+    uint32_t* d_start = reinterpret_cast<uint32_t*>(base + kOffStart);
     uint32_t* d_tok = reinterpret_cast<uint32_t*>(base + kOffTok);
     uint32_t* d_queue = reinterpret_cast<uint32_t*>(base + kOffQueue);
-    if (token_words_per_part() != kTokWords || pass1_warps(kNaMaxParts, 4) > kNaMaxParts) return PGZ_E_ARG;
 
     KParams kp{};
     pgz_config cfg;
@@ -180,7 +181,7 @@ extern "C" int pgz_decompress_noalloc(const uint8_t* gz, uint64_t gz_len, uint8_
     for (int attempt = 0; attempt <= kNaMaxRetries; ++attempt) {
         if (replan) {                                  // n parts of equal compressed size
             const uint64_t per = (csize + n - 1) / n;
-            const uint64_t cap = (kNaSymbols / n) / 8 * 8;
+            const uint64_t cap = (kNaSymbols / n) / 32 * 32;
             memset(plan, 0, sizeof plan);
             for (uint64_t i = 0; i < n; ++i) {
                 ChunkDesc& C = plan[i];
@@ -195,6 +196,10 @@ extern "C" int pgz_decompress_noalloc(const uint8_t* gz, uint64_t gz_len, uint8_
             }
             replan = false;
         }
+        // the largest team whose 256 rows of tokens fit the array for n parts
+        kp.team = n <= kNaMaxParts / 8 ? 16 : (n <= kNaMaxParts / 4 ? 8 : (n <= kNaMaxParts / 2 ? 4 : 2));
+        kp.tok_rows = 256;
+        static_assert(kTokWords * 8 == 16 * 32 * 256, "a team of 16 warps takes eight parts' shares");
         uint64_t gsz = 1;
         while (gsz * gsz < n) ++gsz;
         int32_t g0[kNaMaxGroups], gn[kNaMaxGroups], gfile[kNaMaxGroups];
@@ -229,9 +234,10 @@ extern "C" int pgz_decompress_noalloc(const uint8_t* gz, uint64_t gz_len, uint8_
         cudaMemcpyAsync(d_gn, gn, ng * sizeof(int32_t), cudaMemcpyHostToDevice, s);
         cudaMemcpyAsync(d_gfile, gfile, ng * sizeof(int32_t), cudaMemcpyHostToDevice, s);
         cudaMemcpyAsync(d_seg0, &seg0, sizeof seg0, cudaMemcpyHostToDevice, s);
-        launch_sync(d_files, d_chunks, (int)n, d_sym, d_tok, d_queue, nullptr, kp, s);
-        launch_inflate(d_files, d_chunks, (int)n, d_sym, d_tok, d_queue + 1, nullptr, kp, s);
-        launch_exec(d_files, d_chunks, (int)n, d_sym, d_queue + 2, nullptr, kp, s);
+        cudaMemsetAsync(d_start, 0, kNaSymbols / 8, s);
+        launch_sync(d_files, d_chunks, (int)n, d_sym, d_start, d_tok, d_queue, nullptr, kp, s);
+        launch_inflate(d_files, d_chunks, (int)n, d_sym, d_start, d_tok, d_queue + 1, nullptr, kp, s);
+        launch_exec(d_files, d_chunks, (int)n, d_sym, d_start, d_queue + 2, nullptr, kp, s);
         launch_plan(d_files, d_chunks, 1, s);
         launch_chain(d_files, d_chunks, 1, ng, d_g0, d_gn, d_gfile, d_sym, d_gmaps, d_wstart, d_windows, s);
         launch_translate(d_files, d_chunks, (int)n, plan[0].cap, d_sym, d_windows, nullptr, s);

@@ -1,5 +1,7 @@
 """Pass 1 at the edges of its kernels' tiles: passes of the copy-map executor and segments of the block decoder."""
+import base64
 import functools
+import zlib
 
 import numpy as np
 import pytest
@@ -55,3 +57,44 @@ def test_copies_across_the_executors_passes(members, tail):
                 assert s == 0 and k == len(t) and o[:k].cpu().numpy().tobytes() == t
     finally:
         ctx.close()
+
+
+@functools.lru_cache(maxsize=None)
+def _dense(kind):
+    """Members whose blocks stress the block decoder's segments: tokens of very few bits, codes of one length (parses
+    that start wrong stay wrong), fixed codes, and many small blocks."""
+    rng = np.random.default_rng(len(kind))
+    if kind == "runs":
+        text = b"A" * 3_000_000 + b"AC" * 400_000
+        c = zlib.compressobj(9, zlib.DEFLATED, 31)
+    elif kind == "base64":
+        text = base64.b64encode(rng.integers(0, 256, 400_000, dtype=np.uint8).tobytes())
+        c = zlib.compressobj(6, zlib.DEFLATED, 31)
+    elif kind == "one_length":
+        text = rng.choice(np.frombuffer(bytes(range(33, 97)), dtype=np.uint8), 500_000).tobytes()
+        c = zlib.compressobj(6, zlib.DEFLATED, 31, 8, zlib.Z_HUFFMAN_ONLY)
+    elif kind == "two_literals":
+        text = (rng.random(600_000) < 0.3).astype(np.uint8).tobytes().replace(b"\0", b"x").replace(b"\1", b"y")
+        c = zlib.compressobj(6, zlib.DEFLATED, 31, 8, zlib.Z_HUFFMAN_ONLY)
+    elif kind == "fixed":
+        text = synth.fastq(700_000, 100, 0.001, 4)
+        c = zlib.compressobj(6, zlib.DEFLATED, 31, 8, zlib.Z_FIXED)
+    else:                                            # memLevel 1: blocks of 127 tokens
+        text = synth.fastq(500_000, 100, 0.001, 5)
+        c = zlib.compressobj(6, zlib.DEFLATED, 31, 1)
+    return c.compress(text) + c.flush(), text
+
+
+@pytest.mark.parametrize("wpb", [2, 4, 8])
+@pytest.mark.parametrize("kind", ["runs", "base64", "one_length", "two_literals", "fixed", "small_blocks"])
+def test_block_decoder_edges(kind, wpb):
+    """Every team size (16 warps with few parts, the configured size with many), one part and many."""
+    gz, text = _dense(kind)
+    for n in [1, 5, 310, 700, 2500]:
+        ctx = Ctx(n_chunks=n, warps_per_block=wpb, min_block=16)
+        try:
+            st, out, k, _ = ctx.decompress(gz, out_cap=len(text) + 1000)
+            assert st == 0, (n, ctx.pgz.pgz_strerror(st))
+            assert k == len(text) and out == text, n
+        finally:
+            ctx.close()
