@@ -1456,34 +1456,40 @@ __global__ void __launch_bounds__(32 * NW, pass1_min_blocks(NW))
 // One block of NT threads per part, in passes of 8 NT positions (a thread takes
 // 8 consecutive ones: one 16-byte load, one 16-byte store; a warp's 256 begin at
 // a multiple of kRestart, so the code in force at each comes from the start
-// bits and codes of its own lanes).  The last 32 KiB of
-// the part's symbols and the pass itself live in a ring in shared memory
-// (32768 + 8 NT u16 entries, so that a pass never overwrites a source it can
-// still need).  A position's entry is its symbol when the source lies before the
-// pass (read from the ring; U_j when it lies before the part), else kPtr | the
+// bits and codes of its own lanes).  The last 32 KiB of the part's symbols live
+// in a ring in shared memory, the pass itself in a stage beside it.  A
+// position's stage entry is its symbol when the source lies before the pass
+// (read from the ring; U_j when it lies before the part), else kPtr | the
 // source's index inside the pass.  After one barrier every thread follows its
 // own pointers; each step shortens the chain the next reader follows (an entry
 // is replaced by the entry it points to), an entry only ever changes to an
 // earlier source or to its symbol, and indices strictly decrease, so the chase
-// needs no further barrier and ends, overlapping copies included.
-// Bound: shared-memory latency and the two barriers of a pass.  1.00 ms for the 1024 parts of a 256 MiB file
-// (268 G symbols/s; the map is read and the symbols written once, 1.1 TB/s), 0.064 ms for 8 parts of 128 K
-// symbols.  A warp that executed its tokens out of the part's output in L2 (one kernel for decoding and
-// executing) took 8.5 ms for the block starts and decoding of the same file, against 4.5 ms for decoding to
-// a map and 1.0 ms here.
+// needs no further barrier and ends, overlapping copies included.  The pass's
+// symbols then go to the ring, whose places they take are no longer read.
+// Bound: instruction issue (about 25 instructions a position for the entry, 6 more per chase step; 2.8 steps a
+// pass on level-1 FASTQ).  0.74 ms for the 1024 parts of a 256 MiB file (364 G symbols/s); 1.05 ms with a branch per
+// position and entry in the chase, whose loads then wait for one another.
 constexpr uint32_t kPtr = 0x4000u;    // neither a byte nor a placeholder; the index takes 14 bits
 
 template <int NT>
 constexpr size_t exec_smem() { return (kWin + 8 * NT) * sizeof(uint16_t); }
 
+__device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
+    uint16_t v;
+    asm volatile("ld.volatile.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
+    return v;
+}
+
 template <int NT>
-__global__ void __launch_bounds__(NT, NT == 1024 ? 1 : (NT == 512 ? 2 : 3))
+__global__ void __launch_bounds__(NT, NT == 512 ? 2 : 3)
     k_exec(const FileDesc* __restrict__ files, ChunkDesc* chunks, int nchunks, uint16_t* symbuf,
            const uint32_t* __restrict__ start_bits, uint32_t* queue, const uint32_t* __restrict__ order, int tail) {
-    extern __shared__ __align__(16) uint16_t ring[];
+    extern __shared__ __align__(16) uint16_t ring[];     // kWin symbols, then the stage
     __shared__ int s_q;
-    constexpr uint32_t P = 8 * NT, R = kWin + P;
-    static_assert(R % P == 0 && P <= kPtr, "whole passes in the ring, indices in 14 bits");
+    constexpr uint32_t P = 8 * NT;
+    static_assert(kWin % P == 0 && P <= kPtr, "whole passes in the ring, indices in 14 bits");
+    uint16_t* stage = ring + kWin;
+    const uint32_t ring_a = (uint32_t)__cvta_generic_to_shared(ring), stage_a = ring_a + 2 * kWin;
     static_assert(kRestart == 256, "a warp's positions of a pass");
     const uint32_t t8 = 8u * threadIdx.x;
     const uint32_t below = (1u << (threadIdx.x & 31)) - 1u;
@@ -1508,66 +1514,69 @@ __global__ void __launch_bounds__(NT, NT == 1024 ? 1 : (NT == 512 ? 2 : 3))
             nx = *reinterpret_cast<const uint4*>(sym + t8);
             nst = start[t8 >> 3];
         }
-        uint32_t sA = 0;                             // ring slot of the pass's first position
         for (uint32_t A = 0; A < n; A += P) {
             const uint32_t p0 = A + t8;
-            const uint32_t w4[4] = {nx.x, nx.y, nx.z, nx.w}, st = nst;
+            uint32_t w4[4] = {nx.x, nx.y, nx.z, nx.w}, st = nst;
             if (p0 + P < n) {
                 nx = *reinterpret_cast<const uint4*>(sym + p0 + P);
                 nst = start[(p0 + P) >> 3];
-            } else {
-                nst = 0;
+            }
+            if (A + P > n) {                         // the last pass: byte 0 past the part's end
+                const uint32_t nv = p0 < n ? min(n - p0, 8u) : 0u;
+                st = (st & ((1u << nv) - 1u)) | (0xffu & (0xffu << nv));
+#pragma unroll
+                for (uint32_t k = 0; k < 4; ++k)
+                    w4[k] = 2 * k + 1 < nv ? w4[k] : (2 * k < nv ? w4[k] & 0xffffu : 0u);
             }
             // the last code of the lanes below is in force at my first position
-            const uint32_t top = st ? 31u - __clz(st) : 0u, tw = w4[0], th = 16u * (top & 1u);
-            const uint32_t mine = (top < 4 ? (top < 2 ? tw : w4[1]) : (top < 6 ? w4[2] : w4[3])) >> th;
+            const uint32_t top = st ? 31u - __clz(st) : 0u;
+            const uint32_t last = (top < 4 ? (top < 2 ? w4[0] : w4[1]) : (top < 6 ? w4[2] : w4[3])) >> (16u * (top & 1u));
             const uint32_t has = __ballot_sync(FULL, st != 0) & below;
-            uint32_t v = __shfl_sync(FULL, mine, has ? 31 - __clz(has) : 0) & 0xffffu;
-            uint32_t e[8], slot[8];
-            uint32_t open = 0;                       // bit u: e[u] is a pointer into the pass
+            uint32_t code = __shfl_sync(FULL, last, has ? 31 - __clz(has) : 0) & 0xffffu;
             // (selections, not branches: the eight loads of a thread are in flight together, here and below)
+            uint32_t e[8], ptr[8];
+            int32_t q[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                if ((st >> u) & 1u) v = (u & 1) ? w4[u >> 1] >> 16 : w4[u >> 1] & 0xffffu;
-                e[u] = p0 + (uint32_t)u < n ? v : 0u;
-                const int32_t rel = (int32_t)(t8 + u) - (int32_t)(e[u] & 0x7fffu) - 1;   // a match's source, from A
-                const int32_t a = (int32_t)sA + rel;
-                slot[u] = (e[u] & kPH) && rel < 0 ? (uint32_t)(a < 0 ? a + (int32_t)R : a) : sA;
+                const uint32_t c = (u & 1) ? w4[u >> 1] >> 16 : w4[u >> 1] & 0xffffu;
+                code = (st >> u) & 1u ? c : code;
+                e[u] = code;
+                q[u] = (int32_t)(p0 + u) - 1 - (int32_t)(code & 0x7fffu);   // a match's source
+                ptr[u] = lds_u16(ring_a + 2u * ((uint32_t)q[u] & (kWin - 1u)));
             }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) slot[u] = ring[slot[u]];
+            uint32_t open = 0;
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                if (e[u] & kPH) {
-                    const int32_t rel = (int32_t)(t8 + u) - (int32_t)(e[u] & 0x7fffu) - 1;
-                    const bool in = rel >= 0;
-                    open |= in ? 1u << u : 0u;
-                    e[u] = in ? kPtr | (uint32_t)rel
-                              : ((int32_t)A + rel < 0 ? kPH | (uint32_t)((int32_t)kWin + (int32_t)A + rel) : slot[u]);
-                }
+                const bool match = e[u] >> 15, in = match && q[u] >= (int32_t)A;
+                const uint32_t val = q[u] < 0 ? ((uint32_t)q[u] & 0x7fffu) | kPH : ptr[u], rel = (uint32_t)q[u] - A;
+                e[u] = in ? kPtr | rel : (match ? val : e[u]);
+                ptr[u] = stage_a + 2u * (in ? rel : t8 + u);                // a resolved entry reads itself
+                open |= in;
             }
             uint4 v4;
-            v4.x = e[0] | (e[1] << 16);
-            v4.y = e[2] | (e[3] << 16);
-            v4.z = e[4] | (e[5] << 16);
-            v4.w = e[6] | (e[7] << 16);
-            *reinterpret_cast<uint4*>(ring + sA + t8) = v4;
-            __syncthreads();
-            volatile uint16_t* pass = ring + sA;
-            while (__any_sync(FULL, open)) {
-#pragma unroll
-                for (int u = 0; u < 8; ++u) slot[u] = pass[(open >> u) & 1u ? e[u] & (kPtr - 1u) : t8 + u];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    e[u] = (open >> u) & 1u ? slot[u] : e[u];
-                    if ((e[u] >> 14) != 1u) open &= ~(1u << u);
-                }
+            auto pack = [&]() {
                 v4.x = e[0] | (e[1] << 16);
                 v4.y = e[2] | (e[3] << 16);
                 v4.z = e[4] | (e[5] << 16);
                 v4.w = e[6] | (e[7] << 16);
-                *reinterpret_cast<uint4*>(ring + sA + t8) = v4;   // a thread's entries change only by its own hand
+            };
+            pack();
+            *reinterpret_cast<uint4*>(stage + t8) = v4;
+            __syncthreads();
+            while (__any_sync(FULL, open)) {
+                open = 0;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) e[u] = lds_u16(ptr[u]);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const bool more = (e[u] & 0xc000u) == kPtr;
+                    ptr[u] = more ? stage_a - 2u * kPtr + 2u * e[u] : ptr[u];
+                    open |= more;
+                }
+                pack();
+                *reinterpret_cast<uint4*>(stage + t8) = v4;   // a thread's entries change only by its own hand
             }
+            *reinterpret_cast<uint4*>(ring + ((A + t8) & (kWin - 1u))) = v4;
             if (det == 0xffffffffu && track && A >= ph_end + kWin) det = A;
             if (track) {
                 const uint32_t any = (v4.x | v4.y | v4.z | v4.w) & (kPH | (kPH << 16));
@@ -1585,7 +1594,6 @@ __global__ void __launch_bounds__(NT, NT == 1024 ? 1 : (NT == 512 ? 2 : 3))
                     *reinterpret_cast<uint4*>(sym + p0) = v4;
                 }
             }
-            sA = sA + P == R ? 0u : sA + P;
         }
         if (threadIdx.x == 0 && det != 0xffffffffu) C.det = det;
     }
@@ -2394,9 +2402,12 @@ void launch_exec(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t
                  const uint32_t* order, const KParams& p, cudaStream_t s) {
     if (nchunks <= 0) return;
     cudaMemsetAsync(queue, 0, sizeof(uint32_t), s);
-    // up to one block per SM, the block of 1024 threads: half the passes, so half the barriers, of a part
-    if (nchunks <= exec_resident<1024>()) launch_exec_t<1024>(files, chunks, nchunks, sym, start, queue, order, p, s);
-    else launch_exec_t<512>(files, chunks, nchunks, sym, start, queue, order, p, s);
+    // With at most one part per SM, blocks of 512 threads: half the passes of a part (file of 8 parts: 53 us, against
+    // 59 us with 256).  With more, 256: three fit an SM (two of 512), and shorter passes hold fewer sources inside
+    // them, so they take fewer chase steps (1024 parts of 256 MiB: 737 us, against 873 us with 512 and 996 us with
+    // 1024).
+    if (nchunks <= exec_resident<512>() / 2) launch_exec_t<512>(files, chunks, nchunks, sym, start, queue, order, p, s);
+    else launch_exec_t<256>(files, chunks, nchunks, sym, start, queue, order, p, s);
 }
 
 void launch_plan(FileDesc* files, ChunkDesc* chunks, int nfiles, cudaStream_t s) {
