@@ -233,6 +233,9 @@ struct Plan {
     std::vector<FileDesc> files;
     std::vector<ChunkDesc> chunks;
     std::vector<int32_t> g0, gn, gfile;
+    std::vector<int32_t> upper;   // the chain's upper levels: s0, sn, sfile per supergroup, then f0, fn, ffile per member
+    size_t nsupers = 0;
+    bool many = false, deep = false;   // some member has several groups, several supergroups
     std::vector<uint64_t> seg0;
     std::vector<uint32_t> order;  // the parts in the order the pass-1 work queue hands them out
     uint64_t sym_total = 0, max_cap = 0, total_seg = 0;
@@ -240,15 +243,17 @@ struct Plan {
     bool results_valid = false;   // the device chunk array holds the last run's results
     int wpb = 4;                  // warps per block of the pass-1 kernels (sizes the token scratch)
     const uint8_t* fill = nullptr;   // device window of fill bytes (mode 1)
-    DBuf d_files, d_chunks, d_g0, d_gn, d_gfile, d_seg0, d_sym, d_windows, d_gmaps, d_wstart, d_tok, d_start, d_queue, d_order;
+    DBuf d_files, d_chunks, d_g0, d_gn, d_gfile, d_upper, d_seg0, d_sym, d_windows, d_gmaps, d_wstart, d_tok, d_start, d_queue, d_order;
     PBuf h_files, h_chunks, h_static;
     cudaGraphExec_t graph = nullptr;
+    uint64_t graph_launches = 0;  // kernels of the last enqueued run (a graph replays them)
     void release() {
         d_files.release();
         d_chunks.release();
         d_g0.release();
         d_gn.release();
         d_gfile.release();
+        d_upper.release();
         d_seg0.release();
         d_sym.release();
         d_windows.release();
@@ -373,8 +378,7 @@ void plan_member(pgz_ctx* ctx, Plan& P, const uint8_t* gz, uint64_t gz_len, uint
         C.sync = kNone;
         P.chunks.push_back(C);
     }
-    // window-chain groups of about sqrt(n) parts
-    const uint64_t gsz = std::max<uint64_t>(1, (uint64_t)std::ceil(std::sqrt((double)n)));
+    const uint64_t gsz = (uint64_t)chain_group_size((int)n);     // window-chain groups
     F.group0 = (int32_t)P.g0.size();
     F.ngroups = 0;
     for (uint64_t a = 0; a < n; a += gsz) {
@@ -420,12 +424,35 @@ int layout(Plan& P) {
         return wa > wb;
     });
     const size_t nf = P.files.size(), nc = P.chunks.size(), ng = P.g0.size();
+    std::vector<int32_t> lv[6];                      // the chain's upper levels
+    P.many = P.deep = false;
+    for (size_t f = 0; f < nf; ++f) {
+        FileDesc& F = P.files[f];
+        const int ssz = std::max(1, chain_super_size(F.ngroups));
+        F.super0 = (int32_t)lv[0].size();
+        for (int a = 0; a < F.ngroups; a += ssz) {
+            lv[0].push_back(F.group0 + a);
+            lv[1].push_back(std::min(ssz, F.ngroups - a));
+            lv[2].push_back((int32_t)f);
+        }
+        F.nsupers = (int32_t)lv[0].size() - F.super0;
+        P.many |= F.ngroups > 1;
+        P.deep |= F.nsupers > 1;
+        lv[3].push_back(F.super0);
+        lv[4].push_back(F.nsupers);
+        lv[5].push_back((int32_t)f);
+    }
+    P.nsupers = lv[0].size();
+    P.upper.clear();
+    for (const auto& v : lv) P.upper.insert(P.upper.end(), v.begin(), v.end());
+    const size_t nm = ng + P.nsupers;                // maps and first windows of both levels
     cudaError_t e = cudaSuccess;
     if (!e) e = P.d_files.ensure(nf * sizeof(FileDesc));
     if (!e) e = P.d_chunks.ensure(nc * sizeof(ChunkDesc));
     if (!e) e = P.d_g0.ensure(ng * sizeof(int32_t));
     if (!e) e = P.d_gn.ensure(ng * sizeof(int32_t));
     if (!e) e = P.d_gfile.ensure(ng * sizeof(int32_t));
+    if (!e) e = P.d_upper.ensure(P.upper.size() * sizeof(int32_t));
     if (!e) e = P.d_seg0.ensure(nf * sizeof(uint64_t));
     if (!e) e = P.d_sym.ensure(P.sym_total * sizeof(uint16_t));
     if (!e) e = P.d_tok.ensure((size_t)token_words((int)nc, P.wpb) * sizeof(uint32_t));
@@ -433,12 +460,12 @@ int layout(Plan& P) {
     if (!e) e = P.d_queue.ensure(3 * sizeof(uint32_t));
     if (!e) e = P.d_order.ensure(nc * sizeof(uint32_t));
     if (!e && P.chain) e = P.d_windows.ensure(nc * (size_t)kWin);
-    if (!e && P.chain) e = P.d_gmaps.ensure(ng * (size_t)kWin * sizeof(uint16_t));
-    if (!e && P.chain) e = P.d_wstart.ensure(ng * (size_t)kWin);
+    if (!e && P.chain) e = P.d_gmaps.ensure(nm * (size_t)kWin * sizeof(uint16_t));
+    if (!e && P.chain) e = P.d_wstart.ensure(nm * (size_t)kWin);
     if (!e) e = P.h_files.ensure(nf * sizeof(FileDesc));
     if (!e) e = P.h_chunks.ensure(nc * sizeof(ChunkDesc));
     if (!e) e = P.h_static.ensure(3 * round_up(ng * sizeof(int32_t), 16) + round_up(nf * sizeof(uint64_t), 16) +
-                                  round_up(nc * sizeof(uint32_t), 16));
+                                  round_up(P.upper.size() * sizeof(int32_t), 16) + round_up(nc * sizeof(uint32_t), 16));
     return cuda_status(e);
 }
 
@@ -460,6 +487,7 @@ void upload_static(Plan& P, cudaStream_t s) {
     put(P.d_g0.p, P.g0.data(), ng * sizeof(int32_t));
     put(P.d_gn.p, P.gn.data(), ng * sizeof(int32_t));
     put(P.d_gfile.p, P.gfile.data(), ng * sizeof(int32_t));
+    put(P.d_upper.p, P.upper.data(), P.upper.size() * sizeof(int32_t));
     put(P.d_seg0.p, P.seg0.data(), nf * sizeof(uint64_t));
     put(P.d_order.p, P.order.data(), nc * sizeof(uint32_t));
 }
@@ -496,9 +524,13 @@ int enqueue(pgz_ctx* ctx, Plan& P, cudaStream_t s, bool timed, cudaStream_t up =
     k += 4;
     if (timed) cudaEventRecord(ctx->ev[2], s);
     if (P.chain) {
-        launch_chain(df, dc, (int)nf, (int)ng, P.d_g0.as<int32_t>(), P.d_gn.as<int32_t>(), P.d_gfile.as<int32_t>(),
-                     sym, P.d_gmaps.as<uint16_t>(), P.d_wstart.as<uint8_t>(), P.d_windows.as<uint8_t>(), s);
-        k += 3;
+        const int32_t* u = P.d_upper.as<int32_t>();
+        const size_t ns = P.nsupers;
+        const ChainPlan cp{(int)ng, (int)ns, P.many, P.deep, P.d_g0.as<int32_t>(), P.d_gn.as<int32_t>(), P.d_gfile.as<int32_t>(),
+                           u, u + ns, u + 2 * ns, u + 3 * ns, u + 3 * ns + nf, u + 3 * ns + 2 * nf};
+        launch_chain(df, dc, (int)nf, cp, sym, P.d_gmaps.as<uint16_t>(), P.d_wstart.as<uint8_t>(),
+                     P.d_windows.as<uint8_t>(), s);
+        k += 1 + (P.many ? 2 : 0) + (P.deep ? 2 : 0);
     }
     if (timed) cudaEventRecord(ctx->ev[3], s);
     if (P.translate) {
@@ -514,6 +546,7 @@ int enqueue(pgz_ctx* ctx, Plan& P, cudaStream_t s, bool timed, cudaStream_t up =
     if (timed) cudaEventRecord(ctx->ev[5], s);
     cudaMemcpyAsync(P.h_files.p, P.d_files.p, nf * sizeof(FileDesc), cudaMemcpyDeviceToHost, s);
     ctx->launches += (uint64_t)k;
+    P.graph_launches = (uint64_t)k;
     return cuda_status(cudaGetLastError());
 }
 
@@ -771,7 +804,7 @@ void plan_segment(pgz_ctx* ctx, Plan& P, const uint8_t* win, uint64_t win_len, u
         P.chunks.push_back(C);
     }
     F.out_cap = cap_sum;                              // the caller sizes the output buffer to it
-    const uint64_t gsz = std::max<uint64_t>(1, (uint64_t)std::ceil(std::sqrt((double)np)));
+    const uint64_t gsz = (uint64_t)chain_group_size((int)np);
     F.group0 = (int32_t)P.g0.size();
     F.ngroups = 0;
     for (uint64_t a = 0; a < np; a += gsz) {
@@ -1570,7 +1603,7 @@ int pgz_batch_run(pgz_batch* b, pgz_job* jobs, pgz_stats* st) {
         cudaEventRecord(ctx->ev[6], ctx->stream);
     }
     if (cudaGraphLaunch(P.graph, ctx->stream) != cudaSuccess) return PGZ_E_CUDA;
-    ctx->launches += (uint64_t)kernels_per_run();
+    ctx->launches += P.graph_launches;
     if (st) cudaEventRecord(ctx->ev[7], ctx->stream);
     if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return PGZ_E_CUDA;
     const FileDesc* hf = P.h_files.as<FileDesc>();

@@ -56,7 +56,8 @@ struct FileDesc {
     uint32_t crc_expect;
     uint32_t isize_expect;
     int32_t chunk0, nchunks;
-    int32_t group0, ngroups;
+    int32_t group0, ngroups;   // window-chain groups of consecutive parts
+    int32_t super0, nsupers;   // groups of consecutive groups
     uint64_t seg0, nseg;   // 4 KiB CRC segments of the output
     uint32_t mode;         // 0 whole member; 1 from a bit offset (no CRC/ISIZE); 2 byte range of the output;
                            // 3 one segment of a streamed member (bit positions relative to the segment's bytes)
@@ -132,9 +133,21 @@ uint64_t token_words(int nchunks, int wpb);
 int pass1_team(int nchunks, int wpb);   // warps per part for a launch of nchunks parts
 int pass1_parts(int wpb);               // parts resident at once with many parts (teams of wpb warps)
 void launch_plan(FileDesc* files, ChunkDesc* chunks, int nfiles, cudaStream_t s);
-void launch_chain(const FileDesc* files, const ChunkDesc* chunks, int nfiles, int ngroups,
-                  const int32_t* group_chunk0, const int32_t* group_n, const int32_t* group_file,
-                  const uint16_t* sym, uint16_t* gmaps, uint8_t* wstart, uint8_t* windows, cudaStream_t s);
+// The window chain's levels: groups of parts (g0: first part, gn: parts, gfile: member), supergroups of groups, and
+// per member its supergroups.  gmaps and wstart hold ngroups + nsupers maps (kWin u16) and windows (kWin bytes).
+struct ChainPlan {
+    int ngroups, nsupers;
+    bool many, deep;       // some member has more than one group, more than one supergroup
+    const int32_t *g0, *gn, *gfile, *s0, *sn, *sfile, *f0, *fn, *ffile;
+};
+// Parts per group of a member of n parts, and groups per supergroup: a step (one item of a group) takes about 3 us
+// whatever the level, the groups of a level run side by side, so the lengths of the levels are balanced: one group up
+// to 12 parts (a chain of 12 steps costs less than two more launches and their steps), two levels up to 64, else
+// three.
+int chain_group_size(int n);
+int chain_super_size(int ngroups);
+void launch_chain(const FileDesc* files, const ChunkDesc* chunks, int nfiles, const ChainPlan& C, const uint16_t* sym,
+                  uint16_t* gmaps, uint8_t* wstart, uint8_t* windows, cudaStream_t s);
 void launch_translate(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint64_t max_cap,
                       const uint16_t* sym, const uint8_t* windows, const uint8_t* fill_window, cudaStream_t s);
 // total_seg: CRC segments of crc_segment_bytes() output bytes over all members (FileDesc::seg0, nseg)
@@ -147,7 +160,6 @@ void launch_sequences(const uint16_t* sym, uint64_t n, uint32_t min_len, uint64_
                       unsigned long long* counts, cudaStream_t s);
 // ChunkDesc::nph and last_ph from the symbols of every finished part (statistics and inspection only)
 void launch_count_ph(ChunkDesc* chunks, int nchunks, const uint16_t* sym, cudaStream_t s);
-int kernels_per_run();
 void upload_crc_tables();
 
 // Recovery after a failed run (pgz_host.cu), shared by every entry point.  For the member F whose parts are

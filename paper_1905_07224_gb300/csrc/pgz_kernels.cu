@@ -27,8 +27,8 @@
 //   k_chain_*   pass 2a: w_{i+1} from w_i and the tail of D_i (Section "Full
 //               file decompression in two passes").  Each part's tail is a map
 //               from w_i to w_{i+1} whose entries are bytes or indices; maps
-//               compose, so groups of parts are composed in parallel, walked
-//               across groups, then expanded per part.
+//               compose, so groups of parts (and groups of groups) are composed
+//               in parallel, then expanded level by level.
 //   k_translate pass 2b: U_j -> w_i[j] for every symbol, written to the
 //               final output with 8-byte aligned stores (HBM-bound).
 //   k_crc       CRC-32 (RFC 1952) of the output: raw CRCs of 128-byte pieces,
@@ -39,6 +39,7 @@
 // No kernel waits on another block or warp; every read of the compressed
 // data, the symbol scratch and the output is bounds-checked.
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -1696,107 +1697,154 @@ __device__ __forceinline__ uint16_t map_entry(const uint16_t* d, uint64_t n, uin
     return (uint64_t)t >= det ? reinterpret_cast<const uint8_t*>(d)[det + (uint64_t)t] : d[t];   // det: the tail
 }
 
-// Every thread handles entries tid + 1024*j; eight loads are in flight at once.
+// The items of a run of the chain, in order: PARTS, the finished parts c0 .. c0 + n - 1 of the plan (others hold
+// nothing and are skipped), else the composed maps c0 .. at `maps`.
+template <bool PARTS>
+struct ChainItem {
+    const uint16_t* d = nullptr;
+    uint64_t n = 0, det = 0;
+    int c = 0;                    // the item (past the last: end)
+    __device__ __forceinline__ void find(int from, int end, const ChunkDesc* chunks, const uint16_t* base) {
+        c = from;
+        if (!PARTS) {
+            d = base + (uint64_t)c * kWin;
+            return;
+        }
+        for (; c < end; ++c) {
+            const ChunkDesc& C = chunks[c];
+            if (C.state == CS_DONE && C.n != 0) {
+                d = base + C.sym_base;
+                n = C.n;
+                det = C.det;
+                return;
+            }
+        }
+    }
+    // whole entries in memory, entry k at plain()[k] (a part with 32 Ki u16 symbols or more): loads without a branch
+    __device__ __forceinline__ bool is_plain() const { return !PARTS || (n >= kWin && det >= n); }
+    __device__ __forceinline__ const uint16_t* plain() const { return PARTS ? d + (n - kWin) : d; }
+    __device__ __forceinline__ uint32_t entry(uint32_t k) const { return PARTS ? map_entry(d, n, det, k) : d[k]; }
+};
+
+// Each thread handles the entries tid + 1024 j, j < 32.  A step's 32 loads of a thread were issued during the step
+// before (each register is refilled as soon as its entry is used), so a step costs its shared-memory gathers, about
+// 3 us, and not the latency of the symbols.
+constexpr int kChainPer = kWin / 1024;
+
+// m: the entries of `it`, if it is an item (else left alone)
+template <bool PARTS>
+__device__ __forceinline__ void chain_fill(uint32_t (&m)[kChainPer], const ChainItem<PARTS>& it, int end) {
+    if (it.c >= end) return;
+    if (it.is_plain()) {
+        const uint16_t* p = it.plain() + threadIdx.x;
+#pragma unroll
+        for (int j = 0; j < kChainPer; ++j) m[j] = p[1024 * j];
+    } else {
+#pragma unroll
+        for (int j = 0; j < kChainPer; ++j) m[j] = it.entry(threadIdx.x + 1024u * j);
+    }
+}
+
+// One step: put(k, e) for every entry e = m[j] of k = tid + 1024 j, and m refilled with the next item's (next.c <
+// end) entries on the way.
+template <bool PARTS, typename Put>
+__device__ __forceinline__ void chain_step(uint32_t (&m)[kChainPer], const ChainItem<PARTS>& next, int end, Put put) {
+    if (next.c < end && next.is_plain()) {
+        const uint16_t* p = next.plain() + threadIdx.x;
+#pragma unroll
+        for (int j = 0; j < kChainPer; ++j) {
+            const uint32_t e = m[j];
+            m[j] = p[1024 * j];
+            put(threadIdx.x + 1024u * j, e);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < kChainPer; ++j) put(threadIdx.x + 1024u * j, m[j]);
+        chain_fill<PARTS>(m, next, end);
+    }
+}
+
+// the composed map of each group's items; the last group of a member has no successor, so no one reads its map
+template <bool PARTS>
 __global__ void __launch_bounds__(1024) k_chain_compose(const FileDesc* __restrict__ files,
                                                         const ChunkDesc* __restrict__ chunks, const int32_t* g0,
                                                         const int32_t* gn, const int32_t* gfile,
-                                                        const uint16_t* __restrict__ sym, uint16_t* gmaps) {
+                                                        const uint16_t* __restrict__ src, uint16_t* gmaps) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint16_t* acc = reinterpret_cast<uint16_t*>(smem_raw);
     uint16_t* tmp = acc + kWin;
     const int g = blockIdx.x;
-    if (files[gfile[g]].status != PGZ_OK) return;
+    const FileDesc& F = files[gfile[g]];
+    if (F.status != PGZ_OK || g + 1 == (PARTS ? F.group0 + F.ngroups : F.super0 + F.nsupers)) return;
     const uint32_t tid = threadIdx.x;
+    const int end = g0[g] + gn[g];
+    uint16_t* dst = gmaps + (uint64_t)g * kWin;
+    ChainItem<PARTS> it;
+    it.find(g0[g], end, chunks, src);
+    if (it.c >= end) {
+        for (uint32_t k = tid; k < kWin; k += 1024) dst[k] = (uint16_t)(kPH | k);
+        return;
+    }
+    uint32_t m[kChainPer];
+    chain_fill<PARTS>(m, it, end);
     bool have = false;
-    for (int c = g0[g]; c < g0[g] + gn[g]; ++c) {
-        const ChunkDesc& C = chunks[c];
-        if (C.state != CS_DONE || C.n == 0) continue;
-        const uint16_t* d = sym + C.sym_base;
-        const uint64_t n = C.n;
-        for (uint32_t j0 = 0; j0 < kWin / 1024; j0 += 8) {
-            uint16_t m[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) m[u] = map_entry(d, n, C.det, tid + 1024u * (j0 + u));
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                uint16_t e = m[u];
-                if (have && (e & kPH)) e = acc[e & (kWin - 1)];
-                tmp[tid + 1024u * (j0 + u)] = e;
-            }
-        }
+    for (;;) {
+        it.find(it.c + 1, end, chunks, src);
+        const bool more = it.c < end;
+        uint16_t* to = more ? tmp : dst;
+        if (have)
+            chain_step<PARTS>(m, it, end, [&](uint32_t k, uint32_t e) {
+                const uint32_t w = acc[e & (kWin - 1)];
+                to[k] = (uint16_t)((e & kPH) ? w : e);
+            });
+        else
+            chain_step<PARTS>(m, it, end, [&](uint32_t k, uint32_t e) { to[k] = (uint16_t)e; });
+        if (!more) return;
         __syncthreads();
         uint16_t* x = acc;
         acc = tmp;
         tmp = x;
         have = true;
     }
-    uint16_t* dst = gmaps + (uint64_t)g * kWin;
-    for (uint32_t k = tid; k < kWin; k += 1024) dst[k] = have ? acc[k] : (uint16_t)(kPH | k);
 }
 
-__global__ void __launch_bounds__(1024) k_chain_walk(const FileDesc* __restrict__ files, const uint16_t* __restrict__ gmaps,
-                                                     uint8_t* wstart) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    uint8_t* W = smem_raw;
-    uint8_t* W2 = smem_raw + kWin;
-    const FileDesc& F = files[blockIdx.x];
-    if (F.status != PGZ_OK) return;
-    const uint32_t tid = threadIdx.x;
-    for (uint32_t k = tid; k < kWin; k += 1024) W[k] = F.win0 ? F.win0[k] : 0;   // before the member: never referenced
-    __syncthreads();
-    for (int g = F.group0; g < F.group0 + F.ngroups; ++g) {
-        uint8_t* ws = wstart + (uint64_t)g * kWin;
-        const uint16_t* m = gmaps + (uint64_t)g * kWin;
-        for (uint32_t j0 = 0; j0 < kWin / 1024; j0 += 8) {
-            uint16_t e[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) e[u] = m[tid + 1024u * (j0 + u)];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const uint32_t k = tid + 1024u * (j0 + u);
-                ws[k] = W[k];
-                W2[k] = (e[u] & kPH) ? W[e[u] & (kWin - 1)] : (uint8_t)e[u];
-            }
-        }
-        __syncthreads();
-        uint8_t* x = W;
-        W = W2;
-        W2 = x;
-    }
-}
-
+// Resolved windows along each group's items, from the window before its first: out[item] = the window before that
+// item (PARTS: every part of the group, skipped ones too).  win (null: each member's own start, FileDesc::win0 or
+// nothing) holds the groups' first windows.
+template <bool PARTS>
 __global__ void __launch_bounds__(1024) k_chain_expand(const FileDesc* __restrict__ files,
                                                        const ChunkDesc* __restrict__ chunks, const int32_t* g0,
                                                        const int32_t* gn, const int32_t* gfile,
-                                                       const uint16_t* __restrict__ sym, const uint8_t* wstart,
-                                                       uint8_t* windows) {
+                                                       const uint16_t* __restrict__ src, const uint8_t* win,
+                                                       uint8_t* out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint8_t* W = smem_raw;
     uint8_t* W2 = smem_raw + kWin;
     const int g = blockIdx.x;
-    if (files[gfile[g]].status != PGZ_OK) return;
+    const FileDesc& F = files[gfile[g]];
+    if (F.status != PGZ_OK) return;
     const uint32_t tid = threadIdx.x;
-    const uint8_t* ws = wstart + (uint64_t)g * kWin;
+    const int c0 = g0[g], end = c0 + gn[g];
+    ChainItem<PARTS> it;
+    it.find(c0, end, chunks, src);
+    uint32_t m[kChainPer];
+    chain_fill<PARTS>(m, it, end - 1);                   // the last item's own map leads out of the group
+    const uint8_t* ws = win ? win + (uint64_t)g * kWin : F.win0;
     for (uint32_t k = tid; k < kWin / 16; k += 1024)
-        reinterpret_cast<uint4*>(W)[k] = reinterpret_cast<const uint4*>(ws)[k];
+        reinterpret_cast<uint4*>(W)[k] = ws ? reinterpret_cast<const uint4*>(ws)[k] : make_uint4(0, 0, 0, 0);
     __syncthreads();
-    for (int c = g0[g]; c < g0[g] + gn[g]; ++c) {
-        const ChunkDesc& C = chunks[c];
-        uint4* wc = reinterpret_cast<uint4*>(windows + (uint64_t)c * kWin);
-        for (uint32_t k = tid; k < kWin / 16; k += 1024) wc[k] = reinterpret_cast<const uint4*>(W)[k];
-        if (C.state != CS_DONE || C.n == 0) continue;
-        const uint16_t* d = sym + C.sym_base;
-        const uint64_t n = C.n;
-        for (uint32_t j0 = 0; j0 < kWin / 1024; j0 += 8) {
-            uint16_t m[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) m[u] = map_entry(d, n, C.det, tid + 1024u * (j0 + u));
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const uint16_t e = m[u];
-                W2[tid + 1024u * (j0 + u)] = (e & kPH) ? W[e & (kWin - 1)] : (uint8_t)e;
-            }
-        }
+    int c = c0;                                          // next item whose window is not written
+    for (;;) {
+        const int last = min(it.c, end - 1);             // the items up to the next finished part share this window
+        for (; c <= last; ++c)
+            for (uint32_t k = tid; k < kWin / 16; k += 1024)
+                reinterpret_cast<uint4*>(out + (uint64_t)c * kWin)[k] = reinterpret_cast<const uint4*>(W)[k];
+        if (c >= end) return;
+        it.find(it.c + 1, end, chunks, src);
+        chain_step<PARTS>(m, it, end - 1, [&](uint32_t k, uint32_t e) {
+            const uint32_t w = W[e & (kWin - 1)];
+            W2[k] = (uint8_t)((e & kPH) ? w : e);
+        });
         __syncthreads();
         uint8_t* x = W;
         W = W2;
@@ -2415,24 +2463,46 @@ void launch_plan(FileDesc* files, ChunkDesc* chunks, int nfiles, cudaStream_t s)
     k_plan<<<nfiles, 1024, 0, s>>>(files, chunks);
 }
 
-void launch_chain(const FileDesc* files, const ChunkDesc* chunks, int nfiles, int ngroups,
-                  const int32_t* g0, const int32_t* gn, const int32_t* gfile, const uint16_t* sym,
+// Parts -> group maps -> (supergroup maps ->) the windows before the first items, member by member, then group by
+// group (through the supergroups), then part by part.
+void launch_chain(const FileDesc* files, const ChunkDesc* chunks, int nfiles, const ChainPlan& C, const uint16_t* sym,
                   uint16_t* gmaps, uint8_t* wstart, uint8_t* windows, cudaStream_t s) {
-    if (ngroups <= 0) return;
+    if (C.ngroups <= 0) return;
     static bool attr[64] = {};                            // the shared-memory limits are raised per device
     int dev = 0;
     cudaGetDevice(&dev);
     const int slot = dev >= 0 && dev < 64 ? dev : 0;
     if (!attr[slot]) {
-        attr[slot] =
-            cudaFuncSetAttribute(k_chain_compose, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kWin) ==
-                cudaSuccess &&
-            cudaFuncSetAttribute(k_chain_walk, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kWin) == cudaSuccess &&
-            cudaFuncSetAttribute(k_chain_expand, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kWin) == cudaSuccess;
+        const auto raise = [](const void* f, int n) {
+            return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, n) == cudaSuccess;
+        };
+        attr[slot] = raise((const void*)k_chain_compose<true>, 4 * kWin) &&
+                     raise((const void*)k_chain_compose<false>, 4 * kWin) &&
+                     raise((const void*)k_chain_expand<true>, 2 * kWin) &&
+                     raise((const void*)k_chain_expand<false>, 2 * kWin);
     }
-    k_chain_compose<<<ngroups, 1024, 4 * kWin, s>>>(files, chunks, g0, gn, gfile, sym, gmaps);
-    k_chain_walk<<<nfiles, 1024, 2 * kWin, s>>>(files, gmaps, wstart);
-    k_chain_expand<<<ngroups, 1024, 2 * kWin, s>>>(files, chunks, g0, gn, gfile, sym, wstart, windows);
+    if (C.many) k_chain_compose<true><<<C.ngroups, 1024, 4 * kWin, s>>>(files, chunks, C.g0, C.gn, C.gfile, sym, gmaps);
+    const uint8_t* first = nullptr;
+    if (C.deep) {
+        uint16_t* smaps = gmaps + (uint64_t)C.ngroups * kWin;
+        uint8_t* swin = wstart + (uint64_t)C.ngroups * kWin;
+        k_chain_compose<false><<<C.nsupers, 1024, 4 * kWin, s>>>(files, chunks, C.s0, C.sn, C.sfile, gmaps, smaps);
+        k_chain_expand<false><<<nfiles, 1024, 2 * kWin, s>>>(files, chunks, C.f0, C.fn, C.ffile, smaps, nullptr, swin);
+        first = swin;
+    }
+    if (C.many)
+        k_chain_expand<false><<<C.nsupers, 1024, 2 * kWin, s>>>(files, chunks, C.s0, C.sn, C.sfile, gmaps, first, wstart);
+    k_chain_expand<true><<<C.ngroups, 1024, 2 * kWin, s>>>(files, chunks, C.g0, C.gn, C.gfile, sym,
+                                                           C.many ? wstart : nullptr, windows);
+}
+
+int chain_group_size(int n) {
+    if (n <= 12) return n;
+    const double g = n <= 64 ? std::sqrt((double)n) : std::cbrt((double)n);
+    return (int)std::ceil(g);
+}
+int chain_super_size(int ngroups) {
+    return ngroups <= 12 ? ngroups : (int)std::ceil(std::sqrt((double)ngroups));
 }
 
 void launch_translate(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint64_t max_cap,
@@ -2490,7 +2560,6 @@ void launch_finalize(FileDesc* files, int nfiles, cudaStream_t s) {
     k_finalize<<<(nfiles + 127) / 128, 128, 0, s>>>(files, nfiles);
 }
 
-int kernels_per_run() { return 10; }
 
 // CRC-32 constants from the polynomial (RFC 1952 section 8)
 static uint32_t h_mul(uint32_t a, uint32_t b) {

@@ -38,7 +38,7 @@ constexpr uint64_t kNaMaxOut = 4ull << 20;          // largest output (ISIZE) ac
 constexpr uint64_t kNaMaxIn = kNaMaxOut + (kNaMaxOut >> 6) + 4096;   // stored blocks cost ~0.03 %
 constexpr uint64_t kNaMaxHeader = 4096;
 constexpr int kNaMaxParts = 64;
-constexpr int kNaMaxGroups = 8;
+constexpr int kNaMaxGroups = 8;                     // chain_group_size gives at most 8 groups for 64 parts
 constexpr uint64_t kNaSymbols = 2 * kNaMaxOut;       // u16 symbols shared by the parts
 constexpr uint64_t kNaPartBytes = 32 << 10;          // compressed bytes per part
 constexpr int kNaMaxRetries = 32;
@@ -49,11 +49,12 @@ constexpr size_t kOffChunks = a256(kOffFiles + sizeof(FileDesc));
 constexpr size_t kOffG0 = a256(kOffChunks + kNaMaxParts * sizeof(ChunkDesc));
 constexpr size_t kOffGn = a256(kOffG0 + kNaMaxGroups * sizeof(int32_t));
 constexpr size_t kOffGfile = a256(kOffGn + kNaMaxGroups * sizeof(int32_t));
-constexpr size_t kOffSeg0 = a256(kOffGfile + kNaMaxGroups * sizeof(int32_t));
+constexpr size_t kOffUpper = a256(kOffGfile + kNaMaxGroups * sizeof(int32_t));
+constexpr size_t kOffSeg0 = a256(kOffUpper + 6 * sizeof(int32_t));
 constexpr size_t kOffWindows = a256(kOffSeg0 + sizeof(uint64_t));
 constexpr size_t kOffGmaps = a256(kOffWindows + (size_t)kNaMaxParts * kWin);
-constexpr size_t kOffWstart = a256(kOffGmaps + (size_t)kNaMaxGroups * kWin * sizeof(uint16_t));
-constexpr size_t kOffSym = a256(kOffWstart + (size_t)kNaMaxGroups * kWin);
+constexpr size_t kOffWstart = a256(kOffGmaps + (size_t)(kNaMaxGroups + 1) * kWin * sizeof(uint16_t));
+constexpr size_t kOffSym = a256(kOffWstart + (size_t)(kNaMaxGroups + 1) * kWin);
 constexpr size_t kOffStart = a256(kOffSym + kNaSymbols * sizeof(uint16_t));
 constexpr size_t kTokWords = 32 * 512;                // token rows of one of kNaMaxParts parts
 constexpr size_t kOffTok = a256(kOffStart + kNaSymbols / 8);
@@ -153,6 +154,7 @@ extern "C" int pgz_decompress_noalloc(const uint8_t* gz, uint64_t gz_len, uint8_
     int32_t* d_gn = reinterpret_cast<int32_t*>(base + kOffGn);
     int32_t* d_gfile = reinterpret_cast<int32_t*>(base + kOffGfile);
     uint64_t* d_seg0 = reinterpret_cast<uint64_t*>(base + kOffSeg0);
+    int32_t* d_upper = reinterpret_cast<int32_t*>(base + kOffUpper);
     uint8_t* d_windows = base + kOffWindows;
     uint16_t* d_gmaps = reinterpret_cast<uint16_t*>(base + kOffGmaps);
     uint8_t* d_wstart = base + kOffWstart;
@@ -200,8 +202,7 @@ extern "C" int pgz_decompress_noalloc(const uint8_t* gz, uint64_t gz_len, uint8_
         kp.team = n <= kNaMaxParts / 8 ? 16 : (n <= kNaMaxParts / 4 ? 8 : (n <= kNaMaxParts / 2 ? 4 : 2));
         kp.tok_rows = 256;
         static_assert(kTokWords * 8 == 16 * 32 * 256, "a team of 16 warps takes eight parts' shares");
-        uint64_t gsz = 1;
-        while (gsz * gsz < n) ++gsz;
+        const uint64_t gsz = (uint64_t)chain_group_size((int)n);
         int32_t g0[kNaMaxGroups], gn[kNaMaxGroups], gfile[kNaMaxGroups];
         int ng = 0;
         for (uint64_t a = 0; a < n; a += gsz, ++ng) {
@@ -222,6 +223,7 @@ extern "C" int pgz_decompress_noalloc(const uint8_t* gz, uint64_t gz_len, uint8_
         F.nchunks = (int32_t)n;
         F.group0 = 0;
         F.ngroups = ng;
+        F.nsupers = 1;                                 // at most 8 groups: one supergroup
         F.seg0 = 0;
         F.nseg = ((out_cap < (uint64_t)kNaMaxOut ? out_cap : (uint64_t)kNaMaxOut) + crc_segment_bytes() - 1) /
                  crc_segment_bytes();
@@ -233,13 +235,17 @@ extern "C" int pgz_decompress_noalloc(const uint8_t* gz, uint64_t gz_len, uint8_
         cudaMemcpyAsync(d_g0, g0, ng * sizeof(int32_t), cudaMemcpyHostToDevice, s);
         cudaMemcpyAsync(d_gn, gn, ng * sizeof(int32_t), cudaMemcpyHostToDevice, s);
         cudaMemcpyAsync(d_gfile, gfile, ng * sizeof(int32_t), cudaMemcpyHostToDevice, s);
+        const int32_t upper[6] = {0, ng, 0, 0, 1, 0};
+        cudaMemcpyAsync(d_upper, upper, sizeof upper, cudaMemcpyHostToDevice, s);
         cudaMemcpyAsync(d_seg0, &seg0, sizeof seg0, cudaMemcpyHostToDevice, s);
         cudaMemsetAsync(d_start, 0, kNaSymbols / 8, s);
         launch_sync(d_files, d_chunks, (int)n, d_sym, d_start, d_tok, d_queue, nullptr, kp, s);
         launch_inflate(d_files, d_chunks, (int)n, d_sym, d_start, d_tok, d_queue + 1, nullptr, kp, s);
         launch_exec(d_files, d_chunks, (int)n, d_sym, d_start, d_queue + 2, nullptr, kp, s);
         launch_plan(d_files, d_chunks, 1, s);
-        launch_chain(d_files, d_chunks, 1, ng, d_g0, d_gn, d_gfile, d_sym, d_gmaps, d_wstart, d_windows, s);
+        const ChainPlan cp{ng, 1, ng > 1, false, d_g0, d_gn, d_gfile, d_upper, d_upper + 1, d_upper + 2, d_upper + 3, d_upper + 4,
+                           d_upper + 5};
+        launch_chain(d_files, d_chunks, 1, cp, d_sym, d_gmaps, d_wstart, d_windows, s);
         launch_translate(d_files, d_chunks, (int)n, plan[0].cap, d_sym, d_windows, nullptr, s);
         launch_crc(d_files, 1, F.nseg, d_seg0, s);
         launch_finalize(d_files, 1, s);
