@@ -68,7 +68,9 @@ __constant__ uint32_t c_seg_shift[4][256]; // [j][b]: (byte b at byte j of a reg
 // the payload -- LIT: the token (bytes in its low 16 bits, their count above),
 // two literals when both codes fit the lookup width; LEN, DIST: the base to
 // which the extra bits are added.
-enum : uint32_t { K_LIT = 0, K_LEN = 1, K_DIST = 2, K_EOB = 3, K_LONG = 4, K_BAD = 5 };
+// Kinds from K_EOB on (bit 11 of the entry set) are rare: they end a parse, or need the longer codes.
+enum : uint32_t { K_LIT = 0, K_LEN = 1, K_DIST = 2, K_EOB = 4, K_LONG = 5, K_BAD = 6 };
+constexpr uint32_t kRare = 4u << 9;
 
 // Shared memory of a team: the NW warps of one block, all on one part.
 template <int NW>
@@ -516,8 +518,6 @@ __device__ __forceinline__ uint32_t entry_kind(uint32_t e) { return (e >> 9) & 7
 __device__ __forceinline__ uint32_t entry_value(uint32_t e, uint32_t x) {
     return (e >> 12) + ((x & ((1u << (e & 31u)) - 1u)) >> ((e >> 5) & 15u));
 }
-// output length of a literal entry (one or two)
-__device__ __forceinline__ uint32_t lit_count(uint32_t e) { return e >> 28; }
 
 // The first tokens of a candidate's block, by one warp whose lanes decode the
 // same bits: a false candidate fails after a few tokens (its literals must be
@@ -583,40 +583,62 @@ struct LaneParse {
     uint32_t st;
 };
 
-// The token at P.p of the lanes with `go` (two literals at once if PAIRS), kept in tok[P.n]; false at a symbol that
-// ends the parse (P.p stays at it; P.st says why).  One step for a literal, a match, or two literals: the words
-// around P.p are loaded anew (three loads that conflict little cost less than carrying them from step to step).
+__device__ __forceinline__ void st_global_if(bool on, uint32_t* a, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.global.u32 [%1], %2;\n\t}" ::"r"((uint32_t)on), "l"(a), "r"(v)
+                 : "memory");
+}
+__device__ __forceinline__ void st_global_u16_if(bool on, uint16_t* a, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.global.u16 [%1], %2;\n\t}" ::"r"((uint32_t)on), "l"(a),
+                 "h"((uint16_t)v)
+                 : "memory");
+}
+__device__ __forceinline__ void or_shared_if(bool on, uint32_t a, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p red.shared.or.b32 [%1], %2;\n\t}" ::"r"((uint32_t)on), "r"(a),
+                 "r"(v)
+                 : "memory");
+}
+
+// The token at P.p of a lane with `go` (two literals at once if PAIRS), kept in tok[P.n]; go becomes false at a
+// symbol that ends the parse (P.p stays at it; P.st says why).  One step for a literal, a match, or two literals, and
+// no branch but one for the rare entries: a step's time is the chain of its three shared-memory reads (the words, the
+// first entry, the distance's), about 250 cycles, against 650 with a branch for every kind.
 template <int NW, bool PAIRS>
-__device__ __forceinline__ bool next_token(const TeamSmem<NW>& S, LaneParse& P, uint32_t* tok) {
+__device__ __forceinline__ void next_token(const TeamSmem<NW>& S, LaneParse& P, bool& go, uint32_t* tok) {
     const uint32_t* w = S.bits + (P.p >> 5);
     const uint32_t w0 = w[0], w1 = w[1], w2 = w[2];
     const uint32_t x = __funnelshift_r(w0, w1, P.p);
     uint32_t e = S.tab[x & ((1u << LB) - 1u)];
-    if (entry_kind(e) == K_LONG) e = long_entry<NW>(S, x, 0);
-    uint32_t kind = entry_kind(e);
-    uint32_t t = PAIRS ? e >> 12 : 0x10000u | ((e >> 12) & 0xffu), drop = PAIRS ? e & 31u : (e >> 5) & 15u;
-    if (kind == K_LEN) {
-        const uint32_t q = (P.p & 31u) + (e & 31u);
-        const uint32_t y = __funnelshift_r(q < 32 ? w0 : w1, q < 32 ? w1 : w2, q);
-        uint32_t d = S.tab[(1u << LB) + (y & ((1u << DB) - 1u))];
-        if (entry_kind(d) == K_LONG) d = long_entry<NW>(S, y, 1);
-        kind = entry_kind(d);
-        t = 0x80000000u | (entry_value(e, x) << 16) | (entry_value(d, y) - 1u);
-        drop = (e & 31u) + (d & 31u);
+    uint32_t q = (P.p & 31u) + (e & 31u);
+    uint32_t y = __funnelshift_r(q < 32 ? w0 : w1, q < 32 ? w1 : w2, q);   // the bits after the code
+    uint32_t d = S.tab[(1u << LB) + (y & ((1u << DB) - 1u))];
+    bool len = e & (K_LEN << 9);
+    if (go && ((e | (len ? d : 0u)) & kRare)) {
+        if (entry_kind(e) == K_LONG) {
+            e = long_entry<NW>(S, x, 0);
+            q = (P.p & 31u) + (e & 31u);
+            y = __funnelshift_r(q < 32 ? w0 : w1, q < 32 ? w1 : w2, q);
+            d = S.tab[(1u << LB) + (y & ((1u << DB) - 1u))];
+        }
+        len = entry_kind(e) == K_LEN;
+        if (len && entry_kind(d) == K_LONG) d = long_entry<NW>(S, y, 1);
+        const uint32_t kind = len ? entry_kind(d) : entry_kind(e);
+        if (kind >= K_EOB) {
+            P.st = kind == K_EOB ? PS_EOB : PS_ERR;
+            go = false;
+        }
     }
-    if (kind >= K_EOB) {
-        P.st = kind == K_EOB ? PS_EOB : PS_ERR;
-        return false;
-    }
-    P.p += drop;
-    P.out_len += token_len(t);
-    tok[P.n] = t;
-    P.n += 32 * NW;
-    return true;
+    const uint32_t lit = PAIRS ? e >> 12 : 0x10000u | ((e >> 12) & 0xffu);
+    const uint32_t t = len ? 0x80000000u | (entry_value(e, x) << 16) | (entry_value(d, y) - 1u) : lit;
+    const uint32_t drop = len ? (e & 31u) + (d & 31u) : (PAIRS ? e & 31u : (e >> 5) & 15u);
+    st_global_if(go, tok + P.n, t);
+    P.p += go ? drop : 0u;
+    P.out_len += go ? token_len(t) : 0u;
+    P.n += go ? 32u * NW : 0u;
 }
 
-// In the loops below the lanes of a warp take every step together (the vote at its end): left to themselves, lanes
-// that took different branches run apart for the rest of the loop, and the warp does each group's steps in turn.
+// In the loops below the lanes of a warp take every step together (the vote every second one): left to themselves,
+// lanes that took different branches run apart for the rest of the loop, and the warp does each group's steps in
+// turn.
 
 // A: the tokens that start before p0 + seg, kept in tok[0], tok[T], ... up to tok[cap]
 template <int NW>
@@ -626,18 +648,15 @@ __device__ __forceinline__ void parse_own(TeamSmem<NW>& S, LaneParse& P, uint32_
     const uint32_t p0 = P.p, p1 = p0 + seg;
     uint8_t* list = &S.list[0][0] + tl;
     bool go = true;
-    while (__any_sync(FULL, go)) {
-        if (go) {
-            const uint32_t rel = P.p - p0, n = P.n;
-            go = next_token<NW, true>(S, P, tok);
-            if (!(n & T) && n < 2 * TeamSmem<NW>::kList * T) list[n / 2] = (uint8_t)rel;
-            if (P.n >= cap) {
-                P.st = PS_CAP;
-                go = false;
-            }
-            go = go && P.p < p1;
+    do {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (go && !(P.n & T) && P.n < 2 * TeamSmem<NW>::kList * T) list[P.n / 2] = (uint8_t)(P.p - p0);
+            next_token<NW, true>(S, P, go, tok);
+            go = go && P.p < p1 && P.n < cap;
         }
-    }
+    } while (__any_sync(FULL, go));
+    if (P.st == PS_OK && P.p < p1) P.st = PS_CAP;
 }
 
 // B: on through the segments after lane tl's (rel: the place in the first), literals one at a time, until a listed
@@ -650,33 +669,45 @@ __device__ __forceinline__ void parse_on(TeamSmem<NW>& S, LaneParse& P, bool go,
                                          uint32_t* tok, uint32_t cap, uint32_t& m, uint32_t& j) {
     constexpr uint32_t T = 32 * NW;
     const uint32_t give_up = min(T, tl + 2 + kMeetBits / seg);
-    m = tl + 1;
+    m = min(tl + 1, T - 1);
     j = 0;
-    uint32_t at = 0, cnt = m < T ? S.r_cnt[m] : 0u;    // place of entry j of lane m's list; its entries
+    uint32_t at = 0, cnt = S.r_cnt[m];                 // place of entry j of lane m's list; its entries
+    uint32_t nx = S.list[1][m];                        // its next entry
     while (__any_sync(FULL, go)) {
-        if (go) {
-            if (rel >= seg) {
-                rel -= seg;
-                ++m;
-                j = at = 0;
-                cnt = m < T ? S.r_cnt[m] : 0u;
-            }
-            while (at < rel && j + 1 < cnt) {
-                ++j;
-                at += (S.list[j][m] - at) & 255u;
-            }
-            if (m >= give_up || P.n >= cap) {
+        if (go && rel >= seg) {                        // the next lane's segment
+            rel -= seg;
+            ++m;
+            if (m >= give_up) {
                 P.st = PS_NOSYNC;
                 go = false;
-            } else if (at == rel) {
-                P.st = PS_SYNC;
-                go = false;
             } else {
-                const uint32_t p = P.p;
-                go = next_token<NW, false>(S, P, tok);
-                rel += P.p - p;
+                j = at = 0;
+                cnt = S.r_cnt[m];
+                nx = S.list[1][m];
             }
         }
+        if (go && P.n >= cap) {
+            P.st = PS_NOSYNC;
+            go = false;
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {                  // along the list, to the first entry at or after rel
+            const bool adv = go && at < rel && j + 1 < cnt;
+            at += adv ? (nx - at) & 255u : 0u;
+            j += adv ? 1u : 0u;
+            if (adv && j + 1 < cnt) nx = S.list[j + 1][m];
+        }
+        const bool behind = at < rel && j + 1 < cnt;   // not there yet: no token in this step
+        if (go && at == rel) {
+            P.st = PS_SYNC;
+            go = false;
+        }
+        bool step = go && !behind;
+        const bool was = step;
+        const uint32_t p = P.p;
+        next_token<NW, false>(S, P, step, tok);
+        rel += P.p - p;
+        go = go && (step || !was);
     }
 }
 
@@ -707,18 +738,22 @@ __device__ __noinline__ bool tokens_allowed(const TeamSmem<NW>& S, const uint32_
     return ok;
 }
 
-// C: the copy map of the tokens [n, z), from position `pos` on.  Only the places where a token starts are written
+// C: the copy map of the tokens [n, z), from position base + pos on (map and words from position base on, a multiple
+// of kRestart).  Only the places where a token starts are written
 // (a u16 each, and its start bit): k_exec spreads the matches, many threads to each.  The start bits go to shared
-// memory (sb, from bit 0 of position pos0's word on) when the round's fit there (sb not null), else to `start`.
+// memory (SHARED: words from the round's first on), when the round's fit there, else to the part's own words.
 // Returns false if (check) a literal is not an allowed byte.
-template <int NW>
+template <int NW, bool SHARED>
 __device__ __forceinline__ bool write_map(const TeamSmem<NW>& S, const uint32_t* tok, uint32_t n, uint32_t z,
-                                          uint16_t* map, uint32_t* start, uint32_t* sb, uint32_t pos0, uint32_t pos,
-                                          bool check, bool& neg) {
+                                          uint16_t* map, uint32_t* words, uint32_t pos, uint32_t base, bool check, bool& neg) {
     constexpr uint32_t T = 32 * NW;
     constexpr int kAhead = 4;
+    const uint32_t words_a = SHARED ? (uint32_t)__cvta_generic_to_shared(words) : 0u;
+    auto set = [&](bool on, uint32_t word, uint32_t bits) {
+        if (SHARED) or_shared_if(on, words_a + 4 * word, bits);
+        else if (on) atomicOr(words + word, bits);
+    };
     bool ok = true;
-    uint32_t* words = sb ? sb - (pos0 >> 5) : start;
     uint32_t nx[kAhead];
 #pragma unroll
     for (int k = 0; k < kAhead; ++k) nx[k] = n + k * T < z ? tok[n + k * T] : 0u;
@@ -735,20 +770,21 @@ __device__ __forceinline__ bool write_map(const TeamSmem<NW>& S, const uint32_t*
             const bool match = t >> 31, two = !match && len > 1;
             const uint32_t code = match ? kPH | d : t & 0xffu, b1 = (t >> 8) & 0xffu;
             if (check && !match && len) ok &= allowed_has(S.allowed, code) && (!two || allowed_has(S.allowed, b1));
-            neg |= match && pos <= d;
-            if (len) {
-                atomicOr(words + (pos >> 5), (two ? 3u : 1u) << (pos & 31u));
-                map[pos] = (uint16_t)code;
-            }
-            if (two) map[pos + 1] = (uint16_t)b1;
+            neg |= match && base + pos <= d;
+            set(len != 0, pos >> 5, (two ? 3u : 1u) << (pos & 31u));
+            st_global_u16_if(len != 0, map + pos, code);
+            st_global_u16_if(two, map + pos + 1, b1);
             const uint32_t r = (pos | (kRestart - 1)) + 1, e = pos + len;
-            if (r < e) {                        // the second literal, or the match, starts anew at r
-                for (uint32_t a = r; a < e; a += kRestart) {
-                    if (match) map[a] = (uint16_t)code;
-                    atomicOr(words + (a >> 5), 1u);
+            if (r < e || (two && !(~pos & 31u))) {
+                // the match starts anew at every multiple of kRestart; the second literal's bit is the next word's
+                if (match) {
+                    for (uint32_t a = r; a < e; a += kRestart) {
+                        map[a] = (uint16_t)code;
+                        set(true, a >> 5, 1u);
+                    }
+                } else {
+                    set(true, (pos >> 5) + 1, 1u);
                 }
-            } else if (two && !(~pos & 31u)) {  // the second literal's bit is the next word's
-                atomicOr(words + (pos >> 5) + 1, 1u);
             }
             pos = e;
         }
@@ -867,19 +903,21 @@ __device__ int par_block(TeamSmem<NW>& S, const Input& in, uint64_t s0, uint64_t
         bool neg = false;
         o.hi = max(o.hi, o.n + total);
         // the round's start bits, in the lists' place if they fit
-        const uint32_t pos0 = (uint32_t)o.n, nw = (uint32_t)((o.n + total + 31) / 32 - o.n / 32);
+        const uint32_t pos0 = (uint32_t)o.n, map0 = pos0 & ~(kRestart - 1);
+        const uint32_t nw = (uint32_t)((o.n + total + 31) / 32) - map0 / 32;
         uint32_t* sb = nw <= sizeof(S.list) / 4 ? reinterpret_cast<uint32_t*>(&S.list[0][0]) : nullptr;
         if (sb) {
             for (uint32_t k = tl; k < nw; k += T) sb[k] = 0;
             team_sync<NW>();
         }
-        const bool ok = write_map<NW>(S, tok, skip, mine ? n : skip, o.sym, o.start, sb, pos0,
-                                      pos0 + before + incl - len, check, neg);
+        const uint32_t to = mine ? n : skip, at = pos0 + before + incl - len;
+        const bool ok = sb ? write_map<NW, true>(S, tok, skip, to, o.sym + map0, sb, at - map0, map0, check, neg)
+                           : write_map<NW, false>(S, tok, skip, to, o.sym, o.start, at, 0, check, neg);
         const bool bad = team_or<NW>(!ok);
         if (sb)
             for (uint32_t k = tl; k < nw; k += T) {
-                uint32_t* g = o.start + (pos0 >> 5) + k;
-                if (k == 0 || k + 1 == nw) atomicOr(g, sb[k]);    // words shared with the rounds before and after
+                uint32_t* g = o.start + (map0 >> 5) + k;
+                if (k <= (pos0 - map0) >> 5 || k + 1 == nw) atomicOr(g, sb[k]);   // words shared with other rounds
                 else *g = sb[k];
             }
         o.neg |= neg;
