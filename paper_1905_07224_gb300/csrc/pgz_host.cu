@@ -134,6 +134,7 @@ namespace {
 
 constexpr uint64_t kMaxPartSymbols = (1ull << 31) - 256;   // part positions are 32-bit in the kernels
 constexpr int kMaxRetries = 32;
+constexpr uint64_t kAtPartBytes = 64 << 10;                // parts of pgz_decompress_at when n_chunks is set
 
 struct DBuf {
     void* p = nullptr;
@@ -243,6 +244,11 @@ struct Plan {
     bool results_valid = false;   // the device chunk array holds the last run's results
     int wpb = 4;                  // warps per block of the pass-1 kernels (sizes the token scratch)
     const uint8_t* fill = nullptr;   // device window of fill bytes (mode 1)
+    // mode 1 in several parts: where its symbols and bytes go (launch_resolve_at), and its counts (2 u64)
+    uint16_t* at_sym = nullptr;
+    uint8_t* at_bytes = nullptr;
+    uint8_t at_fill = 0;
+    DBuf d_at;
     DBuf d_files, d_chunks, d_g0, d_gn, d_gfile, d_upper, d_seg0, d_sym, d_windows, d_gmaps, d_wstart, d_tok, d_start, d_queue, d_order;
     PBuf h_files, h_chunks, h_static;
     cudaGraphExec_t graph = nullptr;
@@ -263,6 +269,7 @@ struct Plan {
         d_start.release();
         d_queue.release();
         d_order.release();
+        d_at.release();
         h_files.release();
         h_chunks.release();
         h_static.release();
@@ -278,6 +285,7 @@ struct pgz_ctx {
     KParams kp;
     cudaStream_t stream = nullptr;
     Plan plan;                 // the last call's plan (kept for inspection)
+    Plan at_plan;              // pgz_decompress_at: the run in several parts (its result becomes `plan`'s one part)
     PBuf hdr;                  // header / trailer staging
     DBuf in_buf, out_buf, fill_buf;
     DBuf carry_win;            // streaming: the resolved window a segment leaves for the next
@@ -446,6 +454,7 @@ int layout(Plan& P) {
     P.upper.clear();
     for (const auto& v : lv) P.upper.insert(P.upper.end(), v.begin(), v.end());
     const size_t nm = ng + P.nsupers;                // maps and first windows of both levels
+    const size_t wb = P.at_sym ? 2 * (size_t)kWin : (size_t)kWin;   // bytes of a window
     cudaError_t e = cudaSuccess;
     if (!e) e = P.d_files.ensure(nf * sizeof(FileDesc));
     if (!e) e = P.d_chunks.ensure(nc * sizeof(ChunkDesc));
@@ -457,11 +466,12 @@ int layout(Plan& P) {
     if (!e) e = P.d_sym.ensure(P.sym_total * sizeof(uint16_t));
     if (!e) e = P.d_tok.ensure((size_t)token_words((int)nc, P.wpb) * sizeof(uint32_t));
     if (!e) e = P.d_start.ensure(P.sym_total / 8);
+    if (!e && P.at_sym) e = P.d_at.ensure(2 * sizeof(uint64_t));
     if (!e) e = P.d_queue.ensure(3 * sizeof(uint32_t));
     if (!e) e = P.d_order.ensure(nc * sizeof(uint32_t));
-    if (!e && P.chain) e = P.d_windows.ensure(nc * (size_t)kWin);
+    if (!e && P.chain) e = P.d_windows.ensure(nc * wb);
     if (!e && P.chain) e = P.d_gmaps.ensure(nm * (size_t)kWin * sizeof(uint16_t));
-    if (!e && P.chain) e = P.d_wstart.ensure(nm * (size_t)kWin);
+    if (!e && P.chain) e = P.d_wstart.ensure(nm * wb);
     if (!e) e = P.h_files.ensure(nf * sizeof(FileDesc));
     if (!e) e = P.h_chunks.ensure(nc * sizeof(ChunkDesc));
     if (!e) e = P.h_static.ensure(3 * round_up(ng * sizeof(int32_t), 16) + round_up(nf * sizeof(uint64_t), 16) +
@@ -528,7 +538,12 @@ int enqueue(pgz_ctx* ctx, Plan& P, cudaStream_t s, bool timed, cudaStream_t up =
         const size_t ns = P.nsupers;
         const ChainPlan cp{(int)ng, (int)ns, P.many, P.deep, P.d_g0.as<int32_t>(), P.d_gn.as<int32_t>(), P.d_gfile.as<int32_t>(),
                            u, u + ns, u + 2 * ns, u + 3 * ns, u + 3 * ns + nf, u + 3 * ns + 2 * nf};
-        launch_chain(df, dc, (int)nf, cp, sym, P.d_gmaps.as<uint16_t>(), P.d_wstart.as<uint8_t>(),
+        if (P.at_sym) {
+            launch_resolve_at(df, dc, (int)nc, cp, sym, P.d_gmaps.as<uint16_t>(), P.d_wstart.as<uint16_t>(),
+                              P.d_windows.as<uint16_t>(), P.at_sym, P.at_bytes, P.at_fill,
+                              P.d_at.as<unsigned long long>(), s);
+            k += 1;
+        } else launch_chain(df, dc, (int)nf, cp, sym, P.d_gmaps.as<uint16_t>(), P.d_wstart.as<uint8_t>(),
                      P.d_windows.as<uint8_t>(), s);
         k += 1 + (P.many ? 2 : 0) + (P.deep ? 2 : 0);
     }
@@ -983,6 +998,8 @@ void begin_plan(Plan& P) {
     P.chain = P.translate = P.crc = true;
     P.results_valid = false;
     P.fill = nullptr;
+    P.at_sym = nullptr;
+    P.at_bytes = nullptr;
     if (P.graph) cudaGraphExecDestroy(P.graph);
     P.graph = nullptr;
 }
@@ -1224,6 +1241,7 @@ void pgz_destroy(pgz_ctx* ctx) {
     cudaSetDevice(ctx->cfg.device);
     cudaStreamSynchronize(ctx->stream);
     ctx->plan.release();
+    ctx->at_plan.release();
     ctx->carry_win.release();
     for (int k = 0; k < 2; ++k) {
         ctx->sin[k].release();
@@ -1276,6 +1294,111 @@ int pgz_decompress_host(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, uint8_
     return e;
 }
 
+// Decoding from bit lo (the first block's when at_start) to the member's end in several parts, each with its own block
+// start and symbolic context, the parts' windows then chained as symbols relative to the first part's context.  The
+// result becomes the one part of ctx->plan, as a run in one part leaves it.  Returns PGZ_OK, or anything else when the
+// caller shall run it in one part instead (too short, or an error: what to report is that run's to say).
+static int decompress_at_parts(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, const MemberInfo& mi, uint64_t lo,
+                               bool at_start, uint8_t* byte_out, uint8_t fill, uint64_t out_cap, uint64_t* last_ph) {
+    const uint64_t end_bit = (gz_len - 8) * 8;
+    if (lo >= end_bit) return PGZ_E_NOSYNC;
+    const uint64_t bits = end_bit - lo, csize = bits / 8 + 1;
+    const uint64_t per_bytes = ctx->cfg.n_chunks > 0 ? kAtPartBytes : std::max<uint64_t>(ctx->cfg.chunk_bytes, 4096);
+    const uint64_t n = (csize + per_bytes - 1) / per_bytes;
+    if (n < 2 || n > (1u << 20)) return PGZ_E_NOSYNC;
+    Plan& R = ctx->plan;
+    begin_plan(R);
+    const uint64_t cap1 = round_up(std::max<uint64_t>(out_cap, 65536), 32);
+    if (cap1 > kMaxPartSymbols) return PGZ_E_NOSYNC;
+    if (cuda_status(R.d_sym.ensure(cap1 * sizeof(uint16_t)))) return PGZ_E_NOMEM;
+    Plan& P = ctx->at_plan;
+    begin_plan(P);
+    P.translate = P.crc = false;
+    P.at_sym = R.d_sym.as<uint16_t>();
+    P.at_bytes = byte_out;
+    P.at_fill = fill;
+    FileDesc F{};
+    F.gz = gz;
+    F.gz_len = gz_len;
+    F.out_cap = out_cap;
+    F.s0_bit = mi.s0 * 8;
+    F.end_bit = end_bit;
+    F.mode = 1;
+    F.out_hi = kNone;
+    F.nchunks = (int32_t)n;
+    const uint64_t per = (bits + n - 1) / n;
+    const uint64_t whole = std::max<uint64_t>(1, gz_len - 8 - mi.s0);
+    // symbols expected per part: its share of ISIZE (exact below 4 GiB); 2x the compressed size bounds text otherwise
+    const uint64_t est = std::max<uint64_t>((uint64_t)((double)mi.isize * (double)csize / (double)whole), 2 * csize);
+    for (uint64_t i = 0; i < n; ++i) {
+        ChunkDesc C{};
+        C.lo = lo + i * per;
+        C.hi = std::min<uint64_t>(lo + (i + 1) * per, end_bit);
+        C.disabled = (i > 0 && C.lo >= end_bit) ? 1u : 0u;
+        C.index = (int32_t)(i + (at_start ? 0 : 1));
+        C.cap = std::min<uint64_t>(round_up(2 * est / n + 65536, 32), kMaxPartSymbols);
+        C.stop_hint = kNone;
+        C.sync = kNone;
+        P.chunks.push_back(C);
+    }
+    const uint64_t gsz = (uint64_t)chain_group_size((int)n);
+    for (uint64_t a = 0; a < n; a += gsz) {
+        P.g0.push_back((int32_t)a);
+        P.gn.push_back((int32_t)std::min<uint64_t>(gsz, n - a));
+        P.gfile.push_back(0);
+        F.ngroups++;
+    }
+    P.files.push_back(F);
+    int e = execute(ctx, P, nullptr);
+    if (e) return e;
+    e = read_chunks(ctx, P);
+    if (e) return e;
+    const ChunkDesc* res = P.h_chunks.as<ChunkDesc>();
+    uint64_t first = kNone;
+    for (uint64_t i = 0; i < n && first == kNone; ++i)
+        if (res[i].state == CS_DONE) first = res[i].sync;
+    if (first == kNone) return PGZ_E_NOSYNC;
+    uint64_t counts[2] = {0, 0};
+    if (cudaMemcpyAsync(counts, P.d_at.p, sizeof counts, cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess ||
+        cudaStreamSynchronize(ctx->stream) != cudaSuccess)
+        return PGZ_E_CUDA;
+    // the result as one part
+    FileDesc RF = F;
+    RF.nchunks = 1;
+    RF.ngroups = 0;
+    RF.total = P.files[0].total;
+    RF.status = PGZ_OK;
+    RF.bad_chunk = 0xffffffffu;
+    ChunkDesc C{};
+    C.lo = lo;
+    C.hi = end_bit;
+    C.cap = cap1;
+    C.index = at_start ? 0 : 1;
+    C.stop_hint = kNone;
+    C.sync = first;
+    C.n = RF.total;
+    C.nph = counts[0];
+    C.last_ph = counts[1];
+    C.det = kNone;
+    C.end = end_bit;
+    C.state = CS_DONE;
+    C.final = 1;
+    C.confirmed = 1;
+    C.anyph = counts[0] != 0;
+    R.files.push_back(RF);
+    R.chunks.push_back(C);
+    R.chain = R.crc = false;
+    R.sym_total = cap1;
+    if (cuda_status(R.d_chunks.ensure(sizeof C)) || cuda_status(R.h_chunks.ensure(sizeof C))) return PGZ_E_NOMEM;
+    memcpy(R.h_chunks.p, &C, sizeof C);
+    if (cudaMemcpyAsync(R.d_chunks.p, R.h_chunks.p, sizeof C, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
+        cudaStreamSynchronize(ctx->stream) != cudaSuccess)
+        return PGZ_E_CUDA;
+    R.results_valid = true;
+    *last_ph = counts[1];
+    return PGZ_OK;
+}
+
 int pgz_decompress_at(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, uint64_t start_bit, uint16_t* sym_out,
                       uint8_t* byte_out, uint8_t fill, uint64_t out_cap, uint64_t* out_len, uint64_t* block_bit,
                       uint64_t* first_determined) {
@@ -1285,9 +1408,27 @@ int pgz_decompress_at(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, uint64_t
     MemberInfo mi;
     int e = read_member(ctx, gz, gz_len, &mi);
     if (e) return e;
+    const uint64_t s0_bit = mi.s0 * 8, end_bit = (gz_len - 8) * 8;
+    {
+        uint64_t last = 0;
+        const bool first = start_bit <= s0_bit;
+        e = decompress_at_parts(ctx, gz, gz_len, mi, first ? s0_bit : start_bit, first, byte_out, fill, out_cap, &last);
+        if (e == PGZ_OK) {
+            const ChunkDesc& C = ctx->plan.chunks[0];
+            *out_len = C.n;
+            if (block_bit) *block_bit = C.sync;
+            if (first_determined) *first_determined = last;
+            if (sym_out && C.n &&
+                (cudaMemcpyAsync(sym_out, ctx->plan.d_sym.p, C.n * sizeof(uint16_t), cudaMemcpyDeviceToDevice,
+                                 ctx->stream) != cudaSuccess ||
+                 cudaStreamSynchronize(ctx->stream) != cudaSuccess))
+                return PGZ_E_CUDA;
+            return PGZ_OK;
+        }
+        if (e == PGZ_E_CUDA) return e;
+    }
     Plan& P = ctx->plan;
     begin_plan(P);
-    const uint64_t s0_bit = mi.s0 * 8, end_bit = (gz_len - 8) * 8;
     FileDesc F{};
     if (!byte_out) {                                   // the translation still counts the placeholders
         if (cuda_status(ctx->out_buf.ensure(out_cap))) return PGZ_E_NOMEM;

@@ -148,6 +148,11 @@ int chain_group_size(int n);
 int chain_super_size(int ngroups);
 void launch_chain(const FileDesc* files, const ChunkDesc* chunks, int nfiles, const ChainPlan& C, const uint16_t* sym,
                   uint16_t* gmaps, uint8_t* wstart, uint8_t* windows, cudaStream_t s);
+// The same for one member decoded from a bit offset in several parts (mode 1), its windows u16 symbols relative to the
+// unknown context before its first part (wstart, windows: kWin u16 each), then its symbols in order (k_resolve_at).
+void launch_resolve_at(const FileDesc* files, const ChunkDesc* chunks, int nchunks, const ChainPlan& C,
+                       const uint16_t* sym, uint16_t* gmaps, uint16_t* wstart, uint16_t* windows, uint16_t* sym_out,
+                       uint8_t* byte_out, uint8_t fill, unsigned long long* res, cudaStream_t s);
 void launch_translate(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint64_t max_cap,
                       const uint16_t* sym, const uint8_t* windows, const uint8_t* fill_window, cudaStream_t s);
 // total_seg: CRC segments of crc_segment_bytes() output bytes over all members (FileDesc::seg0, nseg)

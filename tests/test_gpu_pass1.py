@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 
 import deflate_writer as dw
+import oracle
 from gpu_util import Ctx, empty, to_device
 from paper_1905_07224_gb300 import synth
 
@@ -98,3 +99,38 @@ def test_block_decoder_edges(kind, wpb):
             assert k == len(text) and out == text, n
         finally:
             ctx.close()
+
+
+@pytest.mark.parametrize("chunk", [4096, 16384, 65536])
+@pytest.mark.parametrize("kind", ["fastq", "markov", "runs", "tail"])
+def test_decoding_from_an_offset_in_several_parts(kind, chunk):
+    """pgz_decompress_at over one, two and many parts equals the oracle's one symbolic decode: symbols, bytes, block
+    start, last placeholder; so do the inspection calls, which report one part."""
+    import torch
+    text = {"fastq": lambda: synth.fastq(900_001, 150, 0.001, 8), "markov": lambda: synth.markov(400_003, 9),
+            "runs": lambda: (b"@ab\n" * 40_000 + synth.fastq(200_000, 100, 0.0, 3)) * 2,
+            "tail": lambda: synth.fastq(150_000, 100, 0.0, 4)}[kind]()
+    gz = synth.gzip_compress(text, 6)
+    ctx = Ctx(chunk_bytes=chunk)
+    try:
+        d = to_device(gz)
+        cap = len(text) + 1000
+        for start in [0, 8 * len(gz) // 5, 8 * len(gz) // 2 + 3]:
+            ref = oracle.decompress_at(gz, start, fill=ord("?"))
+            sym, byt = torch.zeros(cap, dtype=torch.int16, device="cuda"), empty(cap)
+            st, n, bb, fd = ctx.pgz.pgz_decompress_at(ctx.h, d.data_ptr(), len(gz), start, sym.data_ptr(),
+                                                      byt.data_ptr(), ord("?"), cap)
+            if ref["status"]:
+                assert st != 0
+                continue
+            assert st == 0, ctx.pgz.pgz_strerror(st)
+            assert (n, bb, fd) == (ref["sym"].size, ref["block_bit"], ref["first_determined"])
+            assert np.array_equal(sym[:n].cpu().numpy().view(np.uint16), ref["sym"])
+            assert byt[:n].cpu().numpy().tobytes() == ref["bytes"]
+            sb, ns, nph = ctx.pgz.pgz_inspect_parts(ctx.h)
+            assert list(sb) == [bb] and list(ns) == [n] and list(nph) == [int((ref["sym"] >= 0x8000).sum())]
+            assert np.array_equal(ctx.pgz.pgz_inspect_symbols(ctx.h, 0), ref["sym"])
+            st, n, _, _ = ctx.pgz.pgz_decompress_at(ctx.h, d.data_ptr(), len(gz), start, None, None, 0, n - 1)
+            assert st == ctx.pgz.PGZ_E_CAPACITY and n == ref["sym"].size
+    finally:
+        ctx.close()
