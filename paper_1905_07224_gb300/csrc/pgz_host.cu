@@ -288,6 +288,7 @@ struct pgz_ctx {
     Plan at_plan;              // pgz_decompress_at: the run in several parts (its result becomes `plan`'s one part)
     PBuf hdr;                  // header / trailer staging
     DBuf in_buf, out_buf, fill_buf;
+    DBuf seq_bits;             // sequence extraction: class bits of the symbols
     DBuf carry_win;            // streaming: the resolved window a segment leaves for the next
     DBuf sin[2], sout[2];      // streaming: compressed bytes and output of two segments in flight
     PBuf stage[2];             // streaming: pinned output of two segments
@@ -1252,6 +1253,7 @@ void pgz_destroy(pgz_ctx* ctx) {
     ctx->in_buf.release();
     ctx->out_buf.release();
     ctx->fill_buf.release();
+    ctx->seq_bits.release();
     for (int k = 0; k < 8; ++k)
         if (ctx->ev[k]) cudaEventDestroy(ctx->ev[k]);
     if (ctx->hb_up) cudaStreamSynchronize(ctx->hb_up);
@@ -2194,7 +2196,8 @@ int pgz_extract_sequences(pgz_ctx* ctx, const uint16_t* sym, uint64_t n, uint32_
     *n_spans = *n_undetermined = 0;
     if (cuda_status(ctx->fill_buf.ensure(std::max<size_t>(kWin, 2 * sizeof(unsigned long long))))) return PGZ_E_NOMEM;
     unsigned long long* counts = ctx->fill_buf.as<unsigned long long>();
-    launch_sequences(sym, n, min_len, spans, max_spans, counts, ctx->stream);
+    if (cuda_status(ctx->seq_bits.ensure(sequence_words(n) * sizeof(uint32_t)))) return PGZ_E_NOMEM;
+    launch_sequences(sym, n, min_len, ctx->seq_bits.as<uint32_t>(), spans, max_spans, counts, ctx->stream);
     if (cudaPeekAtLastError() != cudaSuccess) return PGZ_E_CUDA;
     if (cuda_status(ctx->hdr.ensure(2 * sizeof(unsigned long long)))) return PGZ_E_NOMEM;
     unsigned long long* h = ctx->hdr.as<unsigned long long>();
@@ -2203,7 +2206,7 @@ int pgz_extract_sequences(pgz_ctx* ctx, const uint16_t* sym, uint64_t n, uint32_
         return PGZ_E_CUDA;
     *n_spans = h[0];
     *n_undetermined = h[1];
-    ctx->launches += 1;
+    ctx->launches += 2;
     return PGZ_OK;
 }
 

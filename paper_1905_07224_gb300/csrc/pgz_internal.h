@@ -161,8 +161,10 @@ void launch_crc(FileDesc* files, int nfiles, uint64_t total_seg, const uint64_t*
 void launch_finalize(FileDesc* files, int nfiles, cudaStream_t s);
 // DNA sequences among n u16 symbols: spans[2k] = start, spans[2k+1] = length | bit 63 if undetermined
 // symbols lie inside; counts[0] = spans found (may exceed max_spans), counts[1] = those with undetermined
-void launch_sequences(const uint16_t* sym, uint64_t n, uint32_t min_len, uint64_t* spans, uint64_t max_spans,
-                      unsigned long long* counts, cudaStream_t s);
+// (bits: sequence_words(n) u32 of scratch)
+uint64_t sequence_words(uint64_t n);
+void launch_sequences(const uint16_t* sym, uint64_t n, uint32_t min_len, uint32_t* bits, uint64_t* spans,
+                      uint64_t max_spans, unsigned long long* counts, cudaStream_t s);
 // ChunkDesc::nph and last_ph from the symbols of every finished part (statistics and inspection only)
 void launch_count_ph(ChunkDesc* chunks, int nchunks, const uint16_t* sym, cudaStream_t s);
 void upload_crc_tables();

@@ -134,3 +134,25 @@ def test_decoding_from_an_offset_in_several_parts(kind, chunk):
             assert st == ctx.pgz.PGZ_E_CAPACITY and n == ref["sym"].size
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 255, 256, 257, 8191, 8192, 8193, 70001])
+def test_sequences_at_word_and_block_edges(n):
+    """Runs over words of 32 symbols and over the kernels' blocks, ends of the array included, against the oracle."""
+    import torch
+    rng = np.random.default_rng(n)
+    kinds = np.array([ord("A"), ord("C"), 0x8000 | 7, ord("\n"), ord("x")], dtype=np.uint16)
+    ctx = Ctx()
+    try:
+        for weights in [[4, 4, 1, 1, 0.3], [50, 50, 30, 0.3, 0.02], [1, 1, 1, 1, 1], [1, 0, 0, 0, 0], [0, 0, 1, 0, 0]]:
+            p = np.array(weights) / sum(weights)
+            s = kinds[rng.choice(5, size=n, p=p)]
+            d = torch.from_numpy(s.view(np.int16).copy()).cuda()
+            spans = torch.zeros((n + 1, 2), dtype=torch.int64, device="cuda")
+            for min_len in (0, 5):
+                want = oracle.sequences(s, min_len)
+                st, k, nu = ctx.pgz.pgz_extract_sequences(ctx.h, d.data_ptr(), n, min_len, spans.data_ptr(), n + 1)
+                got = sorted((int(a), int(b) & (2**63 - 1), int(b) < 0) for a, b in spans[:k].cpu().tolist())
+                assert st == 0 and got == want and nu == sum(u for _, _, u in want)
+    finally:
+        ctx.close()
