@@ -1943,9 +1943,11 @@ __global__ void __launch_bounds__(512) k_resolve_at(const FileDesc* __restrict__
 // pass 2b: translation U_j -> w_i[j], 8 symbols per thread per step
 // ---------------------------------------------------------------------------
 
-// Persistent: block b translates parts b, b + gridDim.x, ...; the part's
+// Persistent: block b translates units b, b + gridDim.x, ... (a unit is a part, or
+// a piece of one when there are few parts: 18 us for the 8 parts of a 1 MiB file
+// with one block each); the part's
 // window w_i is copied into shared memory (only if the part produced a
-// placeholder) while the block's previous part is translated (two tables).  The shared table is the window followed by the 256 byte
+// placeholder) while the block's previous unit is translated (two tables).  The shared table is the window followed by the 256 byte
 // values, so a symbol s (a byte b < 0x100, or 0x8000 | j for U_j) becomes
 // T[s ^ 0x8000]: window byte j for a placeholder, b for a byte, with no
 // branch.  Parts without any placeholder pack their bytes with byte
@@ -2007,16 +2009,18 @@ __device__ __forceinline__ uint64_t tail8(uint4 q, uint32_t nv) {
 __global__ void __launch_bounds__(kTransThreads, 2) k_translate(const FileDesc* __restrict__ files, ChunkDesc* chunks,
                                                                 int nchunks, const uint16_t* __restrict__ sym,
                                                                 const uint8_t* __restrict__ windows,
-                                                                const uint8_t* __restrict__ fillw) {
+                                                                const uint8_t* __restrict__ fillw, int split) {
     extern __shared__ __align__(16) uint8_t Wbuf[];      // two tables of kWin + 256 bytes (kTransSmem)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     if (threadIdx.x < 256) {
         Wbuf[kWin + threadIdx.x] = (uint8_t)threadIdx.x;
         Wbuf[2 * kWin + 256 + threadIdx.x] = (uint8_t)threadIdx.x;
     }
-    // the window of part c goes into table `buf` by asynchronous copies, one group per part
-    auto fetch = [&](int c, int buf) {
-        if (c < nchunks) {
+    const int nwork = nchunks * split;                   // unit w: piece w % split of part w / split
+    // the window of unit w's part goes into table `buf` by asynchronous copies, one group per unit
+    auto fetch = [&](int w, int buf) {
+        if (w < nwork) {
+            const int c = w / split;
             const ChunkDesc& C = chunks[c];
             if (files[C.file].status == PGZ_OK && C.state == CS_DONE && C.n != 0 && C.anyph) {
                 const uint8_t* src = fillw ? fillw : windows + (uint64_t)c * kWin;
@@ -2028,12 +2032,12 @@ __global__ void __launch_bounds__(kTransThreads, 2) k_translate(const FileDesc* 
     };
     fetch(blockIdx.x, 0);
     int buf = 0;
-    for (int c = blockIdx.x; c < nchunks; c += gridDim.x, buf ^= 1) {
-        fetch(c + gridDim.x, buf ^ 1);                    // the next part's window, while this part runs
-        cp_async_wait<1>();                               // this part's window (this thread's copies) ...
+    for (int w = blockIdx.x; w < nwork; w += gridDim.x, buf ^= 1) {
+        fetch(w + gridDim.x, buf ^ 1);                    // the next unit's window, while this one runs
+        cp_async_wait<1>();                               // this unit's window (this thread's copies) ...
         __syncthreads();                                  // ... and everyone else's
         const uint8_t* W = Wbuf + buf * (kWin + 256);
-        const ChunkDesc& C = chunks[c];
+        const ChunkDesc& C = chunks[w / split];
         const FileDesc& F = files[C.file];
         const bool ph = C.anyph != 0;
         if (F.status == PGZ_OK && C.state == CS_DONE && C.n != 0) {   // uniform per block
@@ -2044,8 +2048,13 @@ __global__ void __launch_bounds__(kTransThreads, 2) k_translate(const FileDesc* 
         const bool vec = F.out_lo == 0 && F.out_hi == kNone && ((reinterpret_cast<uintptr_t>(out) & 7) == 0);
         const uint32_t m = (uint32_t)(C.out_off & 7), sh = 8u * m;
         const uint32_t n32 = (uint32_t)C.n;
-        const uint32_t nsl = (n32 + kTransSlice - 1) / kTransSlice, per = (nsl + nwarp - 1) / nwarp;
-        const uint32_t j0 = min(nsl, per * (uint32_t)warp), j1 = min(nsl, per * (uint32_t)(warp + 1));
+        // the part's slices, those that hold output bytes in [lo, hi) only, in equal runs over the units' warps
+        uint32_t s0 = 0, nsl = (n32 + kTransSlice - 1) / kTransSlice;
+        if (lo > C.out_off) s0 = (uint32_t)min((lo - C.out_off) / kTransSlice, (uint64_t)nsl);
+        if (hi < C.out_off + n32) nsl = hi > C.out_off ? (uint32_t)((hi - C.out_off + kTransSlice - 1) / kTransSlice) : 0u;
+        const uint32_t cnt = nsl > s0 ? nsl - s0 : 0u, runs = (uint32_t)(nwarp * split);
+        const uint32_t per = (cnt + runs - 1) / runs, run = (uint32_t)(w % split) * nwarp + (uint32_t)warp;
+        const uint32_t j0 = s0 + min(cnt, per * run), j1 = s0 + min(cnt, per * (run + 1));
         // the determined tail (symbols from det32 on are bytes at byte det32 + k; det32 is a multiple of 8, so
         // each 8-symbol half lies wholly before or wholly inside it): copied, not translated
         const uint32_t det32 = C.det < (uint64_t)n32 ? (uint32_t)C.det : 0xffffffffu;
@@ -2639,7 +2648,6 @@ int chain_super_size(int ngroups) {
 void launch_translate(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint64_t max_cap,
                       const uint16_t* sym, const uint8_t* windows, const uint8_t* fillw, cudaStream_t s) {
     if (nchunks <= 0) return;
-    (void)max_cap;
     static int resident[64] = {};                         // blocks of k_translate that fit on the device at once
     int dev = 0;
     cudaGetDevice(&dev);
@@ -2656,8 +2664,11 @@ void launch_translate(const FileDesc* files, ChunkDesc* chunks, int nchunks, uin
             cudaGetLastError();
     }
     const int cap = resident[slot] ? resident[slot] : 152 * 2;
-    const int grid = nchunks < cap ? nchunks : cap;
-    k_translate<<<grid, kTransThreads, kTransSmem, s>>>(files, chunks, nchunks, sym, windows, fillw);
+    // pieces of a part: enough units for the resident blocks, each piece worth its window's copy
+    const uint64_t pieces = std::max<uint64_t>(1, max_cap / (2 * kWin));
+    const int split = (int)std::min<uint64_t>({(uint64_t)std::max(1, cap / nchunks), pieces, 16});
+    const int grid = std::min(nchunks * split, cap);
+    k_translate<<<grid, kTransThreads, kTransSmem, s>>>(files, chunks, nchunks, sym, windows, fillw, split);
 }
 
 uint64_t crc_segment_bytes() { return kCrcSeg; }
