@@ -229,6 +229,15 @@ struct MemberInfo {
     uint32_t crc, isize;
 };
 
+// a place inside a device buffer
+struct DView {
+    void* p = nullptr;
+    template <class T>
+    T* as() const {
+        return static_cast<T*>(p);
+    }
+};
+
 // a planned set of members and their parts, with device buffers
 struct Plan {
     std::vector<FileDesc> files;
@@ -249,30 +258,28 @@ struct Plan {
     uint8_t* at_bytes = nullptr;
     uint8_t at_fill = 0;
     DBuf d_at;
-    DBuf d_files, d_chunks, d_g0, d_gn, d_gfile, d_upper, d_seg0, d_sym, d_windows, d_gmaps, d_wstart, d_tok, d_start, d_queue, d_order;
-    PBuf h_files, h_chunks, h_static;
+    // the plan's arrays lie in one device buffer, uploaded from one pinned copy: the work counters, members and
+    // parts first (head_bytes, which a graph uploads again), then what stays the same from run to run
+    DBuf d_plan;
+    PBuf h_plan;
+    DView d_queue, d_files, d_chunks, d_g0, d_gn, d_gfile, d_upper, d_seg0, d_order;
+    size_t plan_bytes = 0, head_bytes = 0;
+    DBuf d_sym, d_windows, d_gmaps, d_wstart, d_tok, d_start;
+    PBuf h_files, h_chunks;       // results read back
     cudaGraphExec_t graph = nullptr;
     uint64_t graph_launches = 0;  // kernels of the last enqueued run (a graph replays them)
     void release() {
-        d_files.release();
-        d_chunks.release();
-        d_g0.release();
-        d_gn.release();
-        d_gfile.release();
-        d_upper.release();
-        d_seg0.release();
+        d_plan.release();
+        h_plan.release();
         d_sym.release();
         d_windows.release();
         d_gmaps.release();
         d_wstart.release();
         d_tok.release();
         d_start.release();
-        d_queue.release();
-        d_order.release();
         d_at.release();
         h_files.release();
         h_chunks.release();
-        h_static.release();
         if (graph) cudaGraphExecDestroy(graph);
         graph = nullptr;
     }
@@ -287,6 +294,7 @@ struct pgz_ctx {
     Plan plan;                 // the last call's plan (kept for inspection)
     Plan at_plan;              // pgz_decompress_at: the run in several parts (its result becomes `plan`'s one part)
     PBuf hdr;                  // header / trailer staging
+    DBuf heads;                // a batch's members, and their headers and trailers gathered
     DBuf in_buf, out_buf, fill_buf;
     DBuf seq_bits;             // sequence extraction: class bits of the symbols
     DBuf carry_win;            // streaming: the resolved window a segment leaves for the next
@@ -347,6 +355,45 @@ int read_member(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, MemberInfo* mi
         mi->isize = t[4] | ((uint32_t)t[5] << 8) | ((uint32_t)t[6] << 16) | ((uint32_t)t[7] << 24);
         return PGZ_OK;
     }
+}
+
+// read_member for the jobs k with st[k] = PGZ_OK, with one kernel and one copy back; st[k] and mi[k] receive the results
+int read_members(pgz_ctx* ctx, int n, const pgz_job* jobs, std::vector<int>& st, std::vector<MemberInfo>& mi) {
+    std::vector<int> idx;
+    for (int k = 0; k < n; ++k) {
+        if (st[(size_t)k] != PGZ_OK) continue;
+        if (jobs[k].gz_len < 18) st[(size_t)k] = PGZ_E_HEADER;
+        else idx.push_back(k);
+    }
+    if (idx.empty()) return PGZ_OK;
+    const size_t m = idx.size(), in = round_up(m * sizeof(MemberRef), 256), row = kHeadBytes + 8;
+    if (cuda_status(ctx->hdr.ensure(in + m * row)) || cuda_status(ctx->heads.ensure(in + m * row))) return PGZ_E_NOMEM;
+    uint8_t *h = ctx->hdr.as<uint8_t>(), *d = ctx->heads.as<uint8_t>();
+    for (size_t i = 0; i < m; ++i) reinterpret_cast<MemberRef*>(h)[i] = MemberRef{jobs[idx[i]].gz, jobs[idx[i]].gz_len};
+    if (cudaMemcpyAsync(d, h, m * sizeof(MemberRef), cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess) return PGZ_E_CUDA;
+    launch_heads(reinterpret_cast<const MemberRef*>(d), (int)m, d + in, ctx->stream);
+    ctx->launches += 1;
+    if (cudaMemcpyAsync(h + in, d + in, m * row, cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess ||
+        cudaStreamSynchronize(ctx->stream) != cudaSuccess)
+        return PGZ_E_CUDA;
+    std::vector<int> again;                          // headers longer than what was read
+    for (size_t i = 0; i < m; ++i) {
+        const int k = idx[i];
+        const uint8_t *b = h + in + i * row, *t = b + kHeadBytes;
+        uint64_t s0 = 0;
+        const int r = parse_header(b, std::min<uint64_t>(kHeadBytes, jobs[k].gz_len), jobs[k].gz_len, &s0);
+        if (r == -1) {
+            again.push_back(k);
+            continue;
+        }
+        st[(size_t)k] = r == PGZ_OK ? PGZ_OK : PGZ_E_HEADER;
+        MemberInfo& M = mi[(size_t)k];
+        M.s0 = s0;
+        M.crc = t[0] | ((uint32_t)t[1] << 8) | ((uint32_t)t[2] << 16) | ((uint32_t)t[3] << 24);
+        M.isize = t[4] | ((uint32_t)t[5] << 8) | ((uint32_t)t[6] << 16) | ((uint32_t)t[7] << 24);
+    }
+    for (const int k : again) st[(size_t)k] = read_member(ctx, jobs[k].gz, jobs[k].gz_len, &mi[(size_t)k]);
+    return PGZ_OK;
 }
 
 // parts of one member: equal compressed size (Section "Full file decompression
@@ -457,62 +504,68 @@ int layout(Plan& P) {
     const size_t nm = ng + P.nsupers;                // maps and first windows of both levels
     const size_t wb = P.at_sym ? 2 * (size_t)kWin : (size_t)kWin;   // bytes of a window
     cudaError_t e = cudaSuccess;
-    if (!e) e = P.d_files.ensure(nf * sizeof(FileDesc));
-    if (!e) e = P.d_chunks.ensure(nc * sizeof(ChunkDesc));
-    if (!e) e = P.d_g0.ensure(ng * sizeof(int32_t));
-    if (!e) e = P.d_gn.ensure(ng * sizeof(int32_t));
-    if (!e) e = P.d_gfile.ensure(ng * sizeof(int32_t));
-    if (!e) e = P.d_upper.ensure(P.upper.size() * sizeof(int32_t));
-    if (!e) e = P.d_seg0.ensure(nf * sizeof(uint64_t));
+    size_t off = 0;
+    auto at = [&](size_t bytes) {
+        const size_t o = off;
+        off += round_up(bytes, 256);
+        return o;
+    };
+    const size_t o_queue = at(3 * sizeof(uint32_t)), o_files = at(nf * sizeof(FileDesc)), o_chunks = at(nc * sizeof(ChunkDesc));
+    P.head_bytes = off;
+    const size_t o_g0 = at(ng * sizeof(int32_t)), o_gn = at(ng * sizeof(int32_t)), o_gfile = at(ng * sizeof(int32_t));
+    const size_t o_upper = at(P.upper.size() * sizeof(int32_t)), o_seg0 = at(nf * sizeof(uint64_t));
+    const size_t o_order = at(nc * sizeof(uint32_t));
+    P.plan_bytes = off;
+    if (!e) e = P.d_plan.ensure(P.plan_bytes);
+    if (!e) e = P.h_plan.ensure(P.plan_bytes);
+    if (e) return cuda_status(e);
+    uint8_t *d = P.d_plan.as<uint8_t>(), *h = P.h_plan.as<uint8_t>();
+    P.d_queue.p = d + o_queue;
+    P.d_files.p = d + o_files;
+    P.d_chunks.p = d + o_chunks;
+    P.d_g0.p = d + o_g0;
+    P.d_gn.p = d + o_gn;
+    P.d_gfile.p = d + o_gfile;
+    P.d_upper.p = d + o_upper;
+    P.d_seg0.p = d + o_seg0;
+    P.d_order.p = d + o_order;
+    auto put = [&](size_t o, const void* src, size_t bytes) {
+        if (bytes) memcpy(h + o, src, bytes);
+    };
+    memset(h + o_queue, 0, 3 * sizeof(uint32_t));
+    put(o_g0, P.g0.data(), ng * sizeof(int32_t));
+    put(o_gn, P.gn.data(), ng * sizeof(int32_t));
+    put(o_gfile, P.gfile.data(), ng * sizeof(int32_t));
+    put(o_upper, P.upper.data(), P.upper.size() * sizeof(int32_t));
+    put(o_seg0, P.seg0.data(), nf * sizeof(uint64_t));
+    put(o_order, P.order.data(), nc * sizeof(uint32_t));
     if (!e) e = P.d_sym.ensure(P.sym_total * sizeof(uint16_t));
     if (!e) e = P.d_tok.ensure((size_t)token_words((int)nc, P.wpb) * sizeof(uint32_t));
     if (!e) e = P.d_start.ensure(P.sym_total / 8);
     if (!e && P.at_sym) e = P.d_at.ensure(2 * sizeof(uint64_t));
-    if (!e) e = P.d_queue.ensure(3 * sizeof(uint32_t));
-    if (!e) e = P.d_order.ensure(nc * sizeof(uint32_t));
     if (!e && P.chain) e = P.d_windows.ensure(nc * wb);
     if (!e && P.chain) e = P.d_gmaps.ensure(nm * (size_t)kWin * sizeof(uint16_t));
     if (!e && P.chain) e = P.d_wstart.ensure(nm * wb);
     if (!e) e = P.h_files.ensure(nf * sizeof(FileDesc));
     if (!e) e = P.h_chunks.ensure(nc * sizeof(ChunkDesc));
-    if (!e) e = P.h_static.ensure(3 * round_up(ng * sizeof(int32_t), 16) + round_up(nf * sizeof(uint64_t), 16) +
-                                  round_up(P.upper.size() * sizeof(int32_t), 16) + round_up(nc * sizeof(uint32_t), 16));
     return cuda_status(e);
 }
 
-// the device-resident part of a run: uploads, every stage, result download
-// the plan's static arrays (outside any graph capture), staged in pinned memory: a copy from pageable memory
-// is staged by the driver and may reach the copy engine after pinned copies issued later (the next group of
-// compressed bytes of a host-buffer batch), so that the run would wait for them
-void upload_static(Plan& P, cudaStream_t s) {
-    const size_t nf = P.files.size(), ng = P.g0.size(), nc = P.order.size();
-    uint8_t* h = P.h_static.as<uint8_t>();
-    size_t off = 0;
-    auto put = [&](void* dst, const void* src, size_t bytes) {
-        if (bytes) {
-            memcpy(h + off, src, bytes);
-            cudaMemcpyAsync(dst, h + off, bytes, cudaMemcpyHostToDevice, s);
-        }
-        off += round_up(bytes, 16);
-    };
-    put(P.d_g0.p, P.g0.data(), ng * sizeof(int32_t));
-    put(P.d_gn.p, P.gn.data(), ng * sizeof(int32_t));
-    put(P.d_gfile.p, P.gfile.data(), ng * sizeof(int32_t));
-    put(P.d_upper.p, P.upper.data(), P.upper.size() * sizeof(int32_t));
-    put(P.d_seg0.p, P.seg0.data(), nf * sizeof(uint64_t));
-    put(P.d_order.p, P.order.data(), nc * sizeof(uint32_t));
-}
-
+// The device-resident part of a run: the plan's upload, every stage, result download.  The upload is one copy from
+// pinned memory (a copy from pageable memory is staged by the driver and may reach the copy engine after pinned copies
+// issued later, the next group of compressed bytes of a host-buffer batch, so that the run would wait for them).
+// static_too: the whole plan, else (a graph's replays) what a run changes.
 // up/up_done (optional): the plan's uploads go on stream `up` instead, and the run waits for them (event
 // up_done); see pgz_decompress_batch_host
-int enqueue(pgz_ctx* ctx, Plan& P, cudaStream_t s, bool timed, cudaStream_t up = nullptr,
+int enqueue(pgz_ctx* ctx, Plan& P, cudaStream_t s, bool timed, bool static_too, cudaStream_t up = nullptr,
             cudaEvent_t up_done = nullptr) {
     const size_t nf = P.files.size(), nc = P.chunks.size(), ng = P.g0.size();
     const cudaStream_t u = up ? up : s;
-    memcpy(P.h_files.p, P.files.data(), nf * sizeof(FileDesc));
-    memcpy(P.h_chunks.p, P.chunks.data(), nc * sizeof(ChunkDesc));
-    cudaMemcpyAsync(P.d_files.p, P.h_files.p, nf * sizeof(FileDesc), cudaMemcpyHostToDevice, u);
-    cudaMemcpyAsync(P.d_chunks.p, P.h_chunks.p, nc * sizeof(ChunkDesc), cudaMemcpyHostToDevice, u);
+    uint8_t* h = P.h_plan.as<uint8_t>();
+    const uint8_t* d = P.d_plan.as<uint8_t>();
+    memcpy(h + (P.d_files.as<uint8_t>() - d), P.files.data(), nf * sizeof(FileDesc));
+    memcpy(h + (P.d_chunks.as<uint8_t>() - d), P.chunks.data(), nc * sizeof(ChunkDesc));
+    cudaMemcpyAsync(P.d_plan.p, h, static_too ? P.plan_bytes : P.head_bytes, cudaMemcpyHostToDevice, u);
     if (up && (cudaEventRecord(up_done, up) != cudaSuccess || cudaStreamWaitEvent(s, up_done, 0) != cudaSuccess))
         return PGZ_E_CUDA;
     FileDesc* df = P.d_files.as<FileDesc>();
@@ -648,8 +701,7 @@ int start_run(pgz_ctx* ctx, Plan& P, bool timed, cudaStream_t up = nullptr, cuda
     reset_results(P);
     int e = layout(P);
     if (e) return e;
-    upload_static(P, up ? up : ctx->stream);
-    return enqueue(ctx, P, ctx->stream, timed, up, up_done);
+    return enqueue(ctx, P, ctx->stream, timed, true, up, up_done);
 }
 
 // the second half: waits for the run, then re-runs with recovery until the plan succeeds or cannot
@@ -964,7 +1016,9 @@ int decompress_members(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, uint8_t
     uint64_t off = 0, total = 0;
     for (;;) {
         uint64_t s0 = 0;
-        int e = member_header_at(ctx, gz, gz_len, off, &s0);
+        int e = -1;
+        if (off == 0) e = parse_header(ctx->hdr.as<uint8_t>(), std::min<uint64_t>(gz_len, 4096), gz_len, &s0);   // read above
+        if (e == -1) e = member_header_at(ctx, gz, gz_len, off, &s0);
         if (e) return off == 0 ? e : PGZ_E_UNSUPPORTED;        // data after a member that is no member
         MemberInfo mi;
         mi.s0 = s0;
@@ -1110,10 +1164,9 @@ int launch_slot(pgz_server* S, SrvSlot& sl, std::vector<pgz_request*>& batch, in
     int e = layout(P);
     if (!e && cuda_status(P.d_windows.ensure(P.chunks.size() * (size_t)kWin))) e = PGZ_E_NOMEM;
     if (!e) {
-        upload_static(P, ctx->stream);
         for (size_t k = 0; k < batch.size(); ++k)
             if (!batch[k]->whole) copy_range_windows(P, S->files[(size_t)batch[k]->file].idx, wins[k], ctx->stream);
-        e = enqueue(ctx, P, ctx->stream, false);
+        e = enqueue(ctx, P, ctx->stream, false, true);
     }
     if (!e && cudaEventRecord(sl.done, ctx->stream) != cudaSuccess) e = PGZ_E_CUDA;
     if (e) {
@@ -1250,6 +1303,7 @@ void pgz_destroy(pgz_ctx* ctx) {
         ctx->stage[k].release();
     }
     ctx->hdr.release();
+    ctx->heads.release();
     ctx->in_buf.release();
     ctx->out_buf.release();
     ctx->fill_buf.release();
@@ -1391,7 +1445,8 @@ static int decompress_at_parts(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len,
     R.chunks.push_back(C);
     R.chain = R.crc = false;
     R.sym_total = cap1;
-    if (cuda_status(R.d_chunks.ensure(sizeof C)) || cuda_status(R.h_chunks.ensure(sizeof C))) return PGZ_E_NOMEM;
+    if (cuda_status(R.d_plan.ensure(sizeof C)) || cuda_status(R.h_chunks.ensure(sizeof C))) return PGZ_E_NOMEM;
+    R.d_chunks.p = R.d_plan.p;
     memcpy(R.h_chunks.p, &C, sizeof C);
     if (cudaMemcpyAsync(R.d_chunks.p, R.h_chunks.p, sizeof C, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
         cudaStreamSynchronize(ctx->stream) != cudaSuccess)
@@ -1495,21 +1550,21 @@ int pgz_decompress_batch(pgz_ctx* ctx, int n, pgz_job* jobs, pgz_stats* st) {
     cudaSetDevice(ctx->cfg.device);
     Plan& P = ctx->plan;
     begin_plan(P);
-    std::vector<int> idx;
+    std::vector<int> idx, bad((size_t)n, PGZ_OK);
+    std::vector<MemberInfo> mi((size_t)n);
     int first_bad = PGZ_OK;
     for (int k = 0; k < n; ++k) {
         jobs[k].out_len = 0;
-        if (!jobs[k].gz || !aligned4(jobs[k].gz) || (!jobs[k].out && jobs[k].out_cap)) {
-            jobs[k].status = PGZ_E_ARG;
+        if (!jobs[k].gz || !aligned4(jobs[k].gz) || (!jobs[k].out && jobs[k].out_cap)) bad[(size_t)k] = PGZ_E_ARG;
+    }
+    const int he = read_members(ctx, n, jobs, bad, mi);
+    if (he) return he;
+    for (int k = 0; k < n; ++k) {
+        if (bad[(size_t)k]) {
+            jobs[k].status = bad[(size_t)k];
             continue;
         }
-        MemberInfo mi;
-        const int e = read_member(ctx, jobs[k].gz, jobs[k].gz_len, &mi);
-        if (e) {
-            jobs[k].status = e;
-            continue;
-        }
-        plan_member(ctx, P, jobs[k].gz, jobs[k].gz_len, jobs[k].out, jobs[k].out_cap, mi, 0);
+        plan_member(ctx, P, jobs[k].gz, jobs[k].gz_len, jobs[k].out, jobs[k].out_cap, mi[(size_t)k], 0);
         idx.push_back(k);
     }
     int e = idx.empty() ? PGZ_OK : execute(ctx, P, st);
@@ -1690,19 +1745,19 @@ int pgz_batch_prepare(pgz_ctx* ctx, int n, const pgz_job* jobs, pgz_batch** out)
     b->jobs.assign(jobs, jobs + n);
     Plan& P = b->plan;
     begin_plan(P);
-    for (int k = 0; k < n; ++k) {
-        if (!jobs[k].gz || !aligned4(jobs[k].gz) || (!jobs[k].out && jobs[k].out_cap)) {
-            delete b;
-            return PGZ_E_ARG;
-        }
-        MemberInfo mi;
-        const int e = read_member(ctx, jobs[k].gz, jobs[k].gz_len, &mi);
-        if (e) {
-            delete b;
-            return e;
-        }
-        plan_member(ctx, P, jobs[k].gz, jobs[k].gz_len, jobs[k].out, jobs[k].out_cap, mi, 0);
+    std::vector<int> bad((size_t)n, PGZ_OK);
+    std::vector<MemberInfo> mi((size_t)n);
+    int he = PGZ_OK;
+    for (int k = 0; k < n; ++k)
+        if (!jobs[k].gz || !aligned4(jobs[k].gz) || (!jobs[k].out && jobs[k].out_cap)) bad[(size_t)k] = PGZ_E_ARG;
+    he = read_members(ctx, n, jobs, bad, mi);
+    for (int k = 0; k < n && !he; ++k) he = bad[(size_t)k];
+    if (he) {
+        delete b;
+        return he;
     }
+    for (int k = 0; k < n; ++k)
+        plan_member(ctx, P, jobs[k].gz, jobs[k].gz_len, jobs[k].out, jobs[k].out_cap, mi[(size_t)k], 0);
     // one untimed run settles the plan (capacities, false starts), then the
     // settled plan is captured
     int e = execute(ctx, P, nullptr);
@@ -1721,7 +1776,7 @@ int pgz_batch_prepare(pgz_ctx* ctx, int n, const pgz_job* jobs, pgz_batch** out)
     cudaGraph_t g = nullptr;
     cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     const uint64_t before = ctx->launches;
-    enqueue(ctx, P, cs, false);
+    enqueue(ctx, P, cs, false, false);
     ctx->launches = before;
     cudaError_t ce = cudaStreamEndCapture(cs, &g);
     if (ce == cudaSuccess) ce = cudaGraphInstantiate(&P.graph, g, 0);

@@ -120,7 +120,7 @@ struct ChunkDesc {
 //        32), zero before launch_sync;
 // tok: token_words(nchunks, p.wpb) u32 of the block decoder's scratch (p.team set: p.tok_rows rows of 32 p.team u32 for
 //      each of at most nchunks teams);
-// queue: one u32 work counter per kernel (zeroed by the launcher on the stream);
+// queue: one u32 work counter per kernel, zero before its launch;
 // order (nullable): the parts in the order the work queue hands them out (nchunks entries).
 void launch_sync(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* start, uint32_t* tok,
                  uint32_t* queue, const uint32_t* order, const KParams& p, cudaStream_t s);
@@ -159,6 +159,13 @@ void launch_translate(const FileDesc* files, ChunkDesc* chunks, int nchunks, uin
 uint64_t crc_segment_bytes();
 void launch_crc(FileDesc* files, int nfiles, uint64_t total_seg, const uint64_t* seg0, cudaStream_t s);
 void launch_finalize(FileDesc* files, int nfiles, cudaStream_t s);
+// members of a batch: out[m] = its first kHeadBytes bytes (zeros past its end), then its last 8 (len >= 8)
+struct MemberRef {
+    const uint8_t* gz;
+    uint64_t len;
+};
+constexpr uint32_t kHeadBytes = 64;
+void launch_heads(const MemberRef* in, int n, uint8_t* out, cudaStream_t s);
 // DNA sequences among n u16 symbols: spans[2k] = start, spans[2k+1] = length | bit 63 if undetermined
 // symbols lie inside; counts[0] = spans found (may exceed max_spans), counts[1] = those with undetermined
 // (bits: sequence_words(n) u32 of scratch)

@@ -1240,7 +1240,7 @@ __device__ __forceinline__ TeamSmem<NW>& team_smem() {
 // different sizes in one launch) balance over the teams.  Position q holds
 // part order[q] (the parts with the most expected output first, so that the
 // short ones fill the end of the launch), or part q without an order.  The
-// counter is zeroed on the stream before each launch.
+// counter is zero before the launch.
 template <int NW>
 __device__ __forceinline__ int next_part(TeamSmem<NW>& S, uint32_t* queue) {
     team_sync<NW>();
@@ -2428,11 +2428,27 @@ __global__ void __launch_bounds__(256) k_sequences(const uint32_t* __restrict__ 
     }
 }
 
+// The first kHeadBytes bytes and the last 8 of every member of a batch, one warp per member, so that the host reads
+// all of them with one copy.
+__global__ void __launch_bounds__(128) k_heads(const MemberRef* __restrict__ in, int n, uint8_t* out) {
+    const int m = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (m >= n) return;
+    const uint8_t* gz = in[m].gz;
+    const uint64_t len = in[m].len;
+    uint8_t* o = out + (uint64_t)m * (kHeadBytes + 8);
+    for (uint32_t k = lane; k < kHeadBytes; k += 32) o[k] = k < len ? gz[k] : 0;
+    if (lane < 8 && len >= 8) o[kHeadBytes + lane] = gz[len - 8 + lane];
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------
 // host wrappers
 // ---------------------------------------------------------------------------
+void launch_heads(const MemberRef* in, int n, uint8_t* out, cudaStream_t s) {
+    if (n > 0) k_heads<<<(n + 3) / 4, 128, 0, s>>>(in, n, out);
+}
+
 uint64_t sequence_words(uint64_t n) { return 3 * ((n + 31) / 32); }
 
 void launch_sequences(const uint16_t* sym, uint64_t n, uint32_t min_len, uint32_t* bits, uint64_t* spans,
@@ -2519,7 +2535,6 @@ static void launch_pass1_any(bool sync, const FileDesc* files, ChunkDesc* chunks
                              uint32_t* start, uint32_t* tok, uint32_t* queue, const uint32_t* order, const KParams& p,
                              cudaStream_t s) {
     if (nchunks <= 0) return;
-    cudaMemsetAsync(queue, 0, sizeof(uint32_t), s);
     switch (p.team ? p.team : pass1_team(nchunks, p.wpb)) {
         case 2: launch_pass1_t<2>(sync, files, chunks, nchunks, sym, start, tok, queue, order, p, s); break;
         case 8: launch_pass1_t<8>(sync, files, chunks, nchunks, sym, start, tok, queue, order, p, s); break;
@@ -2567,7 +2582,6 @@ static void launch_exec_t(const FileDesc* files, ChunkDesc* chunks, int nchunks,
 void launch_exec(const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym, uint32_t* start, uint32_t* queue,
                  const uint32_t* order, const KParams& p, cudaStream_t s) {
     if (nchunks <= 0) return;
-    cudaMemsetAsync(queue, 0, sizeof(uint32_t), s);
     // With at most one part per SM, blocks of 512 threads: half the passes of a part (file of 8 parts: 53 us, against
     // 59 us with 256).  With more, 256: three fit an SM (two of 512), and shorter passes hold fewer sources inside
     // them, so they take fewer chase steps (1024 parts of 256 MiB: 737 us, against 873 us with 512 and 996 us with

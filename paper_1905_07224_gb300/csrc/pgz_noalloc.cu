@@ -51,15 +51,15 @@ constexpr size_t kOffGn = a256(kOffG0 + kNaMaxGroups * sizeof(int32_t));
 constexpr size_t kOffGfile = a256(kOffGn + kNaMaxGroups * sizeof(int32_t));
 constexpr size_t kOffUpper = a256(kOffGfile + kNaMaxGroups * sizeof(int32_t));
 constexpr size_t kOffSeg0 = a256(kOffUpper + 6 * sizeof(int32_t));
-constexpr size_t kOffWindows = a256(kOffSeg0 + sizeof(uint64_t));
+constexpr size_t kOffQueue = a256(kOffSeg0 + sizeof(uint64_t));
+constexpr size_t kOffWindows = a256(kOffQueue + 3 * sizeof(uint32_t));   // all before it is uploaded at once
 constexpr size_t kOffGmaps = a256(kOffWindows + (size_t)kNaMaxParts * kWin);
 constexpr size_t kOffWstart = a256(kOffGmaps + (size_t)(kNaMaxGroups + 1) * kWin * sizeof(uint16_t));
 constexpr size_t kOffSym = a256(kOffWstart + (size_t)(kNaMaxGroups + 1) * kWin);
 constexpr size_t kOffStart = a256(kOffSym + kNaSymbols * sizeof(uint16_t));
 constexpr size_t kTokWords = 32 * 512;                // token rows of one of kNaMaxParts parts
 constexpr size_t kOffTok = a256(kOffStart + kNaSymbols / 8);
-constexpr size_t kOffQueue = a256(kOffTok + (size_t)kNaMaxParts * kTokWords * sizeof(uint32_t));
-constexpr size_t kScratchBytes = a256(kOffQueue + 3 * sizeof(uint32_t));   // about 24 MiB
+constexpr size_t kScratchBytes = a256(kOffTok + (size_t)kNaMaxParts * kTokWords * sizeof(uint32_t));   // about 24 MiB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -229,15 +229,16 @@ extern "C" int pgz_decompress_noalloc(const uint8_t* gz, uint64_t gz_len, uint8_
                  crc_segment_bytes();
         F.out_hi = kNone;
         F.bad_chunk = 0xffffffffu;
-        const uint64_t seg0 = 0;
-        cudaMemcpyAsync(d_files, &F, sizeof F, cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(d_chunks, plan, n * sizeof(ChunkDesc), cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(d_g0, g0, ng * sizeof(int32_t), cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(d_gn, gn, ng * sizeof(int32_t), cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(d_gfile, gfile, ng * sizeof(int32_t), cudaMemcpyHostToDevice, s);
-        const int32_t upper[6] = {0, ng, 0, 0, 1, 0};
-        cudaMemcpyAsync(d_upper, upper, sizeof upper, cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(d_seg0, &seg0, sizeof seg0, cudaMemcpyHostToDevice, s);
+        // the plan's arrays lie before the windows in the scratch: one copy of them all
+        unsigned char up[kOffWindows] = {};
+        const int32_t upper[6] = {0, ng, 0, 0, 1, 0};      // one supergroup of ng groups, the member's only one
+        memcpy(up + kOffFiles, &F, sizeof F);
+        memcpy(up + kOffChunks, plan, n * sizeof(ChunkDesc));
+        memcpy(up + kOffG0, g0, ng * sizeof(int32_t));
+        memcpy(up + kOffGn, gn, ng * sizeof(int32_t));
+        memcpy(up + kOffGfile, gfile, ng * sizeof(int32_t));
+        memcpy(up + kOffUpper, upper, sizeof upper);
+        if (cudaMemcpyAsync(base, up, sizeof up, cudaMemcpyHostToDevice, s) != cudaSuccess) return PGZ_E_CUDA;
         cudaMemsetAsync(d_start, 0, kNaSymbols / 8, s);
         launch_sync(d_files, d_chunks, (int)n, d_sym, d_start, d_tok, d_queue, nullptr, kp, s);
         launch_inflate(d_files, d_chunks, (int)n, d_sym, d_start, d_tok, d_queue + 1, nullptr, kp, s);
