@@ -58,7 +58,7 @@ constexpr uint32_t kPoly = 0xEDB88320u;
 __constant__ uint8_t c_clorder[19] = {16, 17, 18, 0, 8, 7, 9, 6, 10, 5, 11, 4, 12, 3, 13, 2, 14, 1, 15};
 // CRC-32 tables (filled by upload_crc_tables)
 __constant__ uint32_t c_crc_tab[4][256];   // [0][b]: register after byte b from a zero register; [k]: k more zero bytes
-__constant__ uint32_t c_x2k[64];           // x^(2^k) mod P
+__constant__ uint32_t c_x8[5][256];        // [d][v]: x^(8 v 256^d) mod P
 __constant__ uint32_t c_lane_shift[32];    // x^(8*kPiece*k) mod P
 __constant__ uint32_t c_seg_shift[4][256]; // [j][b]: (byte b at byte j of a register) x^(8*kCrcSeg) mod P
 
@@ -2175,11 +2175,14 @@ __device__ __forceinline__ uint32_t gf2_mul(uint32_t a, uint32_t b) {
     return p;
 }
 
-__device__ uint32_t xpow8(uint64_t n) {       // x^(8n) mod P
-    uint64_t e = n << 3;
-    uint32_t r = 0x80000000u;
-    for (int k = 0; e; ++k, e >>= 1)
-        if (e & 1) r = gf2_mul(r, c_x2k[k]);
+// x^(8n) mod P, n < 2^40: a product of one power per byte of n (a multiplication is a serial chain, so their number
+// counts: with powers of two, one per set bit of n, k_crc took 22 us for 1 MiB and 85 us for 256 MiB, now 8 and 71)
+__device__ uint32_t xpow8(uint64_t n) {
+    uint32_t r = c_x8[0][n & 255u];
+    for (int d = 1; d < 5; ++d) {
+        const uint32_t v = (uint32_t)(n >> (8 * d)) & 255u;
+        if (v) r = gf2_mul(r, c_x8[d][v]);
+    }
     return r;
 }
 
@@ -2187,38 +2190,48 @@ constexpr uint32_t kPiece = 32;       // bytes per lane and segment
 constexpr uint32_t kCrcSeg = 32 * kPiece;   // bytes per warp step (one piece per lane)
 constexpr int kCrcAhead = 3;          // segments whose loads are in flight while one is folded
 constexpr int kCrcThreads = 1024;     // one block per SM
-// four byte tables with one copy per lane (128 KiB), then the segment shift's four byte tables, shared (4 KiB)
-constexpr size_t kCrcSmem = (4 * 256 * 32 + 4 * 256) * sizeof(uint32_t);
+// Four byte tables, then the segment shift's four byte tables (4 KiB).  REPL: one copy of the first four per lane
+// (128 KiB), so that the lookups of a warp never share a bank: 72 us instead of 126 for 256 MiB; else one copy (4 KiB),
+// whose lookups conflict but which is filled at once: for 1 MiB (one segment per warp) 8 us instead of 13.  At 12.6 MB
+// (three) the copies take 18 us, the single tables 23.
+template <bool REPL>
+constexpr size_t crc_smem() { return ((REPL ? 32 : 1) * 4 * 256 + 4 * 256) * sizeof(uint32_t); }
+constexpr uint64_t kCrcRepl = 3;      // segments per warp from which the copies pay
 
 // Slicing by four (four table lookups per 32-bit word, RFC 1952 CRC in the
 // reflected form): with x = r ^ w, the register after the word's four bytes
 // is T3[x0] ^ T2[x1] ^ T1[x2] ^ T0[x3], where Tk is the byte table followed
-// by k zero bytes.  Each lane reads its own copy of the tables (entry b of
-// table k of lane l at word 32 * (256 k + b) + l), so the lookups of a warp
-// never share a bank.
-__device__ __forceinline__ uint32_t crc_word(const uint32_t* Tl, uint32_t r, uint32_t w) {
-    const uint32_t x = r ^ w;
-    return Tl[32u * (768u + (x & 0xffu))] ^ Tl[32u * (512u + ((x >> 8) & 0xffu))] ^
-           Tl[32u * (256u + ((x >> 16) & 0xffu))] ^ Tl[32u * (x >> 24)];
-}
+// by k zero bytes.  With copies, entry b of table k of lane l is at word
+// 32 * (256 k + b) + l.
+template <bool REPL>
+struct CrcTable {
+    const uint32_t* t;      // with copies: this lane's
+    __device__ __forceinline__ uint32_t at(uint32_t i) const { return t[REPL ? 32u * i : i]; }
+    __device__ __forceinline__ uint32_t word(uint32_t r, uint32_t w) const {
+        const uint32_t x = r ^ w;
+        return at(768u + (x & 0xffu)) ^ at(512u + ((x >> 8) & 0xffu)) ^ at(256u + ((x >> 16) & 0xffu)) ^ at(x >> 24);
+    }
+};
 
 // raw CRC register (zero start) of a whole piece held in registers
-__device__ __forceinline__ uint32_t crc_piece(const uint32_t* Tl, const uint4 (&v)[kPiece / 16]) {
+template <bool REPL>
+__device__ __forceinline__ uint32_t crc_piece(const CrcTable<REPL>& T, const uint4 (&v)[kPiece / 16]) {
     uint32_t r = 0;
 #pragma unroll
     for (int q = 0; q < (int)(kPiece / 16); ++q) {
-        r = crc_word(Tl, r, v[q].x);
-        r = crc_word(Tl, r, v[q].y);
-        r = crc_word(Tl, r, v[q].z);
-        r = crc_word(Tl, r, v[q].w);
+        r = T.word(r, v[q].x);
+        r = T.word(r, v[q].y);
+        r = T.word(r, v[q].z);
+        r = T.word(r, v[q].w);
     }
     return r;
 }
 
 // raw CRC register (zero start) of n bytes at p, byte by byte
-__device__ __forceinline__ uint32_t crc_bytes(const uint32_t* Tl, const uint8_t* p, uint64_t n) {
+template <bool REPL>
+__device__ __forceinline__ uint32_t crc_bytes(const CrcTable<REPL>& T, const uint8_t* p, uint64_t n) {
     uint32_t r = 0;
-    for (uint64_t i = 0; i < n; ++i) r = Tl[32u * ((r ^ p[i]) & 0xffu)] ^ (r >> 8);
+    for (uint64_t i = 0; i < n; ++i) r = T.at((r ^ p[i]) & 0xffu) ^ (r >> 8);
     return r;
 }
 
@@ -2239,17 +2252,19 @@ __device__ __forceinline__ uint32_t crc_shift_seg(const uint32_t* Y, uint32_t r)
 // 32-byte pieces are one 1 KiB stretch, so each load instruction reads few
 // lines).  A member's last segment, when shorter, is done byte by byte with
 // per-lane shifts, and so is a member whose output is not 16-byte aligned.
+template <bool REPL>
 __global__ void __launch_bounds__(kCrcThreads, 1) k_crc(FileDesc* files, int nfiles, uint64_t total_seg,
                                                         const uint64_t* seg0, uint64_t segs_per_warp) {
-    extern __shared__ uint32_t T[];                       // 4 x 256 x 32 words, then 4 x 256 (the segment shift)
+    extern __shared__ uint32_t T[];                       // 4 x 256 words (x 32 copies), then 4 x 256 (the segment shift)
     __shared__ uint32_t LS[32];
-    for (int k = threadIdx.x; k < 4 * 256 * 32; k += blockDim.x) T[k] = c_crc_tab[k >> 13][(k >> 5) & 255];
-    uint32_t* Y = T + 4 * 256 * 32;
+    constexpr int kCopies = REPL ? 32 : 1;
+    for (int k = threadIdx.x; k < 4 * 256 * kCopies; k += blockDim.x) T[k] = c_crc_tab[k / (256 * kCopies)][k / kCopies & 255];
+    uint32_t* Y = T + 4 * 256 * kCopies;
     for (int k = threadIdx.x; k < 4 * 256; k += blockDim.x) Y[k] = c_seg_shift[k >> 8][k & 255];
     if (threadIdx.x < 32) LS[threadIdx.x] = c_lane_shift[threadIdx.x];
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    const uint32_t* Tl = T + lane;
+    const CrcTable<REPL> Tl{T + (REPL ? lane : 0)};
     const uint64_t w = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const uint64_t s_begin = w * segs_per_warp;
     if (s_begin >= total_seg) return;
@@ -2703,13 +2718,19 @@ void launch_crc(FileDesc* files, int nfiles, uint64_t total_seg, const uint64_t*
         int n = 0;
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) sms[slot] = n;
         else cudaGetLastError();
-        cudaFuncSetAttribute(k_crc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCrcSmem);
+        cudaFuncSetAttribute(k_crc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)crc_smem<true>());
     }
-    const uint64_t wpb = kCrcThreads / 32;
-    const uint64_t target = (uint64_t)(sms[slot] ? sms[slot] : 152) * wpb;   // one block per SM
-    const uint64_t spw = (total_seg + target - 1) / target;
-    const uint64_t warps = (total_seg + spw - 1) / spw;
-    k_crc<<<(unsigned)((warps + wpb - 1) / wpb), kCrcThreads, kCrcSmem, s>>>(files, nfiles, total_seg, seg0, spw);
+    const uint64_t n = (uint64_t)(sms[slot] ? sms[slot] : 152);
+    const uint64_t spw = (total_seg + n * (kCrcThreads / 32) - 1) / (n * (kCrcThreads / 32));   // one block per SM
+    if (spw >= kCrcRepl) {
+        const uint64_t wpb = kCrcThreads / 32, warps = (total_seg + spw - 1) / spw;
+        k_crc<true><<<(unsigned)((warps + wpb - 1) / wpb), kCrcThreads, crc_smem<true>(), s>>>(files, nfiles, total_seg,
+                                                                                              seg0, spw);
+    } else {
+        const uint64_t wpb = 8, warps = (total_seg + spw - 1) / spw;
+        k_crc<false><<<(unsigned)((warps + wpb - 1) / wpb), 32 * wpb, crc_smem<false>(), s>>>(files, nfiles, total_seg,
+                                                                                             seg0, spw);
+    }
 }
 
 void launch_finalize(FileDesc* files, int nfiles, cudaStream_t s) {
@@ -2729,7 +2750,7 @@ static uint32_t h_mul(uint32_t a, uint32_t b) {
 }
 
 void upload_crc_tables() {
-    uint32_t tab[4][256], x2k[64], ls[32];
+    uint32_t tab[4][256], x2k[64], ls[32], x8[5][256];
     for (uint32_t b = 0; b < 256; ++b) {
         uint32_t r = b;
         for (int k = 0; k < 8; ++k) r = (r & 1u) ? (r >> 1) ^ kPoly : (r >> 1);
@@ -2739,6 +2760,10 @@ void upload_crc_tables() {
         for (uint32_t b = 0; b < 256; ++b) tab[k][b] = (tab[k - 1][b] >> 8) ^ tab[0][tab[k - 1][b] & 0xffu];
     x2k[0] = 0x40000000u;                      // x
     for (int k = 1; k < 64; ++k) x2k[k] = h_mul(x2k[k - 1], x2k[k - 1]);
+    for (int d = 0; d < 5; ++d) {              // powers of x^(8 256^d)
+        x8[d][0] = 0x80000000u;
+        for (int v = 1; v < 256; ++v) x8[d][v] = h_mul(x8[d][v - 1], x2k[3 + 8 * d]);
+    }
     for (int l = 0; l < 32; ++l) {             // x^(8*kPiece*l)
         uint64_t e = 8ull * kPiece * (uint64_t)l;
         uint32_t r = 0x80000000u;
@@ -2756,7 +2781,7 @@ void upload_crc_tables() {
     for (int j = 0; j < 4; ++j)
         for (uint32_t b = 0; b < 256; ++b) seg[j][b] = h_mul(b << (8 * j), xseg);
     cudaMemcpyToSymbol(c_crc_tab, tab, sizeof tab);
-    cudaMemcpyToSymbol(c_x2k, x2k, sizeof x2k);
+    cudaMemcpyToSymbol(c_x8, x8, sizeof x8);
     cudaMemcpyToSymbol(c_lane_shift, ls, sizeof ls);
     cudaMemcpyToSymbol(c_seg_shift, seg, sizeof seg);
 }

@@ -156,3 +156,26 @@ def test_sequences_at_word_and_block_edges(n):
                 assert st == 0 and got == want and nu == sum(u for _, _, u in want)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+def test_crc_at_the_edges_of_pieces_segments_and_forms(offset):
+    """CRC-32 of outputs around the sizes of a lane's piece, a warp's segment and the change of the lookup tables' form
+    (9728 segments on 152 SMs), the output aligned or not: the right trailer is accepted, a wrong one is not."""
+    line = np.random.default_rng(5).choice(np.frombuffer(b"ACGT\n", dtype=np.uint8), 1 << 20).tobytes()
+    ctx = Ctx()
+    try:
+        for n in [0, 1, 31, 32, 33, 1023, 1024, 1025, 1056, 262143, 9728 * 1024, 9728 * 1024 + 1]:
+            text = (line * (n // len(line) + 1))[:n]
+            c = zlib.compressobj(1, zlib.DEFLATED, 31)
+            gz = c.compress(text) + c.flush()
+            bad = gz[:-8] + bytes([gz[-8] ^ 0x10]) + gz[-7:]
+            out = empty(n + 16)
+            for data, want in ((gz, 0), (bad, ctx.pgz.PGZ_E_CRC)):
+                d = to_device(data)
+                st, k, _ = ctx.pgz.pgz_decompress(ctx.h, d.data_ptr(), len(data), out.data_ptr() + offset, n, False)
+                assert st == want, (n, ctx.pgz.pgz_strerror(st))
+                if want == 0:
+                    assert k == n and out[offset:offset + n].cpu().numpy().tobytes() == text
+    finally:
+        ctx.close()
