@@ -220,12 +220,13 @@ __device__ __forceinline__ uint32_t dist_entry(uint32_t s, uint32_t L) {
     return ((((2 + (s & 1u)) << E) + 1) << 12) | (K_DIST << 9) | (L << 5) | (L + E);
 }
 
-// the code that prefixes v (15 code bits, first bit most significant): its length (16: none) from the ends of
-// the codes of each length
+// the code that prefixes v (15 code bits, first bit most significant): its length (MAX + 1: none so short) from the
+// ends of the codes of each length
+template <int MAX>
 __device__ __forceinline__ uint32_t code_length(uint32_t v, const uint32_t* lim) {
     uint32_t L = 1;
 #pragma unroll
-    for (int l = 1; l <= 15; ++l) L += v >= lim[l];
+    for (int l = 1; l <= MAX; ++l) L += v >= lim[l];
     return L;
 }
 
@@ -265,6 +266,7 @@ __device__ __forceinline__ void sort_code(const uint8_t* lens, int n, uint32_t* 
     for (int s0 = 0; s0 < n; s0 += 32) {
         const int s = s0 + lane;
         const uint32_t l = (s < n) ? lens[s] : 0u;
+        if (!__any_sync(FULL, l != 0)) continue;       // most values of a byte do not occur in a text
         const uint32_t peers = __match_any_sync(FULL, l);
         const uint32_t rank = __popc(peers & ((1u << lane) - 1u));
         const uint32_t base = cnt[l];
@@ -294,12 +296,12 @@ __device__ void build_tables(TeamSmem<NW>& S, uint32_t hlit, uint32_t hdist) {
     team_sync<NW>();
     for (uint32_t x = tid; x < (1u << LB); x += 32 * NW) {         // x: stream bits, the first least significant
         const uint32_t v = __brev(x) >> 17;                        // the same, left-aligned in 15 bits
-        const uint32_t L = code_length(v, S.lim[0]);
+        const uint32_t L = code_length<LB>(v, S.lim[0]);
         uint32_t e = K_LONG << 9;
         if (L <= LB) {
             e = S.ent[(int32_t)(v >> (15 - L)) + S.sb[0][L]];
             if (((e >> 9) & 7u) == K_LIT) {                        // a second literal inside the lookup width?
-                const uint32_t v2 = (v << L) & 0x7fffu, L2 = code_length(v2, S.lim[0]);
+                const uint32_t v2 = (v << L) & 0x7fffu, L2 = code_length<LB>(v2, S.lim[0]);
                 if (L + L2 <= LB) {
                     const uint32_t e2 = S.ent[(int32_t)(v2 >> (15 - L2)) + S.sb[0][L2]];
                     if (((e2 >> 9) & 7u) == K_LIT)
@@ -311,7 +313,7 @@ __device__ void build_tables(TeamSmem<NW>& S, uint32_t hlit, uint32_t hdist) {
     }
     for (uint32_t x = tid; x < (1u << DB); x += 32 * NW) {
         const uint32_t v = __brev(x) >> 17;
-        const uint32_t L = code_length(v, S.lim[1]);
+        const uint32_t L = code_length<DB>(v, S.lim[1]);
         S.tab[(1 << LB) + x] = L <= DB ? S.ent[(int32_t)(v >> (15 - L)) + S.sb[1][L]] : K_LONG << 9;
     }
     team_sync<NW>();
@@ -394,8 +396,11 @@ __device__ int read_lengths(TeamSmem<NW>& S, Bits& br, int lane, uint32_t& hlit,
     __syncwarp();
     // the lengths, 32 symbols at a time: places by a prefix sum of the counts, a repeat's value from the last
     // symbol before it that is no repeat
+    // (a run of zeros would take up to 138 turns: they are written beforehand)
     uint32_t at0 = 0, prev_val = 0xffu;
     bool bad = false;
+    for (int k = lane; k < 320 / 4; k += 32) reinterpret_cast<uint32_t*>(S.lens)[k] = 0;
+    __syncwarp();
     for (uint32_t k0 = 0; k0 < n; k0 += 32) {
         const uint32_t h = k0 + lane < n ? S.hs[k0 + lane] : 0u, y = h & 31u, rep = h >> 5;
         uint32_t incl = rep;
@@ -409,7 +414,7 @@ __device__ int read_lengths(TeamSmem<NW>& S, Bits& br, int lane, uint32_t& hlit,
         const uint32_t val = own ? from : prev_val;
         bad |= val == 0xffu && rep;                    // a repeat before the first length
         const uint32_t at1 = at0 + incl - rep;
-        for (uint32_t j = 0; j < rep; ++j) S.lens[at1 + j] = (uint8_t)val;
+        for (uint32_t j = 0; j < (val ? rep : 0u); ++j) S.lens[at1 + j] = (uint8_t)val;
         at0 += __shfl_sync(FULL, incl, 31);
         prev_val = __shfl_sync(FULL, val, 31);
     }
