@@ -54,10 +54,10 @@ METRIC = "decompressed GB/s on 1 GB300 (batched vs plain), %HBM roofline; served
 HEADLINE_DESC = ("512 synthetic gzip members, log-uniform 64 KiB-64 MiB (seed 3), FASTQ 150 bp / order-2 Markov "
                  "text, gzip -1/-6/-9")
 TUNE_CHUNKS_BATCH = [128 << 10, 256 << 10, 512 << 10]   # the autotuner's part sizes on the 512 members
-                                                        # (and the sizes of 1-4 whole waves of pass-1 warps)
+                                                        # (and the sizes of 1-4 whole waves of pass-1 teams)
 TUNE_WPB_BATCH = [2, 4]
 SERVED_REQUESTS = 240         # requests per offered load in the default run (the full served run uses 2000)
-# DRAM bytes (read + write) of pass 1 (k_sync + k_inflate) per decompressed byte, from one-pass ncu captures
+# DRAM bytes (read + write) of pass 1 (k_sync + k_inflate + k_exec) per decompressed byte, from one-pass ncu captures
 # of the current kernels.  The two 256 MiB FASTQ files as one batch, by (part size, warps per block, pipelined
 # execution) (profiles/pass1_traffic_fastq256.md) ...
 PASS1_TRAFFIC_PER_OUT_BYTE = {
@@ -391,7 +391,7 @@ def run_pgz(args, rank, world):
                   "ms_per_step": round(ms_plain, 3), "parts_per_file": PLAIN_PARTS,
                   "form": "one file at a time through pgz_decompress", "per_level": per_level},
         "stages_ms": {k: round(v, 3) for k, v in stage.items()},
-        "roofline": {"bound": "hbm", "kernel": "pass 1 (k_sync + k_inflate)", "achieved": round(ach1, 2),
+        "roofline": {"bound": "hbm", "kernel": "pass 1 (k_sync + k_inflate + k_exec)", "achieved": round(ach1, 2),
                      "peak": hbm, "unit": "GB/s", "frac": round(ach1 / hbm, 5),
                      "traffic": round(traffic1) if traffic1 else None, "peak_source": peak_src},
         "roofline_translate": {"bound": "hbm", "kernel": "k_translate", "achieved": round(ach4, 1) if ach4 else None,
@@ -470,7 +470,7 @@ def rooflines(stage, total_in, total_out, window_bytes, hbm, traffic_per_out_byt
     ach4 = alg4 / (stage["ms_translate"] * 1e-3) / 1e9 if stage["ms_translate"] > 0 else None
     ach5 = total_out / (stage["ms_crc"] * 1e-3) / 1e9 if stage["ms_crc"] > 0 else None
     traffic = round(traffic_per_out_byte * total_out) if traffic_per_out_byte else None
-    return ({"bound": "hbm", "kernel": "pass 1 (k_sync + k_inflate)", "achieved": round(ach1, 2), "peak": hbm,
+    return ({"bound": "hbm", "kernel": "pass 1 (k_sync + k_inflate + k_exec)", "achieved": round(ach1, 2), "peak": hbm,
              "unit": "GB/s", "frac": round(ach1 / hbm, 5), "traffic": traffic, "algorithmic_bytes": alg1,
              "ms": round(pass1_ms, 3)},
             {"bound": "hbm", "kernel": "k_translate", "achieved": round(ach4, 1) if ach4 else None, "peak": hbm,
@@ -568,7 +568,7 @@ def _stage_line(stage, total_in, total_out, window_bytes, hbm):
 
 
 def wave_sizes(pgz, ctx, jobs, wpbs, waves):
-    """Part sizes that give whole waves of the resident pass-1 warps over these jobs (pgz_wave_chunk_bytes),
+    """Part sizes that give whole waves of the resident pass-1 teams over these jobs (pgz_wave_chunk_bytes),
     for each CTA shape and wave count."""
     out = set()
     for w in wpbs:
@@ -580,14 +580,14 @@ def wave_sizes(pgz, ctx, jobs, wpbs, waves):
 
 
 def autotune(pgz, ctx, jobs, chunks, wpbs):
-    """The library's autotuner over part size x pass-1 CTA shape x pass-1 execution form on these jobs; the
-    context keeps the fastest configuration.  Returns {"best": [chunk, wpb, pipelined], "ms": {...}}."""
-    st, entries, best = pgz.pgz_autotune(ctx, jobs, chunks, wpbs, 2, sweep_exec=True)
+    """The library's autotuner over part size x pass-1 CTA shape on these jobs (its two execution forms are the same
+    code, so they are not swept); the context keeps the fastest configuration.  Returns {"best": [chunk, wpb,
+    pipelined], "ms": {...}}."""
+    st, entries, best = pgz.pgz_autotune(ctx, jobs, chunks, wpbs, 2, sweep_exec=False)
     if st != 0:
         raise RuntimeError(f"pgz_autotune failed: {pgz.pgz_strerror(st)}")
     return {"best": [best["chunk_bytes"], best["warps_per_block"], best["exec_pipelined"]],
-            "ms": {f"{e['chunk_bytes'] >> 10}K/{e['warps_per_block']}w/{'p' if e['exec_pipelined'] else 's'}":
-                   round(e["ms"], 2) for e in entries}}
+            "ms": {f"{e['chunk_bytes'] >> 10}K/{e['warps_per_block']}w": round(e["ms"], 2) for e in entries}}
 
 
 def run_tune4g(args):

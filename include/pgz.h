@@ -168,8 +168,9 @@ typedef int (*pgz_sink)(void* user, const uint8_t* bytes, uint64_t n);
    order; when a later segment fails, the bytes already delivered stay
    delivered and the status says why the rest could not be decoded.
    Device memory in use is bounded by the segment, not by the member: about
-   17 bytes per compressed byte of a segment at 64 KiB parts for data that
-   expands at most 2x (input, symbol scratch, output, windows); more where a
+   18 bytes per compressed byte of a segment at 64 KiB parts for data that
+   expands at most 2x (input, symbol scratch and its start bits, output,
+   windows), and a fixed scratch of about 200 MB; more where a
    segment expands further, its capacities doubling on demand.
    gz [host, gz_len bytes]: one gzip member.  segment_bytes: 0 for 256 MiB,
    else at least 1 MiB (PGZ_E_ARG otherwise).  *out_len: bytes delivered to

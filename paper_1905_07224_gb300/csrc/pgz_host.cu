@@ -1483,6 +1483,10 @@ int pgz_decompress_at(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, uint64_t
             return PGZ_OK;
         }
         if (e == PGZ_E_CUDA) return e;
+        if (e == PGZ_E_NOMEM) {                        // no room for the parts beside the one part: give theirs back
+            ctx->at_plan.release();
+            cudaGetLastError();
+        }
     }
     Plan& P = ctx->plan;
     begin_plan(P);
