@@ -1473,10 +1473,14 @@ __device__ void inflate_part(TeamSmem<NW>& S, const FileDesc* __restrict__ files
     }
 }
 
-// Launch bounds of the pass-1 kernels: shared memory holds 12 teams of 2 warps per SM, 7 of 4, 4 of 8, 2 of 16, and
-// the registers follow (72 a thread for teams of 4; 64, for an eighth team that does not fit, spilled).  With 9 bits
-// of distance lookup instead of 8 fewer steps take the rare branch: k_inflate of a 256 MiB file 1343 -> 1251 us.
-constexpr int pass1_min_blocks(int nw) { return nw == 4 ? 7 : (nw == 2 ? 12 : 32 / nw); }
+// Launch bounds of the pass-1 kernels, the blocks per SM that the registers are to allow: with many parts what shared
+// memory holds, 12 teams of 2 warps and 7 of 4 (72 registers a thread; 64, for an eighth team that does not fit,
+// spilled).  The larger teams are for few parts, where a part's own time counts: at 4 blocks of 8 and 2 of 16 (64
+// registers) they spilled 32 bytes.  With 3 and 1 (k_sync + k_inflate, us): 1 MiB file 433 -> 389, 64 KiB 161 -> 145,
+// eight byte ranges 2380 -> 2130, 160 parts of a 12 MiB text 945 -> 850; single files of 157 to 611 parts the same.
+// With 9 bits of distance lookup instead of 8 fewer steps take the rare branch: k_inflate of a 256 MiB file 1343 ->
+// 1251 us.
+constexpr int pass1_min_blocks(int nw) { return nw == 2 ? 12 : (nw == 4 ? 7 : (nw == 8 ? 3 : 1)); }
 
 template <int NW>
 __global__ void __launch_bounds__(32 * NW, pass1_min_blocks(NW))
@@ -2531,7 +2535,7 @@ static int pass1_resident(int nw) {
 static uint32_t team_rows(int nw) { return nw <= 8 ? 384 : 256; }
 
 // Warps per part: with few parts the largest team whose launch still holds every part at once (the time of a part
-// falls with its team's size: 8 parts of a 1 MiB file take 0.25 ms of block-start search and 0.2 ms of decoding with
+// falls with its team's size: 8 parts of a 1 MiB file take 0.20 ms of block-start search and 0.19 ms of decoding with
 // teams of 16, against 0.86 and 1.36 ms with one warp each); with more parts than that the configured size, whose
 // rounds spend less on lanes left over.
 int pass1_team(int nchunks, int wpb) {
