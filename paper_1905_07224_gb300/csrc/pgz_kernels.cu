@@ -1473,17 +1473,18 @@ __device__ void inflate_part(TeamSmem<NW>& S, const FileDesc* __restrict__ files
     }
 }
 
-// Launch bounds of the pass-1 kernels, the blocks per SM that the registers are to allow: with many parts what shared
-// memory holds, 12 teams of 2 warps and 7 of 4 (72 registers a thread; 64, for an eighth team that does not fit,
-// spilled).  The larger teams are for few parts, where a part's own time counts: at 4 blocks of 8 and 2 of 16 (64
-// registers) they spilled 32 bytes.  With 3 and 1 (k_sync + k_inflate, us): 1 MiB file 433 -> 389, 64 KiB 161 -> 145,
-// eight byte ranges 2380 -> 2130, 160 parts of a 12 MiB text 945 -> 850; single files of 157 to 611 parts the same.
+// Launch bounds of the pass-1 kernels, the blocks per SM that the registers are to allow (MB): with many parts what
+// shared memory holds, 12 teams of 2 warps and 7 of 4 (72 registers a thread; 64, for an eighth team that does not
+// fit, spilled).  Larger teams are for few parts, where a part's own time counts: 3 of 8 warps (80 registers; at 4,
+// with 64, they spilled; files of 305 to 611 parts take the same time either way).  Teams of 16 have two forms: 2 per
+// SM (64 registers) and, where the parts fill at most half of the SMs, 1 per SM (128), k_sync + k_inflate: 1 MiB file
+// 433 -> 389 us, 64 KiB 161 -> 145, eight byte ranges 2380 -> 2130.
 // With 9 bits of distance lookup instead of 8 fewer steps take the rare branch: k_inflate of a 256 MiB file 1343 ->
 // 1251 us.
-constexpr int pass1_min_blocks(int nw) { return nw == 2 ? 12 : (nw == 4 ? 7 : (nw == 8 ? 3 : 1)); }
+constexpr int pass1_min_blocks(int nw) { return nw == 2 ? 12 : (nw == 4 ? 7 : (nw == 8 ? 3 : 2)); }
 
-template <int NW>
-__global__ void __launch_bounds__(32 * NW, pass1_min_blocks(NW))
+template <int NW, int MB = pass1_min_blocks(NW)>
+__global__ void __launch_bounds__(32 * NW, MB)
     k_sync(const FileDesc* __restrict__ files, ChunkDesc* chunks, int nchunks, uint16_t* symbuf, uint32_t* start_bits,
            uint32_t* tok, uint32_t* queue, const uint32_t* __restrict__ order, KParams p) {
     TeamSmem<NW>& S = team_smem<NW>();
@@ -1495,8 +1496,8 @@ __global__ void __launch_bounds__(32 * NW, pass1_min_blocks(NW))
     }
 }
 
-template <int NW>
-__global__ void __launch_bounds__(32 * NW, pass1_min_blocks(NW))
+template <int NW, int MB = pass1_min_blocks(NW)>
+__global__ void __launch_bounds__(32 * NW, MB)
     k_inflate(const FileDesc* __restrict__ files, ChunkDesc* chunks, int nchunks, uint16_t* symbuf, uint32_t* start_bits,
               uint32_t* tok, uint32_t* queue, const uint32_t* __restrict__ order, KParams p) {
     TeamSmem<NW>& S = team_smem<NW>();
@@ -2508,6 +2509,9 @@ static int pass1_resident_t() {
         const bool ok =
             cudaFuncSetAttribute(k_sync<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
             cudaFuncSetAttribute(k_inflate<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+            (NW != 16 ||
+             (cudaFuncSetAttribute(k_sync<NW, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+              cudaFuncSetAttribute(k_inflate<NW, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess)) &&
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_a, k_sync<NW>, 32 * NW, smem) == cudaSuccess &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_b, k_inflate<NW>, 32 * NW, smem) == cudaSuccess;
@@ -2537,7 +2541,9 @@ static uint32_t team_rows(int nw) { return nw <= 8 ? 384 : 256; }
 // Warps per part: with few parts the largest team whose launch still holds every part at once (the time of a part
 // falls with its team's size: 8 parts of a 1 MiB file take 0.20 ms of block-start search and 0.19 ms of decoding with
 // teams of 16, against 0.86 and 1.36 ms with one warp each); with more parts than that the configured size, whose
-// rounds spend less on lanes left over.
+// rounds spend less on lanes left over.  Teams of 8 instead of two teams of 16 on an SM are faster for
+// one call (160 parts of a 12 MiB text: 1.14 ms against 1.23) but slower for runs side by side (40 requests served in
+// 4 slots: 1.64 against 1.55).
 int pass1_team(int nchunks, int wpb) {
     const int base = wpb == 2 || wpb == 8 ? wpb : 4;
     for (int nw = 16; nw > base; nw >>= 1)
@@ -2561,8 +2567,11 @@ static void launch_pass1_t(bool sync, const FileDesc* files, ChunkDesc* chunks, 
     const int grid = pass1_grid(nchunks, NW);
     KParams q = p;
     if (!p.team) q.tok_rows = team_rows(NW);
-    if (sync) k_sync<NW><<<grid, 32 * NW, sizeof(TeamSmem<NW>), s>>>(files, chunks, nchunks, sym, start, tok, queue, order, q);
-    else k_inflate<NW><<<grid, 32 * NW, sizeof(TeamSmem<NW>), s>>>(files, chunks, nchunks, sym, start, tok, queue, order, q);
+    auto launch = [&](auto kernel) {
+        kernel<<<grid, 32 * NW, sizeof(TeamSmem<NW>), s>>>(files, chunks, nchunks, sym, start, tok, queue, order, q);
+    };
+    if (NW == 16 && nchunks <= pass1_resident(16) / 4) launch(sync ? k_sync<NW, 1> : k_inflate<NW, 1>);
+    else launch(sync ? k_sync<NW> : k_inflate<NW>);
 }
 
 static void launch_pass1_any(bool sync, const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym,
