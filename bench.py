@@ -10,9 +10,9 @@ with inputs and outputs resident in device memory, in two forms:
 
   batched (the reported value): every member in one run of the pass kernels,
       parts taken from a device work queue, captured once in a CUDA graph
-      (pgz_batch_prepare / pgz_batch_run); part size, pass-1 CTA shape and
-      execution form chosen by the library's autotuner (pgz_autotune) on the
-      same members unless --chunk-bytes fixes them;
+      (pgz_batch_prepare / pgz_batch_run); part size and pass-1 CTA shape
+      chosen by the library's autotuner (pgz_autotune) on the same members
+      unless --chunk-bytes fixes them;
   plain: one pgz_decompress call per member (the library's default parts).
 
 e2e times the same members through pgz_decompress_batch_host: pinned host
@@ -59,16 +59,16 @@ TUNE_WPB_BATCH = [2, 4]
 SERVED_REQUESTS = 240         # requests per offered load in the default run (the full served run uses 2000)
 # DRAM bytes (read + write) of pass 1 (k_sync + k_inflate + k_exec) per decompressed byte, from one-pass ncu captures
 # of the current kernels.  The two 256 MiB FASTQ files as one batch, by (part size, warps per block, pipelined
-# execution) (profiles/pass1_traffic_fastq256.md) ...
+# execution, which changes nothing) (profiles/pass1_traffic_fastq256.md) ...
 PASS1_TRAFFIC_PER_OUT_BYTE = {
-    (88162, 2, 0): (0.852781568e9 + 0.524115712e9 + 3.037636864e9 + 1.317603072e9) / 536870912,
-    (88162, 4, 0): (0.854030592e9 + 0.524192512e9 + 3.039483648e9 + 1.317075712e9) / 536870912,
+    (262144, 4, 0): (0.167883008e9 + 0.157478912e9 + 1.515178752e9 + 1.731217152e9 + 1.141309952e9
+                     + 1.009485824e9) / 536870912,
 }
 # ... and the 512-member batch, by (part size, warps per block, pipelined execution, determined tail)
 # (profiles/pass1_traffic_batch512.md).  Other configurations report null.
 PASS1_TRAFFIC_PER_OUT_BYTE_BATCH512 = {
-    (499078, 4, 0, 0): (0.964350464e9 + 0.952157696e9 + 39.964783360e9 + 23.372040960e9) / 4467581835,
-    (499078, 2, 0, 0): (0.966032640e9 + 0.953315840e9 + 39.960246528e9 + 23.372556288e9) / 4467581835,
+    (262144, 2, 0, 0): (1.588861440e9 + 1.700140544e9 + 17.259778304e9 + 19.536223744e9 + 9.498650880e9
+                        + 8.871193600e9) / 4467581835,
 }
 
 
@@ -264,7 +264,7 @@ def run_pgz(args, rank, world):
     window_bytes = int((nph_parts > 0).sum()) * 32768
 
     # ---- plain: one file at a time through pgz_decompress, PLAIN_PARTS equal parts per file, with the
-    # batched form's CTA shape and execution form
+    # batched form's CTA shape
     ctx_p = pgz.pgz_create(pgz.pgz_config_init(device=dev, cuda_stream=stream.cuda_stream, n_chunks=PLAIN_PARTS,
                                                warps_per_block=wpb, exec_pipelined=xp))
 
@@ -1322,7 +1322,7 @@ def main():
     ap.add_argument("--warps-per-block", type=int, default=4, choices=[2, 4, 8],
                     help="pass-1 CTA shape with a fixed --chunk-bytes or --profile-case")
     ap.add_argument("--exec-pipelined", type=int, default=0, choices=[0, 1],
-                    help="pass-1 execution form with a fixed --chunk-bytes (default: autotuned)")
+                    help="accepted for older commands: the two execution forms are the same code")
     ap.add_argument("--served-requests", type=int, default=SERVED_REQUESTS,
                     help="requests per offered load of the served extra (0: leave it out)")
     ap.add_argument("--headline-only", action="store_true",
