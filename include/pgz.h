@@ -412,12 +412,16 @@ uint64_t pgz_kernel_launches(const pgz_ctx* ctx);
    own confirmation passed, decoded past its stop when the run left the
    confirmation open, searched on from the bit after it when it ends a
    streamed segment; a part whose symbols overflowed needs more capacity.
+   Decoding from an offset (mode 1) the first start that passes is kept:
+   invalid data after its window is final, and when it is refused the parts
+   merged on its account are searched again.
    parts [host array of n, part i of the member in order]: the plan fields
    and the run's results on input; on return the plan fields (lo, disabled,
    confirm_ext) hold the next run's plan.  s0_bit: the member's first DEFLATE
    bit (part 0 with lo <= s0_bit is the member start); mode and last_seg as
-   for the member's description (0: a whole member; 3 with last_seg 0: a
-   streamed segment that does not reach the member's end).  Returns
+   for the member's description (0: a whole member; 1: from an offset; 3 with
+   last_seg 0: a streamed segment that does not reach the member's end).
+   Returns
    PGZ_RECOVER_STOP (the parts' errors are final), PGZ_RECOVER_RERUN or
    PGZ_RECOVER_GROW (*grow: the part that needs more symbol capacity), or -1
    for bad arguments; *false_syncs is increased by one for every start the

@@ -73,6 +73,11 @@ int recover_member(const FileDesc& F, ChunkDesc* plan, const ChunkDesc* res, int
         for (int c = c0; c < c1; ++c) {
             if (!searched_start(F, plan[c], res[c])) continue;
             if (confirm_failure(F, res, c, confirm_blocks) > 0) {
+                // decoding from an offset, parts are merged because the chain of blocks from the first start does not
+                // lead to theirs: without that start they are searched again
+                if (F.mode == 1 && next_start(F, res, c0 - 1) == c)
+                    for (int j = c + 1; j < c1; ++j)
+                        if (plan[j].lo < plan[j].hi) plan[j].disabled = 0;
                 plan[c].lo = res[c].sync + 1;
                 plan[c].confirm_ext = 0;
                 again = true;
@@ -121,6 +126,9 @@ int recover_member(const FileDesc& F, ChunkDesc* plan, const ChunkDesc* res, int
             C.confirm_ext = 0;
             return kRecoverRerun;
         }
+        // decoding from an offset: the first start is accepted (its window passed) and its blocks lead to this one, so
+        // the data is invalid; a merge would end with the first start dropped and the decode begun after the damage
+        if (F.mode == 1) return kRecoverStop;
         C.disabled = 1;
         ++*false_syncs;
         return kRecoverRerun;
@@ -1921,6 +1929,7 @@ int pgz_recover_step(int n, pgz_part_state* parts, uint64_t s0_bit, int mode, in
         ChunkDesc& C = plan[(size_t)k];
         C = ChunkDesc{};
         C.lo = q.lo;
+        C.hi = kNone;
         C.index = k;
         C.given = q.given ? 1u : 0u;
         C.probe = q.probe ? 1u : 0u;

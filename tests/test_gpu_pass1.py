@@ -136,6 +136,43 @@ def test_decoding_from_an_offset_in_several_parts(kind, chunk):
         ctx.close()
 
 
+@pytest.mark.parametrize("chunk", [4096, 16384, 65536, 1 << 20])
+def test_decoding_a_damaged_member_from_an_offset(chunk):
+    """One block after another given the reserved type: whatever the parts (1 MiB: a single one), the verdict is the
+    oracle's -- the start is refused if the damage lies in its window of six blocks, else the data is invalid -- and
+    where it is success, so are the block start and the symbols."""
+    import torch
+    c = zlib.compressobj(6, zlib.DEFLATED, 31, 7)
+    text = synth.fastq(800_000, 150, 0.001, 8)
+    gz = c.compress(text) + c.flush()
+    _, _, blocks, _ = oracle.gunzip(gz, max_blocks=1000)
+    start = 8 * (len(gz) // 5)
+    later = [int(b) for b in blocks if b >= start]
+    ctx = Ctx(chunk_bytes=chunk)
+    try:
+        P = ctx.pgz
+        verdicts = {0: 0, -3: P.PGZ_E_DATA, -13: P.PGZ_E_NOSYNC}
+        seen = set()
+        for b in later[:8] + later[8::5] + later[-1:]:
+            bad = bytearray(gz)
+            for k in (1, 2):
+                bad[(b + k) // 8] |= 1 << (b + k) % 8
+            ref = oracle.decompress_at(bytes(bad), start, fill=ord("?"), cap=len(text))
+            sym, byt = torch.zeros(len(text), dtype=torch.int16, device="cuda"), empty(len(text))
+            d = to_device(bytes(bad))
+            st, n, bb, fd = P.pgz_decompress_at(ctx.h, d.data_ptr(), len(bad), start, sym.data_ptr(), byt.data_ptr(),
+                                                ord("?"), len(text))
+            assert st == verdicts[ref["status"]], (b, P.pgz_strerror(st))
+            seen.add(st)
+            if st == 0:
+                assert (n, bb, fd) == (ref["sym"].size, ref["block_bit"], ref["first_determined"])
+                assert np.array_equal(sym[:n].cpu().numpy().view(np.uint16), ref["sym"])
+                assert byt[:n].cpu().numpy().tobytes() == ref["bytes"]
+        assert {0, P.PGZ_E_DATA} <= seen
+    finally:
+        ctx.close()
+
+
 @pytest.mark.parametrize("n", [1, 31, 32, 33, 255, 256, 257, 8191, 8192, 8193, 70001])
 def test_sequences_at_word_and_block_edges(n):
     """Runs over words of 32 symbols and over the kernels' blocks, ends of the array included, against the oracle."""

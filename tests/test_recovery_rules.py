@@ -153,6 +153,39 @@ def test_a_searched_start_failing_past_its_window_is_merged(P):
     assert plan == [(S0, 0, 0), (900, 0, 0), (1900, 1, 0)]
 
 
+def test_from_an_offset_a_failure_past_the_first_starts_window_is_final(P):
+    # decoding from an offset (mode 1, no part is the member start): the decode is the one from the first accepted
+    # start, so invalid data after that start's window is an error, not a reason to drop the start
+    parts = [failed(900, 1000, 2800, 8, P.PGZ_PART_DATA, confirmed=1), done(2900, 3000, 4000, 8)]
+    assert step(P, parts, mode=1) == (P.PGZ_RECOVER_STOP, plan_of(parts), 0, -1)
+    # the same where the first part holds no start, and in a later part that the first start's blocks lead to
+    parts = [dict(lo=200, state=2), failed(900, 1000, 2800, 8, P.PGZ_PART_DATA, confirmed=1), done(2900, 3000, 4000, 8)]
+    assert step(P, parts, mode=1) == (P.PGZ_RECOVER_STOP, plan_of(parts), 0, -1)
+    parts = [done(900, 1000, 2000, 7), failed(1900, 2000, 2800, 8, P.PGZ_PART_DATA, confirmed=1),
+             done(2900, 3000, 4000, 8)]
+    assert step(P, parts, mode=1) == (P.PGZ_RECOVER_STOP, plan_of(parts), 0, -1)
+    # one part alone
+    parts = [failed(900, 1000, 2800, 8, P.PGZ_PART_DATA, confirmed=1)]
+    assert step(P, parts, mode=1) == (P.PGZ_RECOVER_STOP, plan_of(parts), 0, -1)
+
+
+def test_from_an_offset_a_first_start_refused_gives_back_the_parts_merged_on_its_account(P):
+    # part 1 was merged because part 0's start did not lead to its own; part 0's start then fails its confirmation, so
+    # part 1 is searched again beside it
+    parts = [failed(900, 1000, 2600, 2, P.PGZ_PART_CONFIRM), dict(lo=1900, disabled=1, state=2), done(2900, 3000, 4000, 8)]
+    a, plan, fs, g = step(P, parts, mode=1)
+    assert a == P.PGZ_RECOVER_RERUN and fs == 0
+    assert plan == [(1001, 0, 0), (1900, 0, 0), (2900, 0, 0)]
+    # a later start's failure leaves the merged part as it is: the chain from the first start stands
+    parts = [done(900, 1000, 2500, 7), dict(lo=1900, disabled=1, state=2), failed(2400, 2500, 2600, 2, P.PGZ_PART_CONFIRM)]
+    a, plan, fs, g = step(P, parts, mode=1)
+    assert a == P.PGZ_RECOVER_RERUN and plan == [(900, 0, 0), (1900, 1, 0), (2501, 0, 0)]
+    # a whole member's chain begins at its first block: nothing is given back
+    parts = [done(S0, S0, 2500, 7), dict(lo=1900, disabled=1, state=2), failed(2400, 2500, 2600, 2, P.PGZ_PART_CONFIRM)]
+    a, plan, fs, g = step(P, parts)
+    assert a == P.PGZ_RECOVER_RERUN and plan == [(S0, 0, 0), (1900, 1, 0), (2501, 0, 0)]
+
+
 def test_without_confirmation_blocks_a_failed_start_is_still_searched_on(P):
     parts = [done(S0, S0, 1000, 9), failed(900, 1000, 1200, 0, P.PGZ_PART_CONFIRM)]
     a, plan, fs, g = step(P, parts, confirm_blocks=0)
