@@ -11,6 +11,7 @@
 #include <new>
 #include <vector>
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "pgz_internal.h"
@@ -365,43 +366,82 @@ int read_member(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, MemberInfo* mi
     }
 }
 
-// read_member for the jobs k with st[k] = PGZ_OK, with one kernel and one copy back; st[k] and mi[k] receive the results
-int read_members(pgz_ctx* ctx, int n, const pgz_job* jobs, std::vector<int>& st, std::vector<MemberInfo>& mi) {
-    std::vector<int> idx;
+// the device allocation that holds an address, as the driver knows it: [lo, hi)
+struct AllocRange {
+    uint64_t lo = 0, hi = 0;
+    bool holds(uint64_t a, uint64_t n) const { return a >= lo && a < hi && n <= hi - a; }
+    bool find(uint64_t a) {
+        using Fn = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+        static const Fn fn = [] {
+            void* f = nullptr;
+            cudaDriverEntryPointQueryResult q;
+            if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+                q != cudaDriverEntryPointSuccess) {
+                cudaGetLastError();
+                f = nullptr;
+            }
+            return reinterpret_cast<Fn>(f);
+        }();
+        CUdeviceptr base = 0;
+        size_t n = 0;
+        if (!fn || fn(&base, &n, (CUdeviceptr)a) != CUDA_SUCCESS) return false;
+        lo = base;
+        hi = base + n;
+        return true;
+    }
+};
+
+// read_member for the jobs k with st[k] = PGZ_OK, with one kernel and one copy back; st[k] and mi[k] receive the
+// results.  The kernel reads the members' ends through the caller's pointers, so it takes only members that lie in one
+// device allocation, which the driver is asked for; a member whose last byte lies in none is refused, and any other
+// (page-locked memory, a mapping of several allocations) is read by read_member's copies, which the driver checks.
+void read_members(pgz_ctx* ctx, int n, const pgz_job* jobs, std::vector<int>& st, std::vector<MemberInfo>& mi) {
+    std::vector<int> idx, single;                    // members of the kernel; those read one by one
+    AllocRange R;                                    // the last allocation found: members often share one
     for (int k = 0; k < n; ++k) {
         if (st[(size_t)k] != PGZ_OK) continue;
-        if (jobs[k].gz_len < 18) st[(size_t)k] = PGZ_E_HEADER;
-        else idx.push_back(k);
+        const uint64_t a = reinterpret_cast<uintptr_t>(jobs[k].gz), len = jobs[k].gz_len;
+        if (len < 18) st[(size_t)k] = PGZ_E_HEADER;
+        else if (R.holds(a, len)) idx.push_back(k);
+        else if (!R.find(a)) single.push_back(k);
+        else if (R.holds(a, len)) idx.push_back(k);
+        else if (a + len < a || !R.find(a + len - 1)) st[(size_t)k] = PGZ_E_CUDA;
+        else single.push_back(k);
     }
-    if (idx.empty()) return PGZ_OK;
     const size_t m = idx.size(), in = round_up(m * sizeof(MemberRef), 256), row = kHeadBytes + 8;
-    if (cuda_status(ctx->hdr.ensure(in + m * row)) || cuda_status(ctx->heads.ensure(in + m * row))) return PGZ_E_NOMEM;
-    uint8_t *h = ctx->hdr.as<uint8_t>(), *d = ctx->heads.as<uint8_t>();
-    for (size_t i = 0; i < m; ++i) reinterpret_cast<MemberRef*>(h)[i] = MemberRef{jobs[idx[i]].gz, jobs[idx[i]].gz_len};
-    if (cudaMemcpyAsync(d, h, m * sizeof(MemberRef), cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess) return PGZ_E_CUDA;
-    launch_heads(reinterpret_cast<const MemberRef*>(d), (int)m, d + in, ctx->stream);
-    ctx->launches += 1;
-    if (cudaMemcpyAsync(h + in, d + in, m * row, cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess ||
-        cudaStreamSynchronize(ctx->stream) != cudaSuccess)
-        return PGZ_E_CUDA;
-    std::vector<int> again;                          // headers longer than what was read
-    for (size_t i = 0; i < m; ++i) {
-        const int k = idx[i];
-        const uint8_t *b = h + in + i * row, *t = b + kHeadBytes;
-        uint64_t s0 = 0;
-        const int r = parse_header(b, std::min<uint64_t>(kHeadBytes, jobs[k].gz_len), jobs[k].gz_len, &s0);
-        if (r == -1) {
-            again.push_back(k);
-            continue;
-        }
-        st[(size_t)k] = r == PGZ_OK ? PGZ_OK : PGZ_E_HEADER;
-        MemberInfo& M = mi[(size_t)k];
-        M.s0 = s0;
-        M.crc = t[0] | ((uint32_t)t[1] << 8) | ((uint32_t)t[2] << 16) | ((uint32_t)t[3] << 24);
-        M.isize = t[4] | ((uint32_t)t[5] << 8) | ((uint32_t)t[6] << 16) | ((uint32_t)t[7] << 24);
+    if (m && (cuda_status(ctx->hdr.ensure(in + m * row)) || cuda_status(ctx->heads.ensure(in + m * row)))) {
+        single.insert(single.end(), idx.begin(), idx.end());
+        idx.clear();
     }
-    for (const int k : again) st[(size_t)k] = read_member(ctx, jobs[k].gz, jobs[k].gz_len, &mi[(size_t)k]);
-    return PGZ_OK;
+    if (!idx.empty()) {
+        uint8_t *h = ctx->hdr.as<uint8_t>(), *d = ctx->heads.as<uint8_t>();
+        for (size_t i = 0; i < m; ++i) reinterpret_cast<MemberRef*>(h)[i] = MemberRef{jobs[idx[i]].gz, jobs[idx[i]].gz_len};
+        bool ok = cudaMemcpyAsync(d, h, m * sizeof(MemberRef), cudaMemcpyHostToDevice, ctx->stream) == cudaSuccess;
+        if (ok) {
+            launch_heads(reinterpret_cast<const MemberRef*>(d), (int)m, d + in, ctx->stream);
+            ctx->launches += 1;
+            ok = cudaMemcpyAsync(h + in, d + in, m * row, cudaMemcpyDeviceToHost, ctx->stream) == cudaSuccess &&
+                 cudaStreamSynchronize(ctx->stream) == cudaSuccess;
+        }
+        for (size_t i = 0; i < m; ++i) {
+            const int k = idx[i];
+            const uint8_t *b = h + in + i * row, *t = b + kHeadBytes;
+            uint64_t s0 = 0;
+            const int r = ok ? parse_header(b, std::min<uint64_t>(kHeadBytes, jobs[k].gz_len), jobs[k].gz_len, &s0) : PGZ_E_CUDA;
+            if (r == -1) {                           // a header longer than what was read
+                single.push_back(k);
+                continue;
+            }
+            st[(size_t)k] = r == PGZ_OK || r == PGZ_E_CUDA ? r : PGZ_E_HEADER;
+            MemberInfo& M = mi[(size_t)k];
+            M.s0 = s0;
+            M.crc = t[0] | ((uint32_t)t[1] << 8) | ((uint32_t)t[2] << 16) | ((uint32_t)t[3] << 24);
+            M.isize = t[4] | ((uint32_t)t[5] << 8) | ((uint32_t)t[6] << 16) | ((uint32_t)t[7] << 24);
+        }
+    }
+    for (const int k : single) st[(size_t)k] = read_member(ctx, jobs[k].gz, jobs[k].gz_len, &mi[(size_t)k]);
+    for (int k = 0; k < n; ++k)                      // one job's refusal is its own, not the next call's
+        if (st[(size_t)k] == PGZ_E_CUDA || st[(size_t)k] == PGZ_E_NOMEM) cudaGetLastError();
 }
 
 // parts of one member: equal compressed size (Section "Full file decompression
@@ -1569,8 +1609,7 @@ int pgz_decompress_batch(pgz_ctx* ctx, int n, pgz_job* jobs, pgz_stats* st) {
         jobs[k].out_len = 0;
         if (!jobs[k].gz || !aligned4(jobs[k].gz) || (!jobs[k].out && jobs[k].out_cap)) bad[(size_t)k] = PGZ_E_ARG;
     }
-    const int he = read_members(ctx, n, jobs, bad, mi);
-    if (he) return he;
+    read_members(ctx, n, jobs, bad, mi);
     for (int k = 0; k < n; ++k) {
         if (bad[(size_t)k]) {
             jobs[k].status = bad[(size_t)k];
@@ -1762,7 +1801,7 @@ int pgz_batch_prepare(pgz_ctx* ctx, int n, const pgz_job* jobs, pgz_batch** out)
     int he = PGZ_OK;
     for (int k = 0; k < n; ++k)
         if (!jobs[k].gz || !aligned4(jobs[k].gz) || (!jobs[k].out && jobs[k].out_cap)) bad[(size_t)k] = PGZ_E_ARG;
-    he = read_members(ctx, n, jobs, bad, mi);
+    read_members(ctx, n, jobs, bad, mi);
     for (int k = 0; k < n && !he; ++k) he = bad[(size_t)k];
     if (he) {
         delete b;

@@ -2464,7 +2464,7 @@ __global__ void __launch_bounds__(256) k_sequences(const uint32_t* __restrict__ 
 }
 
 // The first kHeadBytes bytes and the last 8 of every member of a batch, one warp per member, so that the host reads
-// all of them with one copy.
+// all of them with one copy (the caller has made sure that they lie in device memory).
 __global__ void __launch_bounds__(128) k_heads(const MemberRef* __restrict__ in, int n, uint8_t* out) {
     const int m = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (m >= n) return;

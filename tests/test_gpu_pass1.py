@@ -173,6 +173,50 @@ def test_decoding_a_damaged_member_from_an_offset(chunk):
         ctx.close()
 
 
+@pytest.mark.parametrize("together", [False, True])
+def test_a_batch_reports_each_job_and_refuses_what_lies_outside_device_memory(together):
+    """Members in allocations of their own or side by side in one: headers within the gathered 64 bytes, longer, and a
+    member shorter than that; a length that runs out of device memory, one below a member's least, a pointer off the
+    alignment.  Each job has its own status, the good ones their output, and the next call is not affected."""
+    import torch
+    text = synth.fastq(60_000, 100, 0.001, 6)
+    raw = zlib.compressobj(6, zlib.DEFLATED, -15)
+    body = raw.compress(text) + raw.flush()
+    good = [(synth.gzip_compress(text, 6), text), (synth.gzip_compress(b"A", 6), b"A"),
+            (dw.gzip_wrap(body, text, flags=8, name=b"n" * 40), text),
+            (dw.gzip_wrap(body, text, flags=8, name=b"n" * 53), text),
+            (dw.gzip_wrap(body, text, flags=2 | 4 | 8 | 16, name=b"n" * 5000, extra=b"e" * 300, comment=b"c"), text)]
+    ctx = Ctx()
+    try:
+        P = ctx.pgz
+        if together:
+            offs = np.cumsum([0] + [(len(g) + 15) // 16 * 16 for g, _ in good])
+            one = to_device(b"".join(g + b"\0" * (-len(g) % 16) for g, _ in good))
+            ptrs = [one.data_ptr() + int(o) for o in offs[:-1]]
+        else:
+            dev = [to_device(g) for g, _ in good]
+            ptrs = [d.data_ptr() for d in dev]
+        outs = [empty(len(t)) for _, t in good]
+        jobs = [(p, len(g), o.data_ptr(), len(t)) for p, o, (g, t) in zip(ptrs, outs, good)]
+        bad = [((ptrs[0], 1 << 62, outs[0].data_ptr(), len(text)), P.PGZ_E_CUDA),
+               ((ptrs[0], 17, outs[0].data_ptr(), len(text)), P.PGZ_E_HEADER),
+               ((ptrs[0] + 1, 100, outs[0].data_ptr(), len(text)), P.PGZ_E_ARG)]
+        for k, (job, want) in enumerate(bad):
+            st, res, _ = P.pgz_decompress_batch(ctx.h, jobs[:k] + [job] + jobs[k:])
+            assert st == want and res[k] == (want, 0)
+            assert [r for i, r in enumerate(res) if i != k] == [(0, len(t)) for _, t in good]
+            for o, (_, t) in zip(outs, good):
+                assert o[:len(t)].cpu().numpy().tobytes() == t
+                o.zero_()
+            with pytest.raises(P.PgzError):
+                P.Batch(ctx.h, jobs + [job])
+        st, res, _ = P.pgz_decompress_batch(ctx.h, jobs)
+        assert st == 0 and all(o[:len(t)].cpu().numpy().tobytes() == t for o, (_, t) in zip(outs, good))
+        torch.cuda.synchronize()
+    finally:
+        ctx.close()
+
+
 @pytest.mark.parametrize("n", [1, 31, 32, 33, 255, 256, 257, 8191, 8192, 8193, 70001])
 def test_sequences_at_word_and_block_edges(n):
     """Runs over words of 32 symbols and over the kernels' blocks, ends of the array included, against the oracle."""
