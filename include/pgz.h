@@ -194,7 +194,11 @@ int pgz_decompress_stream(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, uint
      replaced by `fill` (the undetermined '?' context of Section
      "Undetermined context propagation technique");
    *out_len: symbols decoded; *block_bit: b; *first_determined: one past the
-   last placeholder (0 if none).  PGZ_E_NOSYNC if no block start follows. */
+   last placeholder (0 if none).  PGZ_E_NOSYNC if no block start follows.
+   Scratch: what pgz_decompress takes for the bytes from b on, with windows of
+   64 KiB instead of 32 a part, and 2 bytes per symbol of out_cap; both stay
+   with the context (the latter is given back when a run is short of memory).
+   Without memory for parts the call decodes in one part. */
 int pgz_decompress_at(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, uint64_t start_bit,
                       uint16_t* sym_out, uint8_t* byte_out, uint8_t fill, uint64_t out_cap,
                       uint64_t* out_len, uint64_t* block_bit, uint64_t* first_determined);

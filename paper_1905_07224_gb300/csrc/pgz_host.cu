@@ -267,6 +267,8 @@ struct Plan {
     uint8_t* at_bytes = nullptr;
     uint8_t at_fill = 0;
     DBuf d_at;
+    uint16_t* one = nullptr;      // the symbols of that run as one part, in order (pgz_ctx::at_sym); else null
+    uint16_t* symbols() const { return one ? one : d_sym.as<uint16_t>(); }
     // the plan's arrays lie in one device buffer, uploaded from one pinned copy: the work counters, members and
     // parts first (head_bytes, which a graph uploads again), then what stays the same from run to run
     DBuf d_plan;
@@ -301,7 +303,7 @@ struct pgz_ctx {
     KParams kp;
     cudaStream_t stream = nullptr;
     Plan plan;                 // the last call's plan (kept for inspection)
-    Plan at_plan;              // pgz_decompress_at: the run in several parts (its result becomes `plan`'s one part)
+    DBuf at_sym;               // pgz_decompress_at in several parts: the symbols in order (given back when memory is short)
     PBuf hdr;                  // header / trailer staging
     DBuf heads;                // a batch's members, and their headers and trailers gathered
     DBuf in_buf, out_buf, fill_buf;
@@ -675,7 +677,7 @@ int read_chunks(pgz_ctx* ctx, Plan& P) {
 
 // placeholder counts of the last run's parts (after the run; not timed), then the results
 int count_and_read_chunks(pgz_ctx* ctx, Plan& P) {
-    launch_count_ph(P.d_chunks.as<ChunkDesc>(), (int)P.chunks.size(), P.d_sym.as<uint16_t>(), ctx->stream);
+    launch_count_ph(P.d_chunks.as<ChunkDesc>(), (int)P.chunks.size(), P.symbols(), ctx->stream);
     if (cudaPeekAtLastError() != cudaSuccess) return PGZ_E_CUDA;
     return read_chunks(ctx, P);
 }
@@ -748,6 +750,12 @@ int start_run(pgz_ctx* ctx, Plan& P, bool timed, cudaStream_t up = nullptr, cuda
     P.wpb = ctx->kp.wpb;
     reset_results(P);
     int e = layout(P);
+    if (e == PGZ_E_NOMEM && ctx->at_sym.p && !P.at_sym) {        // give back what pgz_decompress_at kept
+        cudaGetLastError();
+        ctx->at_sym.release();
+        if (ctx->plan.one) ctx->plan.results_valid = false;
+        e = layout(P);
+    }
     if (e) return e;
     return enqueue(ctx, P, ctx->stream, timed, true, up, up_done);
 }
@@ -1101,7 +1109,7 @@ void begin_plan(Plan& P) {
     P.chain = P.translate = P.crc = true;
     P.results_valid = false;
     P.fill = nullptr;
-    P.at_sym = nullptr;
+    P.at_sym = P.one = nullptr;
     P.at_bytes = nullptr;
     if (P.graph) cudaGraphExecDestroy(P.graph);
     P.graph = nullptr;
@@ -1343,7 +1351,7 @@ void pgz_destroy(pgz_ctx* ctx) {
     cudaSetDevice(ctx->cfg.device);
     cudaStreamSynchronize(ctx->stream);
     ctx->plan.release();
-    ctx->at_plan.release();
+    ctx->at_sym.release();
     ctx->carry_win.release();
     for (int k = 0; k < 2; ++k) {
         ctx->sin[k].release();
@@ -1402,6 +1410,8 @@ int pgz_decompress_host(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, uint8_
 // start and symbolic context, the parts' windows then chained as symbols relative to the first part's context.  The
 // result becomes the one part of ctx->plan, as a run in one part leaves it.  Returns PGZ_OK, or anything else when the
 // caller shall run it in one part instead (too short, or an error: what to report is that run's to say).
+// The parts use the context's own plan and scratch, what pgz_decompress takes for the same bytes (windows of u16);
+// beside them only the symbols in order are kept.
 static int decompress_at_parts(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, const MemberInfo& mi, uint64_t lo,
                                bool at_start, uint8_t* byte_out, uint8_t fill, uint64_t out_cap, uint64_t* last_ph) {
     const uint64_t end_bit = (gz_len - 8) * 8;
@@ -1410,15 +1420,13 @@ static int decompress_at_parts(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len,
     const uint64_t per_bytes = ctx->cfg.n_chunks > 0 ? kAtPartBytes : std::max<uint64_t>(ctx->cfg.chunk_bytes, 4096);
     const uint64_t n = (csize + per_bytes - 1) / per_bytes;
     if (n < 2 || n > (1u << 20)) return PGZ_E_NOSYNC;
-    Plan& R = ctx->plan;
-    begin_plan(R);
     const uint64_t cap1 = round_up(std::max<uint64_t>(out_cap, 65536), 32);
     if (cap1 > kMaxPartSymbols) return PGZ_E_NOSYNC;
-    if (cuda_status(R.d_sym.ensure(cap1 * sizeof(uint16_t)))) return PGZ_E_NOMEM;
-    Plan& P = ctx->at_plan;
+    if (cuda_status(ctx->at_sym.ensure(cap1 * sizeof(uint16_t)))) return PGZ_E_NOMEM;
+    Plan& P = ctx->plan;
     begin_plan(P);
     P.translate = P.crc = false;
-    P.at_sym = R.d_sym.as<uint16_t>();
+    P.at_sym = ctx->at_sym.as<uint16_t>();
     P.at_bytes = byte_out;
     P.at_fill = fill;
     FileDesc F{};
@@ -1489,17 +1497,16 @@ static int decompress_at_parts(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len,
     C.final = 1;
     C.confirmed = 1;
     C.anyph = counts[0] != 0;
-    R.files.push_back(RF);
-    R.chunks.push_back(C);
-    R.chain = R.crc = false;
-    R.sym_total = cap1;
-    if (cuda_status(R.d_plan.ensure(sizeof C)) || cuda_status(R.h_chunks.ensure(sizeof C))) return PGZ_E_NOMEM;
-    R.d_chunks.p = R.d_plan.p;
-    memcpy(R.h_chunks.p, &C, sizeof C);
-    if (cudaMemcpyAsync(R.d_chunks.p, R.h_chunks.p, sizeof C, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
+    begin_plan(P);
+    P.files.push_back(RF);
+    P.chunks.push_back(C);
+    P.chain = P.crc = false;
+    P.one = ctx->at_sym.as<uint16_t>();
+    memcpy(P.h_chunks.p, &C, sizeof C);
+    if (cudaMemcpyAsync(P.d_chunks.p, P.h_chunks.p, sizeof C, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
         cudaStreamSynchronize(ctx->stream) != cudaSuccess)
         return PGZ_E_CUDA;
-    R.results_valid = true;
+    P.results_valid = true;
     *last_ph = counts[1];
     return PGZ_OK;
 }
@@ -1524,15 +1531,16 @@ int pgz_decompress_at(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, uint64_t
             if (block_bit) *block_bit = C.sync;
             if (first_determined) *first_determined = last;
             if (sym_out && C.n &&
-                (cudaMemcpyAsync(sym_out, ctx->plan.d_sym.p, C.n * sizeof(uint16_t), cudaMemcpyDeviceToDevice,
+                (cudaMemcpyAsync(sym_out, ctx->plan.symbols(), C.n * sizeof(uint16_t), cudaMemcpyDeviceToDevice,
                                  ctx->stream) != cudaSuccess ||
                  cudaStreamSynchronize(ctx->stream) != cudaSuccess))
                 return PGZ_E_CUDA;
             return PGZ_OK;
         }
         if (e == PGZ_E_CUDA) return e;
-        if (e == PGZ_E_NOMEM) {                        // no room for the parts beside the one part: give theirs back
-            ctx->at_plan.release();
+        if (e == PGZ_E_NOMEM) {                        // no room for the parts: what they hold goes back first
+            ctx->at_sym.release();
+            ctx->plan.release();
             cudaGetLastError();
         }
     }
@@ -1915,7 +1923,7 @@ int pgz_inspect_symbols(pgz_ctx* ctx, int part, uint16_t* host_dst, uint64_t cap
     if (cap < n) return PGZ_E_CAPACITY;
     // u16 symbols before the determined tail; the tail's bytes (symbol k at byte det + k) widened
     const uint64_t nw = C.det < n ? C.det : n;
-    const uint16_t* d = ctx->plan.d_sym.as<uint16_t>() + C.sym_base;
+    const uint16_t* d = ctx->plan.symbols() + C.sym_base;
     if (nw && cudaMemcpy(host_dst, d, nw * sizeof(uint16_t), cudaMemcpyDeviceToHost) != cudaSuccess) return PGZ_E_CUDA;
     if (nw < n) {
         std::vector<uint8_t> t((size_t)(n - nw));

@@ -173,6 +173,31 @@ def test_decoding_a_damaged_member_from_an_offset(chunk):
         ctx.close()
 
 
+def test_decoding_from_an_offset_shares_the_contexts_scratch():
+    """After a file has been decoded, decoding it from an offset takes no more device memory than the symbols in order
+    and the wider windows (32 KiB a part more), with a little room for the allocator's granularity."""
+    import torch
+    text = synth.fastq(8_000_000, 150, 0.001, 8)
+    gz = synth.gzip_compress(text, 6)
+    parts = len(gz) // 4096 + 1
+    ctx = Ctx(chunk_bytes=4096)
+    try:
+        P = ctx.pgz
+        d, out = to_device(gz), empty(len(text))
+        torch.cuda.synchronize()
+        assert P.pgz_decompress(ctx.h, d.data_ptr(), len(gz), out.data_ptr(), len(text), False)[:2] == (0, len(text))
+        before = torch.cuda.mem_get_info()[0]
+        st, n, bb, fd = P.pgz_decompress_at(ctx.h, d.data_ptr(), len(gz), 8 * (len(gz) // 10), None, out.data_ptr(),
+                                            ord("?"), len(text))
+        assert st == 0 and n < len(text)
+        assert before - torch.cuda.mem_get_info()[0] <= 2 * len(text) + 33 * 1024 * parts + (32 << 20)
+        # the context goes on with either call
+        assert P.pgz_decompress(ctx.h, d.data_ptr(), len(gz), out.data_ptr(), len(text), False)[:2] == (0, len(text))
+        assert out[:len(text)].cpu().numpy().tobytes() == text
+    finally:
+        ctx.close()
+
+
 @pytest.mark.parametrize("together", [False, True])
 def test_a_batch_reports_each_job_and_refuses_what_lies_outside_device_memory(together):
     """Members in allocations of their own or side by side in one: headers within the gathered 64 bytes, longer, and a
