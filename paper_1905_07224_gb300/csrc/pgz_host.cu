@@ -260,6 +260,7 @@ struct Plan {
     uint64_t sym_total = 0, max_cap = 0, total_seg = 0;
     bool chain = true, translate = true, crc = true;
     bool results_valid = false;   // the device chunk array holds the last run's results
+    bool spent = false;           // the last run ended with its re-runs used up: its error is not settled
     int wpb = 4;                  // warps per block of the pass-1 kernels (sizes the token scratch)
     const uint8_t* fill = nullptr;   // device window of fill bytes (mode 1)
     // mode 1 in several parts: where its symbols and bytes go (launch_resolve_at), and its counts (2 u64)
@@ -601,6 +602,23 @@ int layout(Plan& P) {
     return cuda_status(e);
 }
 
+// the window chain of a plan whose parts are decoded
+ChainPlan chain_plan(const Plan& P) {
+    const int32_t* u = P.d_upper.as<int32_t>();
+    const size_t nf = P.files.size(), ns = P.nsupers;
+    return ChainPlan{(int)P.g0.size(), (int)ns, P.many, P.deep, P.d_g0.as<int32_t>(), P.d_gn.as<int32_t>(),
+                     P.d_gfile.as<int32_t>(), u, u + ns, u + 2 * ns, u + 3 * ns, u + 3 * ns + nf, u + 3 * ns + 2 * nf};
+}
+int chain_launches(const Plan& P) { return 1 + (P.many ? 2 : 0) + (P.deep ? 2 : 0); }
+
+// pgz_decompress_at in parts: the chain of symbolic windows, then the symbols in order; the kernels launched
+int enqueue_resolve(Plan& P, cudaStream_t s) {
+    launch_resolve_at(P.d_files.as<FileDesc>(), P.d_chunks.as<ChunkDesc>(), (int)P.chunks.size(), chain_plan(P),
+                      P.d_sym.as<uint16_t>(), P.d_gmaps.as<uint16_t>(), P.d_wstart.as<uint16_t>(),
+                      P.d_windows.as<uint16_t>(), P.at_sym, P.at_bytes, P.at_fill, P.d_at.as<unsigned long long>(), s);
+    return chain_launches(P) + 1;
+}
+
 // The device-resident part of a run: the plan's upload, every stage, result download.  The upload is one copy from
 // pinned memory (a copy from pageable memory is staged by the driver and may reach the copy engine after pinned copies
 // issued later, the next group of compressed bytes of a host-buffer batch, so that the run would wait for them).
@@ -609,7 +627,7 @@ int layout(Plan& P) {
 // up_done); see pgz_decompress_batch_host
 int enqueue(pgz_ctx* ctx, Plan& P, cudaStream_t s, bool timed, bool static_too, cudaStream_t up = nullptr,
             cudaEvent_t up_done = nullptr) {
-    const size_t nf = P.files.size(), nc = P.chunks.size(), ng = P.g0.size();
+    const size_t nf = P.files.size(), nc = P.chunks.size();
     const cudaStream_t u = up ? up : s;
     uint8_t* h = P.h_plan.as<uint8_t>();
     const uint8_t* d = P.d_plan.as<uint8_t>();
@@ -637,19 +655,12 @@ int enqueue(pgz_ctx* ctx, Plan& P, cudaStream_t s, bool timed, bool static_too, 
     launch_plan(df, dc, (int)nf, s);
     k += 4;
     if (timed) cudaEventRecord(ctx->ev[2], s);
-    if (P.chain) {
-        const int32_t* u = P.d_upper.as<int32_t>();
-        const size_t ns = P.nsupers;
-        const ChainPlan cp{(int)ng, (int)ns, P.many, P.deep, P.d_g0.as<int32_t>(), P.d_gn.as<int32_t>(), P.d_gfile.as<int32_t>(),
-                           u, u + ns, u + 2 * ns, u + 3 * ns, u + 3 * ns + nf, u + 3 * ns + 2 * nf};
-        if (P.at_sym) {
-            launch_resolve_at(df, dc, (int)nc, cp, sym, P.d_gmaps.as<uint16_t>(), P.d_wstart.as<uint16_t>(),
-                              P.d_windows.as<uint16_t>(), P.at_sym, P.at_bytes, P.at_fill,
-                              P.d_at.as<unsigned long long>(), s);
-            k += 1;
-        } else launch_chain(df, dc, (int)nf, cp, sym, P.d_gmaps.as<uint16_t>(), P.d_wstart.as<uint8_t>(),
+    if (P.at_sym) {
+        k += enqueue_resolve(P, s);
+    } else if (P.chain) {
+        launch_chain(df, dc, (int)nf, chain_plan(P), sym, P.d_gmaps.as<uint16_t>(), P.d_wstart.as<uint8_t>(),
                      P.d_windows.as<uint8_t>(), s);
-        k += 1 + (P.many ? 2 : 0) + (P.deep ? 2 : 0);
+        k += chain_launches(P);
     }
     if (timed) cudaEventRecord(ctx->ev[3], s);
     if (P.translate) {
@@ -765,6 +776,7 @@ int finish_run(pgz_ctx* ctx, Plan& P, pgz_stats* st) {
     uint64_t retries = 0, false_syncs = 0;
     const bool timed = st != nullptr;
     int status = PGZ_OK;
+    P.spent = false;
     for (;;) {
         int e = PGZ_OK;
         if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return PGZ_E_CUDA;
@@ -788,8 +800,9 @@ int finish_run(pgz_ctx* ctx, Plan& P, pgz_stats* st) {
             if (hf[f].bad_chunk != 0xffffffffu && retries < (uint64_t)kMaxRetries &&
                 recover(ctx, P, (int)f, res, &false_syncs)) {
                 again = true;
-            } else if (status == PGZ_OK) {
-                status = (int)hf[f].status;
+            } else {
+                P.spent |= hf[f].bad_chunk != 0xffffffffu && retries >= (uint64_t)kMaxRetries;
+                if (status == PGZ_OK) status = (int)hf[f].status;
             }
         }
         if (again) {
@@ -1408,12 +1421,14 @@ int pgz_decompress_host(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, uint8_
 
 // Decoding from bit lo (the first block's when at_start) to the member's end in several parts, each with its own block
 // start and symbolic context, the parts' windows then chained as symbols relative to the first part's context.  The
-// result becomes the one part of ctx->plan, as a run in one part leaves it.  Returns PGZ_OK, or anything else when the
-// caller shall run it in one part instead (too short, or an error: what to report is that run's to say).
+// result becomes the one part of ctx->plan, as a run in one part leaves it.  *settled: the status returned is the
+// call's (PGZ_OK, or an error that a run in one part would end with too, so that it is not decoded a second time);
+// else the caller runs it in one part (too short for several, no memory, or all re-runs used up).
 // The parts use the context's own plan and scratch, what pgz_decompress takes for the same bytes (windows of u16);
 // beside them only the symbols in order are kept.
 static int decompress_at_parts(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, const MemberInfo& mi, uint64_t lo,
-                               bool at_start, uint8_t* byte_out, uint8_t fill, uint64_t out_cap, uint64_t* last_ph) {
+                               bool at_start, uint8_t* byte_out, uint8_t fill, uint64_t out_cap, uint64_t* last_ph,
+                               bool* settled) {
     const uint64_t end_bit = (gz_len - 8) * 8;
     if (lo >= end_bit) return PGZ_E_NOSYNC;
     const uint64_t bits = end_bit - lo, csize = bits / 8 + 1;
@@ -1462,29 +1477,40 @@ static int decompress_at_parts(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len,
     }
     P.files.push_back(F);
     int e = execute(ctx, P, nullptr);
-    if (e) return e;
-    e = read_chunks(ctx, P);
-    if (e) return e;
+    const uint64_t total = P.files[0].total;
+    if (e == PGZ_E_CUDA || e == PGZ_E_NOMEM || P.spent || (e == PGZ_E_CAPACITY && total > kMaxPartSymbols)) return e;
+    if (e == PGZ_E_CAPACITY) {      // the length is known; the symbols, for inspection only, go to a buffer of that size
+        if (cuda_status(ctx->at_sym.ensure(total * sizeof(uint16_t)))) return PGZ_E_NOMEM;
+        P.at_sym = ctx->at_sym.as<uint16_t>();
+        P.at_bytes = nullptr;
+        FileDesc* hf = P.h_files.as<FileDesc>();
+        hf[0].status = PGZ_OK;
+        if (cudaMemcpyAsync(P.d_files.p, hf, sizeof(FileDesc), cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess)
+            return PGZ_E_CUDA;
+        ctx->launches += (uint64_t)enqueue_resolve(P, ctx->stream);
+        if (cudaPeekAtLastError() != cudaSuccess) return PGZ_E_CUDA;
+    }
+    if (read_chunks(ctx, P)) return PGZ_E_CUDA;
     const ChunkDesc* res = P.h_chunks.as<ChunkDesc>();
     uint64_t first = kNone;
-    for (uint64_t i = 0; i < n && first == kNone; ++i)
-        if (res[i].state == CS_DONE) first = res[i].sync;
-    if (first == kNone) return PGZ_E_NOSYNC;
+    for (uint64_t i = 0; i < n && first == kNone; ++i) first = res[i].sync;
+    if (first == kNone) e = PGZ_E_NOSYNC;
     uint64_t counts[2] = {0, 0};
     if (cudaMemcpyAsync(counts, P.d_at.p, sizeof counts, cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess ||
         cudaStreamSynchronize(ctx->stream) != cudaSuccess)
         return PGZ_E_CUDA;
+    const bool decoded = e == PGZ_OK || e == PGZ_E_CAPACITY;
     // the result as one part
     FileDesc RF = F;
     RF.nchunks = 1;
     RF.ngroups = 0;
-    RF.total = P.files[0].total;
-    RF.status = PGZ_OK;
+    RF.total = decoded ? total : 0;
+    RF.status = (uint32_t)e;
     RF.bad_chunk = 0xffffffffu;
     ChunkDesc C{};
     C.lo = lo;
     C.hi = end_bit;
-    C.cap = cap1;
+    C.cap = std::max(cap1, RF.total);
     C.index = at_start ? 0 : 1;
     C.stop_hint = kNone;
     C.sync = first;
@@ -1493,9 +1519,9 @@ static int decompress_at_parts(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len,
     C.last_ph = counts[1];
     C.det = kNone;
     C.end = end_bit;
-    C.state = CS_DONE;
-    C.final = 1;
-    C.confirmed = 1;
+    C.state = decoded ? CS_DONE : (first == kNone ? CS_EMPTY : CS_ERROR);
+    C.final = decoded;
+    C.confirmed = decoded;
     C.anyph = counts[0] != 0;
     begin_plan(P);
     P.files.push_back(RF);
@@ -1508,7 +1534,8 @@ static int decompress_at_parts(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len,
         return PGZ_E_CUDA;
     P.results_valid = true;
     *last_ph = counts[1];
-    return PGZ_OK;
+    *settled = true;
+    return e;
 }
 
 int pgz_decompress_at(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, uint64_t start_bit, uint16_t* sym_out,
@@ -1523,11 +1550,14 @@ int pgz_decompress_at(pgz_ctx* ctx, const uint8_t* gz, uint64_t gz_len, uint64_t
     const uint64_t s0_bit = mi.s0 * 8, end_bit = (gz_len - 8) * 8;
     {
         uint64_t last = 0;
+        bool settled = false;
         const bool first = start_bit <= s0_bit;
-        e = decompress_at_parts(ctx, gz, gz_len, mi, first ? s0_bit : start_bit, first, byte_out, fill, out_cap, &last);
-        if (e == PGZ_OK) {
+        e = decompress_at_parts(ctx, gz, gz_len, mi, first ? s0_bit : start_bit, first, byte_out, fill, out_cap, &last,
+                                &settled);
+        if (settled) {
             const ChunkDesc& C = ctx->plan.chunks[0];
             *out_len = C.n;
+            if (e) return e;
             if (block_bit) *block_bit = C.sync;
             if (first_determined) *first_determined = last;
             if (sym_out && C.n &&

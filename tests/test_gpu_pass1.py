@@ -173,6 +173,55 @@ def test_decoding_a_damaged_member_from_an_offset(chunk):
         ctx.close()
 
 
+@pytest.mark.parametrize("chunk", [16384, 65536])
+def test_errors_from_an_offset_are_decoded_once(chunk):
+    """A buffer too small, no block start, invalid data past the first start's window: each is reported by the run in
+    parts, with the launches of one run (and, for the length, its symbols put in order once more), and what the
+    inspection calls report is what a run in one part leaves."""
+    c = zlib.compressobj(6, zlib.DEFLATED, 31, 4)
+    text = synth.fastq(600_000, 150, 0.001, 8)
+    noise = np.random.default_rng(4).integers(0, 256, 300_000, dtype=np.uint8).tobytes()
+    gz = c.compress(text + noise) + c.flush()
+    _, _, blocks, _ = oracle.gunzip(gz, max_blocks=5000)
+    start = 8 * (len(gz) // 20)
+    after = [int(b) for b in blocks if b >= start]
+    quiet = 8 * (len(gz) - 200_000)
+    assert oracle.decompress_at(gz, quiet)["status"] == -13
+    bad = bytearray(gz)
+    for k in (1, 2):                                   # the 8th block from the start: past its window, in its part
+        bad[(after[7] + k) // 8] |= 1 << (after[7] + k) % 8
+    assert after[7] < start + 8 * chunk and oracle.decompress_at(bytes(bad), start)["status"] == -3
+    cap = len(text) + len(noise)
+    out = empty(cap)
+    ctx = Ctx(chunk_bytes=chunk)
+    try:
+        P = ctx.pgz
+        d, db = to_device(gz), to_device(bytes(bad))
+
+        def at(dev, bit, cap):
+            k = P.pgz_kernel_launches(ctx.h)
+            r = P.pgz_decompress_at(ctx.h, dev.data_ptr(), len(gz), bit, None, out.data_ptr(), ord("?"), cap)
+            return r[0], r[1], P.pgz_kernel_launches(ctx.h) - k
+
+        ref = oracle.decompress_at(gz, start, cap=cap)
+        st, n, once = at(d, start, cap)
+        assert (st, n) == (0, ref["sym"].size)
+        for small in (n - 1, 1000, 0):
+            st, k, launches = at(d, start, small)
+            assert (st, k) == (P.PGZ_E_CAPACITY, n) and launches < 2 * once
+            sb, ns, nph = P.pgz_inspect_parts(ctx.h)
+            assert list(sb) == [ref["block_bit"]] and list(ns) == [n]
+            assert list(nph) == [int((ref["sym"] >= 0x8000).sum())]
+            assert np.array_equal(P.pgz_inspect_symbols(ctx.h, 0), ref["sym"])
+        for dev, bit, want in ((d, quiet, P.PGZ_E_NOSYNC), (db, start, P.PGZ_E_DATA)):
+            st, k, launches = at(dev, bit, cap)
+            assert (st, k) == (want, 0) and launches <= once
+            sb, ns, nph = P.pgz_inspect_parts(ctx.h)
+            assert list(sb) == [(1 << 64) - 1] and list(ns) == [0] and list(nph) == [0]
+    finally:
+        ctx.close()
+
+
 def test_decoding_from_an_offset_shares_the_contexts_scratch():
     """After a file has been decoded, decoding it from an offset takes no more device memory than the symbols in order
     and the wider windows (32 KiB a part more), with a little room for the allocator's granularity."""
