@@ -314,15 +314,16 @@ typedef struct pgz_tune_entry {
 /* Autotuner.  The number of parts n is a free parameter of the method
    (Section "Full file decompression in two passes": n roughly equal parts);
    this picks the part size and the pass-1 CTA shape for the caller's data.
-   For every pair chunk_bytes[a] x warps_per_block[b] -- and, with
-   sweep_exec, both forms of pass-1 token execution -- it runs
+   For every pair chunk_bytes[a] x warps_per_block[b] it runs
    pgz_decompress_batch on the n_jobs jobs (device buffers, the batch rules;
    one job is one member) once untimed and reps times timed (CUDA events on the
    context's stream), and then sets the context's chunk_bytes, warps_per_block
    and exec_pipelined (n_chunks = 0) to the configuration with the smallest
    median time among those whose calls returned PGZ_OK for every job.
    entries: n_chunk_bytes * n_wpb * (sweep_exec ? 2 : 1) results, ordered by
-   chunk size, then CTA shape, then execution form (NULL: not returned);
+   chunk size, then CTA shape, then execution form (NULL: not returned; the
+   two forms run the same now, so a pair is timed once and sweep_exec lists it
+   under both; the choice is form 0);
    best: the chosen configuration (NULL: not returned).  The jobs' outputs and
    statuses are those of the last call.  Returns PGZ_E_ARG for empty lists,
    chunk sizes below 4 KiB, CTA shapes other than 2, 4 or 8 warps, or reps < 1;

@@ -173,6 +173,29 @@ def test_decoding_a_damaged_member_from_an_offset(chunk):
         ctx.close()
 
 
+def test_the_autotuner_runs_each_configuration_once():
+    """Both execution forms are one: asked for, they are listed with the one time measured, for the same launches."""
+    text = synth.fastq(300_000, 100, 0.001, 7)
+    gz = synth.gzip_compress(text, 6)
+    ctx = Ctx()
+    try:
+        P = ctx.pgz
+        d, out = to_device(gz), empty(len(text))
+        job = [(d.data_ptr(), len(gz), out.data_ptr(), len(text))]
+        launches = []
+        for sweep in (False, True):
+            k = P.pgz_kernel_launches(ctx.h)
+            st, entries, best = P.pgz_autotune(ctx.h, job, [16384, 65536], [4], 2, sweep_exec=sweep)
+            launches.append(P.pgz_kernel_launches(ctx.h) - k)
+            assert st == 0 and len(entries) == (4 if sweep else 2)
+        assert launches[0] == launches[1]
+        assert [e["exec_pipelined"] for e in entries] == [0, 1, 0, 1]
+        assert [e["ms"] for e in entries[::2]] == [e["ms"] for e in entries[1::2]]
+        assert best["ms"] == min(e["ms"] for e in entries)
+    finally:
+        ctx.close()
+
+
 @pytest.mark.parametrize("chunk", [16384, 65536])
 def test_errors_from_an_offset_are_decoded_once(chunk):
     """A buffer too small, no block start, invalid data past the first start's window: each is reported by the run in
