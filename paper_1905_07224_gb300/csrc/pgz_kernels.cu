@@ -118,17 +118,6 @@ struct TeamSmem {
     __device__ __forceinline__ uint16_t* kraft3() { return reinterpret_cast<uint16_t*>(bits + kBits + 2 - 256); }
 };
 
-template <int NW>
-__device__ __forceinline__ void team_sync() {
-    if (NW == 1) __syncwarp();
-    else __syncthreads();
-}
-template <int NW>
-__device__ __forceinline__ bool team_or(bool x) {
-    if (NW == 1) return __any_sync(FULL, x);
-    return __syncthreads_or(x);
-}
-
 __device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) {
     uint32_t lo = __shfl_sync(FULL, (uint32_t)v, src), hi = __shfl_sync(FULL, (uint32_t)(v >> 32), src);
     return ((uint64_t)hi << 32) | lo;
@@ -164,7 +153,7 @@ struct Input {
 template <int NW>
 __device__ void stage(TeamSmem<NW>& S, const Input& in, uint64_t w0, uint32_t n) {
     constexpr uint32_t T = 32 * NW;
-    team_sync<NW>();
+    __syncthreads();
     uint32_t i = threadIdx.x;
     if (w0 + n <= in.nfull) {
         for (; i + 7 * T < n; i += 8 * T) {
@@ -176,7 +165,7 @@ __device__ void stage(TeamSmem<NW>& S, const Input& in, uint64_t w0, uint32_t n)
         }
     }
     for (; i < n; i += T) S.bits[i] = in.word(w0 + i);
-    team_sync<NW>();
+    __syncthreads();
 }
 
 // a reader at bit p of the staged words: 32 bits from p on in x()
@@ -284,16 +273,16 @@ template <int NW>
 __device__ void build_tables(TeamSmem<NW>& S, uint32_t hlit, uint32_t hdist) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid < 32) S.cnt[tid >> 4][tid & 15] = 0;
-    team_sync<NW>();
+    __syncthreads();
     for (uint32_t s = tid; s < hlit + hdist; s += 32 * NW) {
         const uint32_t l = S.lens[s];
         if (l) atomicAdd(&S.cnt[s >= hlit][l], 1u);
     }
-    team_sync<NW>();
+    __syncthreads();
     if (warp == 0) sort_code(S.lens, (int)hlit, S.cnt[0], S.lim[0], S.sb[0], S.ent, 0, lit_entry, lane);
-    if (warp == (NW > 1 ? 1 : 0))
+    if (warp == 1)
         sort_code(S.lens + hlit, (int)hdist, S.cnt[1], S.lim[1], S.sb[1], S.ent, TeamSmem<NW>::kDistEnt, dist_entry, lane);
-    team_sync<NW>();
+    __syncthreads();
     for (uint32_t x = tid; x < (1u << LB); x += 32 * NW) {         // x: stream bits, the first least significant
         const uint32_t v = __brev(x) >> 17;                        // the same, left-aligned in 15 bits
         const uint32_t L = code_length<LB>(v, S.lim[0]);
@@ -316,7 +305,7 @@ __device__ void build_tables(TeamSmem<NW>& S, uint32_t hlit, uint32_t hdist) {
         const uint32_t L = code_length<DB>(v, S.lim[1]);
         S.tab[(1 << LB) + x] = L <= DB ? S.ent[(int32_t)(v >> (15 - L)) + S.sb[1][L]] : K_LONG << 9;
     }
-    team_sync<NW>();
+    __syncthreads();
 }
 
 // A dynamic block's header up to its code lengths, by one warp (RFC 1951
@@ -460,11 +449,11 @@ __device__ int read_dynamic(TeamSmem<NW>& S, uint32_t at, uint32_t* bits) {
             S.table_kind = 0;
         }
     }
-    team_sync<NW>();
+    __syncthreads();
     const int st = S.h_status;
     *bits = S.h_bits;
     if (st) {
-        team_sync<NW>();                       // S.h_* may be rewritten
+        __syncthreads();                       // S.h_* may be rewritten
         return st;
     }
     build_tables<NW>(S, S.h_hlit, S.h_hdist);
@@ -474,11 +463,11 @@ __device__ int read_dynamic(TeamSmem<NW>& S, uint32_t at, uint32_t* bits) {
 // the fixed code of RFC 1951 3.2.6
 template <int NW>
 __device__ void build_fixed(TeamSmem<NW>& S) {
-    team_sync<NW>();
+    __syncthreads();
     for (int s = threadIdx.x; s < 320; s += 32 * NW)
         S.lens[s] = (uint8_t)(s < 144 ? 8 : s < 256 ? 9 : s < 280 ? 7 : s < 288 ? 8 : 5);
     if (threadIdx.x == 0) S.table_kind = 1;
-    team_sync<NW>();
+    __syncthreads();
     build_tables<NW>(S, 288, 32);
 }
 
@@ -834,10 +823,10 @@ __device__ int par_block(TeamSmem<NW>& S, const Input& in, uint64_t s0, uint64_t
         LaneParse P{p0, 0, 0, PS_OK};
         uint32_t* tok = ts.tok + tl;
         const uint32_t cap = ts.cap * T;
-        team_sync<NW>();                               // the lists' place is free
+        __syncthreads();                               // the lists' place is free
         parse_own<NW>(S, P, tl, seg, tok, cap);
         S.r_cnt[tl] = (uint8_t)min((P.n / T + 1) / 2, TeamSmem<NW>::kList);
-        team_sync<NW>();
+        __syncthreads();
         uint32_t m, j;
         parse_on<NW>(S, P, P.st == PS_OK && tl + 1 < T, tl, seg, P.p - p0 - seg, tok, cap, m, j);
         const bool met = P.st == PS_SYNC;
@@ -846,7 +835,7 @@ __device__ int par_block(TeamSmem<NW>& S, const Input& in, uint64_t s0, uint64_t
         S.r_j[tl] = (uint16_t)(2 * j);
         const uint32_t exc = __ballot_sync(FULL, !met || m != tl + 1);
         if (lane == 0) S.r_exc[warp] = exc;
-        team_sync<NW>();
+        __syncthreads();
         // the path from lane 0 (uniform): runs of lanes that met the next one, up to a lane that met another or
         // nobody (the last)
         uint32_t path = 0, last = 0, pred = tl - 1;    // my warp's lanes on the path; mine's predecessor
@@ -885,7 +874,7 @@ __device__ int par_block(TeamSmem<NW>& S, const Input& in, uint64_t s0, uint64_t
             b.seek(S.bits, P.p);
             S.r_end = P.p + (P.st == PS_EOB ? symbol_entry<NW>(S, b.x(), 0) & 31u : 0u);
         }
-        team_sync<NW>();
+        __syncthreads();
         uint32_t before = 0, total = 0;
 #pragma unroll
         for (int v = 0; v < NW; ++v) {
@@ -901,7 +890,7 @@ __device__ int par_block(TeamSmem<NW>& S, const Input& in, uint64_t s0, uint64_t
         else if (o.n + total > o.cap) err = CE_OVERFLOW;
         if (err) {
             // a false candidate is told by its literals before it is given more room
-            if (team_or<NW>(err == CE_OVERFLOW && check && mine && !tokens_allowed<NW>(S, tok, skip, n)))
+            if (__syncthreads_or(err == CE_OVERFLOW && check && mine && !tokens_allowed<NW>(S, tok, skip, n)))
                 return CE_BYTE;
             return err;
         }
@@ -913,12 +902,12 @@ __device__ int par_block(TeamSmem<NW>& S, const Input& in, uint64_t s0, uint64_t
         uint32_t* sb = nw <= sizeof(S.list) / 4 ? reinterpret_cast<uint32_t*>(&S.list[0][0]) : nullptr;
         if (sb) {
             for (uint32_t k = tl; k < nw; k += T) sb[k] = 0;
-            team_sync<NW>();
+            __syncthreads();
         }
         const uint32_t to = mine ? n : skip, at = pos0 + before + incl - len;
         const bool ok = sb ? write_map<NW, true>(S, tok, skip, to, o.sym + map0, sb, at - map0, map0, check, neg)
                            : write_map<NW, false>(S, tok, skip, to, o.sym, o.start, at, 0, check, neg);
-        const bool bad = team_or<NW>(!ok);
+        const bool bad = __syncthreads_or(!ok);
         if (sb)
             for (uint32_t k = tl; k < nw; k += T) {
                 uint32_t* g = o.start + (map0 >> 5) + k;
@@ -927,7 +916,7 @@ __device__ int par_block(TeamSmem<NW>& S, const Input& in, uint64_t s0, uint64_t
             }
         o.neg |= neg;
         if (bad) return CE_BYTE;
-        if (o.known && team_or<NW>(neg)) return CE_DIST;
+        if (o.known && __syncthreads_or(neg)) return CE_DIST;
         o.n += total;
         block_n += total;
         if (round_end > end_bit) return CE_TRUNC;
@@ -968,7 +957,7 @@ __device__ int stored_block(const Input& in, uint64_t& pos, OutState& o, bool ch
         }
     }
     o.hi = max(o.hi, o.n + len);
-    if (team_or<NW>(bad)) return CE_BYTE;
+    if (__syncthreads_or(bad)) return CE_BYTE;
     o.n += len;
     block_n += len;
     pos = p + 32 + 8ull * len;
@@ -1019,9 +1008,9 @@ __device__ int one_block(TeamSmem<NW>& S, const Input& in, uint64_t& pos, TeamSt
                 const int t = trial_prefix<NW>(S, at);
                 if (threadIdx.x == 0) S.h_status = t;
             }
-            team_sync<NW>();
+            __syncthreads();
             st = S.h_status;
-            team_sync<NW>();
+            __syncthreads();
         }
         if (st == CE_OK)
             st = par_block<NW>(S, in, s0, candidate ? s0 : s1, pos, ts, o, check, max_block, end_bit, block_n);
@@ -1172,7 +1161,7 @@ __device__ void scan_step(TeamSmem<NW>& S, const Input& in, uint64_t next, uint6
     static_assert(kWords + 256 <= TeamSmem<NW>::kBits + 2, "a step's words are staged at once");
     const uint64_t T0 = next & ~1023ull;
     uint16_t* kraft3 = S.kraft3();
-    team_sync<NW>();
+    __syncthreads();
     for (uint32_t v = threadIdx.x; v < 512; v += 32 * NW)
         kraft3[v] = (uint16_t)(kraft1(v & 7) + kraft1((v >> 3) & 7) + kraft1(v >> 6));
     stage<NW>(S, in, T0 >> 5, kWords);
@@ -1240,7 +1229,7 @@ __device__ void scan_step(TeamSmem<NW>& S, const Input& in, uint64_t next, uint6
         S.c_done[warp] = at >= end_w;
         S.c_resume[warp] = at;
     }
-    team_sync<NW>();
+    __syncthreads();
 }
 
 template <int NW>
@@ -1257,9 +1246,9 @@ __device__ __forceinline__ TeamSmem<NW>& team_smem() {
 // counter is zero before the launch.
 template <int NW>
 __device__ __forceinline__ int next_part(TeamSmem<NW>& S, uint32_t* queue) {
-    team_sync<NW>();
+    __syncthreads();
     if (threadIdx.x == 0) S.q = (int)min(atomicAdd(queue, 1u), 0x7fffffffu);
-    team_sync<NW>();
+    __syncthreads();
     return S.q;
 }
 
@@ -1267,7 +1256,7 @@ template <int NW>
 __device__ __forceinline__ void init_smem(TeamSmem<NW>& S, const KParams& p) {
     if (threadIdx.x < 8) S.allowed[threadIdx.x] = p.allowed[threadIdx.x];
     if (threadIdx.x == 0) S.table_kind = 0;
-    team_sync<NW>();
+    __syncthreads();
 }
 
 // ---------------------------------------------------------------------------
@@ -1281,10 +1270,10 @@ __device__ __forceinline__ TeamState team_state(uint32_t* tok, const KParams& p,
 // the start bits of a block that failed
 template <int NW>
 __device__ void clear_starts(OutState& o) {
-    team_sync<NW>();
+    __syncthreads();
     for (uint64_t k = threadIdx.x; k < (o.hi + 31) / 32; k += 32 * NW) o.start[k] = 0;
     o.hi = 0;
-    team_sync<NW>();
+    __syncthreads();
 }
 
 // The block start of part c and its first block (Section "Detection of DEFLATE block start positions").
@@ -1347,10 +1336,10 @@ __device__ void sync_part(TeamSmem<NW>& S, const FileDesc& F, ChunkDesc& C, uint
                     break;
                 }
             }
-            team_sync<NW>();                     // S.c_* may be rewritten
+            __syncthreads();                     // S.c_* may be rewritten
         }
     }
-    const bool neg = team_or<NW>(o.neg);
+    const bool neg = __syncthreads_or(o.neg);
     if (threadIdx.x == 0) {
         C.err = err;
         C.sync = sync;
@@ -1386,7 +1375,7 @@ __device__ void inflate_part(TeamSmem<NW>& S, const FileDesc* __restrict__ files
     ChunkDesc& C = chunks[c];
     if (C.state != CS_FOUND) return;
     if (C.probe) {                    // a streamed segment's end: the block start found is all it gives
-        team_sync<NW>();
+        __syncthreads();
         if (threadIdx.x == 0) {
             C.state = CS_DONE;
             C.n = 0;
@@ -1457,7 +1446,7 @@ __device__ void inflate_part(TeamSmem<NW>& S, const FileDesc* __restrict__ files
             }
         }
     }
-    const bool neg = team_or<NW>(o.neg);
+    const bool neg = __syncthreads_or(o.neg);
     if (err == CE_OK && final && F.mode != 2 && !F.open_end) {   // the trailer must follow the final block
         if (((end + 7) >> 3) + 8 != F.gz_len) err = CE_TRAIL;
     }
@@ -2506,12 +2495,12 @@ static int pass1_resident_t() {
     if (!cached[slot]) {
         const int smem = (int)sizeof(TeamSmem<NW>);
         int sms = 0, per_sm_a = 0, per_sm_b = 0;
-        const bool ok =
-            cudaFuncSetAttribute(k_sync<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
-            cudaFuncSetAttribute(k_inflate<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
-            (NW != 16 ||
-             (cudaFuncSetAttribute(k_sync<NW, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
-              cudaFuncSetAttribute(k_inflate<NW, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess)) &&
+        auto raise = [smem](auto kernel) {
+            return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
+        };
+        bool ok = raise(k_sync<NW>) && raise(k_inflate<NW>);
+        if constexpr (NW == 16) ok = ok && raise(k_sync<NW, 1>) && raise(k_inflate<NW, 1>);
+        ok = ok &&
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_a, k_sync<NW>, 32 * NW, smem) == cudaSuccess &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_b, k_inflate<NW>, 32 * NW, smem) == cudaSuccess;
@@ -2570,8 +2559,10 @@ static void launch_pass1_t(bool sync, const FileDesc* files, ChunkDesc* chunks, 
     auto launch = [&](auto kernel) {
         kernel<<<grid, 32 * NW, sizeof(TeamSmem<NW>), s>>>(files, chunks, nchunks, sym, start, tok, queue, order, q);
     };
-    if (NW == 16 && nchunks <= pass1_resident(16) / 4) launch(sync ? k_sync<NW, 1> : k_inflate<NW, 1>);
-    else launch(sync ? k_sync<NW> : k_inflate<NW>);
+    if constexpr (NW == 16) {                    // the form with more registers (see pass1_min_blocks)
+        if (nchunks <= pass1_resident(16) / 4) return launch(sync ? k_sync<NW, 1> : k_inflate<NW, 1>);
+    }
+    launch(sync ? k_sync<NW> : k_inflate<NW>);
 }
 
 static void launch_pass1_any(bool sync, const FileDesc* files, ChunkDesc* chunks, int nchunks, uint16_t* sym,
