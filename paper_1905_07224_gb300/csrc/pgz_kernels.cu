@@ -1463,14 +1463,19 @@ __device__ void inflate_part(TeamSmem<NW>& S, const FileDesc* __restrict__ files
 }
 
 // Launch bounds of the pass-1 kernels, the blocks per SM that the registers are to allow (MB): with many parts what
-// shared memory holds, 12 teams of 2 warps and 7 of 4 (72 registers a thread; 64, for an eighth team that does not
+// shared memory holds, 11 teams of 2 warps (80 registers a thread) and 7 of 4 (72; 64, for an eighth team that does not
 // fit, spilled).  Larger teams are for few parts, where a part's own time counts: 3 of 8 warps (80 registers; at 4,
 // with 64, they spilled; files of 305 to 611 parts take the same time either way).  Teams of 16 have two forms: 2 per
 // SM (64 registers) and, where the parts fill at most half of the SMs, 1 per SM (128), k_sync + k_inflate: 1 MiB file
 // 433 -> 389 us, 64 KiB 161 -> 145, eight byte ranges 2380 -> 2130.
 // With 9 bits of distance lookup instead of 8 fewer steps take the rare branch: k_inflate of a 256 MiB file 1343 ->
 // 1251 us.
-constexpr int pass1_min_blocks(int nw) { return nw == 2 ? 12 : (nw == 4 ? 7 : (nw == 8 ? 3 : 2)); }
+constexpr int pass1_min_blocks(int nw) { return nw == 2 ? 11 : (nw == 4 ? 7 : (nw == 8 ? 3 : 2)); }
+
+// the teams that pass1_min_blocks counts on fit the 228 KiB of an SM (1 KiB of it reserved per block)
+template <int NW>
+constexpr bool team_fits() { return pass1_min_blocks(NW) * (sizeof(TeamSmem<NW>) + 1024) <= 228 * 1024; }
+static_assert(team_fits<2>() && team_fits<4>() && team_fits<8>() && team_fits<16>(), "more teams than shared memory holds");
 
 template <int NW, int MB = pass1_min_blocks(NW)>
 __global__ void __launch_bounds__(32 * NW, MB)
