@@ -67,6 +67,8 @@ PASS1_TRAFFIC_PER_OUT_BYTE = {
 # ... and the 512-member batch, by (part size, warps per block, pipelined execution, determined tail)
 # (profiles/pass1_traffic_batch512.md).  Other configurations report null.
 PASS1_TRAFFIC_PER_OUT_BYTE_BATCH512 = {
+    (524288, 2, 0, 0): (0.804282112e9 + 0.858065152e9 + 17.787428864e9 + 19.834282496e9 + 9.496816384e9
+                        + 8.871113728e9) / 4467581835,
     (262144, 2, 0, 0): (1.588861440e9 + 1.700140544e9 + 17.259778304e9 + 19.536223744e9 + 9.498650880e9
                         + 8.871193600e9) / 4467581835,
 }

@@ -76,8 +76,8 @@ typedef struct pgz_config {
     uint64_t spin_cap;          /* reserved for bounded device waits; 0 = default */
     int warps_per_block;        /* CTA shape of the pass-1 kernels: 2, 4 or 8 warps, together on one part; 0 = 4.
                                    A run with few parts takes larger CTAs by itself */
-    int exec_pipelined;         /* 0 (default) or 1; accepted, kept and swept as before, but pass 1 has one
-                                   execution form now and runs the same either way */
+    int exec_pipelined;         /* 0 (default) or 1; accepted and kept, but pass 1 has one execution form now and
+                                   runs the same either way */
     int determined_tail;        /* 1: once a part's last 32 KiB of output hold no placeholder (none can
                                    follow), pass 1 stores the rest of the part as bytes and the translation
                                    copies them; 0: u16 symbols throughout (default).  The output is the same

@@ -58,7 +58,7 @@ struct FileDesc {
     int32_t chunk0, nchunks;
     int32_t group0, ngroups;   // window-chain groups of consecutive parts
     int32_t super0, nsupers;   // groups of consecutive groups
-    uint64_t seg0, nseg;   // 4 KiB CRC segments of the output
+    uint64_t seg0, nseg;   // CRC segments of crc_segment_bytes() of the output
     uint32_t mode;         // 0 whole member; 1 from a bit offset (no CRC/ISIZE); 2 byte range of the output;
                            // 3 one segment of a streamed member (bit positions relative to the segment's bytes)
     uint32_t open_end;     // mode 0: more members may follow; the member ends after its final block, and its

@@ -595,7 +595,8 @@ __device__ __forceinline__ void or_shared_if(bool on, uint32_t a, uint32_t v) {
 // The token at P.p of a lane with `go` (two literals at once if PAIRS), kept in tok[P.n]; go becomes false at a
 // symbol that ends the parse (P.p stays at it; P.st says why).  One step for a literal, a match, or two literals, and
 // no branch but one for the rare entries: a step's time is the chain of its three shared-memory reads (the words, the
-// first entry, the distance's), about 250 cycles, against 650 with a branch for every kind.
+// first entry, the distance's).  Against a branch for every kind, search and decoding of a 1 MiB file took 443 us for
+// 493, of a 256 MiB file 2086 for 2120.
 template <int NW, bool PAIRS>
 __device__ __forceinline__ void next_token(const TeamSmem<NW>& S, LaneParse& P, bool& go, uint32_t* tok) {
     const uint32_t* w = S.bits + (P.p >> 5);
@@ -1519,8 +1520,8 @@ __global__ void __launch_bounds__(32 * NW, MB)
 // earlier source or to its symbol, and indices strictly decrease, so the chase
 // needs no further barrier and ends, overlapping copies included.  The pass's
 // symbols then go to the ring, whose places they take are no longer read.
-// Bound: instruction issue (about 25 instructions a position for the entry, 6 more per chase step; 2.8 steps a
-// pass on level-1 FASTQ).  0.74 ms for the 1024 parts of a 256 MiB file (364 G symbols/s); 1.05 ms with a branch per
+// Bound: instruction issue (0.60 G warp instructions, all but a few with 32 threads, for the 509 M symbols of 64
+// members: about 37 a position).  0.74 ms for the 1024 parts of a 256 MiB file (364 G symbols/s); 1.05 ms with a branch per
 // position and entry in the chase, whose loads then wait for one another.
 constexpr uint32_t kPtr = 0x4000u;    // neither a byte nor a placeholder; the index takes 14 bits
 

@@ -303,7 +303,8 @@ class Batch:
 
 def pgz_autotune(ctx: int, jobs, chunk_bytes, warps_per_block, reps: int = 3, sweep_exec: bool = False):
     """(status, [entry dicts], best dict); jobs: list of (gz_ptr, gz_len, out_ptr, out_cap) device addresses;
-    sets the context's part size, CTA shape (and, with sweep_exec, the pass-1 execution form)."""
+    sets the context's part size and CTA shape (sweep_exec lists each pair under both execution forms, which run
+    the same)."""
     arr = _jobs(jobs)
     cb = (U64 * len(chunk_bytes))(*chunk_bytes)
     wp = (ctypes.c_int * len(warps_per_block))(*warps_per_block)

@@ -1,8 +1,8 @@
 """A persistent cache of autotuner choices, keyed by (GPU, compression level, size bucket).
 
-pgz_autotune times part sizes x pass-1 CTA shapes x execution forms on the
-caller's data, which costs a few hundred decompressions.  The best choice
-depends on the GPU, on how the data was compressed, and on its size, so a
+pgz_autotune times part sizes x pass-1 CTA shapes on the caller's data (with
+sweep_exec it lists each under both execution forms, which run the same),
+which costs up to a few hundred decompressions.  The best choice depends on the GPU, on how the data was compressed, and on its size, so a
 choice made once is kept in a JSON file and applied to later contexts with
 pgz_set_tuning, with no timing.
 
